@@ -11,8 +11,9 @@
 // of c is the set of pos(c_m) whose translate reproduces c, which gives
 // |Stab| and the compatibility test e^{ik.t} = 1 on it (N_{a,k} > 0 in
 // Alg. 5).  The representatives are sorted by rank (CUB radix sort, a
-// library primitive) and indexed by a prefix table over their two largest
-// sites.
+// library primitive) once for all sectors; each sector takes the compatible
+// ones in order.  The rows of every sector are indexed by their largest sites
+// and buckets of the rank of the others (SecView::pinfo).
 #include <cub/cub.cuh>
 
 #include <algorithm>
@@ -112,9 +113,9 @@ size_t row_kernel_smem(const Basis &B, int /*extra_nd*/) {
 // orbit is taken once, from its designated member, with |Stab| (the moves
 // that give the candidate back) and the compatibility of those moves with K.
 template <int ND>
-__global__ void __launch_bounds__(NTHREADS) k_enum_reps(LatView L, int Kx, int Ky, int Kz, int s0, uint64_t ncand,
-                                                        int emit, unsigned long long *counter,
-                                                        uint64_t *out_rank, uint8_t *out_stab) {
+__global__ void __launch_bounds__(NTHREADS) k_enum_reps(LatView L, int s0, uint64_t ncand, uint64_t cap,
+                                                        unsigned long long *counter, uint64_t *out_rank,
+                                                        uint8_t *out_stab) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *sC = (uint64_t *)smem;
     uint32_t *sxyz = (uint32_t *)(sC + (L.nd + 3) * L.np1);
@@ -123,7 +124,7 @@ __global__ void __launch_bounds__(NTHREADS) k_enum_reps(LatView L, int Kx, int K
     for (int i = threadIdx.x; i < L.N; i += blockDim.x) sxyz[i] = L.xyz[i];
     __syncthreads();
     const int Lx = L.L[0], Ly = L.L[1], Lz = L.L[2];
-    const int G = L.ncell, ns = L.nsub, w = ns - s0;
+    const int ns = L.nsub, w = ns - s0;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t base = (uint64_t)blockIdx.x * blockDim.x; base < ncand; base += stride) {
         const uint64_t j = base + threadIdx.x;
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(NTHREADS) k_enum_reps(LatView L, int Kx, int K
                 Z[m] = p >> 22;
                 SB[m] = ns > 1 ? c[m] % ns : 0;
             }
-            bool designated = true, compat = true;
+            bool designated = true;
 #pragma unroll
             for (int m = 0; m < ND; ++m) {
                 if (SB[m] != s0) continue;
@@ -168,16 +169,10 @@ __global__ void __launch_bounds__(NTHREADS) k_enum_reps(LatView L, int Kx, int K
                 sort_net(sl);
                 const uint64_t rm = rank_of(sl, sC, L.np1);
                 designated &= (rm >= rc);
-                if (rm == rc) {
-                    ++st;
-                    // stabiliser element t = cell(c_m): compatible iff k.t is a multiple of 2 pi
-                    long long num = (long long)Kx * X[m] * (G / Lx) + (long long)Ky * Y[m] * (G / Ly) +
-                                    (long long)Kz * Z[m] * (G / Lz);
-                    compat &= (num % G) == 0;
-                }
+                st += rm == rc;
             }
-            take = designated && compat;
-            if (take && emit) {
+            take = designated;
+            if (take) {
                 int rep[ND];
                 int ax, by, cz;
                 rep_rank = canon(c, L, sxyz, sC, rep, ax, by, cz);
@@ -189,141 +184,424 @@ __global__ void __launch_bounds__(NTHREADS) k_enum_reps(LatView L, int Kx, int K
         unsigned long long basepos = 0;
         if (lane == 0 && mask) basepos = atomicAdd(counter, (unsigned long long)__popc(mask));
         basepos = __shfl_sync(0xffffffffu, basepos, 0);
-        if (take && emit) {
-            const unsigned long long pos = basepos + __popc(mask & ((1u << lane) - 1u));
+        const unsigned long long pos = basepos + __popc(mask & ((1u << lane) - 1u));
+        if (take && pos < cap) {
             out_rank[pos] = rep_rank;
             out_stab[pos] = (uint8_t)st;
         }
     }
 }
 
-template <int ND>
-__global__ void k_prefix(LatView L, const uint64_t *__restrict__ sigma, uint64_t d, uint32_t *__restrict__ P) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t *sC = (uint64_t *)smem;
-    const int nC = (L.nd + 3) * L.np1;
-    for (int i = threadIdx.x; i < nC; i += blockDim.x) sC[i] = L.binom[i];
-    __syncthreads();
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (uint64_t)gridDim.x * blockDim.x) {
-        int c[ND];
-        unrank(sigma[i], sC, L.np1, c);
-        P[i] = prefix_of(c, sC, L.np1);
-    }
-}
-
-// pidx[p] = first i with P[i] >= p, for p in [0, np]
-__global__ void k_pidx(const uint32_t *__restrict__ P, uint64_t d, uint32_t np, uint32_t *__restrict__ pidx) {
-    for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p <= np; p += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t lo = 0, hi = d;
-        while (lo < hi) {
-            uint64_t mid = (lo + hi) >> 1;
-            if (P[mid] < p) lo = mid + 1; else hi = mid;
+// The orbits of the N_down-subsets under the translations, by Burnside's
+// lemma: a translation of order o moves the sites in cycles of o and fixes
+// C(N / o, N_down / o) subsets when o divides N_down, none otherwise.
+static uint64_t count_orbits(const Basis &B, const std::vector<uint64_t> &binom) {
+    auto gcd = [](int a, int b) {
+        while (b) {
+            const int t = a % b;
+            a = b;
+            b = t;
         }
-        pidx[p] = (uint32_t)lo;
-    }
+        return a;
+    };
+    auto order = [&](int L, int t) { return L / gcd(L, t); };
+    unsigned __int128 sum = 0;
+    for (int z = 0; z < B.L[2]; ++z)
+        for (int y = 0; y < B.L[1]; ++y)
+            for (int x = 0; x < B.L[0]; ++x) {
+                int o = order(B.L[0], x);
+                for (int q : {order(B.L[1], y), order(B.L[2], z)}) o = o / gcd(o, q) * q;
+                if (B.nd % o == 0) sum += binom[(size_t)(B.nd / o) * (B.N + 1) + B.N / o];
+            }
+    return (uint64_t)(sum / (unsigned)B.ncell);
 }
 
-// the representatives of momentum K (each orbit once, compatible ones only),
-// sorted by rank0, with |Stab|: d of them in kout / vout
+// the representatives of all orbits, sorted by rank0, with |Stab|: n of them
 template <int ND>
-static int enum_sorted_reps(Basis &B, const int *K, DevBuf &kout, DevBuf &vout, uint64_t &d,
-                            std::vector<uint64_t> &hb, int &nsm) {
-    // per lowest occupied place s0 of the cell: C(M - 1, ND - 1) candidates,
-    // M = (cells) (nsub - s0); one spin per cell: C(N - 1, ND - 1)
-    hb.resize((size_t)(B.nd + 3) * (B.N + 1));
-    QS3_CUDA(cudaMemcpy(hb.data(), B.d_binom.p, hb.size() * sizeof(uint64_t), cudaMemcpyDeviceToHost));
+static int enum_orbits(Basis &B, DevBuf &kout, DevBuf &vout, uint64_t &n) {
+    const std::vector<uint64_t> &hb = B.binom;
     const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8 + (size_t)B.N * 4;
     QS3_CUDA(cudaFuncSetAttribute(k_enum_reps<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-    DevBuf cnt;
-    QS3_TRY(cnt.alloc(sizeof(unsigned long long)));
-    QS3_CUDA(cudaMemset(cnt.p, 0, sizeof(unsigned long long)));
-    int dev = 0;
+    int dev = 0, nsm = 0;
     QS3_CUDA(cudaGetDevice(&dev));
     QS3_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    std::vector<uint64_t> nc(B.nsub, 0);
+    n = count_orbits(B, hb);
+    DevBuf cnt, kin, vin;
+    QS3_TRY(cnt.alloc(sizeof(unsigned long long)));
+    QS3_CUDA(cudaMemset(cnt.p, 0, sizeof(unsigned long long)));
+    QS3_TRY(kin.alloc(n * 8));
+    QS3_TRY(vin.alloc(n));
+    // per lowest occupied place s0 of the cell: C(M - 1, ND - 1) candidates,
+    // M = (cells) (nsub - s0); one spin per cell: C(N - 1, ND - 1)
     for (int s0 = 0; s0 < B.nsub; ++s0) {
         const uint64_t M = (uint64_t)B.ncell * (B.nsub - s0);
-        nc[s0] = (M >= 1 && M - 1 >= (uint64_t)(ND - 1)) ? hb[(size_t)(ND - 1) * (B.N + 1) + (M - 1)] : 0;
-    }
-    auto run = [&](int emit, uint64_t *kp, uint8_t *vp) -> int {
-        for (int s0 = 0; s0 < B.nsub; ++s0) {
-            if (!nc[s0]) continue;
-            const uint64_t want = (nc[s0] + NTHREADS - 1) / NTHREADS;
-            const int grid = (int)std::min<uint64_t>(want ? want : 1, (uint64_t)nsm * 8);
-            k_enum_reps<ND><<<grid, NTHREADS, smem>>>(B.lv, K[0], K[1], K[2], s0, nc[s0], emit,
-                                                      cnt.as<unsigned long long>(), kp, vp);
-            QS3_LAUNCHED();
-        }
-        return QS3_OK;
-    };
-    QS3_TRY(run(0, nullptr, nullptr));
-    d = 0;
-    QS3_CUDA(cudaMemcpy(&d, cnt.p, sizeof(d), cudaMemcpyDeviceToHost));
-    if (d >= (1ull << 32)) return set_err(QS3_ERR_OVERFLOW, "sector dimension %llu exceeds 2^32", (unsigned long long)d);
-    DevBuf kin, vin;
-    QS3_TRY(kin.alloc(d * 8));
-    QS3_TRY(vin.alloc(d));
-    QS3_CUDA(cudaMemset(cnt.p, 0, sizeof(unsigned long long)));
-    QS3_TRY(run(1, kin.as<uint64_t>(), vin.as<uint8_t>()));
-    QS3_TRY(kout.alloc(d * 8));
-    QS3_TRY(vout.alloc(d));
-    if (d > 0) {
-        size_t tb = 0;
-        QS3_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb, kin.as<unsigned long long>(),
-                                                 kout.as<unsigned long long>(), vin.as<uint8_t>(),
-                                                 vout.as<uint8_t>(), (int64_t)d));
-        DevBuf tmp;
-        QS3_TRY(tmp.alloc(tb));
-        QS3_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tb, kin.as<unsigned long long>(),
-                                                 kout.as<unsigned long long>(), vin.as<uint8_t>(),
-                                                 vout.as<uint8_t>(), (int64_t)d));
-    }
-    return QS3_OK;
-}
-
-template <int ND>
-static int build_reps_nd(Basis &B, int s) {
-    const int *K = &B.K[3 * s];
-    std::vector<uint64_t> hb;
-    int nsm = 0;
-    uint64_t d = 0;
-    DevBuf kout, vout;
-    QS3_TRY(enum_sorted_reps<ND>(B, K, kout, vout, d, hb, nsm));
-    // prefix index
-    const uint32_t np = (ND >= 2) ? (uint32_t)hb[2 * (size_t)(B.N + 1) + B.N] : (uint32_t)B.N;   // number of prefixes
-    DevBuf P, pidx;
-    QS3_TRY(P.alloc(d * 4));
-    QS3_TRY(pidx.alloc(((size_t)np + 1) * 4));
-    if (d > 0) {
-        const size_t sm2 = (size_t)(B.nd + 3) * (B.N + 1) * 8;
-        QS3_CUDA(cudaFuncSetAttribute(k_prefix<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-        int g2 = (int)std::min<uint64_t>((d + 255) / 256, (uint64_t)nsm * 8);
-        k_prefix<ND><<<g2, 256, sm2>>>(B.lv, kout.as<uint64_t>(), d, P.as<uint32_t>());
+        const uint64_t nc = (M >= 1 && M - 1 >= (uint64_t)(ND - 1)) ? hb[(size_t)(ND - 1) * (B.N + 1) + (M - 1)] : 0;
+        if (!nc) continue;
+        const int grid = (int)std::min<uint64_t>((nc + NTHREADS - 1) / NTHREADS, (uint64_t)nsm * 8);
+        k_enum_reps<ND><<<grid, NTHREADS, smem>>>(B.lv, s0, nc, n, cnt.as<unsigned long long>(), kin.as<uint64_t>(),
+                                                  vin.as<uint8_t>());
         QS3_LAUNCHED();
     }
-    int g3 = (int)std::min<uint64_t>((np + 256) / 256, (uint64_t)nsm * 8);
-    k_pidx<<<g3, 256>>>(P.as<uint32_t>(), d, np, pidx.as<uint32_t>());
-    QS3_LAUNCHED();
-    QS3_CUDA(cudaDeviceSynchronize());
-    B.dims[s] = d;
-    B.d_sigma[s] = std::move(kout);
-    B.d_stab[s] = std::move(vout);
-    B.d_pidx[s] = std::move(pidx);
+    QS3_TRY(kout.alloc(n * 8));
+    QS3_TRY(vout.alloc(n));
+    // ranks are below C(N, N_down): only those bits are sorted
+    int bits = 1;
+    while (bits < 64 && (hb[(size_t)ND * (B.N + 1) + B.N] >> bits)) ++bits;
+    size_t tb = 0;
+    QS3_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb, kin.as<unsigned long long>(), kout.as<unsigned long long>(),
+                                             vin.as<uint8_t>(), vout.as<uint8_t>(), (int64_t)n, 0, bits));
+    DevBuf tmp;
+    QS3_TRY(tmp.alloc(tb));
+    QS3_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tb, kin.as<unsigned long long>(), kout.as<unsigned long long>(),
+                                             vin.as<uint8_t>(), vout.as<uint8_t>(), (int64_t)n, 0, bits));
+    uint64_t got = 0;
+    QS3_CUDA(cudaMemcpy(&got, cnt.p, sizeof(got), cudaMemcpyDeviceToHost));
+    if (got != n)
+        return set_err(QS3_ERR_CUDA, "enumerated %llu orbits, %llu expected", (unsigned long long)got,
+                       (unsigned long long)n);
     return QS3_OK;
 }
 
-int build_sector_reps(Basis &B, int s) {
-    switch (B.nd) {
-        case 1: return build_reps_nd<1>(B, s);
-        case 2: return build_reps_nd<2>(B, s);
-        case 3: return build_reps_nd<3>(B, s);
-        case 4: return build_reps_nd<4>(B, s);
-        case 5: return build_reps_nd<5>(B, s);
-        case 6: return build_reps_nd<6>(B, s);
-        case 7: return build_reps_nd<7>(B, s);
-        case 8: return build_reps_nd<8>(B, s);
-        default: return set_err(QS3_ERR_INVALID_ARG, "n_down %d", B.nd);
+// flag[i n + g] = 1 when orbit g belongs to the sector of momentum K[i], i <
+// ns: e^{ik.t} = 1 on its stabiliser (N_{a,k} > 0 in Alg. 5).  An orbit with
+// a trivial stabiliser belongs to every sector; the others' stabilisers are
+// among the moves of one spin onto the spins of its place in the cell.
+template <int ND>
+__global__ void __launch_bounds__(NTHREADS) k_members(LatView L, const uint64_t *__restrict__ reps,
+                                                      const uint8_t *__restrict__ stab, uint64_t n, int ns,
+                                                      const int *__restrict__ K, uint32_t *__restrict__ flag) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t *sC = (uint64_t *)smem;
+    uint32_t *sxyz = (uint32_t *)(sC + (L.nd + 3) * L.np1);
+    stage_tables(L, sC, sxyz);
+    __syncthreads();
+    const int Lx = L.L[0], Ly = L.L[1], Lz = L.L[2], G = L.ncell;
+    for (uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (uint64_t)gridDim.x * blockDim.x) {
+        if (__ldg(stab + g) == 1) {
+            for (int i = 0; i < ns; ++i) flag[(uint64_t)i * n + g] = 1u;
+            continue;
+        }
+        int c[ND], X[ND], Y[ND], Z[ND], SB[ND];
+        unrank(__ldg(reps + g), sC, L.np1, c);
+#pragma unroll
+        for (int m = 0; m < ND; ++m) {
+            const uint32_t p = sxyz[c[m]];
+            X[m] = p & 2047u;
+            Y[m] = (p >> 11) & 2047u;
+            Z[m] = p >> 22;
+            SB[m] = L.nsub > 1 ? c[m] % L.nsub : 0;
+        }
+        // the stabiliser's translations, bit m: the move of spin m onto spin 0
+        uint32_t fix = 0;
+#pragma unroll
+        for (int m = 1; m < ND; ++m) {
+            int sl[ND];
+            bool same = SB[m] == SB[0];
+#pragma unroll
+            for (int q = 0; q < ND; ++q) {
+                int x = X[q] + X[0] - X[m], y = Y[q] + Y[0] - Y[m], z = Z[q] + Z[0] - Z[m];
+                x += x < 0 ? Lx : 0; x -= x >= Lx ? Lx : 0;
+                y += y < 0 ? Ly : 0; y -= y >= Ly ? Ly : 0;
+                z += z < 0 ? Lz : 0; z -= z >= Lz ? Lz : 0;
+                sl[q] = SB[q] + L.nsub * (x + Lx * (y + Ly * z));
+            }
+            sort_net(sl);
+#pragma unroll
+            for (int q = 0; q < ND; ++q) same &= sl[q] == c[q];
+            fix |= same ? 1u << m : 0u;
+        }
+        for (int i = 0; i < ns; ++i) {
+            const long long Kx = K[3 * i], Ky = K[3 * i + 1], Kz = K[3 * i + 2];
+            bool ok = true;
+#pragma unroll
+            for (int m = 1; m < ND; ++m) {
+                const long long num = Kx * (X[m] - X[0]) * (G / Lx) + Ky * (Y[m] - Y[0]) * (G / Ly) +
+                                      Kz * (Z[m] - Z[0]) * (G / Lz);
+                ok &= !((fix >> m) & 1u) || num % G == 0;
+            }
+            flag[(uint64_t)i * n + g] = ok ? 1u : 0u;
+        }
     }
+}
+
+__global__ void k_ends(const uint32_t *__restrict__ pos, uint64_t n, int cnt, uint32_t *__restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < cnt) out[i] = pos[(uint64_t)i * n];
+}
+
+// rows of ns sectors from the scanned flags (pos: ns n + 1 entries): the
+// representatives and |Stab| of the members, one sector after another
+__global__ void k_take(const uint32_t *__restrict__ pos, const uint64_t *__restrict__ reps,
+                       const uint8_t *__restrict__ stab, uint64_t n, uint64_t cnt, uint64_t *__restrict__ sigma,
+                       uint8_t *__restrict__ sst) {
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint32_t p = pos[i];
+        if (pos[i + 1] == p) continue;
+        const uint64_t g = i % n;
+        sigma[p] = reps[g];
+        sst[p] = stab[g];
+    }
+}
+
+// the largest x with C(x, 2) <= P
+__device__ __forceinline__ int tri_root(uint32_t P) {
+    int x = (int)(0.5f + sqrtf(0.25f + 2.0f * (float)P));
+    while ((uint64_t)x * (x - 1) / 2 > P) --x;
+    while ((uint64_t)x * (x + 1) / 2 <= P) ++x;
+    return x;
+}
+
+// the buckets of prefix P (SecView::pinfo) when it has so many rows: nq of
+// them, 2^shift low ranks each, at most half as many as rows
+__device__ __forceinline__ int bucket_shift(uint32_t P, uint32_t rows, int nd, int pre2,
+                                            const uint64_t *__restrict__ binom, int np1, uint32_t &nq) {
+    uint64_t w;                            // low ranks
+    if (pre2) {
+        const int x = tri_root(P);
+        w = binom[(size_t)(nd - 2) * np1 + (P - (uint64_t)x * (x - 1) / 2)];
+    } else {
+        w = binom[(size_t)(nd - 1) * np1 + P];
+    }
+    const uint32_t most = rows / 2 > 1 ? rows / 2 : 1;
+    int sh = 0;
+    while (w && ((w - 1) >> sh) + 1 > most) ++sh;
+    nq = w ? (uint32_t)(((w - 1) >> sh) + 1) : 1u;
+    return sh;
+}
+
+// per sector s and prefix P: the first row with a prefix >= P, by a binary
+// search over the sector's rows (first[s (np + 1) + P], P <= np)
+__global__ void k_first(int nd, int np1, int pre2, const SecView *__restrict__ secs, int S, uint32_t np,
+                        const uint64_t *__restrict__ binom, uint32_t *__restrict__ first) {
+    const uint64_t cnt = (uint64_t)S * (np + 1);
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
+        const int s = (int)(i / (np + 1));
+        const uint32_t P = (uint32_t)(i - (uint64_t)s * (np + 1));
+        const uint64_t *sig = secs[s].sigma;
+        uint64_t lo = 0, hi = secs[s].dim;
+        if (P == np) {
+            lo = hi;
+        } else {
+            // the smallest rank with prefix P
+            uint64_t r;
+            if (pre2) {
+                const int x = tri_root(P);
+                r = binom[(size_t)nd * np1 + x] + binom[(size_t)(nd - 1) * np1 + (P - (uint64_t)x * (x - 1) / 2)];
+            } else {
+                r = binom[(size_t)nd * np1 + P];
+            }
+            while (lo < hi) {
+                const uint64_t mid = (lo + hi) >> 1;
+                if (sig[mid] < r) lo = mid + 1; else hi = mid;
+            }
+        }
+        first[i] = (uint32_t)lo;
+    }
+}
+
+// entries of every (sector, prefix): its buckets plus the end
+__global__ void k_bucket_size(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
+                              const uint32_t *__restrict__ first, uint32_t *__restrict__ size) {
+    const uint64_t cnt = (uint64_t)S * np;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t s = i / np;
+        const uint32_t P = (uint32_t)(i - s * np);
+        const uint32_t *f = first + s * (np + 1) + P;
+        uint32_t nq;
+        bucket_shift(P, f[1] - f[0], nd, pre2, binom, np1, nq);
+        size[i] = nq + 1;
+    }
+}
+__global__ void k_bucket_info(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
+                              const uint32_t *__restrict__ first, const uint32_t *__restrict__ off,
+                              uint2 *__restrict__ pinfo, uint32_t *__restrict__ sub) {
+    const uint64_t cnt = (uint64_t)S * np;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t s = i / np;
+        const uint32_t P = (uint32_t)(i - s * np);
+        const uint32_t *f = first + s * (np + 1) + P;
+        uint32_t nq;
+        const int sh = bucket_shift(P, f[1] - f[0], nd, pre2, binom, np1, nq);
+        pinfo[i] = make_uint2(off[i], (uint32_t)sh);
+        // an empty prefix: one empty bucket
+        if (f[0] == f[1])
+            for (uint32_t q = 0; q <= nq; ++q) sub[(uint64_t)off[i] + q] = f[0];
+    }
+}
+
+// the entries of each prefix from its rows: row i writes the buckets that
+// start at it (those after its predecessor's up to its own), the last row of
+// a prefix also the ones after
+template <int ND>
+__global__ void __launch_bounds__(NTHREADS) k_bucket_fill(LatView L, const SecView *__restrict__ secs,
+                                                          const int *__restrict__ tile0, int S, int ntiles, uint32_t np,
+                                                          const uint32_t *__restrict__ first,
+                                                          const uint2 *__restrict__ pinfo, uint32_t *__restrict__ sub) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t *sC = (uint64_t *)smem;
+    stage_tables(L, sC, nullptr);
+    __syncthreads();
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const int s = S == 1 ? 0 : sector_of_tile(tile0, S, t);
+        const uint64_t row = (uint64_t)(t - secs[s].tile0) * TILE + threadIdx.x;
+        if (row >= secs[s].dim) continue;
+        const uint64_t *sig = secs[s].sigma;
+        int c[ND];
+        unrank(sig[row], sC, L.np1, c);
+        uint64_t low;
+        const uint32_t P = prefix_of(c, sC, L.np1, secs[s].pre2, low);
+        const uint32_t *f = first + (uint64_t)s * (np + 1) + P;
+        const uint2 pi = pinfo[(uint64_t)s * np + P];
+        uint32_t *e = sub + pi.x;
+        const uint32_t q = (uint32_t)(low >> pi.y);
+        uint32_t q0 = 0;
+        if (row > f[0]) q0 = (uint32_t)((low - (sig[row] - sig[row - 1])) >> pi.y) + 1;
+        for (uint32_t k = q0; k <= q; ++k) e[k] = (uint32_t)row;
+        if (row + 1 == f[1]) {
+            uint32_t nq;
+            bucket_shift(P, f[1] - f[0], L.nd, secs[s].pre2, L.binom, L.np1, nq);
+            for (uint32_t k = q + 1; k <= nq; ++k) e[k] = (uint32_t)(row + 1);
+        }
+    }
+}
+
+// The sectors of a k-sector basis: the orbits are enumerated and sorted once,
+// and each sector takes the compatible ones in order (a flag per orbit and
+// sector, scanned), as many sectors at a time as 2^27 flags hold.  keep_reps
+// / keep_stab receive the orbits' list for the representative table.
+template <int ND>
+static int build_sectors_nd(Basis &B, DevBuf &keep_reps, DevBuf &keep_stab, uint64_t &n) {
+    QS3_TRY(enum_orbits<ND>(B, keep_reps, keep_stab, n));
+    const int S = B.S;
+    const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8 + (size_t)B.N * 4;
+    QS3_CUDA(cudaFuncSetAttribute(k_members<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+    if (S == 1 && B.K[0] == 0 && B.K[1] == 0 && B.K[2] == 0) {
+        // every orbit; the table's copy is made when there may be one
+        B.dims[0] = n;
+        if (n < (1ull << 20)) {
+            QS3_TRY(B.d_sigma.alloc(n * 8));
+            QS3_TRY(B.d_stab.alloc(n));
+            QS3_CUDA(cudaMemcpy(B.d_sigma.p, keep_reps.p, n * 8, cudaMemcpyDeviceToDevice));
+            QS3_CUDA(cudaMemcpy(B.d_stab.p, keep_stab.p, n, cudaMemcpyDeviceToDevice));
+        } else {
+            B.d_sigma = std::move(keep_reps);
+            B.d_stab = std::move(keep_stab);
+        }
+    } else {
+        QS3_TRY(B.d_sigma.alloc((uint64_t)S * n * 8));
+        QS3_TRY(B.d_stab.alloc((uint64_t)S * n));
+        DevBuf dK, pos, tmp, dends;
+        QS3_TRY(dends.alloc(((size_t)S + 1) * 4));
+        QS3_TRY(dK.upload(B.K.data(), B.K.size() * sizeof(int)));
+        const int grp = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)S, (1ull << 27) / std::max<uint64_t>(n, 1)));
+        QS3_TRY(pos.alloc(((uint64_t)grp * n + 1) * 4));
+        size_t tb = 0;
+        QS3_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, pos.as<uint32_t>(), pos.as<uint32_t>(), (int64_t)((uint64_t)grp * n + 1)));
+        QS3_TRY(tmp.alloc(tb));
+        uint64_t off = 0;
+        std::vector<uint32_t> ends;
+        for (int s0 = 0; s0 < S; s0 += grp) {
+            const int ns = std::min(grp, S - s0);
+            const uint64_t cnt = (uint64_t)ns * n;
+            const int g1 = (int)std::max<uint64_t>(1, std::min<uint64_t>((n + NTHREADS - 1) / NTHREADS, 4096));
+            QS3_CUDA(cudaMemsetAsync(pos.as<uint32_t>() + cnt, 0, 4));
+            k_members<ND><<<g1, NTHREADS, smem>>>(B.lv, keep_reps.as<uint64_t>(), keep_stab.as<uint8_t>(), n, ns,
+                                                  dK.as<int>() + 3 * s0, pos.as<uint32_t>());
+            QS3_LAUNCHED();
+            size_t t2 = tb;
+            QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, t2, pos.as<uint32_t>(), pos.as<uint32_t>(), (int64_t)(cnt + 1)));
+            const int g2 = (int)std::max<uint64_t>(1, std::min<uint64_t>((cnt + 255) / 256, 16384));
+            k_take<<<g2, 256>>>(pos.as<uint32_t>(), keep_reps.as<uint64_t>(), keep_stab.as<uint8_t>(), n, cnt,
+                                B.d_sigma.as<uint64_t>() + off, B.d_stab.as<uint8_t>() + off);
+            QS3_LAUNCHED();
+            k_ends<<<(ns + 256) / 256, 256>>>(pos.as<uint32_t>(), n, ns + 1, dends.as<uint32_t>());
+            QS3_LAUNCHED();
+            ends.assign(ns + 1, 0);
+            QS3_CUDA(cudaMemcpy(ends.data(), dends.p, ends.size() * 4, cudaMemcpyDeviceToHost));
+            for (int i = 0; i < ns; ++i) B.dims[s0 + i] = ends[i + 1] - ends[i];
+            off += ends[ns];
+        }
+    }
+    for (int s = 0; s < S; ++s)
+        if (B.dims[s] >= (1ull << 32))
+            return set_err(QS3_ERR_OVERFLOW, "sector dimension %llu exceeds 2^32", (unsigned long long)B.dims[s]);
+    return QS3_OK;
+}
+
+// the index over every sector's rows (SecView::pinfo, sub)
+template <int ND>
+static int build_index_nd(Basis &B) {
+    const int S = B.S;
+    // two-site prefixes unless that makes many more prefixes than rows
+    const uint64_t np2 = (uint64_t)B.N * (B.N - 1) / 2;
+    const int pre2 = ND >= 2 && (uint64_t)S * np2 / 8 <= B.total ? 1 : 0;
+    const uint32_t np = pre2 ? (uint32_t)np2 : (uint32_t)B.N;
+    const uint64_t cnt = (uint64_t)S * np;
+    for (auto &v : B.secs) v.pre2 = pre2;
+    QS3_CUDA(cudaMemcpy(B.d_secs.p, B.secs.data(), B.secs.size() * sizeof(SecView), cudaMemcpyHostToDevice));
+    DevBuf first, size, off, tmp;
+    QS3_TRY(first.alloc((uint64_t)S * (np + 1) * 4));
+    QS3_TRY(size.alloc((cnt + 1) * 4));
+    QS3_TRY(off.alloc((cnt + 1) * 4));
+    const int g1 = (int)std::max<uint64_t>(1, std::min<uint64_t>((cnt + S + 255) / 256, 16384));
+    const uint64_t *bin = B.d_binom.as<uint64_t>();
+    const SecView *secs = B.d_secs.as<SecView>();
+    k_first<<<g1, 256>>>(B.nd, B.N + 1, pre2, secs, S, np, bin, first.as<uint32_t>());
+    QS3_LAUNCHED();
+    QS3_CUDA(cudaMemsetAsync(size.as<uint32_t>() + cnt, 0, 4));
+    k_bucket_size<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, S, np, first.as<uint32_t>(), size.as<uint32_t>());
+    QS3_LAUNCHED();
+    size_t tb = 0;
+    QS3_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt + 1)));
+    QS3_TRY(tmp.alloc(tb));
+    QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, tb, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt + 1)));
+    // at most rows / 2 + 1 buckets and the end per prefix
+    const uint64_t most = B.total / 2 + 2 * cnt;
+    if (most >= (1ull << 32)) return set_err(QS3_ERR_OVERFLOW, "index of %llu entries", (unsigned long long)most);
+    QS3_TRY(B.d_pinfo.alloc(std::max<uint64_t>(cnt, 1) * sizeof(uint2)));
+    QS3_TRY(B.d_sub.alloc(std::max<uint64_t>(most, 1) * 4));
+    k_bucket_info<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, S, np, first.as<uint32_t>(), off.as<uint32_t>(),
+                               B.d_pinfo.as<uint2>(), B.d_sub.as<uint32_t>());
+    QS3_LAUNCHED();
+    if (B.ntiles > 0) {
+        const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8;
+        QS3_CUDA(cudaFuncSetAttribute(k_bucket_fill<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+        k_bucket_fill<ND><<<std::min(B.ntiles, 8192), NTHREADS, smem>>>(B.lv, secs, B.d_tile0.as<int>(), S, B.ntiles, np,
+                                                                        first.as<uint32_t>(), B.d_pinfo.as<uint2>(),
+                                                                        B.d_sub.as<uint32_t>());
+        QS3_LAUNCHED();
+    }
+    for (int s = 0; s < S; ++s) {
+        B.secs[s].pinfo = B.d_pinfo.as<uint2>() + (uint64_t)s * np;
+        B.secs[s].sub = B.d_sub.as<uint32_t>();
+    }
+    QS3_CUDA(cudaDeviceSynchronize());       // the scratch is released on return
+    return QS3_OK;
+}
+
+#define QS3_ND_CALL(nd, CALL)                                            \
+    switch (nd) {                                                        \
+        case 1: return CALL(1);                                          \
+        case 2: return CALL(2);                                          \
+        case 3: return CALL(3);                                          \
+        case 4: return CALL(4);                                          \
+        case 5: return CALL(5);                                          \
+        case 6: return CALL(6);                                          \
+        case 7: return CALL(7);                                          \
+        case 8: return CALL(8);                                          \
+        default: return set_err(QS3_ERR_INVALID_ARG, "n_down %d", (nd)); \
+    }
+
+static int build_sectors(Basis &B, DevBuf &reps, DevBuf &stab, uint64_t &n) {
+#define QS3_CALL(k) build_sectors_nd<k>(B, reps, stab, n)
+    QS3_ND_CALL(B.nd, QS3_CALL)
+#undef QS3_CALL
+}
+
+static int build_index(Basis &B) {
+#define QS3_CALL(k) build_index_nd<k>(B)
+    QS3_ND_CALL(B.nd, QS3_CALL)
+#undef QS3_CALL
 }
 
 // ---------------------------------------------------- representative table
@@ -402,22 +680,22 @@ __global__ void k_phase_digits(const double2 *__restrict__ ph64, uint64_t n, int
     }
 }
 
+// reps / stab: the orbits' list when the caller has it (n of them; taken over), else empty
 template <int ND>
-static int build_table_nd(Basis &B, size_t max_bytes) {
-    std::vector<uint64_t> hb((size_t)(B.nd + 3) * (B.N + 1));
-    QS3_CUDA(cudaMemcpy(hb.data(), B.d_binom.p, hb.size() * sizeof(uint64_t), cudaMemcpyDeviceToHost));
-    const uint64_t ns = hb[(size_t)ND * (B.N + 1) + B.N];           // C(N, N_down)
+static int build_table_nd(Basis &B, size_t max_bytes, DevBuf &reps, DevBuf &stab, uint64_t n) {
+    const uint64_t ns = B.binom[(size_t)ND * (B.N + 1) + B.N];     // C(N, N_down)
     if (ns >= (1ull << 32)) return set_err(QS3_ERR_OVERFLOW, "C(N, N_down) = %llu states: no table", (unsigned long long)ns);
     const uint64_t n_est = ns / (uint64_t)B.ncell + 1;             // orbits, about C(N, N_down) / (cells)
     if (ns * 4 + n_est * 4 * (uint64_t)B.S > max_bytes)
         return set_err(QS3_ERR_OOM, "representative table of ~%llu bytes exceeds the limit",
                        (unsigned long long)(ns * 4 + n_est * 4 * (uint64_t)B.S));
-    const int K0[3] = {0, 0, 0};                                   // every representative is compatible at k = 0
-    DevBuf reps, stab;
-    uint64_t n = 0;
-    int nsm = 0;
-    std::vector<uint64_t> hb2;
-    QS3_TRY(enum_sorted_reps<ND>(B, K0, reps, stab, n, hb2, nsm));
+    if (!reps.p) {
+        n = count_orbits(B, B.binom);
+        if (n < (1ull << 20)) QS3_TRY(enum_orbits<ND>(B, reps, stab, n));
+    }
+    int dev = 0, nsm = 0;
+    QS3_CUDA(cudaGetDevice(&dev));
+    QS3_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     if (n >= (1ull << 20)) return set_err(QS3_ERR_OVERFLOW, "%llu orbits exceed the table's 20-bit index", (unsigned long long)n);
     if (ns * 4 + n * 4 * (uint64_t)B.S > max_bytes)
         return set_err(QS3_ERR_OOM, "representative table exceeds the limit");
@@ -456,21 +734,18 @@ static int build_table_nd(Basis &B, size_t max_bytes) {
     return QS3_OK;
 }
 
-int build_rep_table(Basis &B, size_t max_bytes) {
+static int build_rep_table(Basis &B, size_t max_bytes, DevBuf &reps, DevBuf &stab, uint64_t n) {
     if (!B.has_k || B.nd == 0 || B.total == 0) return set_err(QS3_ERR_STATE, "the table serves k-sector bases only");
     if (B.N > 4096) return set_err(QS3_ERR_OVERFLOW, "N > 4096");
     if (B.lv.orb) return QS3_OK;
-    switch (B.nd) {
-        case 1: return build_table_nd<1>(B, max_bytes);
-        case 2: return build_table_nd<2>(B, max_bytes);
-        case 3: return build_table_nd<3>(B, max_bytes);
-        case 4: return build_table_nd<4>(B, max_bytes);
-        case 5: return build_table_nd<5>(B, max_bytes);
-        case 6: return build_table_nd<6>(B, max_bytes);
-        case 7: return build_table_nd<7>(B, max_bytes);
-        case 8: return build_table_nd<8>(B, max_bytes);
-        default: return set_err(QS3_ERR_INVALID_ARG, "n_down %d", B.nd);
-    }
+#define QS3_CALL(k) build_table_nd<k>(B, max_bytes, reps, stab, n)
+    QS3_ND_CALL(B.nd, QS3_CALL)
+#undef QS3_CALL
+}
+
+int build_rep_table(Basis &B, size_t max_bytes) {
+    DevBuf reps, stab;
+    return build_rep_table(B, max_bytes, reps, stab, 0);
 }
 
 void drop_rep_table(Basis &B) {
@@ -624,6 +899,7 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     if (!binom_table(N, nd + 3, tb, &cnd, nd))
         return set_err(QS3_ERR_OVERFLOW, "C(%d, %d) does not fit in 63 bits", N, nd);
     QS3_TRY(B.d_binom.upload(tb.data(), tb.size() * 8));
+    B.binom = std::move(tb);
 
     // adjacency (CSR, both directions), diagonal constants
     std::vector<int> deg(N + 1, 0);
@@ -706,6 +982,7 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     for (int a = 0; a < 3; ++a) L.L[a] = B.L[a];
     L.has_k = B.has_k;
     L.key_bits = (bits * nd <= 64) ? bits : 0;
+    L.mask_ok = L.key_bits > 0 && L.L[0] <= 32 && L.L[1] <= 32 && L.L[2] <= 32;
     L.binom = B.d_binom.as<uint64_t>();
     L.adj_ptr = B.d_adj_ptr.as<int>();
     L.adj_nbr = B.d_adj_nbr.as<int>();
@@ -736,24 +1013,20 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
 
     // sectors
     B.dims.assign(nsec, 0);
-    B.d_sigma.resize(nsec);
-    B.d_stab.resize(nsec);
-    B.d_pidx.resize(nsec);
+    DevBuf oreps, ostab;
+    uint64_t n_orb = 0;
     if (!B.has_k) {
         B.dims[0] = cnd;
     } else if (nd == 0) {
-        for (int s = 0; s < nsec; ++s) {
-            const bool k0 = B.K[3 * s] == 0 && B.K[3 * s + 1] == 0 && B.K[3 * s + 2] == 0;
-            B.dims[s] = k0 ? 1 : 0;
-            uint64_t zero = 0;
-            uint8_t one = 1;
-            uint32_t pi[2] = {0, k0 ? 1u : 0u};
-            QS3_TRY(B.d_sigma[s].upload(&zero, 8));
-            QS3_TRY(B.d_stab[s].upload(&one, 1));
-            QS3_TRY(B.d_pidx[s].upload(pi, 8));
-        }
+        // the vacuum, in the sector of momentum 0
+        std::vector<uint64_t> zero(nsec, 0);
+        std::vector<uint8_t> one(nsec, 1);
+        for (int s = 0; s < nsec; ++s)
+            B.dims[s] = B.K[3 * s] == 0 && B.K[3 * s + 1] == 0 && B.K[3 * s + 2] == 0 ? 1 : 0;
+        QS3_TRY(B.d_sigma.upload(zero.data(), zero.size() * 8));
+        QS3_TRY(B.d_stab.upload(one.data(), one.size()));
     } else {
-        for (int s = 0; s < nsec; ++s) QS3_TRY(build_sector_reps(B, s));
+        QS3_TRY(build_sectors(B, oreps, ostab, n_orb));
     }
     B.offs.assign(nsec + 1, 0);
     B.tile0.assign(nsec + 1, 0);
@@ -783,9 +1056,8 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     }
     for (int s = 0; s < nsec; ++s) {
         SecView &v = B.secs[s];
-        v.sigma = B.has_k ? B.d_sigma[s].as<uint64_t>() : nullptr;
-        v.stab = B.has_k ? B.d_stab[s].as<uint8_t>() : nullptr;
-        v.pidx = B.has_k ? B.d_pidx[s].as<uint32_t>() : nullptr;
+        v.sigma = B.has_k ? B.d_sigma.as<uint64_t>() + B.offs[s] : nullptr;
+        v.stab = B.has_k ? B.d_stab.as<uint8_t>() + B.offs[s] : nullptr;
         v.dim = B.dims[s];
         v.off = B.offs[s];
         for (int a = 0; a < 3; ++a) v.K[a] = B.K[3 * s + a];
@@ -797,6 +1069,10 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     QS3_TRY(B.d_secs.upload(B.secs.data(), B.secs.size() * sizeof(SecView)));
     QS3_TRY(B.d_tile0.upload(B.tile0.data(), B.tile0.size() * 4));
     QS3_TRY(B.d_chunk0.upload(B.chunk0.data(), B.chunk0.size() * 4));
+    if (B.has_k && nd > 0) {
+        QS3_TRY(build_index(B));
+        QS3_CUDA(cudaMemcpy(B.d_secs.p, B.secs.data(), B.secs.size() * sizeof(SecView), cudaMemcpyHostToDevice));
+    }
     B.smem_bytes = row_kernel_smem(B, 0);
     if (B.smem_bytes > 200 * 1024)
         return set_err(QS3_ERR_OVERFLOW, "lattice tables need %zu bytes of shared memory", B.smem_bytes);
@@ -807,7 +1083,7 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
         size_t fr = 0, tt = 0;
         QS3_CUDA(cudaMemGetInfo(&fr, &tt));
         const size_t lim = std::min<size_t>(REP_TABLE_AUTO_BYTES, fr / 8);
-        if (build_rep_table(B, lim) != QS3_OK) {
+        if (build_rep_table(B, lim, oreps, ostab, n_orb) != QS3_OK) {
             drop_rep_table(B);
             clear_err();
         }
@@ -864,8 +1140,8 @@ int qs3_basis_ranks(qs3_basis_t b, int32_t s, uint64_t *ranks, uint8_t *stab) {
     if (s < 0 || s >= B.S) return set_err(QS3_ERR_INVALID_ARG, "sector %d", s);
     if (!B.has_k) return set_err(QS3_ERR_INVALID_ARG, "a U(1)-only sector has ranks 0..dim-1");
     if (B.dims[s]) {
-        QS3_CUDA(cudaMemcpy(ranks, B.d_sigma[s].p, B.dims[s] * 8, cudaMemcpyDeviceToHost));
-        if (stab) QS3_CUDA(cudaMemcpy(stab, B.d_stab[s].p, B.dims[s], cudaMemcpyDeviceToHost));
+        QS3_CUDA(cudaMemcpy(ranks, B.secs[s].sigma, B.dims[s] * 8, cudaMemcpyDeviceToHost));
+        if (stab) QS3_CUDA(cudaMemcpy(stab, B.secs[s].stab, B.dims[s], cudaMemcpyDeviceToHost));
     }
     return QS3_OK;
 }

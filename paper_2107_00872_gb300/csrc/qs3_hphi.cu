@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(NTHREADS, (KS && TB && sizeof(VT) == 16) ? 4 :
                         int rep[ND];
                         int ax, by, cz;
                         const uint64_t r2 = canon(tt, L, sm.sxyz, sm.sC, rep, ax, by, cz);
-                        if (!sigma_find(sv, prefix_of(rep, sm.sC, L.np1), r2, idx)) continue;
+                        if (!sigma_find(sv, rep, sm.sC, L.np1, r2, idx)) continue;
                         u = ax + L.L[0] * (by + L.L[1] * cz);
                     }
                     CT p = ph[u];   // generic load (L1-cached)
@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(NTHREADS) k_count(LatView L, const SecView *__
                         int ax, by, cz;
                         const uint64_t r2 = canon(tt, L, sm.sxyz, sm.sC, rep, ax, by, cz);
                         uint32_t idx;
-                        if (sigma_find(sv, prefix_of(rep, sm.sC, L.np1), r2, idx)) ++cnt;
+                        if (sigma_find(sv, rep, sm.sC, L.np1, r2, idx)) ++cnt;
                     }
                 }
             }

@@ -78,6 +78,7 @@ struct LatView {
     int L[3];
     int has_k;
     int key_bits;                 // bits per site of a packed key, 0 -> compare ranks
+    int mask_ok;                  // canon_mask applies: L <= 32 along each axis, keys fit 64 bits
     const uint64_t *binom;
     const int *adj_ptr;           // N + 1
     const int *adj_nbr;           // 2 n_bonds
@@ -116,7 +117,14 @@ struct LatView {
 struct SecView {
     const uint64_t *sigma;        // sorted rank0 of the representatives (NULL: U(1))
     const uint8_t *stab;          // |Stab| of each representative
-    const uint32_t *pidx;         // prefix index over sigma (see build_pidx)
+    // index over sigma: the rows whose representatives share their two largest
+    // sites (pre2; else the largest one), prefix P, are split by the rank of
+    // their other sites into buckets of a few rows: pinfo[P] = (first entry o,
+    // shift), rows of bucket q = low rank >> shift are sub[o + q] .. sub[o + q
+    // + 1] - 1
+    const uint2 *pinfo;
+    const uint32_t *sub;
+    int pre2;
     uint64_t dim;
     uint64_t off;                 // offset of the sector in a concatenated vector
     int K[3];
@@ -144,13 +152,14 @@ struct Basis {
     // host copies of the model
     std::vector<int> bi, bj;
     std::vector<double> jxy, jz, h, pos;
+    std::vector<uint64_t> binom;            // host copy of the binomial rows 0 .. nd + 2
     bool has_h = false;
     // device data
     DevBuf d_binom, d_adj_ptr, d_adj_nbr, d_adj_jxy, d_adj_jz, d_adj_jxy_f, d_u, d_xyz;
     DevBuf d_u_f, d_adj_jz_f;
     DevBuf d_adj_jxy_lo, d_u_lo, d_adj_jz_lo;
     DevBuf d_adj_pad, d_adj_jz_pad;         // fixed-width adjacency (LatView::adj_pad)
-    std::vector<DevBuf> d_sigma, d_stab, d_pidx;
+    DevBuf d_sigma, d_stab, d_pinfo, d_sub;  // every sector's lists, one after another
     DevBuf d_ph64, d_ph32, d_phdf;          // S x N per-site phase tables (k-sectors)
     DevBuf d_secs, d_tile0, d_chunk0;
     LatView lv{};
@@ -342,7 +351,7 @@ __device__ __forceinline__ bool seen_before(const int (&a)[ND], int i, int v) {
 // origin (T^t a' = rep with t = -(ax, by, cz)), and the function returns its
 // rank0.
 template <int ND>
-__device__ __forceinline__ uint64_t canon(const int (&t)[ND], const LatView &L, const uint32_t *__restrict__ sxyz,
+__device__ __forceinline__ uint64_t canon_gen(const int (&t)[ND], const LatView &L, const uint32_t *__restrict__ sxyz,
                                           const uint64_t *__restrict__ sC, int (&rep)[ND], int &ax, int &by,
                                           int &cz) {
     int X[ND], Y[ND], Z[ND], SB[ND];
@@ -487,23 +496,211 @@ __device__ __forceinline__ uint64_t canon(const int (&t)[ND], const LatView &L, 
     return kb ? rank_of(rep, sC, L.np1) : best;
 }
 
-// prefix of a sorted list used by the two-level index over sigma: the colex
-// rank of its two largest sites (its largest site when ND == 1)
+// the highest set bit of the L-bit word m (held twice in a row in mm, L <= 32)
+// rotated right by c
+__device__ __forceinline__ int rot_top(uint64_t mm, uint32_t full, int c) {
+    return 31 - __clz((int)((uint32_t)(mm >> c) & full));
+}
+__device__ __forceinline__ uint64_t twice(uint32_t m, int L) { return (uint64_t)m | ((uint64_t)m << L); }
+__device__ __forceinline__ uint32_t low_ones(int L) { return 0xffffffffu >> (32 - L); }
+
+// the same minimum by occupation masks (LatView::mask_ok: L <= 32 along each
+// axis and packed keys of 64 bits).  Along an axis the spins' coordinates
+// form an L-bit word; the largest coordinate after moving c to 0 is the
+// highest set bit of the word rotated by c, so a level costs a few integer
+// instructions per candidate instead of a pass over all spins (ND^2
+// subtract / wrap / max steps in canon_gen), and the spins at the top are
+// those with one coordinate value.  A candidate whose top (y, x) exceeds the
+// smallest met so far cannot win.  X, Y, Z, SB: the spins' cell coordinates
+// and places in the cell, in any order; best: the packed sorted list of the
+// representative (kb bits per site, the largest site highest).
 template <int ND>
-__device__ __forceinline__ uint32_t prefix_of(const int (&c)[ND], const uint64_t *__restrict__ sC, int np1) {
-    if (ND >= 2) return (uint32_t)(sC[2 * np1 + c[ND - 1]] + (uint64_t)c[ND - 2]);
-    return (uint32_t)c[0];
+__device__ __forceinline__ void canon_mask(const int (&X)[ND], const int (&Y)[ND], const int (&Z)[ND],
+                                           const int (&SB)[ND], const LatView &L, uint64_t &best, int &ax, int &by,
+                                           int &cz) {
+    const int Lx = L.L[0], Ly = L.L[1], Lz = L.L[2];
+    const int kb = L.key_bits;
+    // level z
+    uint32_t mz = 1u;
+    int bz = 0;
+    if (Lz > 1) {
+        uint32_t m = 0;
+#pragma unroll
+        for (int k = 0; k < ND; ++k) m |= 1u << Z[k];
+        const uint64_t mm = twice(m, Lz);
+        const uint32_t full = low_ones(Lz);
+        bz = 32;
+#pragma unroll
+        for (int k = 0; k < ND; ++k) {
+            const int t = rot_top(mm, full, Z[k]);
+            mz = t < bz ? 0u : mz;
+            bz = min(bz, t);
+            mz |= t == bz ? 1u << Z[k] : 0u;
+        }
+    }
+    best = ~0ull;
+    int gy = 32, gx = 32;                  // the smallest top (y, x) so far
+    ax = by = cz = 0;
+    while (mz) {
+        const int zc = __ffs(mz) - 1;
+        mz &= mz - 1;
+        int zt = zc + bz;                  // the z of the top spins
+        zt -= zt >= Lz ? Lz : 0;
+        // level y over the top-z spins
+        uint32_t my = 1u;
+        int byv = 0;
+        if (Ly > 1) {
+            uint32_t m = 0;
+#pragma unroll
+            for (int k = 0; k < ND; ++k) m |= Z[k] == zt ? 1u << Y[k] : 0u;
+            const uint64_t mm = twice(m, Ly);
+            const uint32_t full = low_ones(Ly);
+            byv = 32;
+#pragma unroll
+            for (int k = 0; k < ND; ++k) {
+                const int t = rot_top(mm, full, Y[k]);
+                my = t < byv ? 0u : my;
+                byv = min(byv, t);
+                my |= t == byv ? 1u << Y[k] : 0u;
+            }
+        }
+        if (byv > gy) continue;
+        if (byv < gy) {
+            gy = byv;
+            gx = 32;
+        }
+        while (my) {
+            const int yc = __ffs(my) - 1;
+            my &= my - 1;
+            int yt = yc + byv;
+            yt -= yt >= Ly ? Ly : 0;
+            // level x over the top-(z, y) spins
+            uint32_t mx = 1u;
+            int bxv = 0;
+            if (Lx > 1) {
+                uint32_t m = 0;
+#pragma unroll
+                for (int k = 0; k < ND; ++k) m |= (Z[k] == zt && Y[k] == yt) ? 1u << X[k] : 0u;
+                const uint64_t mm = twice(m, Lx);
+                const uint32_t full = low_ones(Lx);
+                bxv = 32;
+#pragma unroll
+                for (int k = 0; k < ND; ++k) {
+                    const int t = rot_top(mm, full, X[k]);
+                    mx = t < bxv ? 0u : mx;
+                    bxv = min(bxv, t);
+                    mx |= t == bxv ? 1u << X[k] : 0u;
+                }
+            }
+            if (bxv > gx) continue;
+            if (bxv < gx) {
+                gx = bxv;
+                best = ~0ull;
+            }
+            while (mx) {
+                const int xc = __ffs(mx) - 1;
+                mx &= mx - 1;
+                int s[ND];
+#pragma unroll
+                for (int k = 0; k < ND; ++k) {
+                    int dx = X[k] - xc, dy = Y[k] - yc, dz = Z[k] - zc;
+                    dx += dx < 0 ? Lx : 0;
+                    dy += dy < 0 ? Ly : 0;
+                    dz += dz < 0 ? Lz : 0;
+                    s[k] = SB[k] + L.nsub * (dx + Lx * (dy + Ly * dz));
+                }
+                sort_net(s);
+                uint64_t key = 0;
+#pragma unroll
+                for (int k = ND - 1; k >= 0; --k) key = (key << kb) | (uint64_t)s[k];
+                if (key < best) {
+                    best = key;
+                    ax = xc;
+                    by = yc;
+                    cz = zc;
+                }
+            }
+        }
+    }
 }
 
-// position of rank r in sector sv (binary search inside the prefix bucket)
-__device__ __forceinline__ bool sigma_find(const SecView &sv, uint32_t P, uint64_t r, uint32_t &idx) {
-    uint32_t lo = __ldg(sv.pidx + P), hi = __ldg(sv.pidx + P + 1);
-    while (lo < hi) {
-        uint32_t mid = (lo + hi) >> 1;
-        if (__ldg(sv.sigma + mid) < r) lo = mid + 1; else hi = mid;
+// the sorted list of a packed key
+template <int ND>
+__device__ __forceinline__ void unpack_key(uint64_t key, int kb, int (&rep)[ND]) {
+    const uint32_t mask = (1u << kb) - 1u;
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+        rep[k] = (int)((uint32_t)key & mask);
+        key >>= kb;
     }
-    idx = lo;
-    return lo < __ldg(sv.pidx + P + 1) && __ldg(sv.sigma + lo) == r;
+}
+
+// the representative of the site list t, by whichever search applies
+template <int ND>
+__device__ __forceinline__ uint64_t canon(const int (&t)[ND], const LatView &L, const uint32_t *__restrict__ sxyz,
+                                          const uint64_t *__restrict__ sC, int (&rep)[ND], int &ax, int &by,
+                                          int &cz) {
+    if (!L.mask_ok) return canon_gen(t, L, sxyz, sC, rep, ax, by, cz);
+    int X[ND], Y[ND], Z[ND], SB[ND];
+#pragma unroll
+    for (int m = 0; m < ND; ++m) {
+        const uint32_t p = sxyz[t[m]];
+        X[m] = p & 2047u;
+        Y[m] = (p >> 11) & 2047u;
+        Z[m] = p >> 22;
+        SB[m] = L.nsub > 1 ? t[m] % L.nsub : 0;
+    }
+    uint64_t key;
+    canon_mask(X, Y, Z, SB, L, key, ax, by, cz);
+    unpack_key(key, L.key_bits, rep);
+    return rank_of(rep, sC, L.np1);
+}
+
+// prefix of a sorted list used by the index over sigma -- the colex rank of
+// its two largest sites (pre2), or its largest site -- and the rank of the
+// other sites
+template <int ND>
+__device__ __forceinline__ uint32_t prefix_of(const int (&c)[ND], const uint64_t *__restrict__ sC, int np1, int pre2,
+                                              uint64_t &low) {
+    low = 0;
+    if constexpr (ND >= 2) {
+#pragma unroll
+        for (int m = 0; m + 2 < ND; ++m) low += sC[(m + 1) * np1 + c[m]];
+        if (pre2) return (uint32_t)(sC[2 * np1 + c[ND - 1]] + (uint64_t)c[ND - 2]);
+        low += sC[(ND - 1) * np1 + c[ND - 2]];
+    }
+    return (uint32_t)c[ND - 1];
+}
+
+// the row of rank r among rows lo .. hi - 1 of a sector (a bucket of the
+// index): buckets of up to four rows -- nearly all -- are read at once
+__device__ __forceinline__ bool bucket_find(const uint64_t *__restrict__ sigma, uint32_t lo, uint32_t hi, uint64_t r,
+                                            uint32_t &idx) {
+    while (hi - lo > 4u) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (__ldg(sigma + mid) <= r) lo = mid; else hi = mid;
+    }
+    uint64_t v[4];
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i) v[i] = lo + i < hi ? __ldg(sigma + lo + i) : ~0ull;
+    bool found = false;
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i)
+        if (v[i] == r) {
+            found = true;
+            idx = lo + i;
+        }
+    return found;
+}
+
+// position of the representative c, of rank r, in sector sv
+template <int ND>
+__device__ __forceinline__ bool sigma_find(const SecView &sv, const int (&c)[ND], const uint64_t *__restrict__ sC,
+                                           int np1, uint64_t r, uint32_t &idx) {
+    uint64_t low;
+    const uint2 pi = __ldg(sv.pinfo + prefix_of(c, sC, np1, sv.pre2, low));
+    const uint32_t *e = sv.sub + pi.x + (uint32_t)(low >> pi.y);
+    return bucket_find(sv.sigma, __ldg(e), __ldg(e + 1), r, idx);
 }
 
 // stage the binomial table (rows 0..nd+2) and the coordinate table in smem
@@ -542,8 +739,6 @@ void drop_terms(Basis &B);
 int hphi_stored_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t st, const int *active);
 constexpr size_t REP_TABLE_AUTO_BYTES = (size_t)1 << 30;   // built at basis creation up to this size
 void drop_rep_table(Basis &B);
-// implemented in qs3_basis.cu
-int build_sector_reps(Basis &B, int s);
 // implemented in qs3_obs.cu
 int sq_launch(int op, Basis &src, int s_src, const void *phi, Basis &dst, int s_dst, const int *Q, void *psi,
               cudaStream_t st);

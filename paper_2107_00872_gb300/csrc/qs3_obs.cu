@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(NTHREADS) k_corr_k(LatView L, SecView sv, cons
                 int ax, by, cz;
                 const uint64_t r2 = canon(tt, L, sm.sxyz, sm.sC, rep, ax, by, cz);
                 uint32_t idx;
-                if (!sigma_find(sv, prefix_of(rep, sm.sC, L.np1), r2, idx)) continue;
+                if (!sigma_find(sv, rep, sm.sC, L.np1, r2, idx)) continue;
                 // the spin moved by -delta: delta = c_m - j
                 const int d = disp_index(sm.sxyz[j], sm.sxyz[c[m]], L.L);
                 const double2 p = cmul2(cmul2(phk[ax], phy[by]), phz[cz]);
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(NTHREADS) k_smq(LatView Ls, SecView svs, SecVi
                 int ax, by, cz;
                 const uint64_t r2 = canon(rem, Ls, sm.sxyz, sm.sC, rep, ax, by, cz);
                 uint32_t i32;
-                if (!sigma_find(svs, prefix_of(rep, sm.sC, Ls.np1), r2, i32)) continue;
+                if (!sigma_find(svs, rep, sm.sC, Ls.np1, r2, i32)) continue;
                 idx = i32;
                 coef = cmul2(coef, cmul2(cmul2(phk[ax], phy[by]), phz[cz]));
                 const double w = sm.snorm[__ldg(svs.stab + idx)] * rb;
@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(NTHREADS) k_szq(LatView Ls, SecView svs, SecVi
         uint64_t idx = row;
         if constexpr (KS) {
             uint32_t i32;
-            if (!sigma_find(svs, prefix_of(c, sm.sC, Ls.np1), rank, i32)) {
+            if (!sigma_find(svs, c, sm.sC, Ls.np1, rank, i32)) {
                 psi[row] = make_double2(0.0, 0.0);
                 continue;
             }
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(NTHREADS) k_spq(LatView Ls, SecView svs, SecVi
                 int ax, by, cz;
                 const uint64_t r2 = canon(t, Ls, sm.sxyz, sm.sC, rep, ax, by, cz);
                 uint32_t i32;
-                if (!sigma_find(svs, prefix_of(rep, sm.sC, Ls.np1), r2, i32)) continue;
+                if (!sigma_find(svs, rep, sm.sC, Ls.np1, r2, i32)) continue;
                 idx = i32;
                 coef = cmul2(coef, cmul2(cmul2(phk[ax], phy[by]), phz[cz]));
                 const double w = sm.snorm[__ldg(svs.stab + idx)] * rb;

@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(NTHREADS) k_terms(LatView L, const SecView *__
                     int rep[ND];
                     int ax, by, cz;
                     const uint64_t r2 = canon(tt, L, sm.sxyz, sm.sC, rep, ax, by, cz);
-                    if (!sigma_find(sv, prefix_of(rep, sm.sC, L.np1), r2, idx)) continue;
+                    if (!sigma_find(sv, rep, sm.sC, L.np1, r2, idx)) continue;
                     u = ax + L.L[0] * (by + L.L[1] * cz);
                 }
                 if constexpr (FILL) {
