@@ -22,7 +22,6 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
-#include <complex>
 #include <cstring>
 #include <vector>
 
@@ -55,7 +54,6 @@ struct ObsSmem {
     double2 *phk;    // e^{-2 pi i K_alpha v / L_alpha}
     double2 *phq;    // e^{-2 pi i Q_alpha v / L_alpha}
     double *snorm;   // [0..8] sqrt(s), [9..17] 1/sqrt(s)
-    double2 *hist;   // per-block histogram (N entries) or NULL
 };
 
 __host__ __device__ inline size_t obs_smem_bytes(int nd_rows, int N, const int *L, bool hist) {
@@ -67,7 +65,7 @@ __host__ __device__ inline size_t obs_smem_bytes(int nd_rows, int N, const int *
     return s;
 }
 
-__device__ __forceinline__ ObsSmem obs_carve(const LatView &L, unsigned char *smem, bool hist) {
+__device__ __forceinline__ ObsSmem obs_carve(const LatView &L, unsigned char *smem) {
     ObsSmem o;
     const int rows = L.nd + 3;
     o.sC = (uint64_t *)smem;
@@ -77,9 +75,6 @@ __device__ __forceinline__ ObsSmem obs_carve(const LatView &L, unsigned char *sm
     o.phk = (double2 *)(smem + off);
     o.phq = o.phk + (L.L[0] + L.L[1] + L.L[2]);
     o.snorm = (double *)(o.phq + (L.L[0] + L.L[1] + L.L[2]));
-    off += 2 * (size_t)(L.L[0] + L.L[1] + L.L[2]) * 16 + 18 * 8;
-    off = (off + 15) & ~(size_t)15;
-    o.hist = hist ? (double2 *)(smem + off) : nullptr;
     const int nC = rows * L.np1;
     for (int i = threadIdx.x; i < nC; i += blockDim.x) o.sC[i] = L.binom[i];
     for (int i = threadIdx.x; i < L.N; i += blockDim.x) o.sxyz[i] = L.xyz[i];
@@ -87,165 +82,334 @@ __device__ __forceinline__ ObsSmem obs_carve(const LatView &L, unsigned char *sm
         o.snorm[threadIdx.x] = sqrt((double)threadIdx.x);
         o.snorm[9 + threadIdx.x] = threadIdx.x ? 1.0 / sqrt((double)threadIdx.x) : 0.0;
     }
-    if (hist)
-        for (int i = threadIdx.x; i < L.N; i += blockDim.x) o.hist[i] = make_double2(0.0, 0.0);
     return o;
 }
 
-__device__ __forceinline__ int disp_index(uint32_t pa, uint32_t pb, const int *L) {
-    int dx = (int)(pb & 2047u) - (int)(pa & 2047u);
-    int dy = (int)((pb >> 11) & 2047u) - (int)((pa >> 11) & 2047u);
-    int dz = (int)(pb >> 22) - (int)(pa >> 22);
-    dx += dx < 0 ? L[0] : 0;
-    dy += dy < 0 ? L[1] : 0;
-    dz += dz < 0 ? L[2] : 0;
-    return dx + L[0] * (dy + L[1] * dz);
-}
-
 // ---------------------------------------------------------------- U(1): zz
-// G[i*N + j] += |phi_a|^2 for every ordered pair of down spins (i, j) of a
-// (diag_only: only i == j); norm[0] += |phi_a|^2
-template <int ND, typename VT>
-__global__ void __launch_bounds__(NTHREADS) k_occ_u1(LatView L, uint64_t dim, const VT *__restrict__ phi,
-                                                     int diag_only, double *__restrict__ G, double *__restrict__ norm) {
+// G[i*N + j] += |phi_a|^2 for every ordered pair of down spins (i, j) of a;
+// norm[0] += |phi_a|^2.  Consecutive rows share their upper spins, so a warp
+// whose rows agree on c_m adds once for all of them: without that every lane
+// of a shared-memory fp64 atomic (a compare-and-swap loop) hit one address.
+template <int ND>
+__global__ void __launch_bounds__(NTHREADS) k_occ_u1(LatView L, uint64_t dim, const double *__restrict__ phi,
+                                                     double *__restrict__ G, double *__restrict__ norm) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *sC = (uint64_t *)smem;
     double *sh = (double *)(sC + (size_t)(L.nd + 3) * L.np1);
-    const int nC = (L.nd + 3) * L.np1;
-    for (int i = threadIdx.x; i < nC; i += blockDim.x) sC[i] = L.binom[i];
-    for (int i = threadIdx.x; i <= L.N; i += blockDim.x) sh[i] = 0.0;
+    stage_tables(L, sC, nullptr);
+    for (int i = threadIdx.x; i < L.N; i += blockDim.x) sh[i] = 0.0;
     __syncthreads();
-    for (uint64_t row = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; row < dim;
-         row += (uint64_t)gridDim.x * blockDim.x) {
-        const VT v = phi[row];
-        double w;
-        if constexpr (sizeof(VT) == 16) w = ((const double2 &)v).x * ((const double2 &)v).x + ((const double2 &)v).y * ((const double2 &)v).y;
-        else w = (double)(*(const double *)&v) * (double)(*(const double *)&v);
+    const int lane = threadIdx.x & 31;
+    double tot = 0.0;
+    for (uint64_t r0 = (uint64_t)blockIdx.x * blockDim.x; r0 < dim; r0 += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t row = r0 + threadIdx.x;
+        const bool in = row < dim;
+        const double v = in ? phi[row] : 0.0, w = v * v;
         int c[ND];
-        unrank(row, sC, L.np1, c);
-        atomicAdd(sh + L.N, w);
+        unrank(in ? row : dim - 1, sC, L.np1, c);
+        tot += w;
+        double ws = w;
+        bool have = false;
 #pragma unroll
         for (int m = 0; m < ND; ++m) {
-            atomicAdd(sh + c[m], w);
-            if (!diag_only)
+            int same;
+            __match_all_sync(0xffffffffu, c[m], &same);
+            if (same) {
+                if (!have) {
 #pragma unroll
-                for (int q = 0; q < ND; ++q)
-                    if (q != m) atomicAdd(G + (size_t)c[m] * L.N + c[q], w);
+                    for (int o = 16; o; o >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, o);
+                    have = true;
+                }
+                if (lane == 0) atomicAdd(sh + c[m], ws);
+            } else if (in) {
+                atomicAdd(sh + c[m], w);
+            }
+#pragma unroll
+            for (int q = m + 1; q < ND; ++q) {
+                // (c_m, c_q) and (c_q, c_m); both the same for all lanes: once for the warp
+                int sq;
+                __match_all_sync(0xffffffffu, c[q], &sq);
+                if (same && sq) {
+                    if (lane < 2) atomicAdd(G + (lane ? (size_t)c[q] * L.N + c[m] : (size_t)c[m] * L.N + c[q]), ws);
+                } else if (in) {
+                    atomicAdd(G + (size_t)c[m] * L.N + c[q], w);
+                    atomicAdd(G + (size_t)c[q] * L.N + c[m], w);
+                }
+            }
         }
     }
+    __shared__ double red[NTHREADS / 32];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (lane == 0) red[threadIdx.x >> 5] = tot;
     __syncthreads();
     for (int i = threadIdx.x; i < L.N; i += blockDim.x)
         if (sh[i] != 0.0) atomicAdd(G + (size_t)i * L.N + i, sh[i]);
-    if (threadIdx.x == 0) atomicAdd(norm, sh[L.N]);
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < NTHREADS / 32; ++w) t += red[w];
+        atomicAdd(norm, t);
+    }
 }
 
 // --------------------------------------------------------------- U(1): +-
-// M[i*N + j] += conj(phi(a - i + j)) phi(a) for i in a, j not in a
-template <int ND, typename VT>
-__global__ void __launch_bounds__(NTHREADS) k_spsm_u1(LatView L, uint64_t dim, const VT *__restrict__ phi,
-                                                      double2 *__restrict__ M) {
+// M[i*N + j] += phi(a - i + j) phi(a) for i in a, j not in a (real vectors):
+// one warp per row, lanes over the sites j, so that a warp's adds go to
+// consecutive addresses of M
+template <int ND>
+__global__ void __launch_bounds__(NTHREADS) k_spsm_u1(LatView L, uint64_t dim, const double *__restrict__ phi,
+                                                      double *__restrict__ M) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *sC = (uint64_t *)smem;
-    const int nC = (L.nd + 3) * L.np1;
-    for (int i = threadIdx.x; i < nC; i += blockDim.x) sC[i] = L.binom[i];
+    stage_tables(L, sC, nullptr);
     __syncthreads();
-    for (uint64_t row = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; row < dim;
-         row += (uint64_t)gridDim.x * blockDim.x) {
-        double2 x;
-        if constexpr (sizeof(VT) == 16) x = *(const double2 *)(phi + row);
-        else x = make_double2(*(const double *)(phi + row), 0.0);
+    const int lane = threadIdx.x & 31;
+    const uint64_t nw = (uint64_t)gridDim.x * (NTHREADS / 32);
+    for (uint64_t row = (uint64_t)blockIdx.x * (NTHREADS / 32) + (threadIdx.x >> 5); row < dim; row += nw) {
+        const double x = phi[row];
         int c[ND];
         unrank(row, sC, L.np1, c);
+        for (int j = lane; j < L.N; j += 32) {
+            bool occ = false;
 #pragma unroll
-        for (int m = 0; m < ND; ++m) {
-            for (int j = 0; j < L.N; ++j) {
-                bool occ = false;
+            for (int k = 0; k < ND; ++k) occ |= (c[k] == j);
+            if (occ) continue;
+            uint64_t r2[ND];
 #pragma unroll
-                for (int k = 0; k < ND; ++k) occ |= (c[k] == j);
-                if (occ) continue;
+            for (int m = 0; m < ND; ++m) {
                 int tt[ND];
 #pragma unroll
                 for (int k = 0; k < ND; ++k) tt[k] = (k == m) ? j : c[k];
                 sort_net(tt);
-                const uint64_t r2 = rank_of(tt, sC, L.np1);
-                double2 y;
-                if constexpr (sizeof(VT) == 16) y = *(const double2 *)(phi + r2);
-                else y = make_double2(*(const double *)(phi + r2), 0.0);
-                // conj(y) * x
-                const double re = y.x * x.x + y.y * x.y, im = y.x * x.y - y.y * x.x;
-                double2 *dst = M + (size_t)c[m] * L.N + j;
-                atomicAdd(&dst->x, re);
-                atomicAdd(&dst->y, im);
+                r2[m] = rank_of(tt, sC, L.np1);
             }
+#pragma unroll
+            for (int m = 0; m < ND; ++m) atomicAdd(M + (size_t)c[m] * L.N + j, phi[r2[m]] * x);
         }
     }
 }
 
 // ------------------------------------------------------------- k-sectors
-// zz: hist[delta].x += |phi|^2 #{ordered pairs (m, q) at displacement delta}
-// +-: hist[delta] += (1/N) conj(phi_a) (B_delta phi)_a, B_delta = sum_r s^+_r s^-_{r+delta}
-template <int ND>
-__global__ void __launch_bounds__(NTHREADS) k_corr_k(LatView L, SecView sv, const double2 *__restrict__ phi,
-                                                     int do_pm, double2 *__restrict__ hzz, double2 *__restrict__ hpm,
-                                                     double *__restrict__ norm) {
+// For every displacement d of a list: the number of down-spin pairs at d,
+// C(d) = sum_a |phi_a|^2 #{(m, q): c_m - c_q = d}, and the hop sum P(d) = (1/N)
+// conj(phi_a) (B_d phi)_a, B_d = sum_r s^+_r s^-_{r+d}: in row a the spin c_m
+// comes from j = c_m - d.  One thread per row, CD displacements per block:
+// j is occupied (a pair) or a hop whose representative is looked up, so both
+// sums come from one loop; a thread keeps its CD sums in shared memory over
+// all its rows, and the block adds them once, in a fixed order, into
+// part[(chunk * gridDim.x + block) CD + i] = (Re P, Im P, C).  With the
+// representative table a hop costs a rank and two loads, and the displacement
+// -d needs no pass of its own (P(-d) = conj P(d)).  10x10 lattice, N_down = 4,
+// k = 0, all displacements and S(q) at 100 q: the whole call 0.35 ms, against
+// 28.5 ms with the search, fp64 atomics on N addresses and S(q) on the host
+// (7.0 ms of it the kernel).  d = 0 gives C = N_down |phi|^2.
+constexpr int CD = 8;
+constexpr int CORR_SMEM = 226 * 1024;      // the threads' sums (48 KB) beside the row tables
+
+template <int ND, bool TB>
+__global__ void __launch_bounds__(NTHREADS) k_corr_k(LatView L, SecView sv, const double2 *__restrict__ phi, int do_pm,
+                                                     const int *__restrict__ dl, int ndl, double *__restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem[];
-    ObsSmem sm = obs_carve(L, smem, true);
-    __shared__ double snorm_acc;
-    if (threadIdx.x == 0) snorm_acc = 0.0;
-    fill_axis_phases(L.L, sv.K, sm.phk);
+    double *sum = (double *)smem + threadIdx.x;                     // (i, component) at [(3 i + component) NTHREADS]
+    uint64_t *sC = (uint64_t *)((double *)smem + 3 * CD * NTHREADS);
+    uint32_t *sxyz = (uint32_t *)(sC + (L.nd + 3) * L.np1);
+    stage_tables(L, sC, sxyz);
+    __shared__ double snorm[18];
+    if (threadIdx.x < 9) {
+        snorm[threadIdx.x] = sqrt((double)threadIdx.x);
+        snorm[9 + threadIdx.x] = threadIdx.x ? 1.0 / sqrt((double)threadIdx.x) : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < 3 * CD; ++i) sum[i * NTHREADS] = 0.0;
     __syncthreads();
-    const double2 *phk = sm.phk;
-    const double2 *phy = phk + L.L[0], *phz = phk + L.L[0] + L.L[1];
-    // pass 1 (zz) uses sm.hist; pass 2 (+-) goes straight to global memory
+    const int Lx = L.L[0], Ly = L.L[1], Lz = L.L[2];
+    const int i0 = blockIdx.y * CD, n = min(CD, ndl - i0);
     for (uint64_t row = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; row < sv.dim;
          row += (uint64_t)gridDim.x * blockDim.x) {
         const double2 x = phi[row];
         const double w = x.x * x.x + x.y * x.y;
+        const uint64_t rank = __ldg(sv.sigma + row);
         int c[ND];
-        unrank(__ldg(sv.sigma + row), sm.sC, L.np1, c);
-        atomicAdd(&snorm_acc, w);
-#pragma unroll
-        for (int m = 0; m < ND; ++m)
-#pragma unroll
-            for (int q = 0; q < ND; ++q) {
-                const int d = disp_index(sm.sxyz[c[m]], sm.sxyz[c[q]], L.L);
-                atomicAdd(&sm.hist[d].x, w);
-            }
-        if (!do_pm) continue;
-        const double rs = sm.snorm[9 + __ldg(sv.stab + row)];
-#pragma unroll
-        for (int m = 0; m < ND; ++m) {
-            for (int j = 0; j < L.N; ++j) {
+        unrank(rank, sC, L.np1, c);
+        const double rs = snorm[9 + __ldg(sv.stab + row)] / (double)L.N;
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) {
+            const uint32_t dp = sxyz[__ldg(dl + i0 + i)];
+            const int dx = dp & 2047u, dy = (dp >> 11) & 2047u, dz = dp >> 22;
+            int pairs = 0;
+            double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 1
+            for (int m = 0; m < ND; ++m) {
+                const uint32_t p = sxyz[pick(c, m)];
+                int jx = (int)(p & 2047u) - dx, jy = (int)((p >> 11) & 2047u) - dy, jz = (int)(p >> 22) - dz;
+                jx += jx < 0 ? Lx : 0;
+                jy += jy < 0 ? Ly : 0;
+                jz += jz < 0 ? Lz : 0;
+                const int j = jx + Lx * (jy + Ly * jz);
                 bool occ = false;
 #pragma unroll
                 for (int k = 0; k < ND; ++k) occ |= (c[k] == j);
-                if (occ) continue;
+                if (occ) {
+                    ++pairs;
+                    continue;
+                }
+                if (!do_pm) continue;
                 int tt[ND];
 #pragma unroll
                 for (int k = 0; k < ND; ++k) tt[k] = (k == m) ? j : c[k];
-                sort_net(tt);
-                int rep[ND];
-                int ax, by, cz;
-                const uint64_t r2 = canon(tt, L, sm.sxyz, sm.sC, rep, ax, by, cz);
                 uint32_t idx;
-                if (!sigma_find(sv, rep, sm.sC, L.np1, r2, idx)) continue;
-                // the spin moved by -delta: delta = c_m - j
-                const int d = disp_index(sm.sxyz[j], sm.sxyz[c[m]], L.L);
-                const double2 p = cmul2(cmul2(phk[ax], phy[by]), phz[cz]);
-                const double wn = sm.snorm[__ldg(sv.stab + idx)] * rs / (double)L.N;
+                int u;
+                if constexpr (TB) {
+                    sort_net(tt);
+                    const uint32_t e = __ldg(L.orb + rank_of(tt, sC, L.np1));
+                    if ((e >> 12) >= L.n_orb) continue;                  // never for a complete table
+                    const int32_t r2 = __ldg(sv.t2 + (e >> 12));
+                    if (r2 < 0) continue;
+                    idx = (uint32_t)r2;
+                    u = (int)(e & 4095u);
+                } else {
+                    int rep[ND];
+                    int ax, by, cz;
+                    const uint64_t r2 = canon(tt, L, sxyz, sC, rep, ax, by, cz);
+                    if (!sigma_find(sv, rep, sC, L.np1, r2, idx)) continue;
+                    u = ax + Lx * (by + Ly * cz);
+                }
+                double2 ph = sv.ph64[u];
+                const int st = __ldg(sv.stab + idx);
+                if (st != 1) {
+                    ph.x *= snorm[st];
+                    ph.y *= snorm[st];
+                }
                 const double2 y = phi[idx];
-                // conj(x) * p * wn * y
-                const double2 py = cmul2(p, y);
-                const double re = (x.x * py.x + x.y * py.y) * wn, im = (x.x * py.y - x.y * py.x) * wn;
-                atomicAdd(&hpm[d].x, re);
-                atomicAdd(&hpm[d].y, im);
+                acc.x += ph.x * y.x - ph.y * y.y;
+                acc.y += ph.x * y.y + ph.y * y.x;
+            }
+            if (pairs) sum[(3 * i + 2) * NTHREADS] += w * (double)pairs;
+            if (do_pm) {
+                // conj(x) acc, times 1 / (N sqrt |Stab a|)
+                sum[3 * i * NTHREADS] += (x.x * acc.x + x.y * acc.y) * rs;
+                sum[(3 * i + 1) * NTHREADS] += (x.x * acc.y - x.y * acc.x) * rs;
             }
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < L.N; i += blockDim.x)
-        if (sm.hist[i].x != 0.0) atomicAdd(&hzz[i].x, sm.hist[i].x);
-    if (threadIdx.x == 0) atomicAdd(norm, snorm_acc);
+    // warp q sums components q, q + 8, ...
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < 3 * n; i += NTHREADS / 32) {
+        const double *v = (const double *)smem + (size_t)i * NTHREADS;
+        double t = 0.0;
+#pragma unroll
+        for (int q = 0; q < NTHREADS / 32; ++q) t += v[lane + 32 * q];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 3 * CD + i] = t;
+    }
+}
+
+// the correlation functions from the block sums, one warp per displacement
+// dl[i]: cf[d] = <s^z s^z>, cf[N + 2 d] = <s^+ s^-> (re, im) at d and at -d
+// (its complex conjugate); cf[3 N] = |phi|^2 (dl[0] = 0)
+__global__ void k_corr_sum(const double *__restrict__ part, int nb, const int *__restrict__ dl, int ndl, int N, int nd,
+                           int Lx, int Ly, int Lz, double *__restrict__ cf) {
+    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= ndl) return;
+    double t[3] = {0.0, 0.0, 0.0}, t0 = 0.0;
+    for (int b = lane; b < nb; b += 32) {
+        const double *v = part + ((size_t)(i / CD) * nb + b) * 3 * CD + 3 * (i % CD);
+        for (int k = 0; k < 3; ++k) t[k] += v[k];
+        t0 += part[(size_t)b * 3 * CD + 2];            // d = 0
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        for (int k = 0; k < 3; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+        t0 += __shfl_xor_sync(0xffffffffu, t0, o);
+    }
+    if (lane) return;
+    const double norm = t0 / (double)nd;
+    const int d = dl[i];
+    const int x = d % Lx, y = (d / Lx) % Ly, z = d / (Lx * Ly);
+    const int e = (Lx - x) % Lx + Lx * ((Ly - y) % Ly + Ly * ((Lz - z) % Lz));    // -d
+    const double zz = d ? 0.25 - (double)nd / N + t[2] / (N * norm) : 0.25;
+    const double pr = d ? t[0] / norm : 1.0 - (double)nd / N, pi = d ? t[1] / norm : 0.0;
+    cf[d] = cf[e] = zz;
+    cf[N + 2 * e] = pr;
+    cf[N + 2 * e + 1] = -pi;
+    cf[N + 2 * d] = pr;
+    cf[N + 2 * d + 1] = pi;
+    if (i == 0) cf[3 * N] = norm;
+}
+
+// S(q) = (1/N) sum_ij e^{iq.(r_i - r_j)} <O_i O_j> for the q of this block,
+// zz in out[2 q], +- in out[2 q + 1].  KS: the functions of the displacement
+// j - i (cf as k_corr_sum); else from the site-resolved sums G, M and norm.
+// Warps take rows i, lanes columns j.
+template <bool KS>
+__global__ void __launch_bounds__(NTHREADS) k_sq(int N, int Lx, int Ly, int Lz, const double *__restrict__ pos,
+                                                 const double *__restrict__ q, const double *__restrict__ cf,
+                                                 const double *__restrict__ G, const double *__restrict__ M,
+                                                 const double *__restrict__ norm, int pm, double *__restrict__ out) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    double2 *e = (double2 *)smem;                       // e^{iq.r}
+    __shared__ double red[2][NTHREADS / 32];
+    const double qx = q[3 * blockIdx.x], qy = q[3 * blockIdx.x + 1], qz = q[3 * blockIdx.x + 2];
+    for (int r = threadIdx.x; r < N; r += blockDim.x) {
+        double sn, cs;
+        sincos(qx * pos[3 * r] + qy * pos[3 * r + 1] + qz * pos[3 * r + 2], &sn, &cs);
+        e[r] = make_double2(cs, sn);
+    }
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double az = 0.0, ap = 0.0;
+    const double in = KS ? 0.0 : 1.0 / *norm;
+    for (int i = warp; i < N; i += NTHREADS / 32) {
+        const int xi = i % Lx, yi = (i / Lx) % Ly, zi = i / (Lx * Ly);
+        double2 tz = make_double2(0.0, 0.0), tp = tz;
+        const double gi = KS ? 0.0 : G[(size_t)i * N + i] * in;
+        for (int j = lane; j < N; j += 32) {
+            double zz;
+            double2 c = make_double2(0.0, 0.0);
+            if constexpr (KS) {
+                int dx = j % Lx - xi, dy = (j / Lx) % Ly - yi, dz = j / (Lx * Ly) - zi;
+                dx += dx < 0 ? Lx : 0;
+                dy += dy < 0 ? Ly : 0;
+                dz += dz < 0 ? Lz : 0;
+                const int d = dx + Lx * (dy + Ly * dz);
+                zz = cf[d];
+                if (pm) c = make_double2(cf[N + 2 * d], cf[N + 2 * d + 1]);
+            } else {
+                zz = i == j ? 0.25 : 0.25 - 0.5 * (gi + G[(size_t)j * N + j] * in) + G[(size_t)i * N + j] * in;
+                if (pm) c.x = i == j ? 1.0 - gi : M[(size_t)i * N + j] * in;
+            }
+            const double2 ej = e[j];                    // conj(e_j) <O_i O_j>
+            tz.x = fma(zz, ej.x, tz.x);
+            tz.y = fma(-zz, ej.y, tz.y);
+            if (pm) {
+                tp.x = fma(c.x, ej.x, tp.x);
+                tp.y = fma(-c.x, ej.y, tp.y);
+                if (KS) {
+                    tp.x = fma(c.y, ej.y, tp.x);
+                    tp.y = fma(c.y, ej.x, tp.y);
+                }
+            }
+        }
+        az += e[i].x * tz.x - e[i].y * tz.y;
+        ap += e[i].x * tp.x - e[i].y * tp.y;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        az += __shfl_xor_sync(0xffffffffu, az, o);
+        ap += __shfl_xor_sync(0xffffffffu, ap, o);
+    }
+    if (lane == 0) {
+        red[0][warp] = az;
+        red[1][warp] = ap;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double t = 0.0;
+        for (int w = 0; w < NTHREADS / 32; ++w) t += red[threadIdx.x][w];
+        out[2 * blockIdx.x + threadIdx.x] = t / N;
+    }
 }
 
 // ------------------------------------------------------------- S^-_q (K10)
@@ -258,7 +422,7 @@ __global__ void __launch_bounds__(NTHREADS) k_smq(LatView Ls, SecView svs, SecVi
                                                   const double2 *__restrict__ phi, double2 *__restrict__ psi) {
     constexpr int NS = ND - 1;
     extern __shared__ __align__(16) unsigned char smem[];
-    ObsSmem sm = obs_carve(Ls, smem, false);
+    ObsSmem sm = obs_carve(Ls, smem);
     if (KS) fill_axis_phases(Ls.L, svs.K, sm.phk);
     __syncthreads();
     const double2 *phk = sm.phk, *phy = sm.phk + Ls.L[0], *phz = sm.phk + Ls.L[0] + Ls.L[1];
@@ -327,7 +491,7 @@ __global__ void __launch_bounds__(NTHREADS) k_szq(LatView Ls, SecView svs, SecVi
                                                   double inv_sqrt_n, const double2 *__restrict__ phi,
                                                   double2 *__restrict__ psi) {
     extern __shared__ __align__(16) unsigned char smem[];
-    ObsSmem sm = obs_carve(Ls, smem, false);
+    ObsSmem sm = obs_carve(Ls, smem);
     __syncthreads();
     for (uint64_t row = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; row < svd.dim;
          row += (uint64_t)gridDim.x * blockDim.x) {
@@ -362,7 +526,7 @@ __global__ void __launch_bounds__(NTHREADS) k_spq(LatView Ls, SecView svs, SecVi
                                                   const double2 *__restrict__ phi, double2 *__restrict__ psi) {
     constexpr int NS = ND + 1;
     extern __shared__ __align__(16) unsigned char smem[];
-    ObsSmem sm = obs_carve(Ls, smem, false);
+    ObsSmem sm = obs_carve(Ls, smem);
     if (KS) fill_axis_phases(Ls.L, svs.K, sm.phk);
     __syncthreads();
     const double2 *phk = sm.phk, *phy = sm.phk + Ls.L[0], *phz = sm.phk + Ls.L[0] + Ls.L[1];
@@ -476,28 +640,32 @@ static int grid_for(uint64_t n) {
 }
 
 template <int ND>
-static int corr_u1_nd(Basis &B, const double *phi, bool pm, double *G, double2 *M, double *nrm, cudaStream_t st) {
-    const size_t sm1 = (size_t)(B.nd + 3) * (B.N + 1) * 8 + (size_t)(B.N + 1) * 8;
-    QS3_CUDA(cudaFuncSetAttribute(k_occ_u1<ND, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-    const int g = grid_for(B.total);
-    k_occ_u1<ND, double><<<g, NTHREADS, sm1, st>>>(B.lv, B.total, phi, 0, G, nrm);
+static int corr_u1_nd(Basis &B, const double *phi, bool pm, double *G, double *M, double *nrm, cudaStream_t st) {
+    const size_t sm2 = (size_t)(B.nd + 3) * (B.N + 1) * 8, sm1 = sm2 + (size_t)B.N * 8;
+    QS3_CUDA(cudaFuncSetAttribute(k_occ_u1<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+    k_occ_u1<ND><<<grid_for(B.total), NTHREADS, sm1, st>>>(B.lv, B.total, phi, G, nrm);
     QS3_LAUNCHED();
     if (pm) {
-        const size_t sm2 = (size_t)(B.nd + 3) * (B.N + 1) * 8;
-        QS3_CUDA(cudaFuncSetAttribute(k_spsm_u1<ND, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-        k_spsm_u1<ND, double><<<g, NTHREADS, sm2, st>>>(B.lv, B.total, phi, M);
+        QS3_CUDA(cudaFuncSetAttribute(k_spsm_u1<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+        k_spsm_u1<ND><<<grid_for(B.total * 32), NTHREADS, sm2, st>>>(B.lv, B.total, phi, M);
         QS3_LAUNCHED();
     }
     return QS3_OK;
 }
 
+// the block sums of the displacements dl (ndl of them), nb blocks of rows each
 template <int ND>
-static int corr_k_nd(Basis &B, int s, const double2 *phi, bool pm, double2 *hzz, double2 *hpm, double *nrm,
+static int corr_k_nd(Basis &B, int s, const double2 *phi, bool pm, const int *dl, int ndl, int nb, double *part,
                      cudaStream_t st) {
-    const size_t smem = obs_smem_bytes(B.nd + 3, B.N, B.L, true);
-    if (smem > 200 * 1024) return set_err(QS3_ERR_OVERFLOW, "correlation tables need %zu bytes of shared memory", smem);
-    QS3_CUDA(cudaFuncSetAttribute(k_corr_k<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-    k_corr_k<ND><<<grid_for(B.dims[s]), NTHREADS, smem, st>>>(B.lv, B.secs[s], phi, pm ? 1 : 0, hzz, hpm, nrm);
+    const size_t smem = 3 * CD * NTHREADS * 8 + (size_t)(B.nd + 3) * (B.N + 1) * 8 + (size_t)B.N * 4;
+    const dim3 grid(nb, (ndl + CD - 1) / CD);
+    if (B.lv.orb) {
+        QS3_CUDA(cudaFuncSetAttribute(k_corr_k<ND, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, CORR_SMEM));
+        k_corr_k<ND, true><<<grid, NTHREADS, smem, st>>>(B.lv, B.secs[s], phi, pm ? 1 : 0, dl, ndl, part);
+    } else {
+        QS3_CUDA(cudaFuncSetAttribute(k_corr_k<ND, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, CORR_SMEM));
+        k_corr_k<ND, false><<<grid, NTHREADS, smem, st>>>(B.lv, B.secs[s], phi, pm ? 1 : 0, dl, ndl, part);
+    }
     QS3_LAUNCHED();
     return QS3_OK;
 }
@@ -713,34 +881,17 @@ int sq_launch(int op, Basis &S, int ss, const void *phi, Basis &Dd, int sd, cons
     return QS3_OK;
 }
 
-static int dispatch_corr_u1(Basis &B, const double *phi, bool pm, double *G, double2 *M, double *nrm,
-                            cudaStream_t st) {
-    switch (B.nd) {
-        case 1: return corr_u1_nd<1>(B, phi, pm, G, M, nrm, st);
-        case 2: return corr_u1_nd<2>(B, phi, pm, G, M, nrm, st);
-        case 3: return corr_u1_nd<3>(B, phi, pm, G, M, nrm, st);
-        case 4: return corr_u1_nd<4>(B, phi, pm, G, M, nrm, st);
-        case 5: return corr_u1_nd<5>(B, phi, pm, G, M, nrm, st);
-        case 6: return corr_u1_nd<6>(B, phi, pm, G, M, nrm, st);
-        case 7: return corr_u1_nd<7>(B, phi, pm, G, M, nrm, st);
-        case 8: return corr_u1_nd<8>(B, phi, pm, G, M, nrm, st);
-        default: return set_err(QS3_ERR_INVALID_ARG, "n_down %d", B.nd);
-    }
+static int dispatch_corr_u1(Basis &B, const double *phi, bool pm, double *G, double *M, double *nrm, cudaStream_t st) {
+#define QS3_CU(n) corr_u1_nd<n>(B, phi, pm, G, M, nrm, st)
+    QS3_ND_SWITCH(B.nd, QS3_CU)
+#undef QS3_CU
 }
 
-static int dispatch_corr_k(Basis &B, int s, const double2 *phi, bool pm, double2 *hzz, double2 *hpm, double *nrm,
+static int dispatch_corr_k(Basis &B, int s, const double2 *phi, bool pm, const int *dl, int ndl, int nb, double *part,
                            cudaStream_t st) {
-    switch (B.nd) {
-        case 1: return corr_k_nd<1>(B, s, phi, pm, hzz, hpm, nrm, st);
-        case 2: return corr_k_nd<2>(B, s, phi, pm, hzz, hpm, nrm, st);
-        case 3: return corr_k_nd<3>(B, s, phi, pm, hzz, hpm, nrm, st);
-        case 4: return corr_k_nd<4>(B, s, phi, pm, hzz, hpm, nrm, st);
-        case 5: return corr_k_nd<5>(B, s, phi, pm, hzz, hpm, nrm, st);
-        case 6: return corr_k_nd<6>(B, s, phi, pm, hzz, hpm, nrm, st);
-        case 7: return corr_k_nd<7>(B, s, phi, pm, hzz, hpm, nrm, st);
-        case 8: return corr_k_nd<8>(B, s, phi, pm, hzz, hpm, nrm, st);
-        default: return set_err(QS3_ERR_INVALID_ARG, "n_down %d", B.nd);
-    }
+#define QS3_CK(n) corr_k_nd<n>(B, s, phi, pm, dl, ndl, nb, part, st)
+    QS3_ND_SWITCH(B.nd, QS3_CK)
+#undef QS3_CK
 }
 
 static int correlations(Basis &B, int s, const void *gs, int npairs, const int *pairs, double *szsz, double *spsm,
@@ -754,61 +905,88 @@ static int correlations(Basis &B, int s, const void *gs, int npairs, const int *
     for (int p = 0; p < npairs; ++p)
         if (pairs[2 * p] < 0 || pairs[2 * p] >= N || pairs[2 * p + 1] < 0 || pairs[2 * p + 1] >= N)
             return set_err(QS3_ERR_INVALID_ARG, "pair %d outside the lattice", p);
-    // zz(i, j) and pm(i, j) as functions on site pairs
-    std::vector<double> Gh, Ch;
-    std::vector<double2> Mh, Ph;
-    double norm2 = 0.0;
     if (B.dims[s] == 0) return set_err(QS3_ERR_INVALID_ARG, "sector %d is empty", s);
-    if (!B.has_k) {
-        DevBuf G, M, nr;
-        QS3_TRY(G.alloc((size_t)N * N * 8));
-        QS3_CUDA(cudaMemsetAsync(G.p, 0, (size_t)N * N * 8, st));
-        QS3_TRY(nr.alloc(8));
-        QS3_CUDA(cudaMemsetAsync(nr.p, 0, 8, st));
-        QS3_TRY(M.alloc(want_pm ? (size_t)N * N * 16 : 16));
-        QS3_CUDA(cudaMemsetAsync(M.p, 0, M.n, st));
-        if (nd > 0) {
-            QS3_TRY(dispatch_corr_u1(B, (const double *)gs, want_pm, G.as<double>(), M.as<double2>(), nr.as<double>(), st));
-            QS3_CUDA(cudaMemcpyAsync(&norm2, nr.p, 8, cudaMemcpyDeviceToHost, st));
-        } else {
-            double v;
-            QS3_CUDA(cudaMemcpyAsync(&v, gs, 8, cudaMemcpyDeviceToHost, st));
-            QS3_CUDA(cudaStreamSynchronize(st));
-            norm2 = v * v;
+    const bool ks = B.has_k;
+    if (ks && nd > 0 && obs_smem_bytes(nd + 3, N, B.L, true) > 200 * 1024)
+        return set_err(QS3_ERR_OVERFLOW, "correlation tables need %zu bytes of shared memory",
+                       obs_smem_bytes(nd + 3, N, B.L, true));
+    // one displacement of every pair d, -d
+    std::vector<int> dl;
+    if (ks)
+        for (int d = 0; d < N; ++d) {
+            const int Lx = B.L[0], Ly = B.L[1], Lz = B.L[2];
+            const int x = d % Lx, y = (d / Lx) % Ly, z = d / (Lx * Ly);
+            if (d <= (Lx - x) % Lx + Lx * ((Ly - y) % Ly + Ly * ((Lz - z) % Lz))) dl.push_back(d);
         }
-        Gh.resize((size_t)N * N);
-        QS3_CUDA(cudaMemcpyAsync(Gh.data(), G.p, Gh.size() * 8, cudaMemcpyDeviceToHost, st));
-        if (want_pm) {
-            Mh.resize((size_t)N * N);
-            QS3_CUDA(cudaMemcpyAsync(Mh.data(), M.p, Mh.size() * 16, cudaMemcpyDeviceToHost, st));
-        }
-        QS3_CUDA(cudaStreamSynchronize(st));
-    } else {
-        DevBuf hzz, hpm, nr;
-        QS3_TRY(hzz.alloc((size_t)N * 16));
-        QS3_TRY(hpm.alloc((size_t)N * 16));
-        QS3_TRY(nr.alloc(8));
-        QS3_CUDA(cudaMemsetAsync(hzz.p, 0, hzz.n, st));
-        QS3_CUDA(cudaMemsetAsync(hpm.p, 0, hpm.n, st));
-        QS3_CUDA(cudaMemsetAsync(nr.p, 0, 8, st));
-        if (nd > 0) {
-            QS3_TRY(dispatch_corr_k(B, s, (const double2 *)gs, want_pm, hzz.as<double2>(), hpm.as<double2>(),
-                                    nr.as<double>(), st));
-            QS3_CUDA(cudaMemcpyAsync(&norm2, nr.p, 8, cudaMemcpyDeviceToHost, st));
-        } else {
-            double2 v;
-            QS3_CUDA(cudaMemcpyAsync(&v, gs, 16, cudaMemcpyDeviceToHost, st));
-            QS3_CUDA(cudaStreamSynchronize(st));
-            norm2 = v.x * v.x + v.y * v.y;
-        }
-        Ph.resize(N);
-        std::vector<double2> hz(N);
-        QS3_CUDA(cudaMemcpyAsync(hz.data(), hzz.p, N * 16, cudaMemcpyDeviceToHost, st));
-        QS3_CUDA(cudaMemcpyAsync(Ph.data(), hpm.p, N * 16, cudaMemcpyDeviceToHost, st));
-        QS3_CUDA(cudaStreamSynchronize(st));
-        Ch.resize(N);
-        for (int d = 0; d < N; ++d) Ch[d] = hz[d].x;
+    const int ndl = (int)dl.size(), nch = (ndl + CD - 1) / CD;
+    const int nb = ks ? (int)std::max<uint64_t>(1, std::min<uint64_t>((B.dims[s] + NTHREADS - 1) / NTHREADS,
+                                                                     (uint64_t)std::max(8, 4096 / std::max(nch, 1))))
+                      : 0;
+    // device memory, in doubles: results (correlation functions of k-sectors:
+    // 3 N + 1; else the norm; then S(q)), block sums or G and M, positions,
+    // wave vectors, displacements
+    const size_t ncf = ks ? 3 * (size_t)N + 1 : 1, nres = ncf + 2 * (size_t)nq;
+    const size_t nacc = ks ? (size_t)nch * nb * 3 * CD : (want_pm ? 2 : 1) * (size_t)N * N;
+    const size_t nin = 3 * (size_t)(nq > 0 ? N : 0) + 3 * (size_t)nq;
+    DevBuf buf;
+    QS3_TRY(buf.alloc((nres + nacc + nin) * 8 + (size_t)ndl * 4));
+    double *res = buf.as<double>(), *acc = res + nres, *in = acc + nacc;
+    int *ddl = (int *)(in + nin);
+    std::vector<double> hin(nin + (ndl + 1) / 2);
+    if (nq > 0) {
+        for (int r = 0; r < N; ++r) site_pos(B, r, &hin[3 * (size_t)r]);
+        std::memcpy(&hin[3 * (size_t)N], q, 3 * (size_t)nq * 8);
     }
+    if (ndl) std::memcpy(hin.data() + nin, dl.data(), (size_t)ndl * 4);
+    if (nin * 8 + (size_t)ndl * 4 > 0)
+        QS3_CUDA(cudaMemcpyAsync(in, hin.data(), nin * 8 + (size_t)ndl * 4, cudaMemcpyHostToDevice, st));
+    std::vector<double> hres(nres, 0.0);
+    if (nd == 0) {
+        // the vacuum: no down spin anywhere
+        double2 v = make_double2(0.0, 0.0);
+        QS3_CUDA(cudaMemcpyAsync(&v, gs, ks ? 16 : 8, cudaMemcpyDeviceToHost, st));
+        QS3_CUDA(cudaStreamSynchronize(st));
+        hres[ncf - 1] = v.x * v.x + v.y * v.y;
+        if (ks) {
+            for (int d = 0; d < N; ++d) hres[d] = 0.25;
+            hres[N] = 1.0;
+        } else {
+            QS3_CUDA(cudaMemsetAsync(acc, 0, nacc * 8, st));
+        }
+        QS3_CUDA(cudaMemcpyAsync(res, hres.data(), ncf * 8, cudaMemcpyHostToDevice, st));
+    } else if (ks) {
+        QS3_TRY(dispatch_corr_k(B, s, (const double2 *)gs, want_pm, ddl, ndl, nb, acc, st));
+        k_corr_sum<<<(ndl + 7) / 8, NTHREADS, 0, st>>>(acc, nb, ddl, ndl, N, nd, B.L[0], B.L[1], B.L[2], res);
+        QS3_LAUNCHED();
+    } else {
+        QS3_CUDA(cudaMemsetAsync(res, 0, 8, st));
+        QS3_CUDA(cudaMemsetAsync(acc, 0, nacc * 8, st));
+        QS3_TRY(dispatch_corr_u1(B, (const double *)gs, want_pm, acc, acc + (size_t)N * N, res, st));
+    }
+    if (nq > 0) {
+        const size_t smem = (size_t)N * sizeof(double2);
+        const double *p = in, *qd = in + 3 * (size_t)N;
+        double *out = res + ncf;
+        if (ks) {
+            QS3_CUDA(cudaFuncSetAttribute(k_sq<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+            k_sq<true><<<nq, NTHREADS, smem, st>>>(N, B.L[0], B.L[1], B.L[2], p, qd, res, nullptr, nullptr, nullptr,
+                                                   want_pm ? 1 : 0, out);
+        } else {
+            QS3_CUDA(cudaFuncSetAttribute(k_sq<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+            k_sq<false><<<nq, NTHREADS, smem, st>>>(N, 1, 1, 1, p, qd, nullptr, acc, acc + (size_t)N * N, res,
+                                                    want_pm ? 1 : 0, out);
+        }
+        QS3_LAUNCHED();
+    }
+    // site-resolved sums for the pairs and the local values
+    std::vector<double> hacc;
+    if (!ks && (npairs > 0 || szl)) {
+        hacc.resize(npairs > 0 ? nacc : (size_t)N * N);
+        QS3_CUDA(cudaMemcpyAsync(hacc.data(), acc, hacc.size() * 8, cudaMemcpyDeviceToHost, st));
+    }
+    QS3_CUDA(cudaMemcpyAsync(hres.data(), res, nres * 8, cudaMemcpyDeviceToHost, st));
+    QS3_CUDA(cudaStreamSynchronize(st));
+    const double norm2 = hres[ncf - 1];
     if (!(norm2 > 0.0)) return set_err(QS3_ERR_INVALID_ARG, "state has zero norm");
     auto disp = [&](int i, int j) {   // displacement index of j - i
         const int Lx = B.L[0], Ly = B.L[1], Lz = B.L[2];
@@ -816,42 +994,32 @@ static int correlations(Basis &B, int s, const void *gs, int npairs, const int *
         dx += dx < 0 ? Lx : 0; dy += dy < 0 ? Ly : 0; dz += dz < 0 ? Lz : 0;
         return dx + Lx * (dy + Ly * dz);
     };
-    auto n_i = [&](int i) { return B.has_k ? (double)nd / N : Gh[(size_t)i * N + i] / norm2; };
-    auto zz = [&](int i, int j) -> double {
-        if (i == j) return 0.25;
-        if (B.has_k) return 0.25 - (double)nd / N + Ch[disp(i, j)] / (N * norm2);
-        return 0.25 - 0.5 * (n_i(i) + n_i(j)) + Gh[(size_t)i * N + j] / norm2;
-    };
-    auto pm = [&](int i, int j) -> std::complex<double> {
-        if (i == j) return 1.0 - n_i(i);
-        if (B.has_k) { const double2 v = Ph[disp(i, j)]; return std::complex<double>(v.x, v.y) / norm2; }
-        const double2 v = Mh[(size_t)i * N + j];
-        return std::complex<double>(v.x, v.y) / norm2;
-    };
+    auto n_i = [&](int i) { return ks ? (double)nd / N : hacc[(size_t)i * N + i] / norm2; };
     for (int p = 0; p < npairs; ++p) {
         const int i = pairs[2 * p], j = pairs[2 * p + 1];
-        if (szsz) szsz[p] = zz(i, j);
-        if (spsm) { const auto v = pm(i, j); spsm[2 * p] = v.real(); spsm[2 * p + 1] = v.imag(); }
+        double zz = 0.25, pr = 0.0, pi = 0.0;
+        if (ks) {
+            const int d = disp(i, j);
+            zz = hres[d];
+            pr = hres[N + 2 * d];
+            pi = hres[N + 2 * d + 1];
+        } else if (i != j) {
+            zz = 0.25 - 0.5 * (n_i(i) + n_i(j)) + hacc[(size_t)i * N + j] / norm2;
+            if (want_pm) pr = hacc[(size_t)N * N + (size_t)i * N + j] / norm2;
+        } else {
+            pr = 1.0 - n_i(i);
+        }
+        if (szsz) szsz[p] = zz;
+        if (spsm) {
+            spsm[2 * p] = pr;
+            spsm[2 * p + 1] = pi;
+        }
     }
     if (szl)
         for (int i = 0; i < N; ++i) szl[i] = 0.5 - n_i(i);
-    // S(q) = (1/N) sum_{r,r'} e^{iq.(R_r - R_r')} <O_r O_r'>
-    std::vector<double> P((size_t)3 * N);
-    for (int r = 0; r < N; ++r) site_pos(B, r, &P[3 * (size_t)r]);
     for (int n = 0; n < nq; ++n) {
-        std::vector<std::complex<double>> e(N);
-        for (int r = 0; r < N; ++r)
-            e[r] = std::exp(std::complex<double>(0.0, q[3 * n] * P[3 * r] + q[3 * n + 1] * P[3 * r + 1] +
-                                                           q[3 * n + 2] * P[3 * r + 2]));
-        std::complex<double> az = 0.0, ap = 0.0;
-        for (int i = 0; i < N; ++i)
-            for (int j = 0; j < N; ++j) {
-                const std::complex<double> f = e[i] * std::conj(e[j]);
-                if (sqz) az += f * zz(i, j);
-                if (sqp) ap += f * pm(i, j);
-            }
-        if (sqz) sqz[n] = az.real() / N;
-        if (sqp) sqp[n] = ap.real() / N;
+        if (sqz) sqz[n] = hres[ncf + 2 * (size_t)n];
+        if (sqp) sqp[n] = hres[ncf + 2 * (size_t)n + 1];
     }
     return QS3_OK;
 }
