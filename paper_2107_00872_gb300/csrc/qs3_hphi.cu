@@ -409,63 +409,21 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
     }
 }
 
-// The same product batched over sectors (all momenta of one basis share the
-// orbits and their hops; only the phases and the rows differ): one thread per
-// (orbit g, group of OSG sectors) unranks g's representative once, lists its
-// hop targets (orbit, translation, |Stab|) and its diagonal once, then forms
-// g's row in each sector of the group from them: per term one row lookup,
-// the digits of the target and its group exponent, the exact product with
-// the sector's phase digits and the row sum, as in k_hphi_x (whose output it
-// reproduces bit for bit: the terms come in the same order).  The hop lists
-// live in shared memory, maxh entries per thread.
-constexpr int OSG = 8;
-
-template <int ND>
-__global__ void __launch_bounds__(NTHREADS) k_hphi_o(LatView L, const SecView *__restrict__ secs, int S,
-                                                   const uint64_t *__restrict__ oreps,
-                                                   const uint8_t *__restrict__ ostab, uint32_t n_orb, int ngrp,
-                                                   const int4 *__restrict__ phdig, const double2 *__restrict__ phi,
-                                                   const int2 *__restrict__ dg, const int *__restrict__ ge,
-                                                   const int *__restrict__ chunk0, int nchunks, uint64_t D,
-                                                   const int *__restrict__ dx,
-                                                   double2 *__restrict__ psi, const int *__restrict__ active,
-                                                   int maxh) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t *sC = (uint64_t *)smem;
-    double *snorm = (double *)(sC + (L.nd + 3) * L.np1);
-    uint32_t *hl = (uint32_t *)(snorm + 18);                     // hop targets g2 << 12 | u
-    uint8_t *hs = (uint8_t *)(hl + (size_t)maxh * blockDim.x);     // their |Stab|
-    for (int i = threadIdx.x; i < (L.nd + 3) * L.np1; i += blockDim.x) sC[i] = L.binom[i];
-    if (threadIdx.x < 9) {
-        snorm[threadIdx.x] = sqrt((double)threadIdx.x);
-        snorm[9 + threadIdx.x] = threadIdx.x ? 1.0 / sqrt((double)threadIdx.x) : 0.0;
-    }
-    if (dx) {
-        dg += (uint64_t)(*dx) * 2 * D;
-        ge += (uint64_t)(*dx) * nchunks * XW;
-    }
-    __syncthreads();
-    const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= (uint64_t)n_orb * ngrp) return;
-    const uint32_t g = (uint32_t)(tid % n_orb);
-    const int grp = (int)(tid / n_orb);
-    const int s_lo = grp * OSG, s_hi = min(S, s_lo + OSG);
-    bool any = false;
-    for (int s = s_lo; s < s_hi; ++s) any |= (!active || active[s]) && __ldg(secs[s].t2 + g) >= 0;
-    if (!any) return;
-    uint32_t *my = hl + threadIdx.x;                             // entry h at my[h * blockDim.x]
-    uint8_t *mys = hs + threadIdx.x;
-    const uint64_t rank = __ldg(oreps + g);
-    int c[ND];
-    unrank(rank, sC, L.np1, c);
-    const int st_row = __ldg(ostab + g);
-    const double rs = snorm[9 + st_row];
-    double e = L.c0, dd = 0.0;
+// The hops of the representative c (rank0 `rank`) of an orbit, in the order
+// the row kernels visit them: targets g2 << 12 | u at my[h stride], their
+// |Stab| at mys[h stride]; returns their number, and in e, dd the diagonal's
+// site part and the J^z of its down-spin pairs (each met twice).
+template <int ND, typename R>
+__device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const int (&c)[ND],
+                                          const uint64_t *__restrict__ sC, const uint8_t *__restrict__ ostab,
+                                          uint32_t *my, uint8_t *mys, size_t stride, R &e, R &dd) {
+    e = diag_c0<R>(L);
+    dd = 0;
     int nh = 0;
 #pragma unroll 1
     for (int m = 0; m < ND; ++m) {
         const int i = pick(c, m);
-        e += diag_u<double>(L, i);
+        e += diag_u<R>(L, i);
         const int e0 = __ldg(L.adj_ptr + i), e1 = __ldg(L.adj_ptr + i + 1);
         const int lo = m > 0 ? pick(c, m > 0 ? m - 1 : 0) : -1;
         const int hi = m < ND - 1 ? pick(c, m < ND - 1 ? m + 1 : m) : L.np1;
@@ -478,7 +436,7 @@ __global__ void __launch_bounds__(NTHREADS) k_hphi_o(LatView L, const SecView *_
 #pragma unroll
                 for (int k = 0; k < ND; ++k) occ |= (c[k] == j);
                 if (occ) {
-                    dd += diag_jz<double>(L, q);
+                    dd += diag_jz<R>(L, q);
                     continue;
                 }
             }
@@ -493,12 +451,70 @@ __global__ void __launch_bounds__(NTHREADS) k_hphi_o(LatView L, const SecView *_
                 r2 = rank_of(tt, sC, L.np1);
             }
             const uint32_t ee = __ldg(L.orb + r2);
-            if ((ee >> 12) >= n_orb) continue;                   // never for a complete table
-            my[(size_t)nh * blockDim.x] = ee;
-            mys[(size_t)nh * blockDim.x] = __ldg(ostab + (ee >> 12));
+            if ((ee >> 12) >= L.n_orb) continue;                 // never for a complete table
+            my[nh * stride] = ee;
+            mys[nh * stride] = __ldg(ostab + (ee >> 12));
             ++nh;
         }
     }
+    return nh;
+}
+
+// H Phi batched over sectors (all momenta of one basis share the orbits and
+// their hops; only the phases and the rows differ): one thread per (orbit g,
+// group of osg sectors) unranks g's representative once, lists its hop
+// targets (orbit, translation, |Stab|) and its diagonal once in shared
+// memory (maxh entries per thread), then forms g's row in each sector of the
+// group from them.  osg is 8 where that still leaves two rows of blocks per
+// SM, else 4, 2 or 1 (orb_group).
+constexpr int OSG = 8;
+
+// the binary64 engine's product on the integer units: per term one row
+// lookup, the digits of the target and its group exponent, the exact product
+// with the sector's phase digits and the row sum, as in k_hphi_x (whose
+// output it reproduces bit for bit: the terms come in the same order)
+template <int ND>
+__global__ void __launch_bounds__(NTHREADS) k_hphi_o(LatView L, const SecView *__restrict__ secs, int S,
+                                                   const uint64_t *__restrict__ oreps,
+                                                   const uint8_t *__restrict__ ostab, uint32_t n_orb, int ngrp, int osg,
+                                                   const int4 *__restrict__ phdig, const double2 *__restrict__ phi,
+                                                   const int2 *__restrict__ dg, const int *__restrict__ ge,
+                                                   const int *__restrict__ chunk0, int nchunks, uint64_t D,
+                                                   const int *__restrict__ dx,
+                                                   double2 *__restrict__ psi, const int *__restrict__ active,
+                                                   int maxh) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t *sC = (uint64_t *)smem;
+    double *snorm = (double *)(sC + (L.nd + 3) * L.np1);
+    uint32_t *hl = (uint32_t *)(snorm + 18);                     // hop targets g2 << 12 | u
+    uint8_t *hs = (uint8_t *)(hl + (size_t)maxh * blockDim.x);     // their |Stab|
+    stage_tables(L, sC, nullptr);
+    if (threadIdx.x < 9) {
+        snorm[threadIdx.x] = sqrt((double)threadIdx.x);
+        snorm[9 + threadIdx.x] = threadIdx.x ? 1.0 / sqrt((double)threadIdx.x) : 0.0;
+    }
+    if (dx) {
+        dg += (uint64_t)(*dx) * 2 * D;
+        ge += (uint64_t)(*dx) * nchunks * XW;
+    }
+    __syncthreads();
+    const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (tid >= (uint64_t)n_orb * ngrp) return;
+    const uint32_t g = (uint32_t)(tid % n_orb);
+    const int grp = (int)(tid / n_orb);
+    const int s_lo = grp * osg, s_hi = min(S, s_lo + osg);
+    bool any = false;
+    for (int s = s_lo; s < s_hi; ++s) any |= (!active || active[s]) && __ldg(secs[s].t2 + g) >= 0;
+    if (!any) return;
+    uint32_t *my = hl + threadIdx.x;                             // entry h at my[h * blockDim.x]
+    uint8_t *mys = hs + threadIdx.x;
+    const uint64_t rank = __ldg(oreps + g);
+    int c[ND];
+    unrank(rank, sC, L.np1, c);
+    const int st_row = __ldg(ostab + g);
+    const double rs = snorm[9 + st_row];
+    double e, dd;
+    const int nh = orbit_hops<ND, double>(L, rank, c, sC, ostab, my, mys, blockDim.x, e, dd);
     const double ed = e + 0.5 * dd;
     const double juni = L.jh_uniform;
     for (int s = s_lo; s < s_hi; ++s) {
@@ -563,6 +579,96 @@ __global__ void __launch_bounds__(NTHREADS) k_hphi_o(LatView L, const SecView *_
         out.x = fma(ed, x0.x, juni * acch.x);
         out.y = fma(ed, x0.y, juni * acch.y);
         psi[off + (uint32_t)row] = out;
+    }
+}
+
+// the same batching in the vector's own arithmetic (complex128 / complex64
+// FMAs; one hop amplitude on every bond): output identical bit for bit to
+// k_hphi.  Bound by the four fp64 FMAs of a term in complex128; against
+// k_hphi the hop list, the ranks, the site part of the diagonal and its
+// occupied pairs (fp64 additions that any lane made the whole warp take) are
+// paid once per group of sectors instead of per row.
+template <int ND, typename VT>
+__global__ void __launch_bounds__(NTHREADS) k_hphi_of(LatView L, const SecView *__restrict__ secs, int S,
+                                                    const uint64_t *__restrict__ oreps,
+                                                    const uint8_t *__restrict__ ostab, uint32_t n_orb, int ngrp,
+                                                    int osg, const VT *__restrict__ phi, VT *__restrict__ psi,
+                                                    const int *__restrict__ active, int maxh) {
+    using R = typename VTr<VT>::R;
+    using CT = typename VTr<VT>::C;
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t *sC = (uint64_t *)smem;
+    R *snorm = (R *)(sC + (L.nd + 3) * L.np1);                    // 18 of R in the room of 18 doubles
+    uint32_t *hl = (uint32_t *)((double *)snorm + 18);
+    uint8_t *hs = (uint8_t *)(hl + (size_t)maxh * blockDim.x);
+    stage_tables(L, sC, nullptr);
+    if (threadIdx.x < 9) {
+        snorm[threadIdx.x] = (R)sqrt((double)threadIdx.x);
+        snorm[9 + threadIdx.x] = threadIdx.x ? (R)(1.0 / sqrt((double)threadIdx.x)) : (R)0;
+    }
+    __syncthreads();
+    const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (tid >= (uint64_t)n_orb * ngrp) return;
+    const uint32_t g = (uint32_t)(tid % n_orb);
+    const int s_lo = (int)(tid / n_orb) * osg, s_hi = min(S, s_lo + osg);
+    bool any = false;
+    for (int s = s_lo; s < s_hi; ++s) any |= (!active || active[s]) && __ldg(secs[s].t2 + g) >= 0;
+    if (!any) return;
+    uint32_t *my = hl + threadIdx.x;
+    uint8_t *mys = hs + threadIdx.x;
+    const uint64_t rank = __ldg(oreps + g);
+    int c[ND];
+    unrank(rank, sC, L.np1, c);
+    const int st_row = __ldg(ostab + g);
+    const R rs = snorm[9 + st_row];
+    R e, dd;
+    const int nh = orbit_hops<ND, R>(L, rank, c, sC, ostab, my, mys, blockDim.x, e, dd);
+    const R ed = e + (R)0.5 * dd, juni = (R)L.jh_uniform;
+    for (int s = s_lo; s < s_hi; ++s) {
+        if (active && !active[s]) continue;
+        const int32_t *t2 = secs[s].t2;
+        const int32_t row = __ldg(t2 + g);
+        if (row < 0) continue;
+        const VT *__restrict__ ph_in = phi + secs[s].off;
+        const CT *__restrict__ ph = phase_table<CT>(secs[s]);
+        CT acch;
+        acch.x = 0; acch.y = 0;
+        // four terms at a time: their row lookups, then their gathers, are in
+        // flight together; the terms are added in list order
+        for (int h0 = 0; h0 < nh; h0 += 4) {
+            uint32_t ee[4];
+            int32_t r2[4];
+            VT v[4];
+            CT p[4];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const bool in = h0 + b < nh;
+                ee[b] = in ? my[(size_t)(h0 + b) * blockDim.x] : 0u;
+                r2[b] = in ? __ldg(t2 + (ee[b] >> 12)) : -1;
+            }
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                if (r2[b] >= 0) {
+                    v[b] = ph_in[r2[b]];
+                    p[b] = ph[ee[b] & 4095u];
+                }
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                if (r2[b] < 0) continue;
+                const int st = mys[(size_t)(h0 + b) * blockDim.x];
+                if (st != st_row) {
+                    const R f = snorm[st] * rs;
+                    p[b].x *= f;
+                    p[b].y *= f;
+                }
+                acc_add(acch, p[b], v[b]);
+            }
+        }
+        CT acc;
+        acc.x = 0; acc.y = 0;
+        madd_r(acc, juni, acch);
+        madd_r(acc, ed, ph_in[row]);
+        store(psi + secs[s].off + row, acc);
     }
 }
 
@@ -826,27 +932,80 @@ static int hphix_nd(Basis &B, const double2 *phi, const int2 *dg, const int *ge,
     return QS3_OK;
 }
 
+// sectors per thread of the orbit-batched kernels: as many (up to OSG) as
+// leave two resident rows of 2048 threads per SM
+static int orb_group(const Basis &B) {
+    int g = OSG;
+    while (g > 1 && B.n_orb * (uint64_t)((B.S + g - 1) / g) < 2ull * 2048ull * (uint64_t)num_sms()) g >>= 1;
+    return g;
+}
+// shared memory of the hop lists and tables; 0: too many hops per row
+static size_t orb_smem(const Basis &B, int maxh) {
+    const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8 + 18 * 8 + (size_t)maxh * NTHREADS * 5;
+    return smem <= (size_t)MAX_DYN_SMEM ? smem : 0;
+}
+
 template <int ND>
 static int hphio_nd(Basis &B, const double2 *phi, const int2 *dg, const int *ge, const int *dx,
                     double2 *psi, cudaStream_t st, const int *active) {
     const int maxh = std::max(1, B.nd * B.max_degree);
-    const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8 + 18 * 8 + (size_t)maxh * NTHREADS * 5;
-    if (smem > (size_t)MAX_DYN_SMEM) return set_err(QS3_ERR_OVERFLOW, "hop lists of %d entries per row", maxh);
+    const size_t smem = orb_smem(B, maxh);
+    if (!smem) return set_err(QS3_ERR_OVERFLOW, "hop lists of %d entries per row", maxh);
     static std::atomic<int> attr{0};
     if (attr.load(std::memory_order_acquire) == 0) {
         QS3_CUDA(cudaFuncSetAttribute(k_hphi_o<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
         attr.store(1, std::memory_order_release);
     }
-    const int ngrp = (B.S + OSG - 1) / OSG;
+    const int osg = orb_group(B), ngrp = (B.S + osg - 1) / osg;
     const uint64_t nthr = B.n_orb * (uint64_t)ngrp;
     if (nthr == 0) return QS3_OK;
     const int grid = (int)((nthr + NTHREADS - 1) / NTHREADS);
     k_hphi_o<ND><<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.S, B.d_oreps.as<uint64_t>(),
-                                                B.d_ostab.as<uint8_t>(), (uint32_t)B.n_orb, ngrp,
+                                                B.d_ostab.as<uint8_t>(), (uint32_t)B.n_orb, ngrp, osg,
                                                 B.d_phdig.as<int4>(), phi, dg, ge, B.d_chunk0.as<int>(), B.nchunks,
                                                 B.total, dx, psi, active, maxh);
     QS3_LAUNCHED();
     return QS3_OK;
+}
+
+// the orbit-batched FMA kernel serves bases of several sectors with the
+// representative table and one hop amplitude whose hop lists fit
+static bool hphi_of_ok(const Basis &B) {
+    return B.has_k && B.S >= 2 && B.lv.orb && B.d_oreps.p && B.lv.jh_uniform != 0.0 &&
+           orb_smem(B, std::max(1, B.nd * B.max_degree)) > 0;
+}
+
+template <int ND, typename VT>
+static int hphiof_nd(Basis &B, const void *phi, void *psi, cudaStream_t st, const int *active, int dt) {
+    static std::atomic<unsigned long long> cache{0};
+    const int maxh = std::max(1, B.nd * B.max_degree);
+    const size_t smem = orb_smem(B, maxh);
+    int grid = 1, occ = 1;
+    QS3_TRY(launch_rows(k_hphi_of<ND, VT>, B, smem, cache, &grid, &occ));
+    if (B.tune_hphi[dt] == 0) B.tune_hphi[dt] = occ;             // the grid covers all orbits: nothing to tune
+    const int osg = orb_group(B), ngrp = (B.S + osg - 1) / osg;
+    const uint64_t nthr = B.n_orb * (uint64_t)ngrp;
+    if (nthr == 0) return QS3_OK;
+    k_hphi_of<ND, VT><<<(int)((nthr + NTHREADS - 1) / NTHREADS), NTHREADS, smem, st>>>(
+        B.lv, B.d_secs.as<SecView>(), B.S, B.d_oreps.as<uint64_t>(), B.d_ostab.as<uint8_t>(), (uint32_t)B.n_orb, ngrp,
+        osg, (const VT *)phi, (VT *)psi, active, maxh);
+    QS3_LAUNCHED();
+    return QS3_OK;
+}
+
+template <typename VT>
+static int hphiof_vt(Basis &B, const void *phi, void *psi, cudaStream_t st, const int *a, int dt) {
+    switch (B.nd) {
+        case 1: return hphiof_nd<1, VT>(B, phi, psi, st, a, dt);
+        case 2: return hphiof_nd<2, VT>(B, phi, psi, st, a, dt);
+        case 3: return hphiof_nd<3, VT>(B, phi, psi, st, a, dt);
+        case 4: return hphiof_nd<4, VT>(B, phi, psi, st, a, dt);
+        case 5: return hphiof_nd<5, VT>(B, phi, psi, st, a, dt);
+        case 6: return hphiof_nd<6, VT>(B, phi, psi, st, a, dt);
+        case 7: return hphiof_nd<7, VT>(B, phi, psi, st, a, dt);
+        case 8: return hphiof_nd<8, VT>(B, phi, psi, st, a, dt);
+        default: return set_err(QS3_ERR_INVALID_ARG, "n_down %d", B.nd);
+    }
 }
 
 bool hphi_x_ok(const Basis &B) {
@@ -909,6 +1068,10 @@ int hphi_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t
     }
     if (B.has_k) {
         if (B.stored_terms && (dt == QS3_C64 || dt == QS3_C128)) return hphi_stored_launch(B, dt, phi, psi, st, active);
+        if (hphi_of_ok(B)) {
+            if (dt == QS3_C64) return hphiof_vt<float2>(B, phi, psi, st, active, dt);
+            if (dt == QS3_C128) return hphiof_vt<double2>(B, phi, psi, st, active, dt);
+        }
         if (dt == QS3_C64) return hphi_vt<float2, true>(B, phi, psi, st, active);
         if (dt == QS3_C128) return hphi_vt<double2, true>(B, phi, psi, st, active);
     } else {
