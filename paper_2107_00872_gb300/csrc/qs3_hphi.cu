@@ -263,10 +263,9 @@ struct RowAcc {
     long long re = 0, im = 0;
     int r = -100000;
 };
+// x 2^-d rounded to nearest, 0 <= d <= 63, |x| < 2^62 (0 for d = 63)
 __device__ __forceinline__ long long rshift_round(long long x, int d) {
-    if (d <= 0) return x;
-    if (d > 62) return 0;
-    return (x + (1ll << (d - 1))) >> d;
+    return (x + (long long)((1ull << d) >> 1)) >> d;
 }
 __device__ __forceinline__ void row_add(RowAcc &a, long long tr, long long ti, int em) {
     if (em > a.r) {
@@ -275,7 +274,7 @@ __device__ __forceinline__ void row_add(RowAcc &a, long long tr, long long ti, i
         a.im = rshift_round(a.im, d);
         a.r = em;
     }
-    const int d = a.r - em;
+    const int d = min(a.r - em, 63);
     a.re += rshift_round(tr, d);
     a.im += rshift_round(ti, d);
 }
@@ -474,7 +473,7 @@ constexpr int OSG = 8;
 // with the sector's phase digits and the row sum, as in k_hphi_x (whose
 // output it reproduces bit for bit: the terms come in the same order)
 template <int ND>
-__global__ void __launch_bounds__(NTHREADS) k_hphi_o(LatView L, const SecView *__restrict__ secs, int S,
+__global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView *__restrict__ secs, int S,
                                                    const uint64_t *__restrict__ oreps,
                                                    const uint8_t *__restrict__ ostab, uint32_t n_orb, int ngrp, int osg,
                                                    const int4 *__restrict__ phdig, const double2 *__restrict__ phi,
@@ -587,9 +586,12 @@ __global__ void __launch_bounds__(NTHREADS) k_hphi_o(LatView L, const SecView *_
 // k_hphi.  Bound by the four fp64 FMAs of a term in complex128; against
 // k_hphi the hop list, the ranks, the site part of the diagonal and its
 // occupied pairs (fp64 additions that any lane made the whole warp take) are
-// paid once per group of sectors instead of per row.
+// paid once per group of sectors instead of per row.  10x10, N_down = 4, all
+// 100 momenta: 510 us at four resident blocks (64 registers), 877 us at three,
+// 525 at five, against 1099 us of k_hphi; the terms' 4 FMAs alone take 490 us
+// of the fp64 pipe.
 template <int ND, typename VT>
-__global__ void __launch_bounds__(NTHREADS) k_hphi_of(LatView L, const SecView *__restrict__ secs, int S,
+__global__ void __launch_bounds__(NTHREADS, 4) k_hphi_of(LatView L, const SecView *__restrict__ secs, int S,
                                                     const uint64_t *__restrict__ oreps,
                                                     const uint8_t *__restrict__ ostab, uint32_t n_orb, int ngrp,
                                                     int osg, const VT *__restrict__ phi, VT *__restrict__ psi,
