@@ -783,6 +783,14 @@ __global__ void k_phase_tables(int S, int N, int G, int Lx, int Ly, int Lz, cons
     phdf[i] = make_float4(ch, __double2float_rn(cs - (double)ch), sh, __double2float_rn(sn - (double)sh));
 }
 
+__global__ void k_roots(int G, double2 *__restrict__ w) {
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= G) return;
+    double sn, cs;
+    sincospi(-2.0 * (double)n / (double)G, &sn, &cs);
+    w[n] = make_double2(cs, sn);
+}
+
 // ---------------------------------------------------------------- host side
 
 static bool binom_table(int N, int rows, std::vector<uint64_t> &t, uint64_t *cnd, int nd) {
@@ -1051,6 +1059,9 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
         k_phase_tables<<<(tot + 255) / 256, 256>>>(nsec, N, B.ncell, B.L[0], B.L[1], B.L[2], B.d_secs.as<int>(),
                                                    B.d_ph64.as<double2>(), B.d_ph32.as<float2>(),
                                                    B.d_phdf.as<float4>());
+        QS3_LAUNCHED();
+        QS3_TRY(B.d_roots.alloc((size_t)B.ncell * sizeof(double2)));
+        k_roots<<<(B.ncell + 255) / 256, 256>>>(B.ncell, B.d_roots.as<double2>());
         QS3_LAUNCHED();
         QS3_CUDA(cudaDeviceSynchronize());
     }

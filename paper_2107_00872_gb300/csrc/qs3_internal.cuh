@@ -161,6 +161,7 @@ struct Basis {
     DevBuf d_adj_pad, d_adj_jz_pad;         // fixed-width adjacency (LatView::adj_pad)
     DevBuf d_sigma, d_stab, d_pinfo, d_sub;  // every sector's lists, one after another
     DevBuf d_ph64, d_ph32, d_phdf;          // S x N per-site phase tables (k-sectors)
+    DevBuf d_roots;                         // e^{-2 pi i n / ncell}, n < ncell (k-sectors)
     DevBuf d_secs, d_tile0, d_chunk0;
     LatView lv{};
     std::vector<SecView> secs;

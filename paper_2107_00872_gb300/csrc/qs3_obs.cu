@@ -461,6 +461,119 @@ __global__ void __launch_bounds__(NTHREADS) k_smq(LatView Ls, SecView svs, SecVi
     }
 }
 
+// The same with the source's representative table, on lattices whose site
+// positions are the coordinates: S^-_q (UP = false: the source states b \ {s},
+// s in b) and S^+_q (UP: b + {s}, s not in b).  A term costs a rank, two table
+// loads and four fp64 FMAs: both of its phases, e^{ik.u} and e^{-iq.R_s}, are
+// ncell-th roots of unity, so their exponents are added as integers and one
+// table entry multiplies phi (the search, two or three complex phase products
+// and the norm ratio's two square-root products per term made 221 us of S^-_q
+// on the 10x10 lattice, N_down 4 -> 5, 752,875 rows).
+// bytes: binomial rows, roots, exponents
+static size_t root_smem_bytes(const Basis &B) {
+    return (size_t)(B.nd + 3) * (B.N + 1) * 8 + 8 + (size_t)B.ncell * 16 + (size_t)B.N * 4;
+}
+// S^alpha_q takes the table kernel: one spin per cell, coordinates as positions
+static bool root_ok(const Basis &S) {
+    return S.has_k && S.lv.orb && S.nd > 0 && S.nsub == 1 && S.pos.empty() && S.ncell <= 4096 &&
+           root_smem_bytes(S) <= (size_t)MAX_DYN_SMEM;
+}
+
+template <int ND, bool UP>
+__global__ void __launch_bounds__(NTHREADS, 4) k_sq_t(LatView Ls, SecView svs, SecView svd, int qx, int qy, int qz,
+                                                      const double2 *__restrict__ roots, double inv_sqrt_n,
+                                                      const double2 *__restrict__ phi, double2 *__restrict__ psi) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int nC = (Ls.nd + 3) * Ls.np1, G = Ls.ncell, np1 = Ls.np1;
+    uint64_t *sC = (uint64_t *)smem;
+    double2 *w = (double2 *)(sC + nC + (nC & 1));
+    uint32_t *ns = (uint32_t *)(w + G);
+    stage_tables(Ls, sC, nullptr);
+    for (int i = threadIdx.x; i < G; i += blockDim.x) {
+        w[i] = roots[i];
+        const uint32_t p = Ls.xyz[i];
+        const int x = (int)(p & 2047u) * (G / Ls.L[0]), y = (int)((p >> 11) & 2047u) * (G / Ls.L[1]),
+                  z = (int)(p >> 22) * (G / Ls.L[2]);
+        const uint32_t k = (uint32_t)((svs.K[0] * (long long)x + svs.K[1] * (long long)y + svs.K[2] * (long long)z) % G);
+        const uint32_t q = (uint32_t)((qx * (long long)x + qy * (long long)y + qz * (long long)z) % G);
+        ns[i] = k | (q << 16);
+    }
+    __shared__ double snorm[18];
+    if (threadIdx.x < 9) {
+        snorm[threadIdx.x] = sqrt((double)threadIdx.x);
+        snorm[9 + threadIdx.x] = threadIdx.x ? 1.0 / sqrt((double)threadIdx.x) : 0.0;
+    }
+    __syncthreads();
+    for (uint64_t row = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; row < svd.dim;
+         row += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t rank = __ldg(svd.sigma + row);
+        int c[ND];
+        unrank(rank, sC, np1, c);
+        const int st_row = __ldg(svd.stab + row);
+        double2 acc = make_double2(0.0, 0.0);
+        // the source states of up to TB sites s at a time
+        constexpr int TB = UP ? 4 : ND;
+        const int nt = UP ? Ls.N : ND;
+#pragma unroll 1
+        for (int t0 = 0; t0 < nt; t0 += TB) {
+            uint32_t e[TB], q[TB];
+            int32_t r[TB];
+#pragma unroll
+            for (int b = 0; b < TB; ++b) {
+                const int t = t0 + b;
+                int s = t;
+                bool ok = t < nt;
+                uint64_t r2 = 0;
+                if constexpr (UP) {
+                    int p = 0;
+#pragma unroll
+                    for (int k = 0; k < ND; ++k) {
+                        ok &= c[k] != s;
+                        const bool below = c[k] < s;
+                        p += below;
+                        r2 += sC[(below ? k + 1 : k + 2) * np1 + c[k]];
+                    }
+                    if (ok) r2 += sC[(p + 1) * np1 + s];
+                } else {
+                    s = c[b];
+#pragma unroll
+                    for (int k = 0; k < ND; ++k)
+                        if (k != b) r2 += sC[(k < b ? k + 1 : k) * np1 + c[k]];
+                }
+                e[b] = ok ? __ldg(Ls.orb + r2) : 0xffffffffu;
+                q[b] = ok ? ns[s] >> 16 : 0u;
+            }
+#pragma unroll
+            for (int b = 0; b < TB; ++b) r[b] = (e[b] >> 12) < Ls.n_orb ? __ldg(svs.t2 + (e[b] >> 12)) : -1;
+            double2 x[TB];
+            int st[TB];
+#pragma unroll
+            for (int b = 0; b < TB; ++b)
+                if (r[b] >= 0) {
+                    x[b] = phi[r[b]];
+                    st[b] = __ldg(svs.stab + r[b]);
+                }
+#pragma unroll
+            for (int b = 0; b < TB; ++b) {
+                if (r[b] < 0) continue;
+                uint32_t n = (ns[e[b] & 4095u] & 0xffffu) + q[b];
+                n -= n >= (uint32_t)G ? (uint32_t)G : 0u;
+                double2 p = w[n];
+                if (st[b] != st_row) {
+                    const double f = snorm[st[b]] * snorm[9 + st_row];
+                    p.x *= f;
+                    p.y *= f;
+                }
+                acc.x = fma(p.x, x[b].x, acc.x);
+                acc.x = fma(-p.y, x[b].y, acc.x);
+                acc.y = fma(p.x, x[b].y, acc.y);
+                acc.y = fma(p.y, x[b].x, acc.y);
+            }
+        }
+        psi[row] = make_double2(acc.x * inv_sqrt_n, acc.y * inv_sqrt_n);
+    }
+}
+
 // source N_down = 0 (the vacuum, |Stab| = N, momentum 0): psi'_b = N^{-1/2} sqrt(N / |Stab b|) e^{-iq.R} phi_0
 __global__ void k_smq_vac(SecView svd, int ks, int N, const double2 *__restrict__ phsite,
                           const double2 *__restrict__ phi, double2 *__restrict__ psi) {
@@ -670,6 +783,22 @@ static int corr_k_nd(Basis &B, int s, const double2 *phi, bool pm, const int *dl
     return QS3_OK;
 }
 
+// Q reduced into [0, L)
+static void reduced_q(const Basis &S, const int *Q, int (&q)[3]) {
+    for (int a = 0; a < 3; ++a) q[a] = S.L[a] > 0 ? (int)(((long long)Q[a] % S.L[a] + S.L[a]) % S.L[a]) : 0;
+}
+
+template <int ND, bool UP>
+static int sq_t_nd(Basis &S, int ss, Basis &Dd, int sd, const int *Q, const double2 *phi, double2 *psi, cudaStream_t st) {
+    int q[3];
+    reduced_q(S, Q, q);
+    QS3_CUDA(cudaFuncSetAttribute(k_sq_t<ND, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+    k_sq_t<ND, UP><<<grid_for(Dd.dims[sd]), NTHREADS, root_smem_bytes(S), st>>>(
+        S.lv, S.secs[ss], Dd.secs[sd], q[0], q[1], q[2], S.d_roots.as<double2>(), 1.0 / std::sqrt((double)S.N), phi, psi);
+    QS3_LAUNCHED();
+    return QS3_OK;
+}
+
 template <int ND>
 static int smq_nd(Basis &S, int ss, Basis &Dd, int sd, const double2 *phs, const double2 *phi, double2 *psi,
                   cudaStream_t st) {
@@ -691,6 +820,23 @@ static int smq_nd(Basis &S, int ss, Basis &Dd, int sd, const double2 *phs, const
         QS3_LAUNCHED();
         return QS3_OK;
     }
+}
+
+static int dispatch_sq_t(bool up, Basis &S, int ss, Basis &Dd, int sd, const int *Q, const double2 *phi, double2 *psi,
+                         cudaStream_t st) {
+#define QS3_SQT(n) (up ? sq_t_nd<n, true>(S, ss, Dd, sd, Q, phi, psi, st) : sq_t_nd<n, false>(S, ss, Dd, sd, Q, phi, psi, st))
+    switch (Dd.nd) {
+        case 1: return sq_t_nd<1, true>(S, ss, Dd, sd, Q, phi, psi, st);     // S^+ only: S^- starts from N_down > 0
+        case 2: return QS3_SQT(2);
+        case 3: return QS3_SQT(3);
+        case 4: return QS3_SQT(4);
+        case 5: return QS3_SQT(5);
+        case 6: return QS3_SQT(6);
+        case 7: return QS3_SQT(7);
+        case 8: return QS3_SQT(8);
+        default: return set_err(QS3_ERR_INVALID_ARG, "target n_down %d", Dd.nd);
+    }
+#undef QS3_SQT
 }
 
 static int dispatch_smq(Basis &S, int ss, Basis &Dd, int sd, const double2 *phs, const double2 *phi, double2 *psi,
@@ -744,6 +890,11 @@ int smq_launch(Basis &S, int ss, const void *phi, Basis &Dd, int sd, const int *
             if ((((long long)S.K[3 * ss + a] + Q[a]) % S.L[a] + S.L[a]) % S.L[a] != Dd.K[3 * sd + a])
                 return set_err(QS3_ERR_SYMMETRY, "target momentum is not K + Q (axis %d)", a);
     if (Dd.dims[sd] == 0) return QS3_OK;
+    if (S.dims[ss] > 0 && root_ok(S)) {
+        QS3_TRY(dispatch_sq_t(false, S, ss, Dd, sd, Q, (const double2 *)phi, (double2 *)psi, st));
+        QS3_CUDA(cudaStreamSynchronize(st));     // as the form below
+        return QS3_OK;
+    }
     std::vector<double2> ph = site_phases(S, Q);
     DevBuf dph;
     QS3_TRY(dph.upload(ph.data(), ph.size() * sizeof(double2)));
@@ -850,6 +1001,11 @@ int sq_launch(int op, Basis &S, int ss, const void *phi, Basis &Dd, int sd, cons
             if ((((long long)S.K[3 * ss + a] + Q[a]) % S.L[a] + S.L[a]) % S.L[a] != Dd.K[3 * sd + a])
                 return set_err(QS3_ERR_SYMMETRY, "target momentum is not K + Q (axis %d)", a);
     if (Dd.dims[sd] == 0) return QS3_OK;
+    if (op == QS3_OP_SPLUS && Dd.nd > 0 && S.dims[ss] > 0 && root_ok(S)) {
+        QS3_TRY(dispatch_sq_t(true, S, ss, Dd, sd, Q, (const double2 *)phi, (double2 *)psi, st));
+        QS3_CUDA(cudaStreamSynchronize(st));
+        return QS3_OK;
+    }
     std::vector<double2> ph = site_phases(S, Q);
     double2 hs = make_double2(0.0, 0.0);
     for (const double2 &v : ph) { hs.x += 0.5 * v.x; hs.y += 0.5 * v.y; }
@@ -1220,10 +1376,11 @@ static int smq_noalloc(Basis &S, int ss, const void *phi, Basis &Dd, int sd, con
         QS3_CUDA(cudaMemsetAsync(psi, 0, Dd.dims[sd] * 16, st));
         return QS3_OK;
     }
+    if (root_ok(S)) return dispatch_sq_t(false, S, ss, Dd, sd, Q, (const double2 *)phi, (double2 *)psi, st);
     // Q reduced into [0, L) first: the angle is unchanged and the integer
     // products of the phase kernel stay far below 2^63
     int Qr[3];
-    for (int a = 0; a < 3; ++a) Qr[a] = (int)(((long long)Q[a] % S.L[a] + S.L[a]) % S.L[a]);
+    reduced_q(S, Q, Qr);
     k_site_phases<<<(S.N + 255) / 256, 256, 0, st>>>(S.N, S.L[0], S.L[1], S.L[2], Qr[0], Qr[1], Qr[2], ph);
     QS3_LAUNCHED();
     if (S.nd == 0) {
