@@ -23,6 +23,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <utility>
 
@@ -50,9 +51,41 @@ void count_launch(long long n) { g_launches.fetch_add((unsigned long long)n, std
 const char *last_err() { return g_err; }
 
 void DevBuf::release() {
-    if (p) cudaFree(p);
+    if (p) {
+        if (pooled) cudaFreeAsync(p, st); else cudaFree(p);
+    }
     p = nullptr;
     n = 0;
+}
+
+// the pool of the current device (created at its first use, kept by the
+// process), nullptr where the device has none
+static std::mutex g_pool_mu;
+static cudaMemPool_t g_pool[64];
+static bool g_pool_tried[64];
+static cudaMemPool_t device_pool(bool create) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool_tried[dev] && create) {
+        g_pool_tried[dev] = true;
+        cudaMemPoolProps pr = {};
+        pr.allocType = cudaMemAllocationTypePinned;
+        pr.location.type = cudaMemLocationTypeDevice;
+        pr.location.id = dev;
+        cudaMemPool_t mp = nullptr;
+        if (cudaMemPoolCreate(&mp, &pr) == cudaSuccess) {
+            uint64_t keep = POOL_KEEP_BYTES;
+            cudaMemPoolSetAttribute(mp, cudaMemPoolAttrReleaseThreshold, &keep);
+            g_pool[dev] = mp;
+        }
+        cudaGetLastError();
+    }
+    return g_pool[dev];
+}
+void pool_trim() {
+    if (cudaMemPool_t mp = device_pool(false)) cudaMemPoolTrimTo(mp, 0);
+    cudaGetLastError();
 }
 
 // allocation fault injection (qs3_inject_alloc_failure): the number of
@@ -65,14 +98,27 @@ int take_wait_injection() {
     return 0;
 }
 
+// one allocation against the injected budget (true: refused)
+static bool refuse_alloc() {
+    for (long long v = g_alloc_budget.load(); v >= 0;) {
+        if (v == 0) return true;
+        if (g_alloc_budget.compare_exchange_weak(v, v - 1)) break;
+    }
+    return false;
+}
+
 int DevBuf::alloc(size_t bytes) {
     release();
+    pooled = false;
     if (bytes == 0) bytes = 16;
-    for (long long b = g_alloc_budget.load(); b >= 0;) {
-        if (b == 0) return set_err(QS3_ERR_OOM, "device allocation of %zu bytes refused (injected failure)", bytes);
-        if (g_alloc_budget.compare_exchange_weak(b, b - 1)) break;
-    }
+    if (refuse_alloc()) return set_err(QS3_ERR_OOM, "device allocation of %zu bytes refused (injected failure)", bytes);
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        // what the pool holds unused goes back first
+        cudaGetLastError();
+        pool_trim();
+        e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
         p = nullptr;
         cudaGetLastError();
@@ -83,9 +129,41 @@ int DevBuf::alloc(size_t bytes) {
     return QS3_OK;
 }
 
+int DevBuf::alloc(size_t bytes, cudaStream_t stream) {
+    cudaMemPool_t mp = bytes <= POOL_MAX_BYTES ? device_pool(true) : nullptr;
+    if (!mp) return alloc(bytes);
+    release();
+    if (bytes == 0) bytes = 16;
+    if (refuse_alloc()) return set_err(QS3_ERR_OOM, "device allocation of %zu bytes refused (injected failure)", bytes);
+    cudaError_t e = cudaMallocFromPoolAsync(&p, bytes, mp, stream);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        cudaStreamSynchronize(stream);
+        pool_trim();
+        e = cudaMallocFromPoolAsync(&p, bytes, mp, stream);
+    }
+    if (e != cudaSuccess) {
+        p = nullptr;
+        cudaGetLastError();
+        return set_err(e == cudaErrorMemoryAllocation ? QS3_ERR_OOM : QS3_ERR_CUDA, "cudaMallocFromPoolAsync(%zu): %s",
+                       bytes, cudaGetErrorString(e));
+    }
+    n = bytes;
+    pooled = true;
+    st = stream;
+    return QS3_OK;
+}
+
 int DevBuf::upload(const void *src, size_t bytes) {
     QS3_TRY(alloc(bytes));
     if (bytes) QS3_CUDA(cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice));
+    return QS3_OK;
+}
+
+int DevBuf::upload(const void *src, size_t bytes, cudaStream_t stream) {
+    QS3_TRY(alloc(bytes, stream));
+    // src is pageable: the call returns when it has been read
+    if (bytes) QS3_CUDA(cudaMemcpyAsync(p, src, bytes, cudaMemcpyHostToDevice, stream));
     return QS3_OK;
 }
 
@@ -227,10 +305,10 @@ static int enum_orbits(Basis &B, DevBuf &kout, DevBuf &vout, uint64_t &n) {
     QS3_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     n = count_orbits(B, hb);
     DevBuf cnt, kin, vin;
-    QS3_TRY(cnt.alloc(sizeof(unsigned long long)));
+    QS3_TRY(cnt.alloc(sizeof(unsigned long long), (cudaStream_t)0));
     QS3_CUDA(cudaMemset(cnt.p, 0, sizeof(unsigned long long)));
-    QS3_TRY(kin.alloc(n * 8));
-    QS3_TRY(vin.alloc(n));
+    QS3_TRY(kin.alloc(n * 8, (cudaStream_t)0));
+    QS3_TRY(vin.alloc(n, (cudaStream_t)0));
     // per lowest occupied place s0 of the cell: C(M - 1, ND - 1) candidates,
     // M = (cells) (nsub - s0); one spin per cell: C(N - 1, ND - 1)
     for (int s0 = 0; s0 < B.nsub; ++s0) {
@@ -251,7 +329,7 @@ static int enum_orbits(Basis &B, DevBuf &kout, DevBuf &vout, uint64_t &n) {
     QS3_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, tb, kin.as<unsigned long long>(), kout.as<unsigned long long>(),
                                              vin.as<uint8_t>(), vout.as<uint8_t>(), (int64_t)n, 0, bits));
     DevBuf tmp;
-    QS3_TRY(tmp.alloc(tb));
+    QS3_TRY(tmp.alloc(tb, (cudaStream_t)0));
     QS3_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, tb, kin.as<unsigned long long>(), kout.as<unsigned long long>(),
                                              vin.as<uint8_t>(), vout.as<uint8_t>(), (int64_t)n, 0, bits));
     uint64_t got = 0;
@@ -491,13 +569,13 @@ static int build_sectors_nd(Basis &B, DevBuf &keep_reps, DevBuf &keep_stab, uint
         QS3_TRY(B.d_sigma.alloc((uint64_t)S * n * 8));
         QS3_TRY(B.d_stab.alloc((uint64_t)S * n));
         DevBuf dK, pos, tmp, dends;
-        QS3_TRY(dends.alloc(((size_t)S + 1) * 4));
-        QS3_TRY(dK.upload(B.K.data(), B.K.size() * sizeof(int)));
+        QS3_TRY(dends.alloc(((size_t)S + 1) * 4, (cudaStream_t)0));
+        QS3_TRY(dK.upload(B.K.data(), B.K.size() * sizeof(int), (cudaStream_t)0));
         const int grp = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)S, (1ull << 27) / std::max<uint64_t>(n, 1)));
-        QS3_TRY(pos.alloc(((uint64_t)grp * n + 1) * 4));
+        QS3_TRY(pos.alloc(((uint64_t)grp * n + 1) * 4, (cudaStream_t)0));
         size_t tb = 0;
         QS3_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, pos.as<uint32_t>(), pos.as<uint32_t>(), (int64_t)((uint64_t)grp * n + 1)));
-        QS3_TRY(tmp.alloc(tb));
+        QS3_TRY(tmp.alloc(tb, (cudaStream_t)0));
         uint64_t off = 0;
         std::vector<uint32_t> ends;
         for (int s0 = 0; s0 < S; s0 += grp) {
@@ -540,9 +618,9 @@ static int build_index_nd(Basis &B) {
     for (auto &v : B.secs) v.pre2 = pre2;
     QS3_CUDA(cudaMemcpy(B.d_secs.p, B.secs.data(), B.secs.size() * sizeof(SecView), cudaMemcpyHostToDevice));
     DevBuf first, size, off, tmp;
-    QS3_TRY(first.alloc((uint64_t)S * (np + 1) * 4));
-    QS3_TRY(size.alloc((cnt + 1) * 4));
-    QS3_TRY(off.alloc((cnt + 1) * 4));
+    QS3_TRY(first.alloc((uint64_t)S * (np + 1) * 4, (cudaStream_t)0));
+    QS3_TRY(size.alloc((cnt + 1) * 4, (cudaStream_t)0));
+    QS3_TRY(off.alloc((cnt + 1) * 4, (cudaStream_t)0));
     const int g1 = (int)std::max<uint64_t>(1, std::min<uint64_t>((cnt + S + 255) / 256, 16384));
     const uint64_t *bin = B.d_binom.as<uint64_t>();
     const SecView *secs = B.d_secs.as<SecView>();
@@ -553,7 +631,7 @@ static int build_index_nd(Basis &B) {
     QS3_LAUNCHED();
     size_t tb = 0;
     QS3_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt + 1)));
-    QS3_TRY(tmp.alloc(tb));
+    QS3_TRY(tmp.alloc(tb, (cudaStream_t)0));
     QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, tb, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt + 1)));
     // at most rows / 2 + 1 buckets and the end per prefix
     const uint64_t most = B.total / 2 + 2 * cnt;
@@ -1126,6 +1204,7 @@ int qs3_basis_create(const qs3_lattice *lat, int32_t n_down, int32_t n_sectors, 
 int qs3_basis_destroy(qs3_basis_t b) {
     clear_err();
     delete b;
+    pool_trim();
     return QS3_OK;
 }
 

@@ -324,6 +324,34 @@ __global__ void __launch_bounds__(XT)
     if (lane == 0) ge[((uint64_t)j * nchunks + blockIdx.x) * XW + warp] = em;
 }
 
+// the digit image of one interleaved binary64 vector (slot 0 of dg, ge)
+template <typename VT>
+__global__ void __launch_bounds__(XT)
+    k_digitize_il(const VT *__restrict__ x, uint64_t D, typename DigT<VT>::T *__restrict__ dg, int *__restrict__ ge,
+                  const SecView *__restrict__ secs, const int *__restrict__ chunk0, int S) {
+    constexpr int NC = IsC<VT>::v ? 2 : 1;
+    const ChunkInfo ci = chunk_info(secs, chunk0, S, blockIdx.x);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t hw[XR][2], lw[XR][2];
+#pragma unroll
+    for (int k = 0; k < XR; ++k) {
+        const int r = threadIdx.x + k * XT;
+        const double2 v = r < ci.n ? ld2(x + ci.base + r) : make_double2(0.0, 0.0);
+        hw[k][0] = (uint32_t)__double2hiint(v.x);
+        lw[k][0] = (uint32_t)__double2loint(v.x);
+        hw[k][1] = (uint32_t)__double2hiint(v.y);
+        lw[k][1] = (uint32_t)__double2loint(v.y);
+    }
+    int d1[XR][2], d0[XR][2];
+    const int em = fx_group<NC>(hw, lw, d1, d0);
+#pragma unroll
+    for (int k = 0; k < XR; ++k) {
+        const int r = threadIdx.x + k * XT;
+        if (r < ci.n) dig_st(dg, D, ci.base + r, d1[k], d0[k]);
+    }
+    if (lane == 0) ge[(uint64_t)blockIdx.x * XW + warp] = em;
+}
+
 // The exact dot products conj(V_{j0+j}) . w over chunk c, as warp partials:
 // part[((c m + j) XW + q) 3 + {0, 1, 2}] = the re and im sums of warp q (in
 // units of 2^(k - 2098)) and k = em + ew, the sum of its two grid exponents.
@@ -1524,7 +1552,7 @@ struct Engine64 {
     bool loop_graph_ok() const { return graphs; }
     int enable_graphs(bool on) {
         graphs = on && B.nchunks > 0;
-        if (graphs && !xdev.p) QS3_TRY(xdev.alloc(sizeof(int)));
+        if (graphs && !xdev.p) QS3_TRY(xdev.alloc(sizeof(int), st));
         return QS3_OK;
     }
     qs3_dtype dtype() const { return IsC<VT>::v ? QS3_C128 : QS3_F64; }
@@ -1545,29 +1573,29 @@ struct Engine64 {
         cap = cap_;
         nscr = nscratch;
         D = B.total;
-        QS3_TRY(V.alloc((uint64_t)(cap + nscr) * D * sizeof(VT)));
-        QS3_TRY(DG.alloc((uint64_t)(cap + nscr) * D * sizeof(VT) + 16));     // k_dotb reads up to 16 bytes past
-        QS3_TRY(GE.alloc((uint64_t)(cap + nscr) * std::max(B.nchunks, 1) * XW * sizeof(int)));
-        QS3_TRY(wbuf.alloc(std::max<uint64_t>(D, 1) * sizeof(VT)));
-        QS3_TRY(hinb.alloc(std::max<uint64_t>(D, 1) * sizeof(VT)));
-        QS3_TRY(part.alloc((uint64_t)std::max(B.nchunks, 1) * cap * sizeof(double2)));
-        QS3_TRY(partx.alloc((uint64_t)std::max(B.nchunks, 1) * cap * XW * 3 * sizeof(long long)));
+        QS3_TRY(V.alloc((uint64_t)(cap + nscr) * D * sizeof(VT), st));
+        QS3_TRY(DG.alloc((uint64_t)(cap + nscr) * D * sizeof(VT) + 16, st));     // k_dotb reads up to 16 bytes past
+        QS3_TRY(GE.alloc((uint64_t)(cap + nscr) * std::max(B.nchunks, 1) * XW * sizeof(int), st));
+        QS3_TRY(wbuf.alloc(std::max<uint64_t>(D, 1) * sizeof(VT), st));
+        QS3_TRY(hinb.alloc(std::max<uint64_t>(D, 1) * sizeof(VT), st));
+        QS3_TRY(part.alloc((uint64_t)std::max(B.nchunks, 1) * cap * sizeof(double2), st));
+        QS3_TRY(partx.alloc((uint64_t)std::max(B.nchunks, 1) * cap * XW * 3 * sizeof(long long), st));
         {
             const std::vector<int> s0 = reduce_slices(B);
             nslices = s0[B.S];
             slice1 = one_slice(s0);
-            QS3_TRY(slices.upload(s0.data(), s0.size() * sizeof(int)));
-            QS3_TRY(partr.alloc((uint64_t)std::max(nslices, 1) * cap * 5 * sizeof(long long)));
+            QS3_TRY(slices.upload(s0.data(), s0.size() * sizeof(int), st));
+            QS3_TRY(partr.alloc((uint64_t)std::max(nslices, 1) * cap * 5 * sizeof(long long), st));
         }
-        QS3_TRY(h1.alloc((uint64_t)B.S * cap * sizeof(double2)));
-        QS3_TRY(h2.alloc((uint64_t)B.S * cap * sizeof(double2)));
-        QS3_TRY(alpha.alloc((uint64_t)B.S * cap * sizeof(double)));
-        QS3_TRY(beta.alloc((uint64_t)B.S * cap * sizeof(double)));
-        QS3_TRY(nrm.alloc((uint64_t)B.S * sizeof(double2)));
-        QS3_TRY(nrm1.alloc((uint64_t)B.S * sizeof(double2)));
-        QS3_TRY(inv.alloc((uint64_t)B.S * sizeof(double)));
-        QS3_TRY(active.alloc((uint64_t)B.S * sizeof(int)));
-        QS3_TRY(derr.alloc(sizeof(int)));
+        QS3_TRY(h1.alloc((uint64_t)B.S * cap * sizeof(double2), st));
+        QS3_TRY(h2.alloc((uint64_t)B.S * cap * sizeof(double2), st));
+        QS3_TRY(alpha.alloc((uint64_t)B.S * cap * sizeof(double), st));
+        QS3_TRY(beta.alloc((uint64_t)B.S * cap * sizeof(double), st));
+        QS3_TRY(nrm.alloc((uint64_t)B.S * sizeof(double2), st));
+        QS3_TRY(nrm1.alloc((uint64_t)B.S * sizeof(double2), st));
+        QS3_TRY(inv.alloc((uint64_t)B.S * sizeof(double), st));
+        QS3_TRY(active.alloc((uint64_t)B.S * sizeof(int), st));
+        QS3_TRY(derr.alloc(sizeof(int), st));
         QS3_CUDA(cudaMemsetAsync(derr.p, 0, sizeof(int), st));
         QS3_TRY(dotb_prepare<VT>());
         QS3_TRY(updb_prepare<VT>());
@@ -1880,8 +1908,8 @@ struct Engine64 {
         if (nout > MAXOUT) return set_err(QS3_ERR_INVALID_ARG, "at most %d vectors per combination", MAXOUT);
         const int ldc = nin * nout;
         DevBuf dC, dm;
-        QS3_TRY(dC.alloc(C.size() * 8));
-        QS3_TRY(dm.alloc(mask.size() * 4));
+        QS3_TRY(dC.alloc(C.size() * 8, st));
+        QS3_TRY(dm.alloc(mask.size() * 4, st));
         QS3_CUDA(cudaMemcpyAsync(dC.p, C.data(), C.size() * 8, cudaMemcpyHostToDevice, st));
         QS3_CUDA(cudaMemcpyAsync(dm.p, mask.data(), mask.size() * 4, cudaMemcpyHostToDevice, st));
         k_comb64<VT, PLO><<<grid(), NTHREADS, ldc * sizeof(double), st>>>(out, ldo, V.as<ST>(), D, nin, nout,

@@ -897,7 +897,7 @@ int smq_launch(Basis &S, int ss, const void *phi, Basis &Dd, int sd, const int *
     }
     std::vector<double2> ph = site_phases(S, Q);
     DevBuf dph;
-    QS3_TRY(dph.upload(ph.data(), ph.size() * sizeof(double2)));
+    QS3_TRY(dph.upload(ph.data(), ph.size() * sizeof(double2), st));
     if (S.dims[ss] == 0) {
         QS3_CUDA(cudaMemsetAsync(psi, 0, Dd.dims[sd] * 16, st));
         QS3_CUDA(cudaStreamSynchronize(st));
@@ -1010,7 +1010,7 @@ int sq_launch(int op, Basis &S, int ss, const void *phi, Basis &Dd, int sd, cons
     double2 hs = make_double2(0.0, 0.0);
     for (const double2 &v : ph) { hs.x += 0.5 * v.x; hs.y += 0.5 * v.y; }
     DevBuf dph;
-    QS3_TRY(dph.upload(ph.data(), ph.size() * sizeof(double2)));
+    QS3_TRY(dph.upload(ph.data(), ph.size() * sizeof(double2), st));
     if (S.dims[ss] == 0) {
         QS3_CUDA(cudaMemsetAsync(psi, 0, Dd.dims[sd] * 16, st));
     } else if (op == QS3_OP_SZ) {
@@ -1085,7 +1085,7 @@ static int correlations(Basis &B, int s, const void *gs, int npairs, const int *
     const size_t nacc = ks ? (size_t)nch * nb * 3 * CD : (want_pm ? 2 : 1) * (size_t)N * N;
     const size_t nin = 3 * (size_t)(nq > 0 ? N : 0) + 3 * (size_t)nq;
     DevBuf buf;
-    QS3_TRY(buf.alloc((nres + nacc + nin) * 8 + (size_t)ndl * 4));
+    QS3_TRY(buf.alloc((nres + nacc + nin) * 8 + (size_t)ndl * 4, st));
     double *res = buf.as<double>(), *acc = res + nres, *in = acc + nacc;
     int *ddl = (int *)(in + nin);
     std::vector<double> hin(nin + (ndl + 1) / 2);

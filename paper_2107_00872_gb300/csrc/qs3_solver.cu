@@ -1207,7 +1207,7 @@ struct Engine {
     // replay Lanczos steps as CUDA graphs (fp64 engine; ignored otherwise)
     int enable_graphs(bool on) {
         graphs = on && DF && B.nchunks > 0;
-        if (graphs && !xdev.p) QS3_TRY(xdev.alloc(sizeof(int)));
+        if (graphs && !xdev.p) QS3_TRY(xdev.alloc(sizeof(int), st));
         return QS3_OK;
     }
 
@@ -1234,22 +1234,22 @@ struct Engine {
         cap = cap_;
         nscr = nscratch;
         D = B.total;
-        QS3_TRY(V.alloc((uint64_t)(cap + nscr) * D * sizeof(ST)));
-        if (DF) QS3_TRY(ring.alloc(3 * D * sizeof(VT)));
+        QS3_TRY(V.alloc((uint64_t)(cap + nscr) * D * sizeof(ST), st));
+        if (DF) QS3_TRY(ring.alloc(3 * D * sizeof(VT), st));
         if (dfh) {
-            QS3_TRY(wdf.alloc(D * sizeof(float4)));
-            QS3_TRY(hdf.alloc(D * sizeof(float4)));
+            QS3_TRY(wdf.alloc(D * sizeof(float4), st));
+            QS3_TRY(hdf.alloc(D * sizeof(float4), st));
             QS3_CUDA(cudaMemsetAsync(wdf.p, 0, wdf.n, st));
         }
-        QS3_TRY(part.alloc((uint64_t)std::max(B.nchunks, 1) * cap * sizeof(double2)));
-        QS3_TRY(h1.alloc((uint64_t)B.S * cap * sizeof(double2)));
-        QS3_TRY(h2.alloc((uint64_t)B.S * cap * sizeof(double2)));
-        QS3_TRY(alpha.alloc((uint64_t)B.S * cap * sizeof(double)));
-        QS3_TRY(beta.alloc((uint64_t)B.S * cap * sizeof(double)));
-        QS3_TRY(nrm.alloc((uint64_t)B.S * sizeof(double2)));
-        QS3_TRY(nrm1.alloc((uint64_t)B.S * sizeof(double2)));
-        QS3_TRY(inv.alloc((uint64_t)B.S * sizeof(double)));
-        QS3_TRY(active.alloc((uint64_t)B.S * sizeof(int)));
+        QS3_TRY(part.alloc((uint64_t)std::max(B.nchunks, 1) * cap * sizeof(double2), st));
+        QS3_TRY(h1.alloc((uint64_t)B.S * cap * sizeof(double2), st));
+        QS3_TRY(h2.alloc((uint64_t)B.S * cap * sizeof(double2), st));
+        QS3_TRY(alpha.alloc((uint64_t)B.S * cap * sizeof(double), st));
+        QS3_TRY(beta.alloc((uint64_t)B.S * cap * sizeof(double), st));
+        QS3_TRY(nrm.alloc((uint64_t)B.S * sizeof(double2), st));
+        QS3_TRY(nrm1.alloc((uint64_t)B.S * sizeof(double2), st));
+        QS3_TRY(inv.alloc((uint64_t)B.S * sizeof(double), st));
+        QS3_TRY(active.alloc((uint64_t)B.S * sizeof(int), st));
         QS3_CUDA(cudaMemsetAsync(alpha.p, 0, alpha.n, st));
         QS3_CUDA(cudaMemsetAsync(beta.p, 0, beta.n, st));
         h_active.assign(B.S, 0);
@@ -1657,8 +1657,8 @@ struct Engine {
         if (nout > MAXOUT) return set_err(QS3_ERR_INVALID_ARG, "at most %d vectors per combination", MAXOUT);
         const int ldc = nin * nout;
         DevBuf dC, dm;
-        QS3_TRY(dC.alloc(C.size() * 8));
-        QS3_TRY(dm.alloc(mask.size() * 4));
+        QS3_TRY(dC.alloc(C.size() * 8, st));
+        QS3_TRY(dm.alloc(mask.size() * 4, st));
         QS3_CUDA(cudaMemcpyAsync(dC.p, C.data(), C.size() * 8, cudaMemcpyHostToDevice, st));
         QS3_CUDA(cudaMemcpyAsync(dm.p, mask.data(), mask.size() * 4, cudaMemcpyHostToDevice, st));
         // one fp64 result, or one double-float stored vector
@@ -1704,10 +1704,10 @@ static int residuals(Basis &B, const WT *v, const std::vector<double> &e, cudaSt
     rmax = 0.0;
     if (B.nchunks == 0) return QS3_OK;
     DevBuf t, de, part, out;
-    QS3_TRY(t.alloc(B.total * sizeof(WT)));
-    QS3_TRY(de.alloc(B.S * 8));
-    QS3_TRY(part.alloc((uint64_t)B.nchunks * sizeof(double2)));
-    QS3_TRY(out.alloc(B.S * sizeof(double2)));
+    QS3_TRY(t.alloc(B.total * sizeof(WT), st));
+    QS3_TRY(de.alloc(B.S * 8, st));
+    QS3_TRY(part.alloc((uint64_t)B.nchunks * sizeof(double2), st));
+    QS3_TRY(out.alloc(B.S * sizeof(double2), st));
     QS3_CUDA(cudaMemcpyAsync(de.p, e.data(), B.S * 8, cudaMemcpyHostToDevice, st));
     const qs3_dtype dt = sizeof(WT) == 8 ? QS3_F64 : QS3_C128;
     QS3_TRY(hphi_launch(B, dt, v, t.p, st, nullptr));
@@ -1946,14 +1946,14 @@ __device__ void tri_bottom_up_dev(int n, const double *__restrict__ a, const dou
 struct LzState {
     DevBuf eprev, eval, msz, conv, coef, ws, cont, nnz;
     int init(int S, int cap, cudaStream_t st) {
-        QS3_TRY(eprev.alloc((size_t)S * 8));
-        QS3_TRY(eval.alloc((size_t)S * 8));
-        QS3_TRY(msz.alloc((size_t)S * 4));
-        QS3_TRY(conv.alloc((size_t)S * 4));
-        QS3_TRY(coef.alloc((size_t)S * cap * 8));
-        QS3_TRY(ws.alloc((size_t)S * 7 * cap * 8));
-        QS3_TRY(cont.alloc(4));
-        QS3_TRY(nnz.alloc(8));
+        QS3_TRY(eprev.alloc((size_t)S * 8, st));
+        QS3_TRY(eval.alloc((size_t)S * 8, st));
+        QS3_TRY(msz.alloc((size_t)S * 4, st));
+        QS3_TRY(conv.alloc((size_t)S * 4, st));
+        QS3_TRY(coef.alloc((size_t)S * cap * 8, st));
+        QS3_TRY(ws.alloc((size_t)S * 7 * cap * 8, st));
+        QS3_TRY(cont.alloc(4, st));
+        QS3_TRY(nnz.alloc(8, st));
         // eprev = NaN (no previous Ritz value); everything else 0
         QS3_CUDA(cudaMemsetAsync(eprev.p, 0xff, eprev.n, st));
         QS3_CUDA(cudaMemsetAsync(eval.p, 0xff, eval.n, st));
@@ -2190,7 +2190,7 @@ static int lanczos_run(Basis &B, const qs3_solve_opts &o, const typename Wide<VT
     LzState K;
     QS3_TRY(K.init(S, E.cap, st));
     DevBuf dnnz;
-    QS3_TRY(dnnz.upload(B.nnz_sec.data(), (size_t)S * 8));
+    QS3_TRY(dnnz.upload(B.nnz_sec.data(), (size_t)S * 8, st));
     const uint64_t nz0 = hs.nnz;
     int cont = 0;
     auto check = [&](int n) -> int {
@@ -2450,7 +2450,7 @@ static int lanczos_entry(Basis &B, const qs3_solve_opts &o, double *evals, void 
     DevBuf own;
     V64 *out = (V64 *)evecs;
     if (!out) {
-        QS3_TRY(own.alloc(B.total * sizeof(V64)));
+        QS3_TRY(own.alloc(B.total * sizeof(V64), st));
         out = own.as<V64>();
     }
     QS3_CUDA(cudaMemsetAsync(out, 0, B.total * sizeof(V64), st));
@@ -2519,7 +2519,7 @@ static int trl_entry(Basis &B, const qs3_solve_opts &o, double *evals, void *eve
     DevBuf own;
     V64 *out = (V64 *)evecs;
     if (!out) {
-        QS3_TRY(own.alloc((uint64_t)NE * B.total * sizeof(V64)));
+        QS3_TRY(own.alloc((uint64_t)NE * B.total * sizeof(V64), st));
         out = own.as<V64>();
     }
     QS3_CUDA(cudaMemsetAsync(out, 0, (uint64_t)NE * B.total * sizeof(V64), st));
@@ -2534,19 +2534,19 @@ static int trl_entry(Basis &B, const qs3_solve_opts &o, double *evals, void *eve
         o1.eps = std::max(o.eps, 2e-7);
         o1.n_eig = NK;
         DevBuf kept;
-        QS3_TRY(kept.alloc((uint64_t)NK * B.total * sizeof(V64)));
+        QS3_TRY(kept.alloc((uint64_t)NK * B.total * sizeof(V64), st));
         QS3_CUDA(cudaMemsetAsync(kept.p, 0, (uint64_t)NK * B.total * sizeof(V64), st));
         QS3_TRY(trl_run<V32>(B, o1, nullptr, kept.as<V64>(), st, R, hs));
         iters += R.steps;
         restarts += R.restarts;
         DevBuf sum;
-        QS3_TRY(sum.alloc(B.total * sizeof(V64)));
+        QS3_TRY(sum.alloc(B.total * sizeof(V64), st));
         {
             std::vector<double> C((size_t)B.S * NK, 1.0);
             std::vector<int> all(B.S, 1);
             DevBuf dC, dm;
-            QS3_TRY(dC.alloc(C.size() * 8));
-            QS3_TRY(dm.alloc(all.size() * 4));
+            QS3_TRY(dC.alloc(C.size() * 8, st));
+            QS3_TRY(dm.alloc(all.size() * 4, st));
             QS3_CUDA(cudaMemcpyAsync(dC.p, C.data(), C.size() * 8, cudaMemcpyHostToDevice, st));
             QS3_CUDA(cudaMemcpyAsync(dm.p, all.data(), all.size() * 4, cudaMemcpyHostToDevice, st));
             if (B.nchunks) {
@@ -2640,9 +2640,9 @@ static int gs_dots_run(Basis &B, int m, const VT *V, uint64_t ldv, const VT *w, 
     memset(out, 0, (size_t)B.S * m * 2 * sizeof(double));
     if (m == 0 || B.nchunks == 0) return QS3_OK;
     DevBuf pl, dgt, get, part, res, dsl, pr, derr;
-    QS3_TRY(pl.alloc((uint64_t)m * D * sizeof(VT)));
-    QS3_TRY(part.alloc((uint64_t)B.nchunks * m * (mode == 0 ? XW * 3 * sizeof(long long) : sizeof(double2))));
-    QS3_TRY(res.alloc((uint64_t)B.S * m * sizeof(double2)));
+    QS3_TRY(pl.alloc((uint64_t)m * D * sizeof(VT), st));
+    QS3_TRY(part.alloc((uint64_t)B.nchunks * m * (mode == 0 ? XW * 3 * sizeof(long long) : sizeof(double2)), st));
+    QS3_TRY(res.alloc((uint64_t)B.S * m * sizeof(double2), st));
     const int g = (int)std::min<uint64_t>((D + 255) / 256, 4096);
     for (int j = 0; j < m; ++j) {
         k_to_planar<VT><<<g, 256, 0, st>>>(V + (uint64_t)j * ldv, pl.as<T>() + (uint64_t)j * 2 * D, D);
@@ -2652,9 +2652,9 @@ static int gs_dots_run(Basis &B, int m, const VT *V, uint64_t ldv, const VT *w, 
     const int *c0 = B.d_chunk0.as<int>();
     if (mode == 0) {
         using G = typename DigT<VT>::T;
-        QS3_TRY(dgt.alloc((uint64_t)m * D * sizeof(VT) + 16));      // k_dotb reads up to 16 bytes past
-        QS3_TRY(get.alloc((uint64_t)m * B.nchunks * XW * sizeof(int)));
-        QS3_TRY(derr.alloc(sizeof(int)));
+        QS3_TRY(dgt.alloc((uint64_t)m * D * sizeof(VT) + 16, st));      // k_dotb reads up to 16 bytes past
+        QS3_TRY(get.alloc((uint64_t)m * B.nchunks * XW * sizeof(int), st));
+        QS3_TRY(derr.alloc(sizeof(int), st));
         QS3_CUDA(cudaMemsetAsync(derr.p, 0, sizeof(int), st));
         QS3_TRY(dotb_prepare<VT>());
         k_digitize<VT><<<dim3(B.nchunks, m), XT, 0, st>>>(pl.as<T>(), D, 0, dgt.as<G>(), get.as<int>(), B.nchunks,
@@ -2663,8 +2663,8 @@ static int gs_dots_run(Basis &B, int m, const VT *V, uint64_t ldv, const VT *w, 
         QS3_TRY(dotx_launch<VT>(B.tune_nv64 > 0 ? B.tune_nv64 : 2, dgt.as<G>(), get.as<int>(), B.nchunks, D, 0, m,
                                 w, secs, c0, B.S, nullptr, part.as<long long>(), st, nullptr, 0, derr.as<int>()));
         const std::vector<int> s0 = reduce_slices(B);
-        QS3_TRY(dsl.upload(s0.data(), s0.size() * sizeof(int)));
-        QS3_TRY(pr.alloc((uint64_t)std::max(s0[B.S], 1) * m * 5 * sizeof(long long)));
+        QS3_TRY(dsl.upload(s0.data(), s0.size() * sizeof(int), st));
+        QS3_TRY(pr.alloc((uint64_t)std::max(s0[B.S], 1) * m * 5 * sizeof(long long), st));
         QS3_TRY(reducex_launch(part.as<long long>(), pr.as<long long>(), m, m, c0, dsl.as<int>(), s0[B.S], B.S,
                                nullptr, res.as<double2>(), m, st, nullptr, 0, IsC<VT>::v ? 1 : 0, one_slice(s0)));
     } else {
@@ -2723,20 +2723,13 @@ int hphi_x_binary64(Basis &B, const void *phi, void *psi, cudaStream_t st) {
         return set_err(QS3_ERR_STATE, "QS3_C128X needs a k-sector basis with the representative table and one hop "
                                       "amplitude");
     const uint64_t D = B.total;
-    DevBuf pl, dgt, get;
-    QS3_TRY(pl.alloc(D * sizeof(double2)));
-    QS3_TRY(dgt.alloc(D * sizeof(double2)));
-    QS3_TRY(get.alloc((uint64_t)B.nchunks * XW * sizeof(int)));
-    const int g = (int)std::min<uint64_t>((D + 255) / 256, 4096);
-    k_to_planar<double2><<<g, 256, 0, st>>>((const double2 *)phi, pl.as<uint2>(), D);
+    DevBuf dgt, get;
+    QS3_TRY(dgt.alloc(D * sizeof(double2), st));
+    QS3_TRY(get.alloc((uint64_t)B.nchunks * XW * sizeof(int), st));
+    k_digitize_il<double2><<<B.nchunks, XT, 0, st>>>((const double2 *)phi, D, dgt.as<int2>(), get.as<int>(),
+                                                     B.d_secs.as<SecView>(), B.d_chunk0.as<int>(), B.S);
     QS3_LAUNCHED();
-    k_digitize<double2><<<dim3(B.nchunks, 1), XT, 0, st>>>(pl.as<uint2>(), D, 0, dgt.as<int2>(), get.as<int>(),
-                                                           B.nchunks, B.d_secs.as<SecView>(), B.d_chunk0.as<int>(),
-                                                           B.S);
-    QS3_LAUNCHED();
-    QS3_TRY(hphi_x_launch(B, phi, dgt.p, get.as<int>(), nullptr, psi, st, nullptr));
-    QS3_CUDA(cudaStreamSynchronize(st));     // the scratch is released on return
-    return QS3_OK;
+    return hphi_x_launch(B, phi, dgt.p, get.as<int>(), nullptr, psi, st, nullptr);
 }
 
 }  // namespace qs3
@@ -2808,10 +2801,10 @@ int dsf_run(int op, Basis &S, int ss, const void *gs, double e0, Basis &Dd, int 
     }
     if (s_qw && nw > 0) {
         DevBuf dm, dn, dw, dout;
-        QS3_TRY(dm.upload(msz.data(), nq * sizeof(int)));
-        QS3_TRY(dn.upload(nrm2.data(), nq * sizeof(double)));
-        QS3_TRY(dw.upload(omega, nw * sizeof(double)));
-        QS3_TRY(dout.alloc((size_t)nq * nw * sizeof(double)));
+        QS3_TRY(dm.upload(msz.data(), nq * sizeof(int), st));
+        QS3_TRY(dn.upload(nrm2.data(), nq * sizeof(double), st));
+        QS3_TRY(dw.upload(omega, nw * sizeof(double), st));
+        QS3_TRY(dout.alloc((size_t)nq * nw * sizeof(double), st));
         // Zeeman shift of the resolvent: h times the change of N_down
         QS3_TRY(cfrac_launch(nq, E.cap, E.alpha.as<double>(), E.beta.as<double>(), dm.as<int>(), dn.as<double>(), e0,
                              h * (double)(Dd.nd - S.nd), eta, dw.as<double>(), nw, dout.as<double>(), st));
