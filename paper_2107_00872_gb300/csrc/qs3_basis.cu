@@ -421,32 +421,6 @@ __global__ void k_take(const uint32_t *__restrict__ pos, const uint64_t *__restr
     }
 }
 
-// the largest x with C(x, 2) <= P
-__device__ __forceinline__ int tri_root(uint32_t P) {
-    int x = (int)(0.5f + sqrtf(0.25f + 2.0f * (float)P));
-    while ((uint64_t)x * (x - 1) / 2 > P) --x;
-    while ((uint64_t)x * (x + 1) / 2 <= P) ++x;
-    return x;
-}
-
-// the buckets of prefix P (SecView::pinfo) when it has so many rows: nq of
-// them, 2^shift low ranks each, at most half as many as rows
-__device__ __forceinline__ int bucket_shift(uint32_t P, uint32_t rows, int nd, int pre2,
-                                            const uint64_t *__restrict__ binom, int np1, uint32_t &nq) {
-    uint64_t w;                            // low ranks
-    if (pre2) {
-        const int x = tri_root(P);
-        w = binom[(size_t)(nd - 2) * np1 + (P - (uint64_t)x * (x - 1) / 2)];
-    } else {
-        w = binom[(size_t)(nd - 1) * np1 + P];
-    }
-    const uint32_t most = rows / 2 > 1 ? rows / 2 : 1;
-    int sh = 0;
-    while (w && ((w - 1) >> sh) + 1 > most) ++sh;
-    nq = w ? (uint32_t)(((w - 1) >> sh) + 1) : 1u;
-    return sh;
-}
-
 // per sector s and prefix P: the first row with a prefix >= P, by a binary
 // search over the sector's rows (first[s (np + 1) + P], P <= np)
 __global__ void k_first(int nd, int np1, int pre2, const SecView *__restrict__ secs, int S, uint32_t np,
@@ -474,36 +448,6 @@ __global__ void k_first(int nd, int np1, int pre2, const SecView *__restrict__ s
             }
         }
         first[i] = (uint32_t)lo;
-    }
-}
-
-// entries of every (sector, prefix): its buckets plus the end
-__global__ void k_bucket_size(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
-                              const uint32_t *__restrict__ first, uint32_t *__restrict__ size) {
-    const uint64_t cnt = (uint64_t)S * np;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t s = i / np;
-        const uint32_t P = (uint32_t)(i - s * np);
-        const uint32_t *f = first + s * (np + 1) + P;
-        uint32_t nq;
-        bucket_shift(P, f[1] - f[0], nd, pre2, binom, np1, nq);
-        size[i] = nq + 1;
-    }
-}
-__global__ void k_bucket_info(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
-                              const uint32_t *__restrict__ first, const uint32_t *__restrict__ off,
-                              uint2 *__restrict__ pinfo, uint32_t *__restrict__ sub) {
-    const uint64_t cnt = (uint64_t)S * np;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t s = i / np;
-        const uint32_t P = (uint32_t)(i - s * np);
-        const uint32_t *f = first + s * (np + 1) + P;
-        uint32_t nq;
-        const int sh = bucket_shift(P, f[1] - f[0], nd, pre2, binom, np1, nq);
-        pinfo[i] = make_uint2(off[i], (uint32_t)sh);
-        // an empty prefix: one empty bucket
-        if (f[0] == f[1])
-            for (uint32_t q = 0; q <= nq; ++q) sub[(uint64_t)off[i] + q] = f[0];
     }
 }
 
@@ -1175,6 +1119,14 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
         if (build_rep_table(B, lim, oreps, ostab, n_orb) != QS3_OK) {
             drop_rep_table(B);
             clear_err();
+            // without it, the origin forms of the rows
+            oreps.release();
+            ostab.release();
+            QS3_CUDA(cudaMemGetInfo(&fr, &tt));
+            if (build_forms(B, fr / 8) != QS3_OK) {
+                if (cudaPeekAtLastError() != cudaSuccess) return QS3_ERR_CUDA;
+                clear_err();
+            }
         }
     }
     return QS3_OK;

@@ -1070,6 +1070,8 @@ int hphi_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t
     }
     if (B.has_k) {
         if (B.stored_terms && (dt == QS3_C64 || dt == QS3_C128)) return hphi_stored_launch(B, dt, phi, psi, st, active);
+        if (!B.lv.orb && B.d_okey.p && (dt == QS3_C64 || dt == QS3_C128))
+            return hphi_forms_launch(B, dt, phi, psi, st, active);
         if (hphi_of_ok(B)) {
             if (dt == QS3_C64) return hphiof_vt<float2>(B, phi, psi, st, active, dt);
             if (dt == QS3_C128) return hphiof_vt<double2>(B, phi, psi, st, active, dt);

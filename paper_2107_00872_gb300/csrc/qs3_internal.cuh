@@ -93,6 +93,7 @@ struct LatView {
     int L[3];
     int has_k;
     int key_bits;                 // bits per site of a packed key, 0 -> compare ranks
+    int form_bits;                // bits per site of a packed origin form (0: none built)
     int mask_ok;                  // canon_mask applies: L <= 32 along each axis, keys fit 64 bits
     const uint64_t *binom;
     const int *adj_ptr;           // N + 1
@@ -140,6 +141,13 @@ struct SecView {
     const uint2 *pinfo;
     const uint32_t *sub;
     int pre2;
+    // origin forms of the rows (qs3_hphi_search.cu), when built: sorted packed
+    // forms, (row, w | (|Stab| - 1) << 28) of each, and their index
+    const void *okey;
+    const uint2 *oval;
+    const uint2 *finfo;
+    const uint32_t *fsub;
+    int fpre2;
     uint64_t dim;
     uint64_t off;                 // offset of the sector in a concatenated vector
     int K[3];
@@ -175,6 +183,7 @@ struct Basis {
     DevBuf d_adj_jxy_lo, d_u_lo, d_adj_jz_lo;
     DevBuf d_adj_pad, d_adj_jz_pad;         // fixed-width adjacency (LatView::adj_pad)
     DevBuf d_sigma, d_stab, d_pinfo, d_sub;  // every sector's lists, one after another
+    DevBuf d_okey, d_oval, d_finfo, d_fsub;  // origin forms and their index (without a representative table)
     DevBuf d_ph64, d_ph32, d_phdf;          // S x N per-site phase tables (k-sectors)
     DevBuf d_roots;                         // e^{-2 pi i n / ncell}, n < ncell (k-sectors)
     DevBuf d_secs, d_tile0, d_chunk0;
@@ -709,6 +718,32 @@ __device__ __forceinline__ bool bucket_find(const uint64_t *__restrict__ sigma, 
     return found;
 }
 
+// the largest x with C(x, 2) <= P
+__device__ __forceinline__ int tri_root(uint32_t P) {
+    int x = (int)(0.5f + sqrtf(0.25f + 2.0f * (float)P));
+    while ((uint64_t)x * (x - 1) / 2 > P) --x;
+    while ((uint64_t)x * (x + 1) / 2 <= P) ++x;
+    return x;
+}
+
+// the buckets of prefix P (SecView::pinfo) when it has so many rows: nq of
+// them, 2^shift low ranks each, at most half as many as rows
+__device__ __forceinline__ int bucket_shift(uint32_t P, uint32_t rows, int nd, int pre2,
+                                            const uint64_t *__restrict__ binom, int np1, uint32_t &nq) {
+    uint64_t w;                            // low ranks
+    if (pre2) {
+        const int x = tri_root(P);
+        w = binom[(size_t)(nd - 2) * np1 + (P - (uint64_t)x * (x - 1) / 2)];
+    } else {
+        w = binom[(size_t)(nd - 1) * np1 + P];
+    }
+    const uint32_t most = rows / 2 > 1 ? rows / 2 : 1;
+    int sh = 0;
+    while (w && ((w - 1) >> sh) + 1 > most) ++sh;
+    nq = w ? (uint32_t)(((w - 1) >> sh) + 1) : 1u;
+    return sh;
+}
+
 // position of the representative c, of rank r, in sector sv
 template <int ND>
 __device__ __forceinline__ bool sigma_find(const SecView &sv, const int (&c)[ND], const uint64_t *__restrict__ sC,
@@ -727,6 +762,36 @@ __device__ __forceinline__ void stage_tables(const LatView &L, uint64_t *sC, uin
         for (int i = threadIdx.x; i < L.N; i += blockDim.x) sxyz[i] = L.xyz[i];
 }
 
+// entries of every (sector, prefix): its buckets plus the end
+static __global__ void k_bucket_size(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
+                              const uint32_t *__restrict__ first, uint32_t *__restrict__ size) {
+    const uint64_t cnt = (uint64_t)S * np;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t s = i / np;
+        const uint32_t P = (uint32_t)(i - s * np);
+        const uint32_t *f = first + s * (np + 1) + P;
+        uint32_t nq;
+        bucket_shift(P, f[1] - f[0], nd, pre2, binom, np1, nq);
+        size[i] = nq + 1;
+    }
+}
+static __global__ void k_bucket_info(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
+                              const uint32_t *__restrict__ first, const uint32_t *__restrict__ off,
+                              uint2 *__restrict__ pinfo, uint32_t *__restrict__ sub) {
+    const uint64_t cnt = (uint64_t)S * np;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t s = i / np;
+        const uint32_t P = (uint32_t)(i - s * np);
+        const uint32_t *f = first + s * (np + 1) + P;
+        uint32_t nq;
+        const int sh = bucket_shift(P, f[1] - f[0], nd, pre2, binom, np1, nq);
+        pinfo[i] = make_uint2(off[i], (uint32_t)sh);
+        // an empty prefix: one empty bucket
+        if (f[0] == f[1])
+            for (uint32_t q = 0; q <= nq; ++q) sub[(uint64_t)off[i] + q] = f[0];
+    }
+}
+
 size_t row_kernel_smem(const Basis &B, int extra_nd);
 
 // -------------------------------------------------------------- entry points
@@ -737,6 +802,10 @@ int hphi_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t
 // (*dx) ld when dx (device) is given; psi complex128, or double-float when out_df
 int hphi_df_launch(Basis &B, const void *phi, const int *dx, uint64_t ld, void *psi, cudaStream_t st,
                    const int *active = nullptr, bool out_df = false);
+// the same on momentum sectors by origin forms (qs3_hphi_search.cu), built at
+// creation of a basis without a representative table
+int build_forms(Basis &B, size_t max_bytes);
+int hphi_forms_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t st, const int *active);
 int count_nnz(Basis &B, uint64_t *nnz);
 // the binary64 engine's H Phi on the integer units (qs3_hphi.cu, k_hphi_x and the
 // orbit-batched k_hphi_o): phi as binary64 and as its digit-store image (dg, ge:
