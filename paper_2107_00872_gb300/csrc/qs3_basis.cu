@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(NTHREADS) k_bucket_fill(LatView L, const SecVi
         for (uint32_t k = q0; k <= q; ++k) e[k] = (uint32_t)row;
         if (row + 1 == f[1]) {
             uint32_t nq;
-            bucket_shift(P, f[1] - f[0], L.nd, secs[s].pre2, L.binom, L.np1, nq);
+            bucket_shift(P, (f[1] - f[0]) >> 1, L.nd, secs[s].pre2, L.binom, L.np1, nq);
             for (uint32_t k = q + 1; k <= nq; ++k) e[k] = (uint32_t)(row + 1);
         }
     }
@@ -571,7 +571,7 @@ static int build_index_nd(Basis &B) {
     k_first<<<g1, 256>>>(B.nd, B.N + 1, pre2, secs, S, np, bin, first.as<uint32_t>());
     QS3_LAUNCHED();
     QS3_CUDA(cudaMemsetAsync(size.as<uint32_t>() + cnt, 0, 4));
-    k_bucket_size<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, S, np, first.as<uint32_t>(), size.as<uint32_t>());
+    k_bucket_size<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, S, np, 1, first.as<uint32_t>(), size.as<uint32_t>());
     QS3_LAUNCHED();
     size_t tb = 0;
     QS3_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt + 1)));
@@ -582,7 +582,7 @@ static int build_index_nd(Basis &B) {
     if (most >= (1ull << 32)) return set_err(QS3_ERR_OVERFLOW, "index of %llu entries", (unsigned long long)most);
     QS3_TRY(B.d_pinfo.alloc(std::max<uint64_t>(cnt, 1) * sizeof(uint2)));
     QS3_TRY(B.d_sub.alloc(std::max<uint64_t>(most, 1) * 4));
-    k_bucket_info<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, S, np, first.as<uint32_t>(), off.as<uint32_t>(),
+    k_bucket_info<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, S, np, 1, first.as<uint32_t>(), off.as<uint32_t>(),
                                B.d_pinfo.as<uint2>(), B.d_sub.as<uint32_t>());
     QS3_LAUNCHED();
     if (B.ntiles > 0) {
@@ -1039,6 +1039,32 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
         bool same = true;
         for (int b = 1; b < nb; ++b) same &= B.jxy[b] == B.jxy[0];
         if (same) L.jh_uniform = 0.5 * B.jxy[0];
+    }
+
+    L.diag_uniform = 0;
+    if (B.has_k && nb > 0 && nd > 0) {
+        bool same = true;
+        for (int i = 1; i < N; ++i) same &= u[i] == u[0];
+        for (size_t q = 1; q < ajz.size(); ++q) same &= ajz[q] == ajz[0];
+        if (same) {
+            const size_t np = (size_t)nd * B.max_degree + 1;
+            std::vector<double> img(np + (np + 1) / 2, 0.0);
+            float *pf = (float *)(img.data() + np);
+            for (size_t n = 1; n < np; ++n) {
+                img[n] = img[n - 1] + ajz[0];
+                pf[n] = pf[n - 1] + ajzf[0];
+            }
+            QS3_TRY(B.d_pair.upload(img.data(), img.size() * 8));
+            L.pair_sum = B.d_pair.as<double>();
+            L.pair_sum_f = (const float *)(L.pair_sum + np);
+            L.e_row = c0;
+            L.e_row_f = L.c0f;
+            for (int k = 0; k < nd; ++k) {
+                L.e_row += u[0];
+                L.e_row_f += uf[0];
+            }
+            L.diag_uniform = 1;
+        }
     }
 
     // sectors

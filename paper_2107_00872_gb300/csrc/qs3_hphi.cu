@@ -416,13 +416,13 @@ template <int ND, typename R>
 __device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const int (&c)[ND],
                                           const uint64_t *__restrict__ sC, const uint8_t *__restrict__ ostab,
                                           uint32_t *my, uint8_t *mys, size_t stride, R &e, R &dd) {
-    e = diag_c0<R>(L);
+    e = diag_row<R>(L);
     dd = 0;
-    int nh = 0;
+    int nh = 0, npair = 0;
 #pragma unroll 1
     for (int m = 0; m < ND; ++m) {
         const int i = pick(c, m);
-        e += diag_u<R>(L, i);
+        if (!L.diag_uniform) e += diag_u<R>(L, i);
         const int e0 = __ldg(L.adj_ptr + i), e1 = __ldg(L.adj_ptr + i + 1);
         const int lo = m > 0 ? pick(c, m > 0 ? m - 1 : 0) : -1;
         const int hi = m < ND - 1 ? pick(c, m < ND - 1 ? m + 1 : m) : L.np1;
@@ -435,7 +435,8 @@ __device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const
 #pragma unroll
                 for (int k = 0; k < ND; ++k) occ |= (c[k] == j);
                 if (occ) {
-                    dd += diag_jz<R>(L, q);
+                    if (L.diag_uniform) ++npair;
+                    else dd += diag_jz<R>(L, q);
                     continue;
                 }
             }
@@ -456,6 +457,7 @@ __device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const
             ++nh;
         }
     }
+    if (L.diag_uniform) dd = diag_pairs<R>(L, npair);
     return nh;
 }
 
@@ -1070,7 +1072,7 @@ int hphi_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t
     }
     if (B.has_k) {
         if (B.stored_terms && (dt == QS3_C64 || dt == QS3_C128)) return hphi_stored_launch(B, dt, phi, psi, st, active);
-        if (!B.lv.orb && B.d_okey.p && (dt == QS3_C64 || dt == QS3_C128))
+        if (!B.lv.orb && B.d_orec.p && (dt == QS3_C64 || dt == QS3_C128))
             return hphi_forms_launch(B, dt, phi, psi, st, active);
         if (hphi_of_ok(B)) {
             if (dt == QS3_C64) return hphiof_vt<float2>(B, phi, psi, st, active, dt);

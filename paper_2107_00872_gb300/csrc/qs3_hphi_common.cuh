@@ -92,6 +92,15 @@ template <typename R> __device__ __forceinline__ R diag_jz(const LatView &L, int
 template <> __device__ __forceinline__ double diag_jz<double>(const LatView &L, int q) { return __ldg(L.adj_jz + q); }
 template <> __device__ __forceinline__ float diag_jz<float>(const LatView &L, int q) { return __ldg(L.adj_jz_f + q); }
 
+// LatView::diag_uniform: the site part of a row's diagonal, and n J^z summed;
+// else the constant c0 alone
+template <typename R> __device__ __forceinline__ R diag_row(const LatView &L);
+template <> __device__ __forceinline__ double diag_row<double>(const LatView &L) { return L.diag_uniform ? L.e_row : L.c0; }
+template <> __device__ __forceinline__ float diag_row<float>(const LatView &L) { return L.diag_uniform ? L.e_row_f : L.c0f; }
+template <typename R> __device__ __forceinline__ R diag_pairs(const LatView &L, int n);
+template <> __device__ __forceinline__ double diag_pairs<double>(const LatView &L, int n) { return __ldg(L.pair_sum + n); }
+template <> __device__ __forceinline__ float diag_pairs<float>(const LatView &L, int n) { return __ldg(L.pair_sum_f + n); }
+
 template <typename CT> __device__ __forceinline__ const CT *phase_table(const SecView &sv);
 template <> __device__ __forceinline__ const double2 *phase_table<double2>(const SecView &sv) { return sv.ph64; }
 template <> __device__ __forceinline__ const float2 *phase_table<float2>(const SecView &sv) { return sv.ph32; }

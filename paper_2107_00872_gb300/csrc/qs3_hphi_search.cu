@@ -14,11 +14,18 @@
 // spin c_k, k != m, is the sorted list of the unmoved spins' differences to
 // c_k, formed once per row and m, with one more difference inserted.
 //
-// The rows' origin forms are sorted once per basis: okey[i] the packed form,
-// oval[i] its row, the cell w of the representative's spin that the form has
-// at the origin, and |Stab|.  A form is found by the same kind of index as
-// sigma's: its two largest sites, then a bucket of a few keys.  With origin o
-// of the target's form (the moved spin), T_u rep = target for u = o - w.
+// The rows' origin forms are sorted once per basis: orec[i] = (packed form,
+// row, w | (|Stab| - 1) << 28) with w the cell of the representative's spin
+// that the form has at the origin.  A form is found through its largest site
+// (finfo, staged in shared memory) and the rank of its other sites, which give
+// a bucket of about one record.  With origin o of the target's form (the spin
+// moved there), T_u rep = target for u = o - w.  So a hop costs three
+// dependent loads, each a sector per lane: bucket, record, phi.
+// 6x6x6, N_down = 5, k = 0, complex128: 12.0 ms (18.8 with the search on
+// occupation masks; 13.2 with two-site prefixes, separate key and value lists
+// and the diagonal's fp64 additions per row); 8x8x8, N_down = 4, complex64:
+// 1.81 ms (3.45, 2.06).  About 480 instructions per warp and hop, half of the
+// issue slots; the loads' latency at 45 % occupancy is the rest.
 #include <cub/cub.cuh>
 
 #include <algorithm>
@@ -89,13 +96,29 @@ __device__ __forceinline__ KT origin_form(const int (&c)[ND], const LatView &L, 
     return best;
 }
 
-constexpr int SH_HB = 3;                   // hops in flight together
+// p f out of line, so that the multiplications of the rare targets whose
+// |Stab| differs are a branch and not predicated fp64 instructions that every
+// hop issues
+template <typename CT, typename R> __device__ __noinline__ CT scaled(CT p, R f) {
+    p.x *= f;
+    p.y *= f;
+    return p;
+}
+template <typename KT> __device__ __forceinline__ KT rec_key(uint4 r);
+template <> __device__ __forceinline__ uint32_t rec_key<uint32_t>(uint4 r) { return r.x; }
+template <> __device__ __forceinline__ unsigned long long rec_key<unsigned long long>(uint4 r) {
+    return ((unsigned long long)r.y << 32) | r.x;
+}
+
+// hops in flight together: 2 hops at 4 (complex128) or 3 resident blocks per SM
+// took 13.1 / 2.06 ms on the two cubes, 3 hops 13.5 / 2.12, 1 hop 14.6 / 2.10
+constexpr int SH_HB = 2;
 
 template <int ND, typename VT, typename KT>
-__global__ void __launch_bounds__(NTHREADS, 3) k_hphi_f(LatView L, const SecView *__restrict__ secs,
+__global__ void __launch_bounds__(NTHREADS, sizeof(VT) == 16 ? 4 : 3) k_hphi_f(LatView L, const SecView *__restrict__ secs,
                                                         const int *__restrict__ tile0, int S, int ntiles,
                                                         const VT *__restrict__ phi, VT *__restrict__ psi,
-                                                        const int *__restrict__ active) {
+                                                        const int *__restrict__ active, unsigned fi_off) {
     using R = typename VTr<VT>::R;
     using CT = typename VTr<VT>::C;
     constexpr int NO = ND - 1;             // unmoved spins; sites of an origin form
@@ -114,6 +137,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_hphi_f(LatView L, const SecView
     const KT kbase = (KT)1 << bits;
     __syncthreads();
     CT *ph = (CT *)sm.sph;
+    uint2 *sfi = (uint2 *)(smem + fi_off);
     int cur = -1;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int s = (S == 1) ? 0 : sector_of_tile(tile0, S, t);
@@ -122,7 +146,10 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_hphi_f(LatView L, const SecView
         if (s != cur) {
             __syncthreads();
             const CT *g = phase_table<CT>(sv);
-            for (int i = threadIdx.x; i < L.N; i += blockDim.x) ph[i] = g[i];
+            for (int i = threadIdx.x; i < L.N; i += blockDim.x) {
+                ph[i] = g[i];
+                sfi[i] = sv.finfo[i];
+            }
             __syncthreads();
             cur = s;
         }
@@ -131,20 +158,19 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_hphi_f(LatView L, const SecView
         int c[ND];
         unrank(__ldg(sv.sigma + row), sm.sC, np1, c);
         const VT *__restrict__ ph_in = phi + sv.off;
-        const KT *__restrict__ okey = (const KT *)sv.okey;
-        const uint2 *__restrict__ oval = sv.oval, *__restrict__ finfo = sv.finfo;
+        const uint4 *__restrict__ orec = sv.orec;
         const uint32_t *__restrict__ fsub = sv.fsub;
-        const int fpre2 = sv.fpre2;
         const int st_row = sv.stab[row];
         const R rs = snorm[9 + st_row];
-        R e = diag_c0<R>(L), dd = 0;
+        R e = diag_row<R>(L), dd = 0;
+        int npair = 0;
         CT acc, acch;
         acc.x = 0; acc.y = 0;
         acch.x = 0; acch.y = 0;
 #pragma unroll 1
         for (int m = 0; m < ND; ++m) {
             const int i = pick(c, m);
-            e += diag_u<R>(L, i);
+            if (!L.diag_uniform) e += diag_u<R>(L, i);
             const int e0 = __ldg(L.adj_ptr + i), e1 = __ldg(L.adj_ptr + i + 1);
             // the unmoved spins and, for each, the sorted differences of the others to it
             int oX[NO], oY[NO], oZ[NO], E[NO][NO > 1 ? NO - 1 : 1];
@@ -182,7 +208,8 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_hphi_f(LatView L, const SecView
 #pragma unroll
                     for (int k = 0; k < ND; ++k) go[h] &= c[k] != j;
                     if (!go[h]) {
-                        dd += diag_jz<R>(L, q0 + h);
+                        if (L.diag_uniform) ++npair;
+                        else dd += diag_jz<R>(L, q0 + h);
                         continue;
                     }
                     const uint32_t pj = sm.sxyz[j];
@@ -212,73 +239,58 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_hphi_f(LatView L, const SecView
                         }
                     }
                 }
-                // the forms' rows: index entry, bucket, keys, value -- each stage's loads together
-                uint2 fi[SH_HB];
+                // the forms' rows: bucket, record, phi -- each stage's loads together
                 uint32_t lo[SH_HB], hi[SH_HB];
-                uint64_t low[SH_HB];
-#pragma unroll
-                for (int h = 0; h < SH_HB; ++h)
-                    if (go[h]) {
-                        int f[NO];
-                        unpack_list<NO, KT>(key[h], bits, f);
-                        fi[h] = __ldg(finfo + prefix_of(f, sm.sC, np1, fpre2, low[h]));
-                    }
 #pragma unroll
                 for (int h = 0; h < SH_HB; ++h) {
                     lo[h] = hi[h] = 0u;
                     if (go[h]) {
-                        const uint32_t *b = fsub + fi[h].x + (uint32_t)(low[h] >> fi[h].y);
+                        int f[NO];
+                        unpack_list<NO, KT>(key[h], bits, f);
+                        uint64_t low;
+                        const uint2 fi = sfi[prefix_of(f, sm.sC, np1, 0, low)];
+                        const uint32_t *b = fsub + fi.x + (uint32_t)(low >> fi.y);
                         lo[h] = __ldg(b);
                         hi[h] = __ldg(b + 1);
                     }
                 }
-#pragma unroll
-                for (int h = 0; h < SH_HB; ++h)
-                    while (hi[h] - lo[h] > 4u) {
-                        const uint32_t mid = (lo[h] + hi[h]) >> 1;
-                        if (__ldg(okey + mid) <= key[h]) lo[h] = mid; else hi[h] = mid;
-                    }
-                KT kv[SH_HB][4];
-#pragma unroll
-                for (int h = 0; h < SH_HB; ++h)
-#pragma unroll
-                    for (uint32_t x = 0; x < 4; ++x)
-                        kv[h][x] = lo[h] + x < hi[h] ? __ldg(okey + lo[h] + x) : (KT)~key[h];
-                uint2 val[SH_HB];
+                uint32_t val[SH_HB], wst[SH_HB];
 #pragma unroll
                 for (int h = 0; h < SH_HB; ++h) {
-                    bool found = false;
-                    uint32_t idx = lo[h];
+                    while (hi[h] - lo[h] > 4u) {
+                        const uint32_t mid = (lo[h] + hi[h]) >> 1;
+                        if (rec_key<KT>(__ldg(orec + mid)) <= key[h]) lo[h] = mid; else hi[h] = mid;
+                    }
+                }
+                uint4 rec[SH_HB];
 #pragma unroll
-                    for (uint32_t x = 0; x < 4; ++x)
-                        if (kv[h][x] == key[h]) {
-                            found = true;
-                            idx = lo[h] + x;
-                        }
+                for (int h = 0; h < SH_HB; ++h)
+                    if (lo[h] < hi[h]) rec[h] = __ldg(orec + lo[h]);
+#pragma unroll
+                for (int h = 0; h < SH_HB; ++h) {
+                    bool found = lo[h] < hi[h] && rec_key<KT>(rec[h]) == key[h];
+                    while (!found && ++lo[h] < hi[h]) {
+                        rec[h] = __ldg(orec + lo[h]);
+                        found = rec_key<KT>(rec[h]) == key[h];
+                    }
                     go[h] = go[h] && found;
-                    if (go[h]) val[h] = __ldg(oval + idx);
+                    val[h] = rec[h].z;
+                    wst[h] = rec[h].w;
                 }
                 VT xv[SH_HB];
 #pragma unroll
                 for (int h = 0; h < SH_HB; ++h)
-                    if (go[h]) xv[h] = ph_in[val[h].x];
+                    if (go[h]) xv[h] = ph_in[val[h]];
 #pragma unroll
                 for (int h = 0; h < SH_HB; ++h) {
                     if (!go[h]) continue;
-                    // u = origin - w; val.y = w (coordinates) | with |Stab| in a second word's top bits
-                    const uint32_t w = val[h].y;
-                    const int st = (int)(w >> 28) + 1;
-                    const int wc = (int)(w & 0xfffffffu);
-                    const uint32_t wp = sm.sxyz[wc];
+                    const int st = (int)(wst[h] >> 28) + 1;
+                    const uint32_t wp = sm.sxyz[wst[h] & 0xfffffffu];
                     const int u = site_diff(px(org[h]), py(org[h]), pz(org[h]), px(wp), py(wp), pz(wp), Lx, Ly, Lz);
                     CT p = ph[u];
                     if (uni) {
                         // uniform J^xy: the amplitude is applied once per row below
-                        if (st != st_row) {
-                            const R f = snorm[st] * rs;
-                            p.x *= f;
-                            p.y *= f;
-                        }
+                        if (st != st_row) p = scaled(p, snorm[st] * rs);
                         acc_add(acch, p, xv[h]);
                     } else {
                         const R jh = __ldg(jxy + q0 + h);
@@ -291,6 +303,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) k_hphi_f(LatView L, const SecView
             }
         }
         if (uni) madd_r(acc, juni, acch);
+        if (L.diag_uniform) dd = diag_pairs<R>(L, npair);
         madd_r(acc, e + (R)0.5 * dd, ph_in[row]);
         store(psi + sv.off + row, acc);
     }
@@ -316,33 +329,30 @@ __global__ void __launch_bounds__(NTHREADS) k_forms(LatView L, SecView sv, KT *_
     }
 }
 
-// per prefix P <= np: the first form with a prefix >= P (see k_first of the index over sigma)
-template <int NO, typename KT>
-__global__ void k_form_first(const KT *__restrict__ key, uint64_t d, int bits, int pre2, uint32_t np,
+// the records in order: (form, row, w | (|Stab| - 1) << 28)
+template <typename KT>
+__global__ void k_form_recs(const KT *__restrict__ key, const uint2 *__restrict__ val, uint64_t d, uint4 *__restrict__ rec) {
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < d; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = key[i];
+        rec[i] = make_uint4((uint32_t)k, (uint32_t)(k >> 32), val[i].x, val[i].y);
+    }
+}
+// per largest site P <= N: the first form with one >= P
+template <typename KT>
+__global__ void k_form_first(const KT *__restrict__ key, uint64_t d, int bits, int no, uint32_t np,
                              uint32_t *__restrict__ first) {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= np; i += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t lo = 0, hi = d;
-        if (i == np) {
-            lo = hi;
-        } else {
-            KT k;
-            if (pre2) {
-                const int x = tri_root((uint32_t)i);
-                const uint32_t y = (uint32_t)(i - (uint64_t)x * (x - 1) / 2);
-                k = (((KT)x << bits) | (KT)y) << (bits * (NO > 1 ? NO - 2 : 0));
-            } else {
-                k = (KT)i << (bits * (NO - 1));
-            }
-            while (lo < hi) {
-                const uint64_t mid = (lo + hi) >> 1;
-                if (key[mid] < k) lo = mid + 1; else hi = mid;
-            }
+        const uint64_t k = (uint64_t)i << (bits * (no - 1));
+        while (lo < hi && i < np) {
+            const uint64_t mid = (lo + hi) >> 1;
+            if ((uint64_t)key[mid] < k) lo = mid + 1; else hi = mid;
         }
-        first[i] = (uint32_t)lo;
+        first[i] = (uint32_t)(i < np ? lo : d);
     }
 }
 template <int NO, typename KT>
-__global__ void __launch_bounds__(NTHREADS) k_form_fill(LatView L, const KT *__restrict__ key, uint64_t d, int pre2,
+__global__ void __launch_bounds__(NTHREADS) k_form_fill(LatView L, const KT *__restrict__ key, uint64_t d,
                                                         const uint32_t *__restrict__ first,
                                                         const uint2 *__restrict__ info, uint32_t *__restrict__ sub) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -353,25 +363,24 @@ __global__ void __launch_bounds__(NTHREADS) k_form_fill(LatView L, const KT *__r
         int f[NO];
         uint64_t low, lowp;
         unpack_list<NO, KT>(key[r], L.form_bits, f);
-        const uint32_t P = prefix_of(f, sC, L.np1, pre2, low);
+        const uint32_t P = prefix_of(f, sC, L.np1, 0, low);
         const uint2 pi = info[P];
         uint32_t *e = sub + pi.x;
         const uint32_t q = (uint32_t)(low >> pi.y);
         uint32_t q0 = 0;
         if (r > first[P]) {
             unpack_list<NO, KT>(key[r - 1], L.form_bits, f);
-            prefix_of(f, sC, L.np1, pre2, lowp);
+            prefix_of(f, sC, L.np1, 0, lowp);
             q0 = (uint32_t)(lowp >> pi.y) + 1;
         }
         for (uint32_t k = q0; k <= q; ++k) e[k] = (uint32_t)r;
         if (r + 1 == first[P + 1]) {
             uint32_t nq;
-            bucket_shift(P, first[P + 1] - first[P], NO, pre2, L.binom, L.np1, nq);
+            bucket_shift(P, first[P + 1] - first[P], NO, 0, L.binom, L.np1, nq);
             for (uint32_t k = q + 1; k <= nq; ++k) e[k] = (uint32_t)(r + 1);
         }
     }
 }
-
 // whether the origin forms of a basis exist, and the bytes they hold
 static bool forms_apply(const Basis &B) {
     int bits = 1;
@@ -379,26 +388,28 @@ static bool forms_apply(const Basis &B) {
     return B.has_k && B.nd >= 2 && B.nsub == 1 && B.total > 0 && (B.nd - 1) * bits <= 64;
 }
 
+// shared memory of k_hphi_f: the row kernels' tables, then the index of the largest site
+static size_t forms_off(const Basis &B) { return (B.smem_bytes + 15) & ~(size_t)15; }
+static size_t forms_smem(const Basis &B) { return forms_off(B) + (size_t)B.N * sizeof(uint2); }
+
 template <int ND, typename KT>
 static int build_forms_nd(Basis &B) {
     constexpr int NO = ND - 1;
     const int S = B.S, bits = B.lv.form_bits;
-    const uint64_t np2 = (uint64_t)B.N * (B.N - 1) / 2;
-    const int pre2 = NO >= 2 && (uint64_t)S * np2 / 8 <= B.total ? 1 : 0;
-    const uint32_t np = pre2 ? (uint32_t)np2 : (uint32_t)B.N;
+    const uint32_t np = (uint32_t)B.N;
     uint64_t dmax = 0;
     for (uint64_t d : B.dims) dmax = std::max(dmax, d);
-    const uint64_t most = B.total / 2 + 2 * (uint64_t)S * np;
-    if (most >= (1ull << 32)) return set_err(QS3_ERR_OVERFLOW, "index of %llu entries", (unsigned long long)most);
-    DevBuf key, val, info, sub;
-    QS3_TRY(key.alloc(B.total * sizeof(KT)));
-    QS3_TRY(val.alloc(B.total * sizeof(uint2)));
+    // per sector at most a bucket per row or site, and an end per site
+    DevBuf rec, info, sub;
+    QS3_TRY(rec.alloc(B.total * sizeof(uint4)));
     QS3_TRY(info.alloc((uint64_t)S * np * sizeof(uint2)));
-    QS3_TRY(sub.alloc(most * 4));
+    QS3_TRY(sub.alloc((B.total + 2 * (uint64_t)S * np) * 4));
     const cudaStream_t s0 = 0;
-    DevBuf kin, vin, first, size, off, tmp;
+    DevBuf kin, vin, key, val, first, size, off, tmp;
     QS3_TRY(kin.alloc(dmax * sizeof(KT), s0));
     QS3_TRY(vin.alloc(dmax * sizeof(uint2), s0));
+    QS3_TRY(key.alloc(dmax * sizeof(KT), s0));
+    QS3_TRY(val.alloc(dmax * sizeof(uint2), s0));
     QS3_TRY(first.alloc(((uint64_t)np + 1) * 4, s0));
     QS3_TRY(size.alloc(((uint64_t)np + 1) * 4, s0));
     QS3_TRY(off.alloc(((uint64_t)np + 1) * 4, s0));
@@ -413,45 +424,43 @@ static int build_forms_nd(Basis &B) {
     QS3_CUDA(cudaFuncSetAttribute(k_forms<ND, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
     QS3_CUDA(cudaFuncSetAttribute(k_form_fill<NO, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
     const uint64_t *bin = B.d_binom.as<uint64_t>();
-    const int gp = (int)std::min<uint64_t>(((uint64_t)np + 256) / 256, 4096);
+    const int gp = (int)((np + 256) / 256);
     uint64_t base = 0;
     for (int s = 0; s < S; ++s) {
         const uint64_t d = B.dims[s];
         SecView &v = B.secs[s];
-        KT *ks = key.as<KT>() + B.offs[s];
-        uint2 *vs = val.as<uint2>() + B.offs[s], *is = info.as<uint2>() + (uint64_t)s * np;
+        uint2 *is = info.as<uint2>() + (uint64_t)s * np;
+        uint32_t *ss = sub.as<uint32_t>() + base;
         const int g = (int)std::max<uint64_t>(1, std::min<uint64_t>((d + NTHREADS - 1) / NTHREADS, 8192));
         if (d > 0) {
             k_forms<ND, KT><<<g, NTHREADS, smem>>>(B.lv, v, kin.as<KT>(), vin.as<uint2>());
             QS3_LAUNCHED();
             size_t t2 = tb;
-            QS3_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, t2, kin.as<KT>(), ks, vin.as<U64>(), (U64 *)vs, (int64_t)d, 0,
-                                                     bits * NO));
+            QS3_CUDA(cub::DeviceRadixSort::SortPairs(tmp.p, t2, kin.as<KT>(), key.as<KT>(), vin.as<U64>(), val.as<U64>(),
+                                                     (int64_t)d, 0, bits * NO));
+            k_form_recs<KT><<<g, NTHREADS>>>(key.as<KT>(), val.as<uint2>(), d, rec.as<uint4>() + B.offs[s]);
+            QS3_LAUNCHED();
         }
-        k_form_first<NO, KT><<<gp, 256>>>(ks, d, bits, pre2, np, first.as<uint32_t>());
+        k_form_first<KT><<<gp, 256>>>(key.as<KT>(), d, bits, NO, np, first.as<uint32_t>());
         QS3_LAUNCHED();
         QS3_CUDA(cudaMemsetAsync(size.as<uint32_t>() + np, 0, 4));
-        k_bucket_size<<<gp, 256>>>(NO, B.N + 1, pre2, bin, 1, np, first.as<uint32_t>(), size.as<uint32_t>());
+        k_bucket_size<<<gp, 256>>>(NO, B.N + 1, 0, bin, 1, np, 0, first.as<uint32_t>(), size.as<uint32_t>());
         QS3_LAUNCHED();
         size_t t2 = tb;
         QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, t2, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)np + 1));
-        k_bucket_info<<<gp, 256>>>(NO, B.N + 1, pre2, bin, 1, np, first.as<uint32_t>(), off.as<uint32_t>(), is,
-                                   sub.as<uint32_t>() + base);
+        k_bucket_info<<<gp, 256>>>(NO, B.N + 1, 0, bin, 1, np, 0, first.as<uint32_t>(), off.as<uint32_t>(), is, ss);
         QS3_LAUNCHED();
         if (d > 0) {
-            k_form_fill<NO, KT><<<g, NTHREADS, smem>>>(B.lv, ks, d, pre2, first.as<uint32_t>(), is, sub.as<uint32_t>() + base);
+            k_form_fill<NO, KT><<<g, NTHREADS, smem>>>(B.lv, key.as<KT>(), d, first.as<uint32_t>(), is, ss);
             QS3_LAUNCHED();
         }
-        v.okey = ks;
-        v.oval = vs;
+        v.orec = rec.as<uint4>() + B.offs[s];
         v.finfo = is;
-        v.fsub = sub.as<uint32_t>() + base;
-        v.fpre2 = pre2;
-        base += d / 2 + 2 * (uint64_t)np;
+        v.fsub = ss;
+        base += d + 2 * (uint64_t)np;
     }
     QS3_CUDA(cudaDeviceSynchronize());
-    B.d_okey = std::move(key);
-    B.d_oval = std::move(val);
+    B.d_orec = std::move(rec);
     B.d_finfo = std::move(info);
     B.d_fsub = std::move(sub);
     QS3_CUDA(cudaMemcpy(B.d_secs.p, B.secs.data(), B.secs.size() * sizeof(SecView), cudaMemcpyHostToDevice));
@@ -467,9 +476,9 @@ int build_forms(Basis &B, size_t max_bytes) {
     if (!forms_apply(B)) return set_err(QS3_ERR_STATE, "no origin forms for this basis");
     int bits = 1;
     while ((1 << bits) < B.N) ++bits;
-    const size_t ksz = (B.nd - 1) * bits <= 32 ? 4 : 8;
-    // the lists, their index, and the sort's buffers
-    if (B.total * (3 * ksz + 3 * 8 + 2) > max_bytes) return set_err(QS3_ERR_OOM, "origin forms exceed the limit");
+    if (forms_smem(B) > (size_t)MAX_DYN_SMEM) return set_err(QS3_ERR_OVERFLOW, "origin forms need more shared memory");
+    // the records and their index, and the sort's buffers
+    if (B.total * (16 + 4 + 3 * 16) > max_bytes) return set_err(QS3_ERR_OOM, "origin forms exceed the limit");
     B.lv.form_bits = bits;
     switch (B.nd) {
         case 2: return build_forms_k<2>(B);
@@ -487,10 +496,11 @@ template <int ND, typename VT, typename KT>
 static int forms_run(Basis &B, const void *phi, void *psi, cudaStream_t st, const int *active, int dt) {
     static std::atomic<unsigned long long> cache{0};
     int grid = 1, occ = 1;
-    QS3_TRY(launch_rows(k_hphi_f<ND, VT, KT>, B, B.smem_bytes, cache, &grid, &occ));
+    const size_t smem = forms_smem(B);
+    QS3_TRY(launch_rows(k_hphi_f<ND, VT, KT>, B, smem, cache, &grid, &occ));
     if (B.ntiles == 0) return QS3_OK;
-    k_hphi_f<ND, VT, KT><<<grid, NTHREADS, B.smem_bytes, st>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(), B.S,
-                                                               B.ntiles, (const VT *)phi, (VT *)psi, active);
+    k_hphi_f<ND, VT, KT><<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(), B.S, B.ntiles,
+                                                       (const VT *)phi, (VT *)psi, active, (unsigned)forms_off(B));
     QS3_LAUNCHED();
     if (B.tune_hphi[dt] == 0) B.tune_hphi[dt] = occ;             // always the whole occupancy
     return QS3_OK;

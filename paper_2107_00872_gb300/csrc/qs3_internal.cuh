@@ -121,6 +121,14 @@ struct LatView {
     // translation by -u (u the flat site index) takes a to its representative
     const uint32_t *orb;
     uint32_t n_orb;               // orbits in the table (entries >= n_orb << 12 are invalid)
+    // diagonal constants of lattices with one J^z and the same u on every site
+    // (diag_uniform): c0 plus N_down times u, and the sums of 0, 1, ... J^z, all
+    // added one by one as the row kernels do
+    int diag_uniform;
+    double e_row;
+    float e_row_f;
+    const double *pair_sum;
+    const float *pair_sum_f;
     double jh_uniform;            // the hop amplitude J^xy / 2 when every bond has the same one, else 0
     // fixed-width adjacency (largest degree <= 6): pad_w entries per site,
     // (neighbour, fp32 hop amplitude bits) and fp32 J^z; a site with fewer
@@ -141,13 +149,12 @@ struct SecView {
     const uint2 *pinfo;
     const uint32_t *sub;
     int pre2;
-    // origin forms of the rows (qs3_hphi_search.cu), when built: sorted packed
-    // forms, (row, w | (|Stab| - 1) << 28) of each, and their index
-    const void *okey;
-    const uint2 *oval;
+    // origin forms of the rows (qs3_hphi_search.cu), when built: the sorted
+    // records (form, row, w | (|Stab| - 1) << 28), and their index by the
+    // largest site
+    const uint4 *orec;
     const uint2 *finfo;
     const uint32_t *fsub;
-    int fpre2;
     uint64_t dim;
     uint64_t off;                 // offset of the sector in a concatenated vector
     int K[3];
@@ -180,10 +187,11 @@ struct Basis {
     // device data
     DevBuf d_binom, d_adj_ptr, d_adj_nbr, d_adj_jxy, d_adj_jz, d_adj_jxy_f, d_u, d_xyz;
     DevBuf d_u_f, d_adj_jz_f;
+    DevBuf d_pair;                          // LatView::pair_sum, pair_sum_f
     DevBuf d_adj_jxy_lo, d_u_lo, d_adj_jz_lo;
     DevBuf d_adj_pad, d_adj_jz_pad;         // fixed-width adjacency (LatView::adj_pad)
     DevBuf d_sigma, d_stab, d_pinfo, d_sub;  // every sector's lists, one after another
-    DevBuf d_okey, d_oval, d_finfo, d_fsub;  // origin forms and their index (without a representative table)
+    DevBuf d_orec, d_finfo, d_fsub;          // origin forms and their index (without a representative table)
     DevBuf d_ph64, d_ph32, d_phdf;          // S x N per-site phase tables (k-sectors)
     DevBuf d_roots;                         // e^{-2 pi i n / ncell}, n < ncell (k-sectors)
     DevBuf d_secs, d_tile0, d_chunk0;
@@ -726,9 +734,9 @@ __device__ __forceinline__ int tri_root(uint32_t P) {
     return x;
 }
 
-// the buckets of prefix P (SecView::pinfo) when it has so many rows: nq of
-// them, 2^shift low ranks each, at most half as many as rows
-__device__ __forceinline__ int bucket_shift(uint32_t P, uint32_t rows, int nd, int pre2,
+// the buckets of prefix P (SecView::pinfo): nq of them, 2^shift low ranks
+// each, at most `most`
+__device__ __forceinline__ int bucket_shift(uint32_t P, uint32_t most, int nd, int pre2,
                                             const uint64_t *__restrict__ binom, int np1, uint32_t &nq) {
     uint64_t w;                            // low ranks
     if (pre2) {
@@ -737,7 +745,7 @@ __device__ __forceinline__ int bucket_shift(uint32_t P, uint32_t rows, int nd, i
     } else {
         w = binom[(size_t)(nd - 1) * np1 + P];
     }
-    const uint32_t most = rows / 2 > 1 ? rows / 2 : 1;
+    most = most > 1 ? most : 1;
     int sh = 0;
     while (w && ((w - 1) >> sh) + 1 > most) ++sh;
     nq = w ? (uint32_t)(((w - 1) >> sh) + 1) : 1u;
@@ -764,19 +772,19 @@ __device__ __forceinline__ void stage_tables(const LatView &L, uint64_t *sC, uin
 
 // entries of every (sector, prefix): its buckets plus the end
 static __global__ void k_bucket_size(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
-                              const uint32_t *__restrict__ first, uint32_t *__restrict__ size) {
+                              int half, const uint32_t *__restrict__ first, uint32_t *__restrict__ size) {
     const uint64_t cnt = (uint64_t)S * np;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t s = i / np;
         const uint32_t P = (uint32_t)(i - s * np);
         const uint32_t *f = first + s * (np + 1) + P;
         uint32_t nq;
-        bucket_shift(P, f[1] - f[0], nd, pre2, binom, np1, nq);
+        bucket_shift(P, (f[1] - f[0]) >> half, nd, pre2, binom, np1, nq);
         size[i] = nq + 1;
     }
 }
 static __global__ void k_bucket_info(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
-                              const uint32_t *__restrict__ first, const uint32_t *__restrict__ off,
+                              int half, const uint32_t *__restrict__ first, const uint32_t *__restrict__ off,
                               uint2 *__restrict__ pinfo, uint32_t *__restrict__ sub) {
     const uint64_t cnt = (uint64_t)S * np;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
@@ -784,7 +792,7 @@ static __global__ void k_bucket_info(int nd, int np1, int pre2, const uint64_t *
         const uint32_t P = (uint32_t)(i - s * np);
         const uint32_t *f = first + s * (np + 1) + P;
         uint32_t nq;
-        const int sh = bucket_shift(P, f[1] - f[0], nd, pre2, binom, np1, nq);
+        const int sh = bucket_shift(P, (f[1] - f[0]) >> half, nd, pre2, binom, np1, nq);
         pinfo[i] = make_uint2(off[i], (uint32_t)sh);
         // an empty prefix: one empty bucket
         if (f[0] == f[1])
