@@ -975,23 +975,33 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
         QS3_TRY(B.d_u_lo.upload(bu.data(), bu.size() * 4));
         QS3_TRY(B.d_adj_jz_lo.upload(cz.data(), cz.size() * 4));
     }
-    // fixed-width copy of the adjacency for the U(1) fp32 kernel
-    const int padw = B.max_degree <= 4 ? 4 : (B.max_degree <= 6 ? 6 : 0);
+    // fixed-width copies of the adjacency for the U(1) kernels
+    const int padw = K ? 0 : B.max_degree <= 2 ? 2 : B.max_degree <= 4 ? 4 : (B.max_degree <= 6 ? 6 : 0);
+    const size_t np = (size_t)N * padw;
     if (padw) {
-        std::vector<int2> pk((size_t)N * padw);
-        std::vector<float> pz((size_t)N * padw, 0.f);
+        // int4 | fp64 J^z | int2 | int2 transposed | fp32 J^z | fp32 J^z transposed
+        std::vector<unsigned char> img(np * (16 + 8 + 8 + 8 + 4 + 4), 0);
+        int4 *p64 = (int4 *)img.data();
+        double *z64 = (double *)(p64 + np);
+        int2 *p32 = (int2 *)(z64 + np), *t32 = p32 + np;
+        float *z32 = (float *)(t32 + np), *zt = z32 + np;
         for (int i = 0; i < N; ++i)
-            for (int b = 0; b < padw; ++b) {
-                const int q = deg[i] + b;
+            for (int e = 0; e < padw; ++e) {
+                const size_t a = (size_t)i * padw + e, t = (size_t)e * N + i;
+                const int q = deg[i] + e;
                 const bool real = q < deg[i + 1];
-                float jf = real ? ajxyf[q] : 0.f;
-                int bitsf;
-                std::memcpy(&bitsf, &jf, 4);
-                pk[(size_t)i * padw + b] = make_int2(real ? nbr[q] : i, bitsf);
-                pz[(size_t)i * padw + b] = real ? ajzf[q] : 0.f;
+                const float jf = real ? ajxyf[q] : 0.f;
+                const double jd = real ? ajxy[q] : 0.0;
+                int bf, bd[2];
+                std::memcpy(&bf, &jf, 4);
+                std::memcpy(bd, &jd, 8);
+                const int j = real ? nbr[q] : i;
+                p64[a] = make_int4(j, 0, bd[0], bd[1]);
+                z64[a] = real ? ajz[q] : 0.0;
+                p32[a] = t32[t] = make_int2(j, bf);
+                z32[a] = zt[t] = real ? ajzf[q] : 0.f;
             }
-        QS3_TRY(B.d_adj_pad.upload(pk.data(), pk.size() * sizeof(int2)));
-        QS3_TRY(B.d_adj_jz_pad.upload(pz.data(), pz.size() * 4));
+        QS3_TRY(B.d_pad.upload(img.data(), img.size()));
     }
     std::vector<uint32_t> xyz(N);
     for (int r = 0; r < N; ++r) {
@@ -1031,9 +1041,15 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     L.xyz = B.d_xyz.as<uint32_t>();
     L.nsub = B.nsub;
     L.ncell = B.ncell;
-    L.adj_pad = B.d_adj_pad.as<int2>();
-    L.adj_jz_pad = B.d_adj_jz_pad.as<float>();
     L.pad_w = padw;
+    if (padw) {
+        L.adj_pad64 = B.d_pad.as<int4>();
+        L.adj_jz_pad64 = (const double *)(L.adj_pad64 + np);
+        L.adj_pad = (const int2 *)(L.adj_jz_pad64 + np);
+        L.adjt = L.adj_pad + np;
+        L.adj_jz_pad = (const float *)(L.adjt + np);
+        L.adjt_jz = L.adj_jz_pad + np;
+    }
     L.jh_uniform = 0.0;
     if (nb > 0) {
         bool same = true;

@@ -676,88 +676,6 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_of(LatView L, const SecVie
     }
 }
 
-// U(1) H Phi with 32-bit ranks, for C(N, N_down) < 2^32, N_down <= 4, fp32
-// vectors and lattices of degree <= 6: the binomial rows 0..N_down as a
-// 32-bit table in shared memory, one thread per row striding over the single
-// sector, and the fixed-width adjacency (DEGB = 4 or 6 entries per site, a
-// site with fewer padded with itself and zero couplings), one 8-byte load
-// per entry (neighbour, hop amplitude).  The hop of c_m to j keeps its place
-// in the sorted list when c_{m-1} < j < c_{m+1}; then its rank is the row's
-// rank with C(c_m, m+1) replaced by C(j, m+1) -- two compares and one table
-// read, and a padded entry (j = c_m) lands on the row itself with amplitude
-// 0.  Only the other hops (j occupied, or j passing another down spin) take
-// the occupancy test and the re-sort.  Per occupied site the ranks of its
-// DEGB entries are formed before their gathers issue together.  Same
-// signature as k_hphi (the launch and the autotuner treat both alike).
-template <int ND, typename VT, int DEGB>
-__global__ void __launch_bounds__(NTHREADS, DEGB <= 4 ? 6 : 4) k_hphi_u1n(LatView L, const SecView *__restrict__ secs,
-                                                      const int *__restrict__ tile0, int S, int ntiles,
-                                                      const VT *__restrict__ phi, VT *__restrict__ psi,
-                                                      const int *__restrict__ active) {
-    using R = typename VTr<VT>::R;
-    using CT = typename VTr<VT>::C;
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint32_t *sC = (uint32_t *)smem;
-    const int np1 = L.np1;
-    for (int i = threadIdx.x; i < (ND + 1) * np1; i += blockDim.x) sC[i] = (uint32_t)L.binom[i];
-    __syncthreads();
-    if (active && !active[0]) return;
-    const uint64_t dim = secs[0].dim;     // < 2^32
-    const int2 *__restrict__ pad = L.adj_pad;
-    for (uint64_t rw = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; rw < dim; rw += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t row = (uint32_t)rw;
-        int c[ND];
-        unrank32(row, sC, np1, c);
-        const VT x0 = phi[row];
-        R e = diag_c0<R>(L), dd = 0;
-        CT acc;
-        acc.x = 0; acc.y = 0;
-#pragma unroll
-        for (int m = 0; m < ND; ++m) {
-            const int i = c[m];
-            e += diag_u<R>(L, i);
-            const int lo = m > 0 ? c[m > 0 ? m - 1 : 0] : -1;
-            const int hi = m < ND - 1 ? c[m < ND - 1 ? m + 1 : m] : np1;
-            const uint32_t base = row - sC[(m + 1) * np1 + i];
-            const uint32_t *col = sC + (m + 1) * np1;
-            uint32_t r2b[DEGB];
-            R cfb[DEGB];
-#pragma unroll
-            for (int b = 0; b < DEGB; ++b) {
-                const int2 pk = __ldg(pad + i * DEGB + b);
-                const int j = pk.x;
-                const R cf = (R)__int_as_float(pk.y);
-                r2b[b] = base + col[j];
-                cfb[b] = cf;
-                if (!(j > lo && j < hi)) {
-                    // occupied, or passing another down spin
-                    bool occ = false;
-#pragma unroll
-                    for (int k = 0; k < ND; ++k) occ |= (c[k] == j);
-                    if (occ) {
-                        dd += (R)__ldg(L.adj_jz_pad + i * DEGB + b);
-                        cfb[b] = 0;
-                        r2b[b] = row;
-                    } else {
-                        int tt[ND];
-#pragma unroll
-                        for (int k = 0; k < ND; ++k) tt[k] = (k == m) ? j : c[k];
-                        sort_net(tt);
-                        r2b[b] = rank_of32(tt, sC, np1);
-                    }
-                }
-            }
-            VT vb[DEGB];
-#pragma unroll
-            for (int b = 0; b < DEGB; ++b) vb[b] = phi[r2b[b]];
-#pragma unroll
-            for (int b = 0; b < DEGB; ++b) madd_r(acc, cfb[b], vb[b]);
-        }
-        madd_r(acc, e + (R)0.5 * dd, x0);
-        store(psi + row, acc);
-    }
-}
-
 // nnz count per sector: the diagonal plus every hop that lands on a member of the sector
 template <int ND, bool KS>
 __global__ void __launch_bounds__(NTHREADS) k_count(LatView L, const SecView *__restrict__ secs,
@@ -858,37 +776,10 @@ static int hphi_ndt(Basis &B, const void *phi, void *psi, cudaStream_t st, const
     return QS3_OK;
 }
 
-template <int ND, typename VT, int DEGB>
-static int hphi_u1n(Basis &B, const void *phi, void *psi, cudaStream_t st, const int *active) {
-    static std::atomic<unsigned long long> cache{0};
-    const size_t smem = (size_t)(ND + 1) * (B.N + 1) * sizeof(uint32_t);
-    int grid = 1, occ = 1;
-    QS3_TRY(launch_rows(k_hphi_u1n<ND, VT, DEGB>, B, smem, cache, &grid, &occ));
-    if (B.ntiles == 0) return QS3_OK;
-    int &bps = B.tune_hphi[DtIdx<VT>::v];
-    if (bps == 0) {
-        cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
-        QS3_CUDA(cudaStreamIsCapturing(st, &cst));
-        if (cst == cudaStreamCaptureStatusNone) {
-            int b = occ;
-            QS3_TRY(tune_grid(k_hphi_u1n<ND, VT, DEGB>, B, occ, st, (const VT *)phi, (VT *)psi, active, b, smem));
-            bps = b;
-        }
-    }
-    if (bps > 0) grid = std::max(1, std::min(B.ntiles, std::min(bps, occ) * num_sms()));
-    k_hphi_u1n<ND, VT, DEGB><<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(), B.S,
-                                                           B.ntiles, (const VT *)phi, (VT *)psi, active);
-    QS3_LAUNCHED();
-    return QS3_OK;
-}
-
 template <int ND, typename VT, bool KS>
 static int hphi_nd(Basis &B, const void *phi, void *psi, cudaStream_t st, const int *active) {
     if constexpr (KS) {
         if (B.lv.orb) return hphi_ndt<ND, VT, true, true>(B, phi, psi, st, active);
-    } else if constexpr (ND <= 4 && sizeof(typename VTr<VT>::R) == 4) {
-        if (B.narrow_ranks && B.lv.pad_w == 4) return hphi_u1n<ND, VT, 4>(B, phi, psi, st, active);
-        if (B.narrow_ranks && B.lv.pad_w == 6) return hphi_u1n<ND, VT, 6>(B, phi, psi, st, active);
     }
     return hphi_ndt<ND, VT, KS, false>(B, phi, psi, st, active);
 }
@@ -1081,6 +972,9 @@ int hphi_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t
         if (dt == QS3_C64) return hphi_vt<float2, true>(B, phi, psi, st, active);
         if (dt == QS3_C128) return hphi_vt<double2, true>(B, phi, psi, st, active);
     } else {
+        bool done = false;
+        QS3_TRY(hphi_u1_launch(B, dt, phi, psi, st, active, &done));
+        if (done) return QS3_OK;
         if (dt == QS3_F32) return hphi_vt<float, false>(B, phi, psi, st, active);
         if (dt == QS3_F64) return hphi_vt<double, false>(B, phi, psi, st, active);
         if (dt == QS3_C64) return hphi_vt<float2, false>(B, phi, psi, st, active);

@@ -130,12 +130,17 @@ struct LatView {
     const double *pair_sum;
     const float *pair_sum_f;
     double jh_uniform;            // the hop amplitude J^xy / 2 when every bond has the same one, else 0
-    // fixed-width adjacency (largest degree <= 6): pad_w entries per site,
-    // (neighbour, fp32 hop amplitude bits) and fp32 J^z; a site with fewer
-    // neighbours is padded with itself and zero couplings
-    const int2 *adj_pad;
-    const float *adj_jz_pad;
-    int pad_w;                    // 4 or 6; 0 when the table is not built
+    // U(1)-only bases of largest degree <= 6: fixed-width adjacency, pad_w
+    // entries per site, (neighbour, hop amplitude) in one load: fp32 in 8 bytes,
+    // fp64 in 16 (neighbour, -, amplitude); a site with fewer neighbours is
+    // padded with itself and zero couplings.  adjt: the fp32 entries transposed
+    // (entry b of site i at b N + i), so that threads of consecutive
+    // sites read consecutive words
+    int pad_w;                    // 2, 4 or 6; 0 when the tables are not built
+    const int2 *adj_pad, *adjt;
+    const int4 *adj_pad64;
+    const float *adj_jz_pad, *adjt_jz;
+    const double *adj_jz_pad64;
 };
 
 struct SecView {
@@ -189,7 +194,7 @@ struct Basis {
     DevBuf d_u_f, d_adj_jz_f;
     DevBuf d_pair;                          // LatView::pair_sum, pair_sum_f
     DevBuf d_adj_jxy_lo, d_u_lo, d_adj_jz_lo;
-    DevBuf d_adj_pad, d_adj_jz_pad;         // fixed-width adjacency (LatView::adj_pad)
+    DevBuf d_pad;                           // fixed-width adjacency (LatView::adj_pad ...)
     DevBuf d_sigma, d_stab, d_pinfo, d_sub;  // every sector's lists, one after another
     DevBuf d_orec, d_finfo, d_fsub;          // origin forms and their index (without a representative table)
     DevBuf d_ph64, d_ph32, d_phdf;          // S x N per-site phase tables (k-sectors)
@@ -810,6 +815,9 @@ int hphi_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t
 // (*dx) ld when dx (device) is given; psi complex128, or double-float when out_df
 int hphi_df_launch(Basis &B, const void *phi, const int *dx, uint64_t ld, void *psi, cudaStream_t st,
                    const int *active = nullptr, bool out_df = false);
+// H Phi of a U(1)-only basis with 32-bit ranks (qs3_hphi_u1.cu); *done = false
+// when no kernel there takes it (the caller then runs the general one)
+int hphi_u1_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t st, const int *active, bool *done);
 // the same on momentum sectors by origin forms (qs3_hphi_search.cu), built at
 // creation of a basis without a representative table
 int build_forms(Basis &B, size_t max_bytes);
