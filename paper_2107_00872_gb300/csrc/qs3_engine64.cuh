@@ -324,32 +324,27 @@ __global__ void __launch_bounds__(XT)
     if (lane == 0) ge[((uint64_t)j * nchunks + blockIdx.x) * XW + warp] = em;
 }
 
-// the digit image of one interleaved binary64 vector (slot 0 of dg, ge)
-template <typename VT>
-__global__ void __launch_bounds__(XT)
-    k_digitize_il(const VT *__restrict__ x, uint64_t D, typename DigT<VT>::T *__restrict__ dg, int *__restrict__ ge,
-                  const SecView *__restrict__ secs, const int *__restrict__ chunk0, int S) {
-    constexpr int NC = IsC<VT>::v ? 2 : 1;
+// the gather image of one interleaved complex128 vector
+__global__ void __launch_bounds__(XT) k_image(const double2 *__restrict__ x, int4 *__restrict__ hd,
+                                              const SecView *__restrict__ secs, const int *__restrict__ chunk0, int S) {
     const ChunkInfo ci = chunk_info(secs, chunk0, S, blockIdx.x);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t hw[XR][2], lw[XR][2];
 #pragma unroll
     for (int k = 0; k < XR; ++k) {
         const int r = threadIdx.x + k * XT;
-        const double2 v = r < ci.n ? ld2(x + ci.base + r) : make_double2(0.0, 0.0);
+        const double2 v = r < ci.n ? x[ci.base + r] : make_double2(0.0, 0.0);
         hw[k][0] = (uint32_t)__double2hiint(v.x);
         lw[k][0] = (uint32_t)__double2loint(v.x);
         hw[k][1] = (uint32_t)__double2hiint(v.y);
         lw[k][1] = (uint32_t)__double2loint(v.y);
     }
     int d1[XR][2], d0[XR][2];
-    const int em = fx_group<NC>(hw, lw, d1, d0);
+    const int em = fx_group<2>(hw, lw, d1, d0);
 #pragma unroll
     for (int k = 0; k < XR; ++k) {
         const int r = threadIdx.x + k * XT;
-        if (r < ci.n) dig_st(dg, D, ci.base + r, d1[k], d0[k]);
+        if (r < ci.n) hd[ci.base + r] = hd_pack(d1[k][0], d0[k][0], d1[k][1], d0[k][1], em);
     }
-    if (lane == 0) ge[(uint64_t)blockIdx.x * XW + warp] = em;
 }
 
 // The exact dot products conj(V_{j0+j}) . w over chunk c, as warp partials:
@@ -1393,15 +1388,17 @@ template <typename VT> static int updb_prepare() {
 }
 
 // psi_{x+1} = w * inv[s]: into the store's slot (graph mode: slot *dx + 1 of
-// the store at out), its digit-store image (dg, ge) and hin, the interleaved
-// input of the next H Phi.  w may alias hin (the start vector is normalised
-// in place).  One block of XT threads per chunk.
+// the store at out), its digit-store image (dg, ge) and hin, the input of the
+// next H Phi: the gather image of the integer product (hx), else interleaved
+// binary64.  w may alias hin (the start vector is normalised in place: a
+// thread reads its rows before it writes them).  One block of XT threads per
+// chunk.
 template <typename VT>
 __global__ void __launch_bounds__(XT)
     k_scale64(const VT *w, typename PlS<VT>::T *__restrict__ out, typename DigT<VT>::T *__restrict__ dg,
               int *__restrict__ ge, int nchunks, VT *hin, const double *__restrict__ inv,
               const SecView *__restrict__ secs, const int *__restrict__ chunk0, int S, const int *__restrict__ active,
-              const int *__restrict__ dx, uint64_t D) {
+              const int *__restrict__ dx, uint64_t D, int hx) {
     constexpr int NC = IsC<VT>::v ? 2 : 1;
     if (dx) {
         out += (uint64_t)(*dx + 1) * 2 * D;
@@ -1422,7 +1419,7 @@ __global__ void __launch_bounds__(XT)
             v.x *= f;
             v.y *= f;
             pl_st(out, D, ci.base + r, v);
-            st2(hin + ci.base + r, v);
+            if (!hx) st2(hin + ci.base + r, v);
         }
         hw[k][0] = (uint32_t)__double2hiint(v.x);
         lw[k][0] = (uint32_t)__double2loint(v.x);
@@ -1434,7 +1431,10 @@ __global__ void __launch_bounds__(XT)
 #pragma unroll
     for (int k = 0; k < XR; ++k) {
         const int r = threadIdx.x + k * XT;
-        if (r < ci.n) dig_st(dg, D, ci.base + r, d1[k], d0[k]);
+        if (r < ci.n) {
+            dig_st(dg, D, ci.base + r, d1[k], d0[k]);
+            if (NC == 2 && hx) ((int4 *)hin)[ci.base + r] = hd_pack(d1[k][0], d0[k][0], d1[k][1], d0[k][1], em);
+        }
     }
     if (lane == 0) ge[(uint64_t)blockIdx.x * XW + warp] = em;
 }
@@ -1725,7 +1725,7 @@ struct Engine64 {
     int scale_store(const VT *w, int j) {
         if (B.nchunks == 0) return QS3_OK;
         k_scale64<VT><<<grid(), XT, 0, st>>>(w, svec(j), dg(j), ge(j), B.nchunks, hin(0), inv.as<double>(), secs(),
-                                             c0(), B.S, act(), nullptr, D);
+                                             c0(), B.S, act(), nullptr, D, hx());
         QS3_LAUNCHED();
         return QS3_OK;
     }
@@ -1756,13 +1756,15 @@ struct Engine64 {
         for (int s = 0; s < B.S; ++s)
             if (h_active[s]) stats->nnz += B.nnz_sec[s];
     }
-    // w = H psi_x: on the integer units from the digit image of slot x (slot
-    // *dx in graph mode) when the basis allows it and strict64 is off, else
-    // the binary64 FMA kernels
+    // whether H Phi runs on the integer units: hin then holds the gather image
+    int hx() const { return !strict && IsC<VT>::v && hphi_x_ok(B) ? 1 : 0; }
+    // w = H psi_x: on the integer units when the basis allows it and strict64 is
+    // off (the image of psi_x in hin, its values in slot x, *dx in graph mode),
+    // else the binary64 FMA kernels
     int hphi_apply(int x, const int *dx) {
-        if (!strict && IsC<VT>::v && hphi_x_ok(B))
-            return dx ? hphi_x_launch(B, hin(0), DG.p, GE.as<int>(), dx, wv(), st, act())
-                      : hphi_x_launch(B, hin(0), dg(x), ge(x), nullptr, wv(), st, act());
+        if (hx())
+            return hphi_x_launch(B, {(const int4 *)hinb.p, nullptr, (const uint2 *)(dx ? V.as<ST>() : svec(x)), D, dx}, wv(),
+                                 st, act());
         return hphi_launch(B, dtype(), hin(x), wv(), st, act());
     }
     // the Gram-Schmidt dot pass against psi_0 .. psi_x, timed with events
@@ -1813,7 +1815,7 @@ struct Engine64 {
                                                          dx);
         QS3_LAUNCHED();
         k_scale64<VT><<<grid(), XT, 0, st>>>(w, V.as<ST>(), dg(), ge(), B.nchunks, hin(0), inv.as<double>(), secs(),
-                                             c0(), B.S, act(), dx, D);
+                                             c0(), B.S, act(), dx, D, hx());
         QS3_LAUNCHED();
         k_advance<<<1, 1, 0, st>>>(xdev.as<int>());
         QS3_LAUNCHED();

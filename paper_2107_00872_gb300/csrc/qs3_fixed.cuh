@@ -51,6 +51,21 @@ __device__ __forceinline__ long long mad_w(int a, int b, long long c) {
     asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
     return d;
 }
+// The image H Phi gathers: the digits of a complex element and its group's
+// grid exponent in one 16-byte word, so that a hop's target costs one gather
+// (the planes of the digit store and the exponents were three, and seven
+// instructions of address arithmetic).  |P1| <= 2^27 and |P0| <= 2^25 leave
+// room for the 11 bits of the exponent: the low bit of x and five of z and w.
+__device__ __forceinline__ int4 hd_pack(int r1, int r0, int i1, int i0, int em) {
+    return make_int4((int)((unsigned)r1 << 1) | (em >> 10), i1, (int)((unsigned)r0 << 5) | (em & 31),
+                     (int)((unsigned)i0 << 5) | ((em >> 5) & 31));
+}
+__device__ __forceinline__ void hd_unpack(int4 q, int2 &f1, int2 &f0, int &em) {
+    f1 = make_int2(q.x >> 1, q.y);
+    f0 = make_int2(q.z >> 5, q.w >> 5);
+    em = ((q.x & 1) << 10) | ((q.w & 31) << 5) | (q.z & 31);
+}
+
 // a 2^k rounded to the nearest binary64 (ties to even) in integer operations
 // (the fp64 pipe issues one warp instruction per ~70 ALU ones, even for a
 // single active lane); only a result below the normal range takes fp64 ops
@@ -85,7 +100,5 @@ __device__ __forceinline__ double i128_ldexp(__int128 a, int k) {
     return __longlong_as_double((long long)(sgn | ((unsigned long long)(e + 1023) << 52) | (mant & 0xfffffffffffffull)));
 }
 
-// the warp group of row o (0 <= o < BROWS) of a chunk in the digit store
-__host__ __device__ __forceinline__ int dg_group(int o) { return (o & (XT - 1)) >> 5; }
 
 }  // namespace qs3

@@ -242,16 +242,14 @@ __global__ void __launch_bounds__(NTHREADS, (KS && TB && sizeof(VT) == 16) ? 4 :
 
 // H Phi of the binary64 engine on the integer units: k-sectors with the
 // representative table and one hop amplitude J/2 on every bond.  phi comes
-// twice: as binary64 (the diagonal term) and as its digit-store image (dg:
-// the top-digit plane then the low-digit plane, D int2 (re, im) each; ge:
-// the grid exponent of every chunk's warp groups).  Each hop's product
+// twice (HxVec): as binary64 (the diagonal term) and as its gather image
+// (hd_pack).  Each hop's product
 // phase x phi is formed exactly on the images (the phases on the grid 2^-52,
 // staged per sector as digits) with mad.wide.s32, folded at weight 2^52
 // (rounded to nearest) and added to the row sum (RowAcc); terms whose target
 // stabiliser differs from the row's (norm ratio != 1, rare) are summed in
 // binary64 as in k_hphi.  The row sum is rounded to binary64 once, then
-// psi = J/2 sum + diag phi in binary64.  Graph mode (dx): dg and ge are the
-// store's, slot *dx.
+// psi = J/2 sum + diag phi in binary64.
 // the row sum of the integer H Phi: (re, im) 2^(r - 1075), r the group
 // exponent of the largest term so far; a term T 2^(em - 1075) (|T| <= 2^54)
 // is rounded to nearest onto that grid, and a term of a coarser group first
@@ -294,10 +292,7 @@ __device__ __forceinline__ void term_x(int4 p, int2 f1, int2 f0, long long &tr, 
 template <int ND>
 __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView *__restrict__ secs,
                                                        const int *__restrict__ tile0, int S, int ntiles,
-                                                       const double2 *__restrict__ phi, const int2 *__restrict__ dg,
-                                                       const int *__restrict__ ge, const int *__restrict__ chunk0,
-                                                       int nchunks, uint64_t D,
-                                                       const int *__restrict__ dx, double2 *__restrict__ psi,
+                                                       HxVec hv, double2 *__restrict__ psi,
                                                        const int *__restrict__ active) {
     extern __shared__ __align__(16) unsigned char smem[];
     SmemLayout sm = carve(L, smem);
@@ -307,14 +302,11 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
         snorm[threadIdx.x] = sqrt((double)threadIdx.x);
         snorm[9 + threadIdx.x] = threadIdx.x ? 1.0 / sqrt((double)threadIdx.x) : 0.0;
     }
-    if (dx) {
-        dg += (uint64_t)(*dx) * 2 * D;
-        ge += (uint64_t)(*dx) * nchunks * XW;
-    }
+    hv.at_slot();
     const double juni = L.jh_uniform;
     __syncthreads();
     int4 *pd = (int4 *)sm.sph;          // the current sector's phases: (re.P1, re.P0, im.P1, im.P0) on 2^-52
-    int cur = -1, c0s = 0;
+    int cur = -1;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int s = (S == 1) ? 0 : sector_of_tile(tile0, S, t);
         if (active && !active[s]) continue;
@@ -328,7 +320,6 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
                 fx_digits((uint32_t)__double2hiint(p.y), (uint32_t)__double2loint(p.y), 1023, b1, b0);
                 pd[i] = make_int4(a1, a0, b1, b0);
             }
-            c0s = chunk0[s];
             __syncthreads();
             cur = s;
         }
@@ -337,7 +328,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
         const uint64_t rank = __ldg(sv.sigma + row);
         int c[ND];
         unrank(rank, sm.sC, L.np1, c);
-        const double2 x0 = phi[sv.off + row];
+        const double2 x0 = hv.value(sv.off + row);
         const int st_row = sv.stab[row];
         const double rs = snorm[9 + st_row];
         double e = L.c0, dd = 0.0;
@@ -382,9 +373,9 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
                 const int u = (int)(ee & 4095u);
                 const int st = __ldg(sv.stab + idx);
                 if (st == st_row) {
-                    const uint64_t gi = sv.off + idx;
-                    const int2 f1 = dg[gi], f0 = dg[D + gi];
-                    const int em = __ldg(ge + (uint64_t)(c0s + (int)(idx >> 11)) * XW + dg_group((int)(idx & 2047u)));
+                    int2 f1, f0;
+                    int em;
+                    hd_unpack(__ldg(hv.hd + sv.off + idx), f1, f0, em);
                     long long tr, ti;
                     term_x(pd[u], f1, f0, tr, ti);
                     row_add(acc, tr, ti, em);
@@ -393,7 +384,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
                     const double f = snorm[st] * rs;
                     p.x *= f;
                     p.y *= f;
-                    acc_add(acc64, p, phi[sv.off + idx]);
+                    acc_add(acc64, p, hv.value(sv.off + idx));
                 }
             }
         }
@@ -478,10 +469,7 @@ template <int ND>
 __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView *__restrict__ secs, int S,
                                                    const uint64_t *__restrict__ oreps,
                                                    const uint8_t *__restrict__ ostab, uint32_t n_orb, int ngrp, int osg,
-                                                   const int4 *__restrict__ phdig, const double2 *__restrict__ phi,
-                                                   const int2 *__restrict__ dg, const int *__restrict__ ge,
-                                                   const int *__restrict__ chunk0, int nchunks, uint64_t D,
-                                                   const int *__restrict__ dx,
+                                                   const int4 *__restrict__ phdig, HxVec hv,
                                                    double2 *__restrict__ psi, const int *__restrict__ active,
                                                    int maxh) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -494,10 +482,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView
         snorm[threadIdx.x] = sqrt((double)threadIdx.x);
         snorm[9 + threadIdx.x] = threadIdx.x ? 1.0 / sqrt((double)threadIdx.x) : 0.0;
     }
-    if (dx) {
-        dg += (uint64_t)(*dx) * 2 * D;
-        ge += (uint64_t)(*dx) * nchunks * XW;
-    }
+    hv.at_slot();
     __syncthreads();
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (tid >= (uint64_t)n_orb * ngrp) return;
@@ -524,7 +509,6 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView
         const int32_t row = __ldg(t2 + g);
         if (row < 0) continue;
         const uint64_t off = secs[s].off;
-        const int c0s = __ldg(chunk0 + s);
         const int4 *pds = phdig + (size_t)s * L.N;
         RowAcc acc;
         double2 acc64 = make_double2(0.0, 0.0);
@@ -541,41 +525,34 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView
                 stb[b] = in ? mys[(size_t)(h0 + b) * blockDim.x] : 0;
                 r2[b] = in ? __ldg(t2 + (ee[b] >> 12)) : -1;
             }
-            int2 f1[4], f0[4];
-            int em[4];
+            int4 q[4];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                if (r2[b] >= 0 && stb[b] == st_row) {
-                    const uint64_t gi = off + (uint32_t)r2[b];
-                    f1[b] = dg[gi];
-                    f0[b] = dg[D + gi];
-                    em[b] = __ldg(ge + (uint64_t)(c0s + (r2[b] >> 11)) * XW + dg_group(r2[b] & 2047));
-                } else {
-                    f1[b] = f0[b] = make_int2(0, 0);
-                    em[b] = 0;
-                }
-            }
+            for (int b = 0; b < 4; ++b)
+                q[b] = r2[b] >= 0 && stb[b] == st_row ? __ldg(hv.hd + off + (uint32_t)r2[b]) : make_int4(0, 0, 0, 0);
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 if (r2[b] < 0) continue;
                 const int u = (int)(ee[b] & 4095u);
                 if (stb[b] == st_row) {
+                    int2 f1, f0;
+                    int em;
+                    hd_unpack(q[b], f1, f0, em);
                     long long tr, ti;
-                    term_x(__ldg(pds + u), f1[b], f0[b], tr, ti);
-                    row_add(acc, tr, ti, em[b]);
+                    term_x(__ldg(pds + u), f1, f0, tr, ti);
+                    row_add(acc, tr, ti, em);
                 } else {
                     double2 p = secs[s].ph64[u];
                     const double f = snorm[stb[b]] * rs;
                     p.x *= f;
                     p.y *= f;
-                    acc_add(acc64, p, phi[off + (uint32_t)r2[b]]);
+                    acc_add(acc64, p, hv.value(off + (uint32_t)r2[b]));
                 }
             }
         }
         double2 acch;
         acch.x = i128_ldexp(acc.re, acc.r - 1075) + acc64.x;
         acch.y = i128_ldexp(acc.im, acc.r - 1075) + acc64.y;
-        const double2 x0 = phi[off + (uint32_t)row];
+        const double2 x0 = hv.value(off + (uint32_t)row);
         double2 out;
         out.x = fma(ed, x0.x, juni * acch.x);
         out.y = fma(ed, x0.y, juni * acch.y);
@@ -800,22 +777,20 @@ static int hphi_vt(Basis &B, const void *phi, void *psi, cudaStream_t st, const 
 }
 
 template <int ND>
-static int hphix_nd(Basis &B, const double2 *phi, const int2 *dg, const int *ge, const int *dx,
-                    double2 *psi, cudaStream_t st, const int *active) {
+static int hphix_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, const int *active) {
     static std::atomic<unsigned long long> cache{0};
     int grid = 1, occ = 1;
     QS3_TRY(launch_rows(k_hphi_x<ND>, B, B.smem_bytes, cache, &grid, &occ));
     if (B.ntiles == 0) return QS3_OK;
     auto launch = [&](int g) {
         k_hphi_x<ND><<<g, NTHREADS, B.smem_bytes, st>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(), B.S,
-                                                         B.ntiles, phi, dg, ge, B.d_chunk0.as<int>(), B.nchunks,
-                                                         B.total, dx, psi, active);
+                                                         B.ntiles, hv, psi, active);
     };
     int &bps = B.tune_hphix;
     if (bps == 0) {
         cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
         QS3_CUDA(cudaStreamIsCapturing(st, &cst));
-        if (cst == cudaStreamCaptureStatusNone && !dx) {
+        if (cst == cudaStreamCaptureStatusNone && !hv.dx) {
             int b = occ;
             QS3_TRY(tune_blocks(B, occ, st, b, launch));
             bps = b;
@@ -841,8 +816,7 @@ static size_t orb_smem(const Basis &B, int maxh) {
 }
 
 template <int ND>
-static int hphio_nd(Basis &B, const double2 *phi, const int2 *dg, const int *ge, const int *dx,
-                    double2 *psi, cudaStream_t st, const int *active) {
+static int hphio_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, const int *active) {
     const int maxh = std::max(1, B.nd * B.max_degree);
     const size_t smem = orb_smem(B, maxh);
     if (!smem) return set_err(QS3_ERR_OVERFLOW, "hop lists of %d entries per row", maxh);
@@ -857,8 +831,7 @@ static int hphio_nd(Basis &B, const double2 *phi, const int2 *dg, const int *ge,
     const int grid = (int)((nthr + NTHREADS - 1) / NTHREADS);
     k_hphi_o<ND><<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.S, B.d_oreps.as<uint64_t>(),
                                                 B.d_ostab.as<uint8_t>(), (uint32_t)B.n_orb, ngrp, osg,
-                                                B.d_phdig.as<int4>(), phi, dg, ge, B.d_chunk0.as<int>(), B.nchunks,
-                                                B.total, dx, psi, active, maxh);
+                                                B.d_phdig.as<int4>(), hv, psi, active, maxh);
     QS3_LAUNCHED();
     return QS3_OK;
 }
@@ -907,36 +880,33 @@ bool hphi_x_ok(const Basis &B) {
     return B.has_k && B.lv.orb && B.lv.jh_uniform != 0.0 && B.nd > 0 && !B.stored_terms && B.total > 0;
 }
 
-int hphi_x_launch(Basis &B, const void *phi, const void *dg, const int *ge, const int *dx, void *psi, cudaStream_t st,
-                  const int *active) {
+int hphi_x_launch(Basis &B, const HxVec &hv, void *psi, cudaStream_t st, const int *active) {
     if (!hphi_x_ok(B)) return set_err(QS3_ERR_STATE, "the integer H Phi needs a k-sector basis with the "
                                                      "representative table and one hop amplitude");
-    const double2 *p = (const double2 *)phi;
-    const int2 *g = (const int2 *)dg;
     double2 *o = (double2 *)psi;
     // several sectors share the orbits: the orbit-batched kernel
     if (B.S >= 2 && B.d_oreps.p) {
         switch (B.nd) {
-            case 1: return hphio_nd<1>(B, p, g, ge, dx, o, st, active);
-            case 2: return hphio_nd<2>(B, p, g, ge, dx, o, st, active);
-            case 3: return hphio_nd<3>(B, p, g, ge, dx, o, st, active);
-            case 4: return hphio_nd<4>(B, p, g, ge, dx, o, st, active);
-            case 5: return hphio_nd<5>(B, p, g, ge, dx, o, st, active);
-            case 6: return hphio_nd<6>(B, p, g, ge, dx, o, st, active);
-            case 7: return hphio_nd<7>(B, p, g, ge, dx, o, st, active);
-            case 8: return hphio_nd<8>(B, p, g, ge, dx, o, st, active);
+            case 1: return hphio_nd<1>(B, hv, o, st, active);
+            case 2: return hphio_nd<2>(B, hv, o, st, active);
+            case 3: return hphio_nd<3>(B, hv, o, st, active);
+            case 4: return hphio_nd<4>(B, hv, o, st, active);
+            case 5: return hphio_nd<5>(B, hv, o, st, active);
+            case 6: return hphio_nd<6>(B, hv, o, st, active);
+            case 7: return hphio_nd<7>(B, hv, o, st, active);
+            case 8: return hphio_nd<8>(B, hv, o, st, active);
             default: return set_err(QS3_ERR_INVALID_ARG, "n_down %d", B.nd);
         }
     }
     switch (B.nd) {
-        case 1: return hphix_nd<1>(B, p, g, ge, dx, o, st, active);
-        case 2: return hphix_nd<2>(B, p, g, ge, dx, o, st, active);
-        case 3: return hphix_nd<3>(B, p, g, ge, dx, o, st, active);
-        case 4: return hphix_nd<4>(B, p, g, ge, dx, o, st, active);
-        case 5: return hphix_nd<5>(B, p, g, ge, dx, o, st, active);
-        case 6: return hphix_nd<6>(B, p, g, ge, dx, o, st, active);
-        case 7: return hphix_nd<7>(B, p, g, ge, dx, o, st, active);
-        case 8: return hphix_nd<8>(B, p, g, ge, dx, o, st, active);
+        case 1: return hphix_nd<1>(B, hv, o, st, active);
+        case 2: return hphix_nd<2>(B, hv, o, st, active);
+        case 3: return hphix_nd<3>(B, hv, o, st, active);
+        case 4: return hphix_nd<4>(B, hv, o, st, active);
+        case 5: return hphix_nd<5>(B, hv, o, st, active);
+        case 6: return hphix_nd<6>(B, hv, o, st, active);
+        case 7: return hphix_nd<7>(B, hv, o, st, active);
+        case 8: return hphix_nd<8>(B, hv, o, st, active);
         default: return set_err(QS3_ERR_INVALID_ARG, "n_down %d", B.nd);
     }
 }

@@ -824,13 +824,30 @@ int build_forms(Basis &B, size_t max_bytes);
 int hphi_forms_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t st, const int *active);
 int count_nnz(Basis &B, uint64_t *nnz);
 // the binary64 engine's H Phi on the integer units (qs3_hphi.cu, k_hphi_x and the
-// orbit-batched k_hphi_o): phi as binary64 and as its digit-store image (dg, ge:
-// slot *dx of the store when dx is given)
+// orbit-batched k_hphi_o).  Its input: the gather image hd (hd_pack) and the
+// binary64 values, interleaved (phi) or the engine's word-planar slot (plane, D
+// elements per word plane; slot *dx of a store when dx is given)
+struct HxVec {
+    const int4 *hd;
+    const double2 *phi;
+    const uint2 *plane;
+    uint64_t D;
+    const int *dx;
+#ifdef __CUDACC__
+    __device__ __forceinline__ void at_slot() {
+        if (dx) plane += (uint64_t)(*dx) * 2 * D;
+    }
+    __device__ __forceinline__ double2 value(uint64_t i) const {
+        if (phi) return phi[i];
+        const uint2 h = plane[i], l = plane[D + i];
+        return make_double2(__hiloint2double((int)h.x, (int)l.x), __hiloint2double((int)h.y, (int)l.y));
+    }
+#endif
+};
 bool hphi_x_ok(const Basis &B);
-int hphi_x_launch(Basis &B, const void *phi, const void *dg, const int *ge, const int *dx, void *psi, cudaStream_t st,
-                  const int *active = nullptr);
-// qs3_hphi with QS3_C128X: phi's digit image in scratch, then hphi_x_launch
-// (qs3_solver.cu, where the digit kernels live); synchronous on st
+int hphi_x_launch(Basis &B, const HxVec &hv, void *psi, cudaStream_t st, const int *active = nullptr);
+// qs3_hphi with QS3_C128X: phi's image in scratch, then hphi_x_launch
+// (qs3_solver.cu, where the digit kernels live); asynchronous on st
 int hphi_x_binary64(Basis &B, const void *phi, void *psi, cudaStream_t st);
 // representative table: build (QS3_OK, or an error when it cannot be built) / release
 int build_rep_table(Basis &B, size_t max_bytes);

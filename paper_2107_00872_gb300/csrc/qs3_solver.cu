@@ -2716,20 +2716,16 @@ extern "C" int qs3_trlanczos(qs3_basis_t b, const qs3_solve_opts *o, double *eva
 
 namespace qs3 {
 
-// qs3_hphi with QS3_C128X: phi's digit image (the layout of the engine's
-// digit store, one slot) in scratch, then the product
+// qs3_hphi with QS3_C128X: phi's gather image in scratch, then the product
 int hphi_x_binary64(Basis &B, const void *phi, void *psi, cudaStream_t st) {
     if (!hphi_x_ok(B))
         return set_err(QS3_ERR_STATE, "QS3_C128X needs a k-sector basis with the representative table and one hop "
                                       "amplitude");
-    const uint64_t D = B.total;
-    DevBuf dgt, get;
-    QS3_TRY(dgt.alloc(D * sizeof(double2), st));
-    QS3_TRY(get.alloc((uint64_t)B.nchunks * XW * sizeof(int), st));
-    k_digitize_il<double2><<<B.nchunks, XT, 0, st>>>((const double2 *)phi, D, dgt.as<int2>(), get.as<int>(),
-                                                     B.d_secs.as<SecView>(), B.d_chunk0.as<int>(), B.S);
+    DevBuf hd;
+    QS3_TRY(hd.alloc(B.total * sizeof(int4), st));
+    k_image<<<B.nchunks, XT, 0, st>>>((const double2 *)phi, hd.as<int4>(), B.d_secs.as<SecView>(), B.d_chunk0.as<int>(), B.S);
     QS3_LAUNCHED();
-    return hphi_x_launch(B, phi, dgt.p, get.as<int>(), nullptr, psi, st, nullptr);
+    return hphi_x_launch(B, {hd.as<int4>(), (const double2 *)phi, nullptr, B.total, nullptr}, psi, st, nullptr);
 }
 
 }  // namespace qs3
