@@ -163,6 +163,11 @@ __device__ __forceinline__ long long warp_sum_ll(long long t) {
     const long long s2 = __reduce_add_sync(0xffffffffu, l2);
     return s0 + s1 * (1ll << 26) + s2 * (1ll << 52);
 }
+__device__ __forceinline__ __int128 align_round(__int128 v, int d) {
+    if (d <= 0) return v;
+    if (d > 120) return 0;
+    return (v + ((__int128)1 << (d - 1))) >> d;
+}
 // the sum over the warp of a 128-bit value (exact, all lanes)
 __device__ __forceinline__ __int128 warp_sum_i128(__int128 v) {
 #pragma unroll
@@ -352,17 +357,28 @@ __global__ void __launch_bounds__(XT) k_image(const double2 *__restrict__ x, int
 // units of 2^(k - 2098)) and k = em + ew, the sum of its two grid exponents.
 // The stored vectors are read from the digit store (dg, ge), w (interleaved
 // binary64) is put on its warps' grids here.  NV vectors per pass have their
-// loads in flight together.  Graph mode (dx): the range of graph_range.
+// loads in flight together.  A launch of few chunks splits the vectors over
+// blockIdx.y (dotx_split), so that the chip is filled and a block's chain of
+// passes is short.  Graph mode (dx): the range of graph_range.
+// out (sectors of one chunk each): the block reduces its own warp partials and
+// writes the coefficients to out[s ldo + j] (from out + j0 in graph mode),
+// which takes a reduction launch otherwise.
+constexpr int DX_FIN = 32;
 template <typename VT, int NV>
 __global__ void __launch_bounds__(XT, 1)
     k_dotx(const typename DigT<VT>::T *__restrict__ dg, const int *__restrict__ ge, int nchunks, uint64_t D, int j0,
            int m, const VT *__restrict__ w, const SecView *__restrict__ secs, const int *__restrict__ chunk0, int S,
            const int *__restrict__ active, long long *__restrict__ part, const int *__restrict__ dx = nullptr,
-           int ring = 0) {
+           int ring = 0, double2 *__restrict__ out = nullptr, int ldo = 0) {
     using G = typename DigT<VT>::T;
     constexpr bool CX = IsC<VT>::v;
     constexpr int NC = CX ? 2 : 1;
+    __shared__ long long fin[DX_FIN][XW][3];          // out: warp partials of up to DX_FIN vectors
     graph_range(dx, ring, j0, m);
+    // this block's vectors ja .. jb - 1 of the m
+    const int per = ((m + (int)gridDim.y - 1) / (int)gridDim.y + NV - 1) / NV * NV;
+    const int ja = blockIdx.y * per, jb = min(m, ja + per);
+    if (ja >= jb) return;
     const ChunkInfo ci = chunk_info(secs, chunk0, S, blockIdx.x);
     if (active && !active[ci.s]) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -412,24 +428,49 @@ __global__ void __launch_bounds__(XT, 1)
             fx_thread_dot<CX>(b.a1[v], b.a0[v], wd, tr, ti);
             const long long sr = warp_sum_ll(tr);
             const long long si = CX ? warp_sum_ll(ti) : 0ll;
-            if (lane == 0 && jj + v < m) {
-                long long *o = part + (((uint64_t)blockIdx.x * m + jj + v) * XW + warp) * 3;
+            if (lane == 0 && jj + v < jb) {
+                long long *o = out ? fin[(jj + v - ja) % DX_FIN][warp]
+                                   : part + (((uint64_t)blockIdx.x * m + jj + v) * XW + warp) * 3;
                 o[0] = sr;
                 o[1] = si;
                 o[2] = b.em[v] + ew;
             }
         }
     };
+    // out: the block's warps hold the whole sector: the coefficients of the
+    // vectors up to `end` that wait in fin, as k_reducex1 forms them
+    auto finish = [&](int from, int end) {
+        __syncthreads();
+        for (int j = from + warp; j < end; j += XW) {
+            const long long *q = fin[(j - ja) % DX_FIN][lane < XW ? lane : 0];
+            const int K = __reduce_max_sync(0xffffffffu, lane < XW ? (int)q[2] : -1);
+            __int128 ar = lane < XW ? align_round(q[0], K - (int)q[2]) : (__int128)0;
+            __int128 ai = lane < XW ? align_round(q[1], K - (int)q[2]) : (__int128)0;
+            ar = warp_sum_i128(ar);
+            if (CX) ai = warp_sum_i128(ai);
+            if (lane == 0)
+                out[(uint64_t)ci.s * ldo + (dx && ring ? j0 : 0) + j] =
+                    make_double2(i128_ldexp(ar, K - 2098), CX ? i128_ldexp(ai, K - 2098) : 0.0);
+        }
+        __syncthreads();
+    };
     Stage s0, s1;
-    if (m > 0) load(s0, 0);
+    load(s0, ja);
+    int done = ja;
 #pragma unroll 1
-    for (int jj = 0; jj < m; jj += 2 * NV) {
-        if (jj + NV < m) load(s1, jj + NV);
+    for (int jj = ja; jj < jb; jj += 2 * NV) {
+        if (jj + NV < jb) load(s1, jj + NV);
         consume(s0, jj);
-        if (jj + NV >= m) break;
-        if (jj + 2 * NV < m) load(s0, jj + 2 * NV);
-        consume(s1, jj + NV);
+        if (jj + NV < jb) {
+            if (jj + 2 * NV < jb) load(s0, jj + 2 * NV);
+            consume(s1, jj + NV);
+        }
+        if (out && jj + 4 * NV > done + DX_FIN) {
+            finish(done, min(jb, jj + 2 * NV));
+            done = min(jb, jj + 2 * NV);
+        }
     }
+    if (out && done < jb) finish(done, jb);
 }
 
 // The same dot products with the stored vectors' digits brought in by TMA
@@ -677,10 +718,34 @@ static inline bool one_slice(const std::vector<int> &s0) {
     return s0.size() > 1;
 }
 
-__device__ __forceinline__ __int128 align_round(__int128 v, int d) {
-    if (d <= 0) return v;
-    if (d > 120) return 0;
-    return (v + ((__int128)1 << (d - 1))) >> d;
+// the sums of coefficient j over the warp partials p0 .. p1 - 1 (p / XW the
+// chunk, p % XW the warp), aligned to the coarsest grid K among them; one warp
+__device__ __forceinline__ int coef_sums(const long long *__restrict__ part, int m, int j, int p0, int p1,
+                                         __int128 &ar, __int128 &ai) {
+    const int lane = threadIdx.x & 31;
+    int K = -1;
+    for (int p = p0 + lane; p < p1; p += 32) {
+        const long long *q = part + (((uint64_t)(p / XW) * m + j) * XW + p % XW) * 3;
+        K = max(K, (int)q[2]);
+    }
+    K = __reduce_max_sync(0xffffffffu, K);
+    ar = 0;
+    ai = 0;
+    for (int p = p0 + lane; p < p1; p += 32) {
+        const long long *q = part + (((uint64_t)(p / XW) * m + j) * XW + p % XW) * 3;
+        const int d = K - (int)q[2];
+        ar += align_round(q[0], d);
+        ai += align_round(q[1], d);
+    }
+    ar = warp_sum_i128(ar);
+    ai = warp_sum_i128(ai);
+    return K;
+}
+// the sector's sum of chunk partials (the order of k_reduce64); one warp
+__device__ __forceinline__ double sector_sum(const double2 *__restrict__ part, const int *__restrict__ chunk0, int s) {
+    double2 acc = make_double2(0.0, 0.0);
+    for (int c = chunk0[s] + (int)(threadIdx.x & 31); c < chunk0[s + 1]; c += 32) acc.x += part[c].x;
+    return warp_sum2(acc).x;
 }
 
 // out1[(sl m + j) 5 + {0..4}] = re (lo, hi words), im (lo, hi), K of slice sl
@@ -705,21 +770,8 @@ __global__ void k_reducex1(const long long *__restrict__ part, int m, const int 
     const int j = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j >= m) return;
     const int p0 = chunk0[s] * XW + (sl - slice0[s]) * RSL, p1 = min(p0 + RSL, chunk0[s + 1] * XW);
-    int K = -1;
-    for (int p = p0 + lane; p < p1; p += 32) {
-        const long long *q = part + (((uint64_t)(p / XW) * m + j) * XW + p % XW) * 3;
-        K = max(K, (int)q[2]);
-    }
-    K = __reduce_max_sync(0xffffffffu, K);
-    __int128 ar = 0, ai = 0;
-    for (int p = p0 + lane; p < p1; p += 32) {
-        const long long *q = part + (((uint64_t)(p / XW) * m + j) * XW + p % XW) * 3;
-        const int d = K - (int)q[2];
-        ar += align_round(q[0], d);
-        ai += align_round(q[1], d);
-    }
-    ar = warp_sum_i128(ar);
-    ai = warp_sum_i128(ai);
+    __int128 ar, ai;
+    const int K = coef_sums(part, m, j, p0, p1, ar, ai);
     if (out) {
         // one slice per sector: the slice sum is the sector's dot
         if (lane == 0)
@@ -811,6 +863,15 @@ template <typename VT> static int dotb_prepare() {
     return QS3_OK;
 }
 
+// blocks along the vectors: two per SM in all, each with at least two passes
+static int dotx_split(int nchunks, int m, int nv) {
+    int dev = 0, nsm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int most = std::max(1, 2 * nsm / std::max(nchunks, 1));
+    return std::max(1, std::min(most, (m + 2 * nv - 1) / (2 * nv)));
+}
+
 // The dot pass: nv = 1, 2 or 4 stored vectors per pass of k_dotx (register
 // staging), or nv = 8 the copy-engine ring of k_dotb (dg must then have 16
 // readable bytes past its last slot, err a device int; dotb_prepare done).
@@ -818,9 +879,10 @@ template <typename VT> static int dotb_prepare() {
 template <typename VT>
 static int dotx_launch(int nv, const typename DigT<VT>::T *dg, const int *ge, int nchunks, uint64_t D, int j0, int m,
                        const VT *w, const SecView *secs, const int *c0, int S, const int *act, long long *pp,
-                       cudaStream_t st, const int *dx = nullptr, int ring = 0, int *err = nullptr) {
+                       cudaStream_t st, const int *dx = nullptr, int ring = 0, int *err = nullptr,
+                       double2 *out = nullptr, int ldo = 0) {
     const bool small = ring || (!dx && m <= 2);
-    if (nv >= 8 && !small && err) {
+    if (nv >= 8 && !small && err && !out) {
         k_dotb<VT, dotb_ns<VT>()><<<std::max(nchunks, 1), XT + 32, dotb_smem<VT, dotb_ns<VT>()>(), st>>>(
             dg, ge, nchunks, D, j0, m, w, secs, c0, S, act, pp, err, take_wait_injection(), dx, ring);
         QS3_LAUNCHED();
@@ -832,12 +894,13 @@ static int dotx_launch(int nv, const typename DigT<VT>::T *dg, const int *ge, in
     if (ring == 2 || (!dx && m == 1)) nv = 1;
     const int g = std::max(nchunks, 1);
     if (nv == 1) {
-        k_dotx<VT, 1><<<g, XT, 0, st>>>(dg, ge, nchunks, D, j0, m, w, secs, c0, S, act, pp, dx, ring);
+        k_dotx<VT, 1><<<dim3(g, dotx_split(nchunks, m, 1)), XT, 0, st>>>(dg, ge, nchunks, D, j0, m, w, secs, c0, S, act, pp, dx, ring, out, ldo);
     } else if (nv == 2) {
-        k_dotx<VT, 2><<<g, XT, 0, st>>>(dg, ge, nchunks, D, j0, m, w, secs, c0, S, act, pp, dx, ring);
+        k_dotx<VT, 2><<<dim3(g, dotx_split(nchunks, m, 2)), XT, 0, st>>>(dg, ge, nchunks, D, j0, m, w, secs, c0, S, act, pp, dx, ring, out, ldo);
     } else {
         if constexpr (!IsC<VT>::v)
-            k_dotx<VT, 4><<<g, XT, 0, st>>>(dg, ge, nchunks, D, j0, m, w, secs, c0, S, act, pp, dx, ring);
+            k_dotx<VT, 4><<<dim3(g, dotx_split(nchunks, m, 4)), XT, 0, st>>>(dg, ge, nchunks, D, j0, m, w, secs, c0, S, act,
+                                                                             pp, dx, ring, out, ldo);
     }
     QS3_LAUNCHED();
     return QS3_OK;
@@ -878,6 +941,9 @@ __global__ void k_reduce64(const double2 *__restrict__ part, int m, const int *_
 // chunk; the fp32 pass reads UV vectors' top digits per stage, two stages in
 // flight.  Graph mode (dx): the range of graph_range, and for the three-term
 // pass (ring) the coefficients from coef + j0.
+// wpart (sectors of few chunks, Engine64::few): |w|^2 before the update as
+// chunk sums of the three-term part, which the block sums itself
+constexpr int FEW = 8;
 constexpr int UV = 4;
 template <typename VT>
 __global__ void __launch_bounds__(XT)
@@ -885,7 +951,8 @@ __global__ void __launch_bounds__(XT)
             const int *__restrict__ ge, int nchunks, uint64_t D, int j0, int m,
             const double2 *__restrict__ coef, int ldc, const SecView *__restrict__ secs,
             const int *__restrict__ chunk0, int S, const int *__restrict__ active, const double2 *__restrict__ wn2,
-            int strict, double2 *__restrict__ part, const int *__restrict__ dx = nullptr, int ring = 0) {
+            int strict, double2 *__restrict__ part, const int *__restrict__ dx = nullptr, int ring = 0,
+            const double2 *__restrict__ wpart = nullptr) {
     using T = typename PlS<VT>::T;
     constexpr bool CX = IsC<VT>::v;
     if (dx) {
@@ -899,6 +966,11 @@ __global__ void __launch_bounds__(XT)
     const ChunkInfo ci = chunk_info(secs, chunk0, S, blockIdx.x);
     if (active && !active[ci.s]) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ double wn_s;
+    if (wpart && warp == XW - 1) {
+        const double t = sector_sum(wpart, chunk0, ci.s);
+        if (lane == 0) wn_s = t;
+    }
     double cs = 0.0;
     for (int j = threadIdx.x; j < m; j += XT) {
         const double2 c = coef[(uint64_t)ci.s * ldc + j];
@@ -921,7 +993,7 @@ __global__ void __launch_bounds__(XT)
         const int nw = m > 32 ? XW : 1;
         for (int q = 0; q < nw; ++q) t += red[q];
         const double lim = m > 256 ? 0x1p-80 * (256.0 / m) * (256.0 / m) : 0x1p-80;
-        lite_s = (!strict && wn2 && t * t <= lim * wn2[ci.s].x) ? 1 : 0;
+        lite_s = (!strict && (wn2 || wpart) && t * t <= lim * (wpart ? wn_s : wn2[ci.s].x)) ? 1 : 0;
     }
     __syncthreads();
     const bool lite = lite_s != 0;
@@ -1154,7 +1226,8 @@ __global__ void __launch_bounds__(XT + 32, 2)
            const int *__restrict__ ge, int nchunks, uint64_t D, int j0, int m, int ns,
            const double2 *__restrict__ coef, int ldc, const SecView *__restrict__ secs,
            const int *__restrict__ chunk0, int S, const int *__restrict__ active, const double2 *__restrict__ wn2,
-           double2 *__restrict__ part, int *__restrict__ err, int starve, const int *__restrict__ dx = nullptr) {
+           double2 *__restrict__ part, int *__restrict__ err, int starve, const int *__restrict__ dx = nullptr,
+           const double2 *__restrict__ wpart = nullptr) {
     using G = typename DigT<VT>::T;
     using T = typename PlS<VT>::T;
     constexpr bool CX = IsC<VT>::v;
@@ -1193,7 +1266,8 @@ __global__ void __launch_bounds__(XT + 32, 2)
         bulk_g2s(sp + SL, ge + ((uint64_t)(j0 + issued) * nchunks + blockIdx.x) * XW, XW * 4, &full[t]);
         ++issued;
     };
-    if (warp == XW && lane == 0 && wn2 && !starve)
+    __shared__ double wn_s;
+    if (warp == XW && lane == 0 && (wn2 || wpart) && !starve)
         while (issued < m && issued < ns) issue(issued);
     const int nk = (ci.n - (int)threadIdx.x + XT - 1) / XT;
     const uint64_t r0 = ci.base + threadIdx.x;
@@ -1202,6 +1276,10 @@ __global__ void __launch_bounds__(XT + 32, 2)
     if (warp < XW) {
 #pragma unroll
         for (int k = 0; k < XR; ++k) wr[k] = k < nk ? ld2(w + r0 + (uint64_t)k * XT) : make_double2(0.0, 0.0);
+        if (wpart && warp == XW - 1) {
+            const double t = sector_sum(wpart, chunk0, ci.s);
+            if (lane == 0) wn_s = t;
+        }
         double cs = 0.0;
         for (int j = threadIdx.x; j < m; j += XT) {
             const double2 c = coef[(uint64_t)ci.s * ldc + j];
@@ -1225,7 +1303,7 @@ __global__ void __launch_bounds__(XT + 32, 2)
         const int nw = m > 32 ? XW : 1;
         for (int q = 0; q < nw; ++q) t += red[q];
         const double lim = m > 256 ? 0x1p-80 * (256.0 / m) * (256.0 / m) : 0x1p-80;
-        lite_s = (wn2 && t * t <= lim * wn2[ci.s].x) ? 1 : 0;
+        lite_s = ((wn2 || wpart) && t * t <= lim * (wpart ? wn_s : wn2[ci.s].x)) ? 1 : 0;
     }
     __syncthreads();
     const bool lite = lite_s != 0;
@@ -1392,13 +1470,21 @@ template <typename VT> static int updb_prepare() {
 // next H Phi: the gather image of the integer product (hx), else interleaved
 // binary64.  w may alias hin (the start vector is normalised in place: a
 // thread reads its rows before it writes them).  One block of XT threads per
-// chunk.
+// chunk.  With sp.npart (sectors of few chunks) the block also forms the
+// step's scalars, which a reduction and k_step_scalars form otherwise.
+struct StepIn {
+    const double2 *npart = nullptr;
+    const double2 *h = nullptr;
+    double *alpha = nullptr, *beta = nullptr;
+    double brk = 0.0;
+    int cap = 0, x = 0;
+};
 template <typename VT>
 __global__ void __launch_bounds__(XT)
     k_scale64(const VT *w, typename PlS<VT>::T *__restrict__ out, typename DigT<VT>::T *__restrict__ dg,
               int *__restrict__ ge, int nchunks, VT *hin, const double *__restrict__ inv,
               const SecView *__restrict__ secs, const int *__restrict__ chunk0, int S, const int *__restrict__ active,
-              const int *__restrict__ dx, uint64_t D, int hx) {
+              const int *__restrict__ dx, uint64_t D, int hx, StepIn sp = StepIn{}) {
     constexpr int NC = IsC<VT>::v ? 2 : 1;
     if (dx) {
         out += (uint64_t)(*dx + 1) * 2 * D;
@@ -1408,7 +1494,27 @@ __global__ void __launch_bounds__(XT)
     const ChunkInfo ci = chunk_info(secs, chunk0, S, blockIdx.x);
     if (active && !active[ci.s]) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const double f = inv[ci.s];
+    __shared__ double f_s;
+    if (sp.npart) {
+        // the step's scalars (k_step_scalars) from the update's chunk sums; the
+        // sector's first block keeps them
+        if (warp == 0) {
+            const double n2 = sector_sum(sp.npart, chunk0, ci.s);
+            if (lane == 0) {
+                double b;
+                const int x = dx ? *dx : sp.x;
+                const double a = sp.h[(uint64_t)ci.s * sp.cap + x].x;
+                b = step_beta(a, n2, x > 0 ? sp.beta[(uint64_t)ci.s * sp.cap + x - 1] : 0.0, sp.brk);
+                f_s = b > 0.0 ? 1.0 / b : 0.0;
+                if ((int)blockIdx.x == chunk0[ci.s]) {
+                    sp.alpha[(uint64_t)ci.s * sp.cap + x] = a;
+                    sp.beta[(uint64_t)ci.s * sp.cap + x] = b;
+                }
+            }
+        }
+        __syncthreads();
+    }
+    const double f = sp.npart ? f_s : inv[ci.s];
     uint32_t hw[XR][2], lw[XR][2];
 #pragma unroll
     for (int k = 0; k < XR; ++k) {
@@ -1527,9 +1633,13 @@ struct Engine64 {
     HphiStats *stats;
     int cap = 0, nscr = 0;
     uint64_t D = 0;
-    DevBuf V, DG, GE, wbuf, hinb, part, partx, partr, slices, h1, h2, alpha, beta, nrm, nrm1, inv, active, derr;
+    DevBuf V, DG, GE, wbuf, hinb, part, part3, partx, partr, slices, h1, h2, alpha, beta, nrm, nrm1, inv, active, derr;
     int nslices = 0;
     bool slice1 = false;                   // one reduction slice per sector
+    // every sector has at most FEW chunks: the kernels that use a sector's sums
+    // form them per block instead of after a reduction launch; one chunk each
+    // (tiny): the dot pass also writes the coefficients
+    bool few = false, tiny = false;
     std::vector<int> h_active;
     double brk = 1e-12;
     int strict = 0;                        // 1: every update on binary64 FMAs
@@ -1584,6 +1694,11 @@ struct Engine64 {
             const std::vector<int> s0 = reduce_slices(B);
             nslices = s0[B.S];
             slice1 = one_slice(s0);
+            int most = 0;
+            for (int s = 0; s < B.S; ++s) most = std::max(most, B.chunk0[s + 1] - B.chunk0[s]);
+            few = !strict && most <= FEW;
+            tiny = few && most <= 1;
+            QS3_TRY(part3.alloc((uint64_t)std::max(B.nchunks, 1) * sizeof(double2), st));
             QS3_TRY(slices.upload(s0.data(), s0.size() * sizeof(int), st));
             QS3_TRY(partr.alloc((uint64_t)std::max(nslices, 1) * cap * 5 * sizeof(long long), st));
         }
@@ -1633,12 +1748,12 @@ struct Engine64 {
     // the dot products of w against stored vectors j0 .. j0 + m - 1 as chunk
     // partials: k_dotx with nv stored vectors per pass (1, 2 or 4), or under
     // strict64 k_dot64 (binary64 FMA chains); dot_reduce sums them per sector
-    int dot_launch(int nv, int j0, int m, const int *dx = nullptr, int ring = 0) {
+    int dot_launch(int nv, int j0, int m, const int *dx = nullptr, int ring = 0, double2 *out = nullptr, int ldo = 0) {
         const ST *v = V.as<ST>();
         const VT *w = wv();
         if (!strict)
             return dotx_launch<VT>(nv, dg(), ge(), B.nchunks, D, j0, m, w, secs(), c0(), B.S, act(),
-                                   partx.as<long long>(), st, dx, ring, derr.as<int>());
+                                   partx.as<long long>(), st, dx, ring, derr.as<int>(), out, ldo);
         k_dot64<VT, 2><<<grid(), NTHREADS, 0, st>>>(v, D, j0, m, w, secs(), c0(), B.S, act(), part.as<double2>(), dx,
                                                      ring);
         QS3_LAUNCHED();
@@ -1653,8 +1768,14 @@ struct Engine64 {
     // dot products of w against stored vectors j0 .. j0 + m - 1 into out (S x ldo)
     int mdot(int j0, int m, double2 *out, int ldo) {
         if (B.nchunks == 0) return QS3_OK;
-        QS3_TRY(dot_launch(B.tune_nv64 > 0 ? B.tune_nv64 : 2, j0, m));
-        return dot_reduce(m, out, ldo);
+        return dots(j0, m, m, out, ldo, nullptr, 0);
+    }
+    // the dot pass and its sector sums (mg: the coefficients a graph launch provides for)
+    int dots(int j0, int m, int mg, double2 *out, int ldo, const int *dx, int ring) {
+        const int nv = dx && ring ? 2 : B.tune_nv64 > 0 ? B.tune_nv64 : 2;
+        if (tiny) return dot_launch(nv, j0, m, dx, ring, out, ldo);
+        QS3_TRY(dot_launch(nv, j0, m, dx, ring));
+        return dot_reduce(m, out, ldo, dx, ring, mg);
     }
     // the dot pass: time k_dotx with 1, 2 and 4 vectors per pass and the
     // k_dotb ring (8) on min(cap, 48) zeroed slots and keep the fastest
@@ -1700,26 +1821,27 @@ struct Engine64 {
     // dot pass (dot_vectors64 = 8), when the fp32 correction is possible
     // (wn2 given, strict64 off), the pass is longer than the three-term one
     // and the ring fits beside mmax coefficients
-    bool updb_ok(const double2 *wn2, int m, int mmax) const {
+    bool updb_ok(bool wn2, int m, int mmax) const {
         return B.tune_nv64 == 8 && !strict && wn2 && m > 2 && updb_ns<VT>(mmax) > 0;
     }
-    // w -= sum_j psi_{j0+j} cf[s][j]; nrm_out: per-sector |w|^2 after it;
-    // wn2: |w|^2 before it (enables the fp32 correction of tiny coefficients)
-    int mupdate(int j0, int m, const double2 *cf, int ldc, double2 *nrm_out, const double2 *wn2 = nullptr) {
+    // w -= sum_j psi_{j0+j} cf[s][j]; nrm_out: per-sector |w|^2 after it (NULL:
+    // its chunk sums stay in part); wn2: |w|^2 before it (enables the fp32
+    // correction of tiny coefficients), or wpart its chunk sums
+    int mupdate(int j0, int m, const double2 *cf, int ldc, double2 *nrm_out, const double2 *wn2 = nullptr,
+                const double2 *wpart = nullptr) {
         if (B.nchunks == 0) return QS3_OK;
-        if (updb_ok(wn2, m, m)) {
+        if (updb_ok(wn2 || wpart, m, m)) {
             const int ns = updb_ns<VT>(m);
             k_updb<VT><<<grid(), XT + 32, (size_t)ns * updb_stage<VT>() + (size_t)m * 24, st>>>(
                 wv(), V.as<ST>(), dg(), ge(), B.nchunks, D, j0, m, ns, cf, ldc, secs(), c0(), B.S, act(), wn2,
-                part.as<double2>(), derr.as<int>(), take_wait_injection());
-            QS3_LAUNCHED();
-            return reduce(1, nrm_out, 1);
+                part.as<double2>(), derr.as<int>(), take_wait_injection(), nullptr, wpart);
+        } else {
+            k_upd64<VT><<<grid(), XT, (size_t)m * (sizeof(double2) + sizeof(float2)), st>>>(
+                wv(), V.as<ST>(), dg(), ge(), B.nchunks, D, j0, m, cf, ldc, secs(), c0(), B.S, act(), wn2, strict,
+                part.as<double2>(), nullptr, 0, wpart);
         }
-        k_upd64<VT><<<grid(), XT, (size_t)m * (sizeof(double2) + sizeof(float2)), st>>>(
-            wv(), V.as<ST>(), dg(), ge(), B.nchunks, D, j0, m, cf, ldc, secs(), c0(), B.S, act(), wn2, strict,
-            part.as<double2>());
         QS3_LAUNCHED();
-        return reduce(1, nrm_out, 1);
+        return nrm_out ? reduce(1, nrm_out, 1) : QS3_OK;
     }
     // psi_j = w * inv (per sector) into slot j and hin
     int scale_store(const VT *w, int j) {
@@ -1790,33 +1912,35 @@ struct Engine64 {
         VT *w = wv();
         double2 *hh1 = h1.as<double2>(), *n1 = nrm1.as<double2>();
         QS3_TRY(hphi_apply(0, dx));
-        QS3_TRY(dot_launch(2, 0, 1, dx, 2));
-        QS3_TRY(dot_reduce(1, hh1, cap, dx, 2, 1));
-        k_upd3<VT><<<grid(), XT, 0, st>>>(w, V.as<ST>(), D, 0, hh1, beta.as<double>(), cap, secs(), c0(), B.S,
-                                          act(), part.as<double2>(), dx);
-        QS3_LAUNCHED();
-        QS3_TRY(reduce(1, n1, 1));
-        QS3_TRY(dot_launch(B.tune_nv64 > 0 ? B.tune_nv64 : 2, 0, cap, dx, 0));
-        QS3_TRY(dot_reduce(cap, h2.as<double2>(), cap, dx, 0, cap));
-        if (updb_ok(n1, cap, cap)) {
+        QS3_TRY(dots(0, 1, 1, hh1, cap, dx, 2));
+        QS3_TRY(three_term(0, dx));
+        if (!few) QS3_TRY(reduce(1, n1, 1));
+        QS3_TRY(dots(0, cap, cap, h2.as<double2>(), cap, dx, 0));
+        const double2 *wpart = few ? part3.as<double2>() : nullptr;
+        const double2 *wn2 = few ? nullptr : n1;
+        if (updb_ok(true, cap, cap)) {
             const int ns = updb_ns<VT>(cap);
             k_updb<VT><<<grid(), XT + 32, (size_t)ns * updb_stage<VT>() + (size_t)cap * 24, st>>>(
                 w, V.as<ST>(), dg(), ge(), B.nchunks, D, 0, cap, ns, h2.as<double2>(), cap, secs(), c0(), B.S, act(),
-                n1, part.as<double2>(), derr.as<int>(), take_wait_injection(), dx);
+                wn2, part.as<double2>(), derr.as<int>(), take_wait_injection(), dx, wpart);
         } else {
             k_upd64<VT><<<grid(), XT, (size_t)cap * (sizeof(double2) + sizeof(float2)), st>>>(
-                w, V.as<ST>(), dg(), ge(), B.nchunks, D, 0, cap, h2.as<double2>(), cap, secs(), c0(), B.S, act(), n1,
-                strict, part.as<double2>(), dx, 0);
+                w, V.as<ST>(), dg(), ge(), B.nchunks, D, 0, cap, h2.as<double2>(), cap, secs(), c0(), B.S, act(), wn2,
+                strict, part.as<double2>(), dx, 0, wpart);
         }
         QS3_LAUNCHED();
-        QS3_TRY(reduce(1, nrm.as<double2>(), 1));
-        k_step_scalars<<<(B.S + 127) / 128, 128, 0, st>>>(B.S, 0, cap, hh1, nrm.as<double2>(), act(),
-                                                         alpha.as<double>(), beta.as<double>(), inv.as<double>(), brk,
-                                                         dx);
-        QS3_LAUNCHED();
-        k_scale64<VT><<<grid(), XT, 0, st>>>(w, V.as<ST>(), dg(), ge(), B.nchunks, hin(0), inv.as<double>(), secs(),
-                                             c0(), B.S, act(), dx, D, hx());
-        QS3_LAUNCHED();
+        if (few) {
+            QS3_TRY(scale_step(0, dx));
+        } else {
+            QS3_TRY(reduce(1, nrm.as<double2>(), 1));
+            k_step_scalars<<<(B.S + 127) / 128, 128, 0, st>>>(B.S, 0, cap, hh1, nrm.as<double2>(), act(),
+                                                             alpha.as<double>(), beta.as<double>(), inv.as<double>(),
+                                                             brk, dx);
+            QS3_LAUNCHED();
+            k_scale64<VT><<<grid(), XT, 0, st>>>(w, V.as<ST>(), dg(), ge(), B.nchunks, hin(0), inv.as<double>(), secs(),
+                                                 c0(), B.S, act(), dx, D, hx());
+            QS3_LAUNCHED();
+        }
         k_advance<<<1, 1, 0, st>>>(xdev.as<int>());
         QS3_LAUNCHED();
         return QS3_OK;
@@ -1873,25 +1997,51 @@ struct Engine64 {
         QS3_CUDA(cudaEventRecord(ev.second, st));
         stats->pend.push_back(ev);
         count_hphi();
-        double2 *n1 = nrm1.as<double2>();
+        double2 *n1 = nrm1.as<double2>(), *hh1 = h1.as<double2>();
         if (full2) {
             // after a thick restart: a full first pass with complex coefficients
-            QS3_TRY(mdot(0, x + 1, h1.as<double2>(), cap));
-            QS3_TRY(mupdate(0, x + 1, h1.as<double2>(), cap, n1));
+            QS3_TRY(mdot(0, x + 1, hh1, cap));
+            QS3_TRY(mupdate(0, x + 1, hh1, cap, n1));
         } else {
             // alpha_x = Re psi_x^H w, then w -= beta_{x-1} psi_{x-1} + alpha_x psi_x
-            QS3_TRY(mdot(x, 1, h1.as<double2>() + x, cap));
-            k_upd3<VT><<<grid(), XT, 0, st>>>(w, V.as<ST>(), D, x, h1.as<double2>(), beta.as<double>(), cap, secs(),
-                                              c0(), B.S, act(), part.as<double2>());
-            QS3_LAUNCHED();
-            QS3_TRY(reduce(1, n1, 1));
+            QS3_TRY(mdot(x, 1, hh1 + x, cap));
+            QS3_TRY(three_term(x, nullptr));
+            if (!few) QS3_TRY(reduce(1, n1, 1));
         }
         QS3_TRY(gs_dots(x));
+        if (few && !full2) {
+            QS3_TRY(mupdate(0, x + 1, h2.as<double2>(), cap, nullptr, nullptr, part3.as<double2>()));
+            return scale_step(x, nullptr);
+        }
         QS3_TRY(mupdate(0, x + 1, h2.as<double2>(), cap, nrm.as<double2>(), n1));
-        k_step_scalars<<<(B.S + 127) / 128, 128, 0, st>>>(B.S, x, cap, h1.as<double2>(), nrm.as<double2>(), act(),
-                                                         alpha.as<double>(), beta.as<double>(), inv.as<double>(), brk);
+        k_step_scalars<<<(B.S + 127) / 128, 128, 0, st>>>(B.S, x, cap, hh1, nrm.as<double2>(), act(), alpha.as<double>(),
+                                                         beta.as<double>(), inv.as<double>(), brk);
         QS3_LAUNCHED();
         return scale_store(w, x + 1);
+    }
+    // the three-term part of step x (*dx in graph mode): with few chunks |w|^2
+    // stays as chunk sums in part3
+    int three_term(int x, const int *dx) {
+        k_upd3<VT><<<grid(), XT, 0, st>>>(wv(), V.as<ST>(), D, x, h1.as<double2>(), beta.as<double>(), cap, secs(), c0(),
+                                          B.S, act(), few ? part3.as<double2>() : part.as<double2>(), dx);
+        QS3_LAUNCHED();
+        return QS3_OK;
+    }
+    // the scalars of step x and psi_{x+1} (few chunks)
+    int scale_step(int x, const int *dx) {
+        StepIn sp;
+        sp.npart = part.as<double2>();
+        sp.h = h1.as<double2>();
+        sp.alpha = alpha.as<double>();
+        sp.beta = beta.as<double>();
+        sp.brk = brk;
+        sp.cap = cap;
+        sp.x = x;
+        const int j = dx ? 0 : x + 1;
+        k_scale64<VT><<<grid(), XT, 0, st>>>(wv(), svec(j), dg(j), ge(j), B.nchunks, hin(0), inv.as<double>(), secs(), c0(),
+                                             B.S, act(), dx, D, hx(), sp);
+        QS3_LAUNCHED();
+        return QS3_OK;
     }
     int fetch(std::vector<double> &a, std::vector<double> &b) {
         a.resize((size_t)B.S * cap);

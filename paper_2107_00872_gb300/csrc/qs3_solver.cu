@@ -232,6 +232,12 @@ __global__ void __launch_bounds__(NTHREADS) k_mupdate(VT *__restrict__ w, const 
     }
 }
 
+// beta_x from alpha_x, |w|^2 and beta_{x-1}; 0 when the Krylov space is exhausted
+__device__ __forceinline__ double step_beta(double a, double nrm2, double bprev, double brk) {
+    const double b = sqrt(fmax(nrm2, 0.0));
+    return !(b > brk * (fabs(a) + bprev)) || !isfinite(b) ? 0.0 : b;      // invariant subspace reached
+}
+
 // per-sector scalars after a step: alpha_x, beta_x (with breakdown), 1/beta
 __global__ void k_step_scalars(int S, int x, int cap, const double2 *__restrict__ h, const double2 *__restrict__ nrm2,
                                const int *__restrict__ active, double *__restrict__ alpha, double *__restrict__ beta,
@@ -240,9 +246,7 @@ __global__ void k_step_scalars(int S, int x, int cap, const double2 *__restrict_
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= S || (active && !active[s])) return;
     const double a = h[(uint64_t)s * cap + x].x;
-    double b = sqrt(fmax(nrm2[s].x, 0.0));
-    const double bprev = x > 0 ? beta[(uint64_t)s * cap + x - 1] : 0.0;
-    if (!(b > brk * (fabs(a) + bprev)) || !isfinite(b)) b = 0.0;      // invariant subspace reached
+    const double b = step_beta(a, nrm2[s].x, x > 0 ? beta[(uint64_t)s * cap + x - 1] : 0.0, brk);
     alpha[(uint64_t)s * cap + x] = a;
     beta[(uint64_t)s * cap + x] = b;
     inv[s] = b > 0.0 ? 1.0 / b : 0.0;
@@ -1746,10 +1750,13 @@ static int residuals(Basis &B, const WT *v, const std::vector<double> &e, cudaSt
 // [2^-500, 2^500], which keeps every ratio exact.  A vanishing p_i takes the
 // sign opposite to p_{i-1} (one change, as for a zero pivot of T - x I = L D L^T
 // counted negative).
-__device__ int sturm_count_dev(int n, const double *__restrict__ a, const double *__restrict__ bb, double x) {
+__device__ int sturm_count_dev(int n, const double *__restrict__ a, const double *__restrict__ bb, double x, bool mild) {
     // bb[i] = b_{i-1}^2 (bb[0] unused).  Signs, zeros and the rescaling test
     // read the bit pattern in integer instructions, so the only fp64 work on
-    // the dependent chain is the fma of each step.
+    // the dependent chain is the fma of each step.  mild (every |a - x| and b^2
+    // within [.., 2^100]): the test runs every fourth step only, at 2^400, which
+    // four steps take to 2^1000 at most (the test's integer chain and branch cost
+    // as much as the fma).
     int cnt = 0, sp = 1;
     double pm = 0.0, p = 1.0;
     for (int i = 0; i < n; ++i) {
@@ -1762,9 +1769,12 @@ __device__ int sturm_count_dev(int n, const double *__restrict__ a, const double
         sp = sn;
         pm = p;
         p = pn;
-        const int e = (int)((bits >> 52) & 0x7ff);
-        if (e > 1523 || (e < 523 && !zero)) {        // |p| >= 2^501 or 0 < |p| < 2^-500
-            const double f = e > 1523 ? 0x1p-500 : 0x1p500;
+        if (mild && (i & 3) != 3) continue;
+        // the larger of the two: a p near zero is no reason to rescale
+        const int e = max((int)((bits >> 52) & 0x7ff), mild ? (int)((__double_as_longlong(pm) >> 52) & 0x7ff) : 0);
+        const int lim = mild ? 400 : 500;
+        if (e > 1023 + lim || (e < 1023 - lim && (mild || !zero))) {
+            const double f = e > 1023 ? 0x1p-500 : 0x1p500;
             p *= f;
             pm *= f;
         }
@@ -1793,6 +1803,7 @@ __device__ double tri_lowest_warp(int n, const double *__restrict__ a, const dou
         hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     }
     const double w = fmax(hi - lo, 1e-300);
+    const bool mild = w < 0x1p40 && w > 0x1p-40;      // |a - x| <= 2 w, b <= w
     lo -= 1e-3 * w;
     hi += 1e-3 * w;
     if (isfinite(e_prev) && e_prev > lo && e_prev < hi) {
@@ -1802,7 +1813,7 @@ __device__ double tri_lowest_warp(int n, const double *__restrict__ a, const dou
         // so the last ladder point without an eigenvalue below it and the
         // first with one bracket it to within a factor of four of that move
         const double t = lane == 0 ? e_prev + 1e-12 * w : e_prev - ldexp(1e-6 * w, -2 * (lane - 1));
-        const int c = sturm_count_dev(n, a, bb, t);
+        const int c = sturm_count_dev(n, a, bb, t, mild);
         const unsigned some = __ballot_sync(0xffffffffu, lane > 0 && c > 0);   // counts rise with t
         const unsigned none = __ballot_sync(0xffffffffu, lane > 0 && c == 0);
         const int c0 = __shfl_sync(0xffffffffu, c, 0);
@@ -1822,7 +1833,7 @@ __device__ double tri_lowest_warp(int n, const double *__restrict__ a, const dou
     for (int it = 0; it < 64; ++it) {
         const double h = (hi - lo) / 32.0;
         const double xl = lo + h * (double)(lane + 1);
-        const int cnt = (lane < 31 && xl > lo && xl < hi) ? sturm_count_dev(n, a, bb, xl) : 0;
+        const int cnt = (lane < 31 && xl > lo && xl < hi) ? sturm_count_dev(n, a, bb, xl, mild) : 0;
         const unsigned mk = __ballot_sync(0xffffffffu, lane < 31 && cnt > 0);
         const int j = mk ? __ffs(mk) - 1 : 31;
         const double nlo = j == 0 ? lo : fmax(lo, lo + h * (double)j);
