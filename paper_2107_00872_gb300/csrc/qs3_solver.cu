@@ -1743,47 +1743,66 @@ static int residuals(Basis &B, const WT *v, const std::vector<double> &e, cudaSt
 // reads one flag every check_every steps (direct mode).  Both run the same
 // kernels, so their results are identical.
 
-// number of eigenvalues of the symmetric tridiagonal (a, b) below x: the sign
-// changes of the Sturm sequence p_0 = 1, p_i = (a_{i-1} - x) p_{i-1} -
-// b_{i-2}^2 p_{i-2} (the leading principal minors of T - x I).  No division:
-// p_i and p_{i-1} are rescaled together by a power of two when |p_i| leaves
-// [2^-500, 2^500], which keeps every ratio exact.  A vanishing p_i takes the
-// sign opposite to p_{i-1} (one change, as for a zero pivot of T - x I = L D L^T
-// counted negative).
-__device__ int sturm_count_dev(int n, const double *__restrict__ a, const double *__restrict__ bb, double x, bool mild) {
-    // bb[i] = b_{i-1}^2 (bb[0] unused).  Signs, zeros and the rescaling test
-    // read the bit pattern in integer instructions, so the only fp64 work on
-    // the dependent chain is the fma of each step.  mild (every |a - x| and b^2
-    // within [.., 2^100]): the test runs every fourth step only, at 2^400, which
-    // four steps take to 2^1000 at most (the test's integer chain and branch cost
-    // as much as the fma).
-    int cnt = 0, sp = 1;
+// whether the symmetric tridiagonal (a, b) has an eigenvalue below x (or at x):
+// T - x I is not positive definite.  Its leading principal minors p_i = (a_{i-1}
+// - x) p_{i-1} - b_{i-2}^2 p_{i-2}, p_0 = 1, are followed from the top to the
+// middle row k, the trailing ones q_i from the bottom, as two independent
+// chains: the dependent fma of a step (about 130 cycles on this GPU) bounds
+// the count, and two chains of half the length take half the time.  T - x I is
+// positive definite when all of them are positive and so is the middle row's
+// pivot, (a_k - x) - b_{k-1}^2 p_{k-1} / p_k - b_k^2 q_{k+2} / q_{k+1}, taken
+// times p_k q_{k+1}.  No division: a value and its predecessor are rescaled
+// together by a power of two when they leave [2^-lim, 2^lim], which keeps every
+// ratio exact.  bb[i] = b_{i-1}^2.  mild (|a - x| and b within [2^-41, 2^41]):
+// the test runs every fourth step only, at 2^400, which four steps take to
+// 2^724 at most.
+struct Minor {
     double pm = 0.0, p = 1.0;
-    for (int i = 0; i < n; ++i) {
-        const double t = i ? bb[i] * pm : 0.0;
-        const double pn = fma(a[i] - x, p, -t);
-        const long long bits = __double_as_longlong(pn);
-        const bool zero = (bits << 1) == 0;
-        const int sn = zero ? -sp : (bits < 0 ? -1 : 1);
-        cnt += sn != sp;
-        sp = sn;
+    bool neg = false;
+    __device__ __forceinline__ void step(double ax, double b2) {
+        const double t = b2 * pm;
+        const double pn = fma(ax, p, -t);
+        neg |= __double_as_longlong(pn) <= 0;            // negative or +-0
         pm = p;
         p = pn;
-        if (mild && (i & 3) != 3) continue;
-        // the larger of the two: a p near zero is no reason to rescale
-        const int e = max((int)((bits >> 52) & 0x7ff), mild ? (int)((__double_as_longlong(pm) >> 52) & 0x7ff) : 0);
-        const int lim = mild ? 400 : 500;
-        if (e > 1023 + lim || (e < 1023 - lim && (mild || !zero))) {
+    }
+    __device__ __forceinline__ void rescale(int lim) {
+        const int e = max((int)((__double_as_longlong(p) >> 52) & 0x7ff), (int)((__double_as_longlong(pm) >> 52) & 0x7ff));
+        if (e > 1023 + lim || e < 1023 - lim) {
             const double f = e > 1023 ? 0x1p-500 : 0x1p500;
             p *= f;
             pm *= f;
         }
     }
-    return cnt;
+    // p and pm times the power of two that takes p (> 0) to [1, 2)
+    __device__ __forceinline__ void normalise() {
+        const int e = (int)((__double_as_longlong(p) >> 52) & 0x7ff);
+        const double f = __longlong_as_double((long long)(2046 - e) << 52);
+        p *= f;
+        pm *= f;
+    }
+};
+__device__ int sturm_below_dev(int n, const double *__restrict__ a, const double *__restrict__ bb, double x, bool mild) {
+    const int k = n / 2, nb = n - 1 - k;                 // k minors from the top, nb from the bottom (nb <= k)
+    Minor P, Q;
+    for (int i = 0; i < k; ++i) {
+        P.step(a[i] - x, i ? bb[i] : 0.0);
+        if (i < nb) Q.step(a[n - 1 - i] - x, i ? bb[n - i] : 0.0);
+        if (mild && (i & 3) != 3) continue;
+        P.rescale(mild ? 400 : 500);
+        Q.rescale(mild ? 400 : 500);
+    }
+    if (P.neg || Q.neg) return 1;
+    P.normalise();
+    Q.normalise();
+    double g = (a[k] - x) * P.p * Q.p;
+    if (k > 0) g = fma(-bb[k] * P.pm, Q.p, g);
+    if (nb > 0) g = fma(-bb[k + 1] * Q.pm, P.p, g);
+    return __double_as_longlong(g) <= 0 ? 1 : 0;
 }
 
 // lowest eigenvalue of the tridiagonal of order n by multisection: the warp
-// evaluates the Sturm count at 31 interior points of a bracket and keeps
+// tests (sturm_below_dev) 31 interior points of a bracket and keeps
 // the first sub-interval that holds an eigenvalue, until the bracket stops
 // shrinking in fp64 (all lanes return the same value).  The bracket starts
 // around e_prev when given (the lowest Ritz value of a shorter Krylov space,
@@ -1813,7 +1832,7 @@ __device__ double tri_lowest_warp(int n, const double *__restrict__ a, const dou
         // so the last ladder point without an eigenvalue below it and the
         // first with one bracket it to within a factor of four of that move
         const double t = lane == 0 ? e_prev + 1e-12 * w : e_prev - ldexp(1e-6 * w, -2 * (lane - 1));
-        const int c = sturm_count_dev(n, a, bb, t, mild);
+        const int c = sturm_below_dev(n, a, bb, t, mild);
         const unsigned some = __ballot_sync(0xffffffffu, lane > 0 && c > 0);   // counts rise with t
         const unsigned none = __ballot_sync(0xffffffffu, lane > 0 && c == 0);
         const int c0 = __shfl_sync(0xffffffffu, c, 0);
@@ -1833,7 +1852,7 @@ __device__ double tri_lowest_warp(int n, const double *__restrict__ a, const dou
     for (int it = 0; it < 64; ++it) {
         const double h = (hi - lo) / 32.0;
         const double xl = lo + h * (double)(lane + 1);
-        const int cnt = (lane < 31 && xl > lo && xl < hi) ? sturm_count_dev(n, a, bb, xl, mild) : 0;
+        const int cnt = (lane < 31 && xl > lo && xl < hi) ? sturm_below_dev(n, a, bb, xl, mild) : 0;
         const unsigned mk = __ballot_sync(0xffffffffu, lane < 31 && cnt > 0);
         const int j = mk ? __ffs(mk) - 1 : 31;
         const double nlo = j == 0 ? lo : fmax(lo, lo + h * (double)j);
