@@ -29,6 +29,30 @@
 
 namespace qs3 {
 
+// what these kernels read of the lattice (LatView is four times as large, and
+// the smallest products are bound by their launch)
+struct U1View {
+    int N, np1;
+    const uint64_t *binom;
+    double c0;
+    float c0f;
+    const double *u;
+    const float *u_f;
+    const int2 *adj_pad, *adjt;
+    const int4 *adj_pad64;
+    const float *adj_jz_pad, *adjt_jz;
+    const double *adj_jz_pad64;
+};
+static U1View u1_view(const LatView &L) {
+    return {L.N, L.np1, L.binom, L.c0, L.c0f, L.u, L.u_f, L.adj_pad, L.adjt, L.adj_pad64, L.adj_jz_pad, L.adjt_jz, L.adj_jz_pad64};
+}
+template <typename R> __device__ __forceinline__ R diag_c0(const U1View &L);
+template <> __device__ __forceinline__ double diag_c0<double>(const U1View &L) { return L.c0; }
+template <> __device__ __forceinline__ float diag_c0<float>(const U1View &L) { return L.c0f; }
+template <typename R> __device__ __forceinline__ R diag_u(const U1View &L, int i);
+template <> __device__ __forceinline__ double diag_u<double>(const U1View &L, int i) { return __ldg(L.u + i); }
+template <> __device__ __forceinline__ float diag_u<float>(const U1View &L, int i) { return __ldg(L.u_f + i); }
+
 // entry b of site i's fixed-width adjacency (one load): the neighbour and the
 // hop amplitude, padded with the site itself and amplitude 0
 template <typename R> struct Nbr {
@@ -43,10 +67,10 @@ __device__ __forceinline__ Nbr<double> nbr_at(const int4 *__restrict__ t, int at
     const int4 v = __ldg(t + at);
     return {v.x, __hiloint2double(v.w, v.z)};
 }
-__device__ __forceinline__ const int2 *pad_table(const LatView &L, float) { return L.adj_pad; }
-__device__ __forceinline__ const int4 *pad_table(const LatView &L, double) { return L.adj_pad64; }
-__device__ __forceinline__ float pad_jz(const LatView &L, int at, float) { return __ldg(L.adj_jz_pad + at); }
-__device__ __forceinline__ double pad_jz(const LatView &L, int at, double) { return __ldg(L.adj_jz_pad64 + at); }
+__device__ __forceinline__ const int2 *pad_table(const U1View &L, float) { return L.adj_pad; }
+__device__ __forceinline__ const int4 *pad_table(const U1View &L, double) { return L.adj_pad64; }
+__device__ __forceinline__ float pad_jz(const U1View &L, int at, float) { return __ldg(L.adj_jz_pad + at); }
+__device__ __forceinline__ double pad_jz(const U1View &L, int at, double) { return __ldg(L.adj_jz_pad64 + at); }
 
 // one hop of an upper spin of a segment: the rank of the target of c_1 = 0
 // (B(U')), the site j, the hop amplitude and J^z
@@ -79,7 +103,7 @@ template <int ND> struct Seg {
 
 // the rows c_1 = x + lane + 32 r of a segment (FULL: all of them exist)
 template <int ND, typename VT, int DEG, int RL, bool FULL>
-__device__ __forceinline__ void seg_rows(const LatView &L, const uint32_t *sC, const SegHop *hop,
+__device__ __forceinline__ void seg_rows(const U1View &L, const uint32_t *sC, const SegHop *hop,
                                          const Seg<ND> &sg, int x, int lane,
                                          const VT *__restrict__ phi, VT *__restrict__ psi) {
     using R = typename VTr<VT>::R;
@@ -180,7 +204,7 @@ __device__ __forceinline__ void seg_rows(const LatView &L, const uint32_t *sC, c
 }
 
 template <int ND, typename VT, int DEG>
-__global__ void __launch_bounds__(NTHREADS, 4) k_hphi_u1s(LatView L, uint32_t nseg, const VT *__restrict__ phi,
+__global__ void __launch_bounds__(NTHREADS, 4) k_hphi_u1s(U1View L, uint32_t nseg, const VT *__restrict__ phi,
                                                           VT *__restrict__ psi, const int *__restrict__ active) {
     using R = float;
     constexpr int NU = ND - 1, H = NU * DEG, RL = seg_r<VT>();
@@ -275,7 +299,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_u1s(LatView L, uint32_t ns
 }
 
 template <int ND, typename VT, int DEGB>
-__global__ void __launch_bounds__(NTHREADS, sizeof(typename VTr<VT>::R) == 8 || DEGB > 4 ? 4 : 6) k_hphi_u1n(LatView L, uint32_t dim,
+__global__ void __launch_bounds__(NTHREADS, sizeof(typename VTr<VT>::R) == 8 || DEGB > 4 ? 4 : 6) k_hphi_u1n(U1View L, uint32_t dim,
                                                                          const VT *__restrict__ phi,
                                                                          VT *__restrict__ psi,
                                                                          const int *__restrict__ active) {
@@ -360,7 +384,7 @@ static int u1_run(KF kern, Basis &B, size_t smem, uint64_t blocks, uint32_t n, c
     int grid = 1, occ = 1;
     QS3_TRY(launch_rows(kern, B, smem, cache, &grid, &occ));
     auto launch = [&](int g) {
-        kern<<<std::max(1, (int)std::min<uint64_t>(blocks, (uint64_t)g)), NTHREADS, smem, st>>>(B.lv, n, phi, psi,
+        kern<<<std::max(1, (int)std::min<uint64_t>(blocks, (uint64_t)g)), NTHREADS, smem, st>>>(u1_view(B.lv), n, phi, psi,
                                                                                               active);
     };
     int &bps = B.tune_hphi[dt];
