@@ -457,8 +457,7 @@ __device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const
 // group of osg sectors) unranks g's representative once, lists its hop
 // targets (orbit, translation, |Stab|) and its diagonal once in shared
 // memory (maxh entries per thread), then forms g's row in each sector of the
-// group from them.  osg is 8 where that still leaves two rows of blocks per
-// SM, else 4, 2 or 1 (orb_group).
+// group from them (osg from orb_group).
 constexpr int OSG = 8;
 
 // the binary64 engine's product on the integer units: per term one row
@@ -802,12 +801,22 @@ static int hphix_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
     return QS3_OK;
 }
 
-// sectors per thread of the orbit-batched kernels: as many (up to OSG) as
-// leave two resident rows of 2048 threads per SM
-static int orb_group(const Basis &B) {
-    int g = OSG;
-    while (g > 1 && B.n_orb * (uint64_t)((B.S + g - 1) / g) < 2ull * 2048ull * (uint64_t)num_sms()) g >>= 1;
-    return g;
+// sectors per thread of the orbit-batched kernels: the power of two g up to
+// OSG that makes (waves of resident blocks + 1/2 for the last one) times
+// (listing an orbit's hops + g sectors) smallest; the listing costs about as
+// much as one sector in fp32, half of one in binary64 and on the integer
+// units.  10x10, N_down = 4, 20 sectors, 1 / 2 / 4 per thread: c64 83 / 57 /
+// 57 us, c128 146 / 128 / 135, integer 146 / 114 / 120; all 100, 4 / 8 per
+// thread: c64 188 / 169, c128 507 / 519, integer 417 / 410.
+static int orb_group(const Basis &B, bool fp32) {
+    const uint64_t wave = 4ull * NTHREADS * (uint64_t)num_sms();
+    uint64_t least = ~0ull;
+    int best = 1;
+    for (int g = 1; g <= OSG; g *= 2) {
+        const uint64_t c = (2 * B.n_orb * (uint64_t)((B.S + g - 1) / g) + wave) * (uint64_t)(2 * g + (fp32 ? 2 : 1));
+        if (c < least) { least = c; best = g; }
+    }
+    return best;
 }
 // shared memory of the hop lists and tables; 0: too many hops per row
 static size_t orb_smem(const Basis &B, int maxh) {
@@ -825,7 +834,7 @@ static int hphio_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
         QS3_CUDA(cudaFuncSetAttribute(k_hphi_o<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
         attr.store(1, std::memory_order_release);
     }
-    const int osg = orb_group(B), ngrp = (B.S + osg - 1) / osg;
+    const int osg = orb_group(B, false), ngrp = (B.S + osg - 1) / osg;
     const uint64_t nthr = B.n_orb * (uint64_t)ngrp;
     if (nthr == 0) return QS3_OK;
     const int grid = (int)((nthr + NTHREADS - 1) / NTHREADS);
@@ -851,7 +860,7 @@ static int hphiof_nd(Basis &B, const void *phi, void *psi, cudaStream_t st, cons
     int grid = 1, occ = 1;
     QS3_TRY(launch_rows(k_hphi_of<ND, VT>, B, smem, cache, &grid, &occ));
     if (B.tune_hphi[dt] == 0) B.tune_hphi[dt] = occ;             // the grid covers all orbits: nothing to tune
-    const int osg = orb_group(B), ngrp = (B.S + osg - 1) / osg;
+    const int osg = orb_group(B, sizeof(VT) == 8), ngrp = (B.S + osg - 1) / osg;
     const uint64_t nthr = B.n_orb * (uint64_t)ngrp;
     if (nthr == 0) return QS3_OK;
     k_hphi_of<ND, VT><<<(int)((nthr + NTHREADS - 1) / NTHREADS), NTHREADS, smem, st>>>(
