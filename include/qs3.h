@@ -135,17 +135,27 @@ int qs3_basis_nnz(qs3_basis_t b, uint64_t *nnz);
  *   mode = 1: build it (any size that fits); OVERFLOW when C(N, N_down) >= 2^32
  *             or there are 2^20 orbits or more, OOM when it does not fit,
  *             STATE on a U(1)-only basis or N_down = 0;
- *   mode = 0: release it (H Phi runs the search);
+ *   mode = 0: release it (H Phi, S^-_q, S^+_q and the correlations then run
+ *             the search);
  *   mode = -1: query only.
  * *active (may be NULL) receives 1 if the table is in use afterwards.  The
  * table occupies C(N, N_down) * 4 + n_sectors * n_orbits * 4 bytes of device
- * memory, library-owned, released with the basis. */
+ * memory, library-owned, released with the basis.  A basis created without
+ * it (N_down >= 2, one spin per unit cell, N_down - 1 packed sites within 64
+ * bits) gets, where an eighth of the free memory holds them, the sorted origin
+ * forms of its rows instead (about 20 bytes per row): C64 and C128 products
+ * then find a target by its origin form, without the search and with
+ * identical results. */
 int qs3_basis_rep_table(qs3_basis_t b, int32_t mode, int32_t *active);
 /* Autotuned launch choices of a basis (no counterpart in the paper).  On the
  * first direct (not stream-captured) use, the library times:
- *   - H Phi with 1..4 fewer resident 256-row blocks per SM than the occupancy
- *     limit (the persistent grid, i.e. rows in flight per SM), per vector
- *     dtype, and keeps the fastest;
+ *   - H Phi of the per-row k-sector kernels (one sector or no uniform J^xy
+ *     with the table, the search, C128DF, one-sector C128X) with 1..4 fewer
+ *     resident 256-row blocks per SM than the occupancy limit (the persistent
+ *     grid, i.e. rows in flight per SM), per vector dtype, and keeps the
+ *     fastest.  The orbit-batched, origin-form and U(1) kernels take their
+ *     blocks from a rule and record them without trials; the persistent ones
+ *     follow an imposed choice;
  *   - the dot products of the Gram-Schmidt pass with 1, 2 or 4 basis vectors
  *     per pass (loads in flight together): dot_vectors for the double-float
  *     engine and the fp32 phase, dot_vectors64 for the binary64 engine, which
@@ -181,7 +191,9 @@ int qs3_basis_store_terms(qs3_basis_t b, int32_t mode, uint64_t *bytes);
  * sectors, within a few 2^-48 relative of the exact product per term.
  * phi and psi are device vectors of the basis' total dimension and must not
  * alias.  F32/C64 use fp32 matrix elements and fp32 row accumulation.
- * C128X allocates device scratch of twice the vector size per call.
+ * C128X takes device scratch of about one vector per call, in stream order:
+ * the call neither synchronises nor, once the pool of up to 512 MB kept per
+ * device is warm, allocates (vectors above 256 MB are allocated and freed).
  * Errors: STATE (real dtype on a k-sector basis, C128DF on a U(1)-only one,
  * C128X without the representative table or with bond-dependent J^xy). */
 int qs3_hphi(qs3_basis_t b, qs3_dtype dtype, const void *phi, void *psi, void *stream);

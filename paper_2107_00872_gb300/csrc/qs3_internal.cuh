@@ -360,14 +360,6 @@ __device__ __forceinline__ int pick(const int (&a)[ND], int i) {
     return v;
 }
 
-template <int ND>
-__device__ __forceinline__ bool seen_before(const int (&a)[ND], int i, int v) {
-    bool s = false;
-#pragma unroll
-    for (int m = 0; m < ND - 1; ++m) s |= (m < i) && (a[m] == v);
-    return s;
-}
-
 // Minimum-rank translate of the site list t (the representative of its
 // orbit, Alg. 7), found without trying every translation.  Translations move
 // unit cells; a site is spin sb of cell (x, y, z), index sb + nsub (x + Lx

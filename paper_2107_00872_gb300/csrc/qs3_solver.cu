@@ -49,10 +49,6 @@ __device__ __forceinline__ void st2(double2 *p, double2 v) { *p = v; }
 __device__ __forceinline__ double2 cdot(double2 a, double2 b) {
     return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
 }
-__device__ __forceinline__ double2 cmad(double2 acc, double2 a, double2 b) {   // acc + a * b
-    return make_double2(acc.x + a.x * b.x - a.y * b.y, acc.y + a.x * b.y + a.y * b.x);
-}
-
 template <typename VT> struct Is64 { static constexpr bool v = false; };
 template <> struct Is64<double> { static constexpr bool v = true; };
 template <> struct Is64<double2> { static constexpr bool v = true; };
