@@ -404,8 +404,8 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
 // |Stab| at mys[h stride]; returns their number, and in e, dd the diagonal's
 // site part and the J^z of its down-spin pairs (each met twice).
 template <int ND, typename R>
-__device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const int (&c)[ND],
-                                          const uint64_t *__restrict__ sC, const uint8_t *__restrict__ ostab,
+__device__ __forceinline__ int orbit_hops(const LatView &L, uint32_t rank, const int (&c)[ND],
+                                          const uint32_t *__restrict__ sC, const uint8_t *__restrict__ ostab,
                                           uint32_t *my, uint8_t *mys, size_t stride, R &e, R &dd) {
     e = diag_row<R>(L);
     dd = 0;
@@ -417,7 +417,7 @@ __device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const
         const int e0 = __ldg(L.adj_ptr + i), e1 = __ldg(L.adj_ptr + i + 1);
         const int lo = m > 0 ? pick(c, m > 0 ? m - 1 : 0) : -1;
         const int hi = m < ND - 1 ? pick(c, m < ND - 1 ? m + 1 : m) : L.np1;
-        const uint64_t base = rank - sC[(m + 1) * L.np1 + i];
+        const uint32_t base = rank - sC[(m + 1) * L.np1 + i];
         for (int q = e0; q < e1; ++q) {
             const int j = __ldg(L.adj_nbr + q);
             const bool inpl = j > lo && j < hi;
@@ -431,7 +431,7 @@ __device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const
                     continue;
                 }
             }
-            uint64_t r2;
+            uint32_t r2;
             if (inpl) {
                 r2 = base + sC[(m + 1) * L.np1 + j];
             } else {
@@ -439,7 +439,7 @@ __device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const
 #pragma unroll
                 for (int k = 0; k < ND; ++k) tt[k] = (k == m) ? j : c[k];
                 sort_net(tt);
-                r2 = rank_of(tt, sC, L.np1);
+                r2 = rank_of32(tt, sC, L.np1);
             }
             const uint32_t ee = __ldg(L.orb + r2);
             if ((ee >> 12) >= L.n_orb) continue;                 // never for a complete table
@@ -458,6 +458,10 @@ __device__ __forceinline__ int orbit_hops(const LatView &L, uint64_t rank, const
 // targets (orbit, translation, |Stab|) and its diagonal once in shared
 // memory (maxh entries per thread), then forms g's row in each sector of the
 // group from them (osg from orb_group).
+// A table has fewer than 2^32 states, so ranks and binomials (rows 0 .. N_down)
+// are 32-bit words: 16 KB instead of 48 KB staged per block at N = 1000, and four
+// resident blocks instead of three (10x10x10, N_down = 3, 28 sectors: integer 674
+// -> 491 us, c128 720 -> 630, c64 406 -> 233, with the group rule's staging term).
 constexpr int OSG = 8;
 
 // the binary64 engine's product on the integer units: per term one row
@@ -472,11 +476,11 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView
                                                    double2 *__restrict__ psi, const int *__restrict__ active,
                                                    int maxh) {
     extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t *sC = (uint64_t *)smem;
-    double *snorm = (double *)(sC + (L.nd + 3) * L.np1);
+    uint32_t *sC = (uint32_t *)smem;                             // binomial rows 0 .. N_down
+    double *snorm = (double *)(sC + (((ND + 1) * L.np1 + 1) & ~1));
     uint32_t *hl = (uint32_t *)(snorm + 18);                     // hop targets g2 << 12 | u
     uint8_t *hs = (uint8_t *)(hl + (size_t)maxh * blockDim.x);     // their |Stab|
-    stage_tables(L, sC, nullptr);
+    for (int i = threadIdx.x; i < (ND + 1) * L.np1; i += blockDim.x) sC[i] = (uint32_t)L.binom[i];
     if (threadIdx.x < 9) {
         snorm[threadIdx.x] = sqrt((double)threadIdx.x);
         snorm[9 + threadIdx.x] = threadIdx.x ? 1.0 / sqrt((double)threadIdx.x) : 0.0;
@@ -493,11 +497,10 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView
     if (!any) return;
     uint32_t *my = hl + threadIdx.x;                             // entry h at my[h * blockDim.x]
     uint8_t *mys = hs + threadIdx.x;
-    const uint64_t rank = __ldg(oreps + g);
+    const uint32_t rank = (uint32_t)__ldg(oreps + g);            // a table has fewer than 2^32 states
     int c[ND];
-    unrank(rank, sC, L.np1, c);
+    unrank32(rank, sC, L.np1, c);
     const int st_row = __ldg(ostab + g);
-    const double rs = snorm[9 + st_row];
     double e, dd;
     const int nh = orbit_hops<ND, double>(L, rank, c, sC, ostab, my, mys, blockDim.x, e, dd);
     const double ed = e + 0.5 * dd;
@@ -514,25 +517,24 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView
         // four terms at a time: their row lookups, then their digit gathers,
         // are in flight together; the terms are added in list order
         for (int h0 = 0; h0 < nh; h0 += 4) {
-            uint32_t ee[4];
+            int us[4];                                           // u | |Stab| << 12
             int32_t r2[4];
-            int stb[4];
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 const bool in = h0 + b < nh;
-                ee[b] = in ? my[(size_t)(h0 + b) * blockDim.x] : 0u;
-                stb[b] = in ? mys[(size_t)(h0 + b) * blockDim.x] : 0;
-                r2[b] = in ? __ldg(t2 + (ee[b] >> 12)) : -1;
+                const uint32_t ee = in ? my[(size_t)(h0 + b) * blockDim.x] : 0u;
+                us[b] = (int)(ee & 4095u) | (in ? (int)mys[(size_t)(h0 + b) * blockDim.x] << 12 : 0);
+                r2[b] = in ? __ldg(t2 + (ee >> 12)) : -1;
             }
             int4 q[4];
 #pragma unroll
             for (int b = 0; b < 4; ++b)
-                q[b] = r2[b] >= 0 && stb[b] == st_row ? __ldg(hv.hd + off + (uint32_t)r2[b]) : make_int4(0, 0, 0, 0);
+                q[b] = r2[b] >= 0 && us[b] >> 12 == st_row ? __ldg(hv.hd + off + (uint32_t)r2[b]) : make_int4(0, 0, 0, 0);
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
                 if (r2[b] < 0) continue;
-                const int u = (int)(ee[b] & 4095u);
-                if (stb[b] == st_row) {
+                const int u = us[b] & 4095;
+                if (us[b] >> 12 == st_row) {
                     int2 f1, f0;
                     int em;
                     hd_unpack(q[b], f1, f0, em);
@@ -541,7 +543,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView
                     row_add(acc, tr, ti, em);
                 } else {
                     double2 p = secs[s].ph64[u];
-                    const double f = snorm[stb[b]] * rs;
+                    const double f = snorm[us[b] >> 12] * snorm[9 + st_row];
                     p.x *= f;
                     p.y *= f;
                     acc_add(acc64, p, hv.value(off + (uint32_t)r2[b]));
@@ -577,11 +579,11 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_of(LatView L, const SecVie
     using R = typename VTr<VT>::R;
     using CT = typename VTr<VT>::C;
     extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t *sC = (uint64_t *)smem;
-    R *snorm = (R *)(sC + (L.nd + 3) * L.np1);                    // 18 of R in the room of 18 doubles
+    uint32_t *sC = (uint32_t *)smem;                             // binomial rows 0 .. N_down
+    R *snorm = (R *)(sC + (((ND + 1) * L.np1 + 1) & ~1));         // 18 of R in the room of 18 doubles
     uint32_t *hl = (uint32_t *)((double *)snorm + 18);
     uint8_t *hs = (uint8_t *)(hl + (size_t)maxh * blockDim.x);
-    stage_tables(L, sC, nullptr);
+    for (int i = threadIdx.x; i < (ND + 1) * L.np1; i += blockDim.x) sC[i] = (uint32_t)L.binom[i];
     if (threadIdx.x < 9) {
         snorm[threadIdx.x] = (R)sqrt((double)threadIdx.x);
         snorm[9 + threadIdx.x] = threadIdx.x ? (R)(1.0 / sqrt((double)threadIdx.x)) : (R)0;
@@ -596,9 +598,9 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_of(LatView L, const SecVie
     if (!any) return;
     uint32_t *my = hl + threadIdx.x;
     uint8_t *mys = hs + threadIdx.x;
-    const uint64_t rank = __ldg(oreps + g);
+    const uint32_t rank = (uint32_t)__ldg(oreps + g);            // a table has fewer than 2^32 states
     int c[ND];
-    unrank(rank, sC, L.np1, c);
+    unrank32(rank, sC, L.np1, c);
     const int st_row = __ldg(ostab + g);
     const R rs = snorm[9 + st_row];
     R e, dd;
@@ -803,25 +805,29 @@ static int hphix_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
 
 // sectors per thread of the orbit-batched kernels: the power of two g up to
 // OSG that makes (waves of resident blocks + 1/2 for the last one) times
-// (listing an orbit's hops + g sectors) smallest; the listing costs about as
-// much as one sector in fp32, half of one in binary64 and on the integer
-// units.  10x10, N_down = 4, 20 sectors, 1 / 2 / 4 per thread: c64 83 / 57 /
-// 57 us, c128 146 / 128 / 135, integer 146 / 114 / 120; all 100, 4 / 8 per
-// thread: c64 188 / 169, c128 507 / 519, integer 417 / 410.
+// (setting a thread up + g sectors) smallest.  Listing an orbit's hops costs
+// about as much as one sector in fp32, half of one in binary64 and on the
+// integer units, staging the binomials half of one per four loads a thread.
+// 10x10, N_down = 4, 20 sectors, 1 / 2 / 4 per thread: c64 83 / 57 / 57 us,
+// c128 146 / 128 / 135, integer 146 / 114 / 120; all 100, 4 / 8 per thread: c64
+// 188 / 169, c128 507 / 519, integer 417 / 410; 10x10x10, N_down = 3 (16 loads a
+// thread), 28 sectors, 2 / 4 / 8: c64 347 / 268 / 233, integer 594 / 520 / 491.
 static int orb_group(const Basis &B, bool fp32) {
     const uint64_t wave = 4ull * NTHREADS * (uint64_t)num_sms();
+    const int setup = (fp32 ? 2 : 1) + (B.nd + 1) * (B.N + 1) / (4 * NTHREADS);     // in half sectors
     uint64_t least = ~0ull;
     int best = 1;
     for (int g = 1; g <= OSG; g *= 2) {
-        const uint64_t c = (2 * B.n_orb * (uint64_t)((B.S + g - 1) / g) + wave) * (uint64_t)(2 * g + (fp32 ? 2 : 1));
+        const uint64_t c = (2 * B.n_orb * (uint64_t)((B.S + g - 1) / g) + wave) * (uint64_t)(2 * g + setup);
         if (c < least) { least = c; best = g; }
     }
     return best;
 }
-// shared memory of the hop lists and tables; 0: too many hops per row
+// shared memory of the 32-bit binomials and the hop lists; 0: too many hops per row
 static size_t orb_smem(const Basis &B, int maxh) {
-    const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8 + 18 * 8 + (size_t)maxh * NTHREADS * 5;
-    return smem <= (size_t)MAX_DYN_SMEM ? smem : 0;
+    const size_t lists = 18 * 8 + (size_t)maxh * NTHREADS * 5;
+    if ((size_t)(B.nd + 3) * (B.N + 1) * 8 + lists > (size_t)MAX_DYN_SMEM) return 0;
+    return (((size_t)(B.nd + 1) * (B.N + 1) + 1) & ~(size_t)1) * 4 + lists;
 }
 
 template <int ND>
