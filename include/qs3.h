@@ -149,8 +149,8 @@ int qs3_basis_nnz(qs3_basis_t b, uint64_t *nnz);
 int qs3_basis_rep_table(qs3_basis_t b, int32_t mode, int32_t *active);
 /* Autotuned launch choices of a basis (no counterpart in the paper).  On the
  * first direct (not stream-captured) use, the library times:
- *   - H Phi of the per-row k-sector kernels (one sector or no uniform J^xy
- *     with the table, the search, C128DF, one-sector C128X) with 1..4 fewer
+ *   - H Phi of the per-row k-sector kernels (no uniform J^xy with the table,
+ *     the search, C128DF, hop lists beyond shared memory) with 1..4 fewer
  *     resident 256-row blocks per SM than the occupancy limit (the persistent
  *     grid, i.e. rows in flight per SM), per vector dtype, and keeps the
  *     fastest.  The orbit-batched, origin-form and U(1) kernels take their

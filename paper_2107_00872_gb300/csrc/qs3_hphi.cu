@@ -851,10 +851,12 @@ static int hphio_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
     return QS3_OK;
 }
 
-// the orbit-batched FMA kernel serves bases of several sectors with the
-// representative table and one hop amplitude whose hop lists fit
+// the orbit-batched FMA kernel serves bases with the representative table and
+// one hop amplitude whose hop lists fit, of one sector too (c128 k_hphi /
+// k_hphi_of: 10x10, N_down = 4 31 / 27 us a call, 12x12 53 / 37, 10x10x10, N_down =
+// 3 71 / 54; c64 21 / 18, 23 / 21, 44 / 38)
 static bool hphi_of_ok(const Basis &B) {
-    return B.has_k && B.S >= 2 && B.lv.orb && B.d_oreps.p && B.lv.jh_uniform != 0.0 &&
+    return B.has_k && B.lv.orb && B.d_oreps.p && B.lv.jh_uniform != 0.0 &&
            orb_smem(B, std::max(1, B.nd * B.max_degree)) > 0;
 }
 
@@ -899,8 +901,10 @@ int hphi_x_launch(Basis &B, const HxVec &hv, void *psi, cudaStream_t st, const i
     if (!hphi_x_ok(B)) return set_err(QS3_ERR_STATE, "the integer H Phi needs a k-sector basis with the "
                                                      "representative table and one hop amplitude");
     double2 *o = (double2 *)psi;
-    // several sectors share the orbits: the orbit-batched kernel
-    if (B.S >= 2 && B.d_oreps.p) {
+    // the orbit-batched kernel, except one sector with hop lists that do not
+    // fit (one sector, k_hphi_x / k_hphi_o: 10x10, N_down = 4 36 / 34 us a call,
+    // 10x10x10, N_down = 3 61 / 51, 12x12 40 / 40)
+    if (B.d_oreps.p && (B.S >= 2 || orb_smem(B, std::max(1, B.nd * B.max_degree)) > 0)) {
         switch (B.nd) {
             case 1: return hphio_nd<1>(B, hv, o, st, active);
             case 2: return hphio_nd<2>(B, hv, o, st, active);

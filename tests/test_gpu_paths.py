@@ -106,7 +106,10 @@ def test_batched_sectors_equal_single(spec, nd, nk):
         for s, k in enumerate(ks):
             one = lib_basis(spec, nd, [k])
             lo, hi = b.offsets[s], b.offsets[s + 1]
-            assert torch.equal(one.hphi(phi[lo:hi].contiguous()), got[lo:hi])
+            x = phi[lo:hi].contiguous()
+            assert torch.equal(one.hphi(x), got[lo:hi])
+            one.rep_table(0)                            # the row kernel with the search
+            assert torch.equal(one.hphi(x), got[lo:hi])
 
 
 # two-point functions and S^-_q, S^+_q by the table and by the search.  Each is a
