@@ -270,28 +270,55 @@ __global__ void __launch_bounds__(NTHREADS) k_enum_reps(LatView L, int s0, uint6
     }
 }
 
-// The orbits of the N_down-subsets under the translations, by Burnside's
-// lemma: a translation of order o moves the sites in cycles of o and fixes
-// C(N / o, N_down / o) subsets when o divides N_down, none otherwise.
-static uint64_t count_orbits(const Basis &B, const std::vector<uint64_t> &binom) {
-    auto gcd = [](int a, int b) {
-        while (b) {
-            const int t = a % b;
-            a = b;
-            b = t;
+static int gcd_of(int a, int b) {
+    while (b) {
+        const int t = a % b;
+        a = b;
+        b = t;
+    }
+    return a;
+}
+
+// The rows of the sector of momentum K, exactly: the orbits on whose
+// stabiliser e^{ik.t} = 1, which by the character sum are (1 / G) sum_t
+// e^{ik.t} Fix(t) (for K = 0 Burnside's count of all orbits).  A translation of
+// order o moves the sites in cycles of o and fixes C(N / o, N_down / o)
+// subsets when o divides N_down, none otherwise.  The translations with o t =
+// 0 are the multiples of L_a / g_a along each axis, g_a = gcd(o, L_a), so e^{ik.t}
+// sums over them to prod g_a when every g_a divides K_a and to 0 otherwise;
+// Moebius inversion over the divisors of o leaves those of order o.
+static uint64_t sector_dim(const Basis &B, const int *K) {
+    auto moebius = [](int n) {
+        int m = 1;
+        for (int p = 2; p <= n; ++p) {
+            if (n % p) continue;
+            n /= p;
+            if (n % p == 0) return 0;
+            m = -m;
         }
-        return a;
+        return m;
     };
-    auto order = [&](int L, int t) { return L / gcd(L, t); };
-    unsigned __int128 sum = 0;
-    for (int z = 0; z < B.L[2]; ++z)
-        for (int y = 0; y < B.L[1]; ++y)
-            for (int x = 0; x < B.L[0]; ++x) {
-                int o = order(B.L[0], x);
-                for (int q : {order(B.L[1], y), order(B.L[2], z)}) o = o / gcd(o, q) * q;
-                if (B.nd % o == 0) sum += binom[(size_t)(B.nd / o) * (B.N + 1) + B.N / o];
-            }
-    return (uint64_t)(sum / (unsigned)B.ncell);
+    auto killed_by = [&](int o) {
+        long long f = 1;
+        for (int a = 0; a < 3; ++a) {
+            const int g = gcd_of(o, B.L[a]);
+            f *= K[a] % g == 0 ? g : 0;
+        }
+        return f;
+    };
+    __int128 sum = 0;
+    for (int o = 1; o <= B.nd; ++o) {
+        if (B.nd % o) continue;
+        long long e = 0;
+        for (int d = 1; d <= o; ++d)
+            if (o % d == 0) e += moebius(o / d) * killed_by(d);
+        if (e) sum += (__int128)e * B.binom[(size_t)(B.nd / o) * (B.N + 1) + B.N / o];
+    }
+    return (uint64_t)(sum / B.ncell);
+}
+static uint64_t count_orbits(const Basis &B) {
+    const int K0[3] = {0, 0, 0};
+    return sector_dim(B, K0);
 }
 
 // the representatives of all orbits, sorted by rank0, with |Stab|: n of them
@@ -303,7 +330,7 @@ static int enum_orbits(Basis &B, DevBuf &kout, DevBuf &vout, uint64_t &n) {
     int dev = 0, nsm = 0;
     QS3_CUDA(cudaGetDevice(&dev));
     QS3_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    n = count_orbits(B, hb);
+    n = count_orbits(B);
     DevBuf cnt, kin, vin;
     QS3_TRY(cnt.alloc(sizeof(unsigned long long), (cudaStream_t)0));
     QS3_CUDA(cudaMemset(cnt.p, 0, sizeof(unsigned long long)));
@@ -402,19 +429,15 @@ __global__ void __launch_bounds__(NTHREADS) k_members(LatView L, const uint64_t 
     }
 }
 
-__global__ void k_ends(const uint32_t *__restrict__ pos, uint64_t n, int cnt, uint32_t *__restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < cnt) out[i] = pos[(uint64_t)i * n];
-}
-
 // rows of ns sectors from the scanned flags (pos: ns n + 1 entries): the
-// representatives and |Stab| of the members, one sector after another
+// representatives and |Stab| of the members, one sector after another (room
+// for cap of them)
 __global__ void k_take(const uint32_t *__restrict__ pos, const uint64_t *__restrict__ reps,
-                       const uint8_t *__restrict__ stab, uint64_t n, uint64_t cnt, uint64_t *__restrict__ sigma,
-                       uint8_t *__restrict__ sst) {
+                       const uint8_t *__restrict__ stab, uint64_t n, uint64_t cnt, uint64_t cap,
+                       uint64_t *__restrict__ sigma, uint8_t *__restrict__ sst) {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t p = pos[i];
-        if (pos[i + 1] == p) continue;
+        if (pos[i + 1] == p || p >= cap) continue;
         const uint64_t g = i % n;
         sigma[p] = reps[g];
         sst[p] = stab[g];
@@ -487,66 +510,65 @@ __global__ void __launch_bounds__(NTHREADS) k_bucket_fill(LatView L, const SecVi
     }
 }
 
-// The sectors of a k-sector basis: the orbits are enumerated and sorted once,
-// and each sector takes the compatible ones in order (a flag per orbit and
-// sector, scanned), as many sectors at a time as 2^27 flags hold.  keep_reps
-// / keep_stab receive the orbits' list for the representative table.
+// The sectors of a k-sector basis (B.dims set, each below 2^32): the orbits
+// are enumerated and sorted once, and each sector takes the compatible ones in
+// order (a flag per orbit and sector, scanned), as many sectors at a time as
+// 2^27 flags hold and at least one, whose rows 32-bit positions number.
+// keep_reps / keep_stab receive the orbits' list for the representative table.
 template <int ND>
 static int build_sectors_nd(Basis &B, DevBuf &keep_reps, DevBuf &keep_stab, uint64_t &n) {
     QS3_TRY(enum_orbits<ND>(B, keep_reps, keep_stab, n));
     const int S = B.S;
-    const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8 + (size_t)B.N * 4;
-    QS3_CUDA(cudaFuncSetAttribute(k_members<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-    if (S == 1 && B.K[0] == 0 && B.K[1] == 0 && B.K[2] == 0) {
+    if (S == 1 && B.dims[0] == n) {
         // every orbit; the table's copy is made when there may be one
-        B.dims[0] = n;
         if (n < (1ull << 20)) {
             QS3_TRY(B.d_sigma.alloc(n * 8));
             QS3_TRY(B.d_stab.alloc(n));
-            QS3_CUDA(cudaMemcpy(B.d_sigma.p, keep_reps.p, n * 8, cudaMemcpyDeviceToDevice));
-            QS3_CUDA(cudaMemcpy(B.d_stab.p, keep_stab.p, n, cudaMemcpyDeviceToDevice));
+            QS3_CUDA(cudaMemcpyAsync(B.d_sigma.p, keep_reps.p, n * 8, cudaMemcpyDeviceToDevice));
+            QS3_CUDA(cudaMemcpyAsync(B.d_stab.p, keep_stab.p, n, cudaMemcpyDeviceToDevice));
         } else {
             B.d_sigma = std::move(keep_reps);
             B.d_stab = std::move(keep_stab);
         }
-    } else {
-        QS3_TRY(B.d_sigma.alloc((uint64_t)S * n * 8));
-        QS3_TRY(B.d_stab.alloc((uint64_t)S * n));
-        DevBuf dK, pos, tmp, dends;
-        QS3_TRY(dends.alloc(((size_t)S + 1) * 4, (cudaStream_t)0));
-        QS3_TRY(dK.upload(B.K.data(), B.K.size() * sizeof(int), (cudaStream_t)0));
-        const int grp = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)S, (1ull << 27) / std::max<uint64_t>(n, 1)));
-        QS3_TRY(pos.alloc(((uint64_t)grp * n + 1) * 4, (cudaStream_t)0));
-        size_t tb = 0;
-        QS3_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, pos.as<uint32_t>(), pos.as<uint32_t>(), (int64_t)((uint64_t)grp * n + 1)));
-        QS3_TRY(tmp.alloc(tb, (cudaStream_t)0));
-        uint64_t off = 0;
-        std::vector<uint32_t> ends;
-        for (int s0 = 0; s0 < S; s0 += grp) {
-            const int ns = std::min(grp, S - s0);
-            const uint64_t cnt = (uint64_t)ns * n;
-            const int g1 = (int)std::max<uint64_t>(1, std::min<uint64_t>((n + NTHREADS - 1) / NTHREADS, 4096));
-            QS3_CUDA(cudaMemsetAsync(pos.as<uint32_t>() + cnt, 0, 4));
-            k_members<ND><<<g1, NTHREADS, smem>>>(B.lv, keep_reps.as<uint64_t>(), keep_stab.as<uint8_t>(), n, ns,
-                                                  dK.as<int>() + 3 * s0, pos.as<uint32_t>());
-            QS3_LAUNCHED();
-            size_t t2 = tb;
-            QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, t2, pos.as<uint32_t>(), pos.as<uint32_t>(), (int64_t)(cnt + 1)));
-            const int g2 = (int)std::max<uint64_t>(1, std::min<uint64_t>((cnt + 255) / 256, 16384));
-            k_take<<<g2, 256>>>(pos.as<uint32_t>(), keep_reps.as<uint64_t>(), keep_stab.as<uint8_t>(), n, cnt,
-                                B.d_sigma.as<uint64_t>() + off, B.d_stab.as<uint8_t>() + off);
-            QS3_LAUNCHED();
-            k_ends<<<(ns + 256) / 256, 256>>>(pos.as<uint32_t>(), n, ns + 1, dends.as<uint32_t>());
-            QS3_LAUNCHED();
-            ends.assign(ns + 1, 0);
-            QS3_CUDA(cudaMemcpy(ends.data(), dends.p, ends.size() * 4, cudaMemcpyDeviceToHost));
-            for (int i = 0; i < ns; ++i) B.dims[s0 + i] = ends[i + 1] - ends[i];
-            off += ends[ns];
-        }
+        return QS3_OK;
     }
-    for (int s = 0; s < S; ++s)
-        if (B.dims[s] >= (1ull << 32))
-            return set_err(QS3_ERR_OVERFLOW, "sector dimension %llu exceeds 2^32", (unsigned long long)B.dims[s]);
+    const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8 + (size_t)B.N * 4;
+    QS3_CUDA(cudaFuncSetAttribute(k_members<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+    uint64_t total = 0;
+    for (uint64_t d : B.dims) total += d;
+    QS3_TRY(B.d_sigma.alloc(total * 8));
+    QS3_TRY(B.d_stab.alloc(total));
+    DevBuf dK, pos, tmp;
+    QS3_TRY(dK.upload(B.K.data(), B.K.size() * sizeof(int), (cudaStream_t)0));
+    const int grp = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)S, (1ull << 27) / std::max<uint64_t>(n, 1)));
+    QS3_TRY(pos.alloc(((uint64_t)grp * n + 1) * 4, (cudaStream_t)0));
+    size_t tb = 0;
+    QS3_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, pos.as<uint32_t>(), pos.as<uint32_t>(), (int64_t)((uint64_t)grp * n + 1)));
+    QS3_TRY(tmp.alloc(tb, (cudaStream_t)0));
+    uint64_t off = 0;
+    for (int s0 = 0; s0 < S; s0 += grp) {
+        const int ns = std::min(grp, S - s0);
+        const uint64_t cnt = (uint64_t)ns * n;
+        uint64_t rows = 0;
+        for (int s = s0; s < s0 + ns; ++s) rows += B.dims[s];
+        const int g1 = (int)std::max<uint64_t>(1, std::min<uint64_t>((n + NTHREADS - 1) / NTHREADS, 4096));
+        QS3_CUDA(cudaMemsetAsync(pos.as<uint32_t>() + cnt, 0, 4));
+        k_members<ND><<<g1, NTHREADS, smem>>>(B.lv, keep_reps.as<uint64_t>(), keep_stab.as<uint8_t>(), n, ns,
+                                              dK.as<int>() + 3 * s0, pos.as<uint32_t>());
+        QS3_LAUNCHED();
+        size_t t2 = tb;
+        QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, t2, pos.as<uint32_t>(), pos.as<uint32_t>(), (int64_t)(cnt + 1)));
+        const int g2 = (int)std::max<uint64_t>(1, std::min<uint64_t>((cnt + 255) / 256, 16384));
+        k_take<<<g2, 256>>>(pos.as<uint32_t>(), keep_reps.as<uint64_t>(), keep_stab.as<uint8_t>(), n, cnt, rows,
+                            B.d_sigma.as<uint64_t>() + off, B.d_stab.as<uint8_t>() + off);
+        QS3_LAUNCHED();
+        uint32_t end = 0;
+        QS3_CUDA(cudaMemcpy(&end, pos.as<uint32_t>() + cnt, 4, cudaMemcpyDeviceToHost));
+        if (end != rows)
+            return set_err(QS3_ERR_CUDA, "%u rows of sectors %d .. %d, %llu expected", end, s0, s0 + ns - 1,
+                           (unsigned long long)rows);
+        off += rows;
+    }
     return QS3_OK;
 }
 
@@ -712,7 +734,7 @@ static int build_table_nd(Basis &B, size_t max_bytes, DevBuf &reps, DevBuf &stab
         return set_err(QS3_ERR_OOM, "representative table of ~%llu bytes exceeds the limit",
                        (unsigned long long)(ns * 4 + n_est * 4 * (uint64_t)B.S));
     if (!reps.p) {
-        n = count_orbits(B, B.binom);
+        n = count_orbits(B);
         if (n < (1ull << 20)) QS3_TRY(enum_orbits<ND>(B, reps, stab, n));
     }
     int dev = 0, nsm = 0;
@@ -928,8 +950,30 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     uint64_t cnd = 0;
     if (!binom_table(N, nd + 3, tb, &cnd, nd))
         return set_err(QS3_ERR_OVERFLOW, "C(%d, %d) does not fit in 63 bits", N, nd);
-    QS3_TRY(B.d_binom.upload(tb.data(), tb.size() * 8));
     B.binom = std::move(tb);
+
+    // the sectors' rows, and what they are limited to, before anything is allocated
+    B.dims.assign(nsec, 0);
+    B.offs.assign(nsec + 1, 0);
+    B.tile0.assign(nsec + 1, 0);
+    B.chunk0.assign(nsec + 1, 0);
+    for (int s = 0; s < nsec; ++s) {
+        const int *k = &B.K[3 * s];
+        if (!B.has_k) B.dims[s] = cnd;
+        else if (nd == 0) B.dims[s] = k[0] == 0 && k[1] == 0 && k[2] == 0 ? 1 : 0;   // the vacuum
+        else B.dims[s] = sector_dim(B, k);
+        if (B.has_k && B.dims[s] >= (1ull << 32))
+            return set_err(QS3_ERR_OVERFLOW, "sector dimension %llu exceeds 2^32", (unsigned long long)B.dims[s]);
+        B.offs[s + 1] = B.offs[s] + B.dims[s];
+        const uint64_t nt = (B.dims[s] + TILE - 1) / TILE;
+        if ((uint64_t)B.tile0[s] + nt > (1ull << 31) - 1) return set_err(QS3_ERR_OVERFLOW, "too many rows");
+        B.tile0[s + 1] = B.tile0[s] + (int)nt;
+        B.chunk0[s + 1] = B.chunk0[s] + (int)((B.dims[s] + BROWS - 1) / BROWS);
+    }
+    B.total = B.offs[nsec];
+    B.ntiles = B.tile0[nsec];
+    B.nchunks = B.chunk0[nsec];
+    QS3_TRY(B.d_binom.upload(B.binom.data(), B.binom.size() * 8));
 
     // adjacency (CSR, both directions), diagonal constants
     std::vector<int> deg(N + 1, 0);
@@ -1084,35 +1128,16 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     }
 
     // sectors
-    B.dims.assign(nsec, 0);
     DevBuf oreps, ostab;
     uint64_t n_orb = 0;
-    if (!B.has_k) {
-        B.dims[0] = cnd;
-    } else if (nd == 0) {
-        // the vacuum, in the sector of momentum 0
+    if (B.has_k && nd == 0) {
         std::vector<uint64_t> zero(nsec, 0);
         std::vector<uint8_t> one(nsec, 1);
-        for (int s = 0; s < nsec; ++s)
-            B.dims[s] = B.K[3 * s] == 0 && B.K[3 * s + 1] == 0 && B.K[3 * s + 2] == 0 ? 1 : 0;
         QS3_TRY(B.d_sigma.upload(zero.data(), zero.size() * 8));
         QS3_TRY(B.d_stab.upload(one.data(), one.size()));
-    } else {
+    } else if (B.has_k) {
         QS3_TRY(build_sectors(B, oreps, ostab, n_orb));
     }
-    B.offs.assign(nsec + 1, 0);
-    B.tile0.assign(nsec + 1, 0);
-    B.chunk0.assign(nsec + 1, 0);
-    for (int s = 0; s < nsec; ++s) {
-        B.offs[s + 1] = B.offs[s] + B.dims[s];
-        uint64_t nt = (B.dims[s] + TILE - 1) / TILE;
-        if ((uint64_t)B.tile0[s] + nt > (1ull << 31) - 1) return set_err(QS3_ERR_OVERFLOW, "too many rows");
-        B.tile0[s + 1] = B.tile0[s] + (int)nt;
-        B.chunk0[s + 1] = B.chunk0[s] + (int)((B.dims[s] + BROWS - 1) / BROWS);
-    }
-    B.total = B.offs[nsec];
-    B.ntiles = B.tile0[nsec];
-    B.nchunks = B.chunk0[nsec];
     B.secs.resize(nsec);
     if (B.has_k) {
         QS3_TRY(B.d_ph64.alloc((size_t)nsec * N * sizeof(double2)));
