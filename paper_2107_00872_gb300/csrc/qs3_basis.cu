@@ -479,15 +479,15 @@ __global__ void k_first(int nd, int np1, int pre2, const SecView *__restrict__ s
 // a prefix also the ones after
 template <int ND>
 __global__ void __launch_bounds__(NTHREADS) k_bucket_fill(LatView L, const SecView *__restrict__ secs,
-                                                          const int *__restrict__ tile0, int S, int ntiles, uint32_t np,
-                                                          const uint32_t *__restrict__ first,
+                                                          const int *__restrict__ tile0, int S, int t0, int t1,
+                                                          uint32_t np, const uint32_t *__restrict__ first,
                                                           const uint2 *__restrict__ pinfo, uint32_t *__restrict__ sub) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *sC = (uint64_t *)smem;
     stage_tables(L, sC, nullptr);
     __syncthreads();
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int s = S == 1 ? 0 : sector_of_tile(tile0, S, t);
+    for (int64_t t = (int64_t)t0 + blockIdx.x; t < t1; t += gridDim.x) {
+        const int s = S == 1 ? 0 : sector_of_tile(tile0, S, (int)t);
         const uint64_t row = (uint64_t)(t - secs[s].tile0) * TILE + threadIdx.x;
         if (row >= secs[s].dim) continue;
         const uint64_t *sig = secs[s].sigma;
@@ -572,7 +572,11 @@ static int build_sectors_nd(Basis &B, DevBuf &keep_reps, DevBuf &keep_stab, uint
     return QS3_OK;
 }
 
-// the index over every sector's rows (SecView::pinfo, sub)
+// the index over every sector's rows (SecView::pinfo, sub), as many sectors at
+// a time as INDEX_GROUP entries hold and at least one: the offsets in a group
+// are 32 bits (a sector of fewer than 2^32 rows has at most 2^31 + 2 np
+// entries), the groups' places in d_sub 64
+constexpr uint64_t INDEX_GROUP = (uint64_t)1 << 22;
 template <int ND>
 static int build_index_nd(Basis &B) {
     const int S = B.S;
@@ -580,44 +584,62 @@ static int build_index_nd(Basis &B) {
     const uint64_t np2 = (uint64_t)B.N * (B.N - 1) / 2;
     const int pre2 = ND >= 2 && (uint64_t)S * np2 / 8 <= B.total ? 1 : 0;
     const uint32_t np = pre2 ? (uint32_t)np2 : (uint32_t)B.N;
-    const uint64_t cnt = (uint64_t)S * np;
     for (auto &v : B.secs) v.pre2 = pre2;
     QS3_CUDA(cudaMemcpy(B.d_secs.p, B.secs.data(), B.secs.size() * sizeof(SecView), cudaMemcpyHostToDevice));
-    DevBuf first, size, off, tmp;
-    QS3_TRY(first.alloc((uint64_t)S * (np + 1) * 4, (cudaStream_t)0));
-    QS3_TRY(size.alloc((cnt + 1) * 4, (cudaStream_t)0));
-    QS3_TRY(off.alloc((cnt + 1) * 4, (cudaStream_t)0));
-    const int g1 = (int)std::max<uint64_t>(1, std::min<uint64_t>((cnt + S + 255) / 256, 16384));
-    const uint64_t *bin = B.d_binom.as<uint64_t>();
-    const SecView *secs = B.d_secs.as<SecView>();
-    k_first<<<g1, 256>>>(B.nd, B.N + 1, pre2, secs, S, np, bin, first.as<uint32_t>());
-    QS3_LAUNCHED();
-    QS3_CUDA(cudaMemsetAsync(size.as<uint32_t>() + cnt, 0, 4));
-    k_bucket_size<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, S, np, 1, first.as<uint32_t>(), size.as<uint32_t>());
-    QS3_LAUNCHED();
-    size_t tb = 0;
-    QS3_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt + 1)));
-    QS3_TRY(tmp.alloc(tb, (cudaStream_t)0));
-    QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, tb, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt + 1)));
     // at most rows / 2 + 1 buckets and the end per prefix
-    const uint64_t most = B.total / 2 + 2 * cnt;
-    if (most >= (1ull << 32)) return set_err(QS3_ERR_OVERFLOW, "index of %llu entries", (unsigned long long)most);
-    QS3_TRY(B.d_pinfo.alloc(std::max<uint64_t>(cnt, 1) * sizeof(uint2)));
-    QS3_TRY(B.d_sub.alloc(std::max<uint64_t>(most, 1) * 4));
-    k_bucket_info<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, S, np, 1, first.as<uint32_t>(), off.as<uint32_t>(),
-                               B.d_pinfo.as<uint2>(), B.d_sub.as<uint32_t>());
-    QS3_LAUNCHED();
-    if (B.ntiles > 0) {
-        const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8;
-        QS3_CUDA(cudaFuncSetAttribute(k_bucket_fill<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-        k_bucket_fill<ND><<<std::min(B.ntiles, 8192), NTHREADS, smem>>>(B.lv, secs, B.d_tile0.as<int>(), S, B.ntiles, np,
-                                                                        first.as<uint32_t>(), B.d_pinfo.as<uint2>(),
-                                                                        B.d_sub.as<uint32_t>());
-        QS3_LAUNCHED();
-    }
+    auto entries = [&](int s) { return B.dims[s] / 2 + 2 * (uint64_t)np; };
+    std::vector<int> g0{0};
+    uint64_t most = 0, in_group = 0, cnt_max = 0;
     for (int s = 0; s < S; ++s) {
-        B.secs[s].pinfo = B.d_pinfo.as<uint2>() + (uint64_t)s * np;
-        B.secs[s].sub = B.d_sub.as<uint32_t>();
+        if (s > g0.back() && in_group + entries(s) > INDEX_GROUP) {
+            g0.push_back(s);
+            in_group = 0;
+        }
+        in_group += entries(s);
+        most += entries(s);
+        cnt_max = std::max(cnt_max, (uint64_t)(s + 1 - g0.back()) * np);
+    }
+    g0.push_back(S);
+    QS3_TRY(B.d_pinfo.alloc(std::max<uint64_t>((uint64_t)S * np, 1) * sizeof(uint2)));
+    QS3_TRY(B.d_sub.alloc(std::max<uint64_t>(most, 1) * 4));
+    DevBuf first, size, off, tmp;
+    QS3_TRY(first.alloc((cnt_max + S) * 4, (cudaStream_t)0));
+    QS3_TRY(size.alloc((cnt_max + 1) * 4, (cudaStream_t)0));
+    QS3_TRY(off.alloc((cnt_max + 1) * 4, (cudaStream_t)0));
+    size_t tb = 0;
+    QS3_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, tb, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt_max + 1)));
+    QS3_TRY(tmp.alloc(tb, (cudaStream_t)0));
+    const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8;
+    QS3_CUDA(cudaFuncSetAttribute(k_bucket_fill<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
+    const uint64_t *bin = B.d_binom.as<uint64_t>();
+    uint64_t base = 0;
+    for (size_t g = 0; g + 1 < g0.size(); ++g) {
+        const int s0 = g0[g], ns = g0[g + 1] - s0;
+        const uint64_t cnt = (uint64_t)ns * np;
+        const int g1 = (int)std::max<uint64_t>(1, std::min<uint64_t>((cnt + ns + 255) / 256, 16384));
+        const SecView *secs = B.d_secs.as<SecView>() + s0;
+        uint2 *pinfo = B.d_pinfo.as<uint2>() + (uint64_t)s0 * np;
+        uint32_t *sub = B.d_sub.as<uint32_t>() + base;
+        k_first<<<g1, 256>>>(B.nd, B.N + 1, pre2, secs, ns, np, bin, first.as<uint32_t>());
+        QS3_LAUNCHED();
+        QS3_CUDA(cudaMemsetAsync(size.as<uint32_t>() + cnt, 0, 4));
+        k_bucket_size<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, ns, np, 1, first.as<uint32_t>(), size.as<uint32_t>());
+        QS3_LAUNCHED();
+        size_t t2 = tb;
+        QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, t2, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt + 1)));
+        k_bucket_info<<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, ns, np, 1, first.as<uint32_t>(), off.as<uint32_t>(), pinfo, sub);
+        QS3_LAUNCHED();
+        const int t0 = B.tile0[s0], t1 = B.tile0[s0 + ns];
+        if (t1 > t0) {
+            k_bucket_fill<ND><<<std::min(t1 - t0, 8192), NTHREADS, smem>>>(B.lv, secs, B.d_tile0.as<int>() + s0, ns, t0, t1,
+                                                                           np, first.as<uint32_t>(), pinfo, sub);
+            QS3_LAUNCHED();
+        }
+        for (int s = s0; s < s0 + ns; ++s) {
+            B.secs[s].pinfo = B.d_pinfo.as<uint2>() + (uint64_t)s * np;
+            B.secs[s].sub = sub;
+            base += entries(s);
+        }
     }
     QS3_CUDA(cudaDeviceSynchronize());       // the scratch is released on return
     return QS3_OK;

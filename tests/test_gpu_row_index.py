@@ -1,0 +1,49 @@
+"""The index over the rows of many sectors, built for a few sectors at a time:
+products that look their targets up in it against the representative table,
+and a basis whose index has more than 2^32 entries."""
+from __future__ import annotations
+
+import math
+
+import numpy as np
+import pytest
+
+import qs3_inputs as qi
+from tests.gpu_common import lib_basis, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def _randn(torch, d, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.view_as_complex(torch.randn(d, 2, generator=g, device="cuda", dtype=torch.float32))
+
+
+# 12x12, N_down = 4, all 144 momenta: about 11.6 million entries, several groups;
+# 9x5 and 6x4 stay within one (two-site and one-site prefixes)
+@pytest.mark.parametrize("dims,nd", [((12, 12), 4), ((9, 5), 4), ((6, 4), 2)])
+def test_index_equals_table(dims, nd):
+    torch = torch_cuda()
+    spec = qi.hypercubic(dims, True, 1.0, 0.8)
+    b = lib_basis(spec, nd, qi.all_k(spec.L))
+    phi = _randn(torch, b.total_dim, 3)
+    assert b.rep_table()
+    ref = b.hphi(phi)
+    assert not b.rep_table(0)
+    assert torch.equal(b.hphi(phi), ref)
+
+
+def test_index_beyond_32_bit_entries():
+    torch = torch_cuda()
+    spec = qi.hypercubic((41, 41), True)
+    n, ks = spec.n_sites, qi.all_k(spec.L)
+    assert math.comb(n, 3) // 2 + 2 * n * (n * (n - 1) // 2) >= 2 ** 32
+    b = lib_basis(spec, 3, ks)
+    assert b.total_dim == math.comb(n, 3) and not b.rep_table()
+    phi = _randn(torch, b.total_dim, 4)
+    psi = b.hphi(phi)
+    for s in (0, 1, 1000, n - 1):
+        one = lib_basis(spec, 3, [ks[s]])           # found by its origin forms
+        lo, hi = b.offsets[s], b.offsets[s + 1]
+        np.testing.assert_array_equal(b.ranks(s)[0], one.ranks()[0])
+        assert torch.equal(one.hphi(phi[lo:hi].contiguous()), psi[lo:hi])
