@@ -105,9 +105,12 @@ typedef struct qs3_basis_s *qs3_basis_t;
  * U(1) symmetry"; Alg. 5-6 for k-sectors).  K = NULL: one U(1)-only sector of
  * dimension C(N, N_down) (n_sectors must be 1).  Otherwise K holds 3 ints per
  * sector (K_alpha in [0, L_alpha)); the representative lists are enumerated,
- * filtered and sorted on the device.  Errors: INVALID_ARG, OVERFLOW,
+ * filtered and sorted on the device.  Errors: INVALID_ARG, OVERFLOW (a momentum
+ * sector of 2^32 rows or more, found before anything is allocated, among others),
  * SYMMETRY (bonds or h not invariant under the translations, K out of range),
- * OOM, CUDA.  The handle owns its device memory until qs3_basis_destroy. */
+ * OOM, CUDA.  The handle owns its device memory until qs3_basis_destroy; scratch
+ * of the library's calls comes from a pool per device, of which a destroyed basis
+ * leaves at most 32 MB unused. */
 int qs3_basis_create(const qs3_lattice *lat, int32_t n_down, int32_t n_sectors, const int32_t *K,
                      qs3_basis_t *out);
 int qs3_basis_destroy(qs3_basis_t b);

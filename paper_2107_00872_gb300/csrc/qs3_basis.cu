@@ -83,8 +83,8 @@ static cudaMemPool_t device_pool(bool create) {
     }
     return g_pool[dev];
 }
-void pool_trim() {
-    if (cudaMemPool_t mp = device_pool(false)) cudaMemPoolTrimTo(mp, 0);
+void pool_trim(size_t keep) {
+    if (cudaMemPool_t mp = device_pool(false)) cudaMemPoolTrimTo(mp, keep);
     cudaGetLastError();
 }
 
@@ -116,7 +116,7 @@ int DevBuf::alloc(size_t bytes) {
     if (e == cudaErrorMemoryAllocation) {
         // what the pool holds unused goes back first
         cudaGetLastError();
-        pool_trim();
+        pool_trim(0);
         e = cudaMalloc(&p, bytes);
     }
     if (e != cudaSuccess) {
@@ -139,7 +139,7 @@ int DevBuf::alloc(size_t bytes, cudaStream_t stream) {
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         cudaStreamSynchronize(stream);
-        pool_trim();
+        pool_trim(0);
         e = cudaMallocFromPoolAsync(&p, bytes, mp, stream);
     }
     if (e != cudaSuccess) {
@@ -538,8 +538,7 @@ static int build_sectors_nd(Basis &B, DevBuf &keep_reps, DevBuf &keep_stab, uint
     for (uint64_t d : B.dims) total += d;
     QS3_TRY(B.d_sigma.alloc(total * 8));
     QS3_TRY(B.d_stab.alloc(total));
-    DevBuf dK, pos, tmp;
-    QS3_TRY(dK.upload(B.K.data(), B.K.size() * sizeof(int), (cudaStream_t)0));
+    DevBuf pos, tmp;
     const int grp = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)S, (1ull << 27) / std::max<uint64_t>(n, 1)));
     QS3_TRY(pos.alloc(((uint64_t)grp * n + 1) * 4, (cudaStream_t)0));
     size_t tb = 0;
@@ -554,7 +553,7 @@ static int build_sectors_nd(Basis &B, DevBuf &keep_reps, DevBuf &keep_stab, uint
         const int g1 = (int)std::max<uint64_t>(1, std::min<uint64_t>((n + NTHREADS - 1) / NTHREADS, 4096));
         QS3_CUDA(cudaMemsetAsync(pos.as<uint32_t>() + cnt, 0, 4));
         k_members<ND><<<g1, NTHREADS, smem>>>(B.lv, keep_reps.as<uint64_t>(), keep_stab.as<uint8_t>(), n, ns,
-                                              dK.as<int>() + 3 * s0, pos.as<uint32_t>());
+                                              B.K_d + 3 * s0, pos.as<uint32_t>());
         QS3_LAUNCHED();
         size_t t2 = tb;
         QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, t2, pos.as<uint32_t>(), pos.as<uint32_t>(), (int64_t)(cnt + 1)));
@@ -572,6 +571,12 @@ static int build_sectors_nd(Basis &B, DevBuf &keep_reps, DevBuf &keep_stab, uint
     return QS3_OK;
 }
 
+// the sectors' views as the kernels read them
+static int put_secs(Basis &B) {
+    QS3_CUDA(cudaMemcpy(B.d_secs.p, B.secs.data(), B.secs.size() * sizeof(SecView), cudaMemcpyHostToDevice));
+    return QS3_OK;
+}
+
 // the index over every sector's rows (SecView::pinfo, sub), as many sectors at
 // a time as INDEX_GROUP entries hold and at least one: the offsets in a group
 // are 32 bits (a sector of fewer than 2^32 rows has at most 2^31 + 2 np
@@ -585,7 +590,7 @@ static int build_index_nd(Basis &B) {
     const int pre2 = ND >= 2 && (uint64_t)S * np2 / 8 <= B.total ? 1 : 0;
     const uint32_t np = pre2 ? (uint32_t)np2 : (uint32_t)B.N;
     for (auto &v : B.secs) v.pre2 = pre2;
-    QS3_CUDA(cudaMemcpy(B.d_secs.p, B.secs.data(), B.secs.size() * sizeof(SecView), cudaMemcpyHostToDevice));
+    QS3_TRY(put_secs(B));
     // at most rows / 2 + 1 buckets and the end per prefix
     auto entries = [&](int s) { return B.dims[s] / 2 + 2 * (uint64_t)np; };
     std::vector<int> g0{0};
@@ -611,7 +616,7 @@ static int build_index_nd(Basis &B) {
     QS3_TRY(tmp.alloc(tb, (cudaStream_t)0));
     const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8;
     QS3_CUDA(cudaFuncSetAttribute(k_bucket_fill<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-    const uint64_t *bin = B.d_binom.as<uint64_t>();
+    const uint64_t *bin = B.lv.binom;
     uint64_t base = 0;
     for (size_t g = 0; g + 1 < g0.size(); ++g) {
         const int s0 = g0[g], ns = g0[g + 1] - s0;
@@ -631,7 +636,7 @@ static int build_index_nd(Basis &B) {
         QS3_LAUNCHED();
         const int t0 = B.tile0[s0], t1 = B.tile0[s0 + ns];
         if (t1 > t0) {
-            k_bucket_fill<ND><<<std::min(t1 - t0, 8192), NTHREADS, smem>>>(B.lv, secs, B.d_tile0.as<int>() + s0, ns, t0, t1,
+            k_bucket_fill<ND><<<std::min(t1 - t0, 8192), NTHREADS, smem>>>(B.lv, secs, B.tile0_d + s0, ns, t0, t1,
                                                                            np, first.as<uint32_t>(), pinfo, sub);
             QS3_LAUNCHED();
         }
@@ -641,7 +646,6 @@ static int build_index_nd(Basis &B) {
             base += entries(s);
         }
     }
-    QS3_CUDA(cudaDeviceSynchronize());       // the scratch is released on return
     return QS3_OK;
 }
 
@@ -779,12 +783,10 @@ static int build_table_nd(Basis &B, size_t max_bytes, DevBuf &reps, DevBuf &stab
     int grid2 = (int)std::min<uint64_t>((tot2 + 255) / 256, (uint64_t)nsm * 8);
     k_orbit_rows<<<std::max(grid2, 1), 256>>>(B.d_secs.as<SecView>(), B.S, reps.as<uint64_t>(), n, t2.as<int32_t>());
     QS3_LAUNCHED();
-    QS3_CUDA(cudaDeviceSynchronize());
     DevBuf phd;
     const uint64_t nph = (uint64_t)B.S * B.N;
     QS3_TRY(phd.alloc(nph * sizeof(int4)));
-    k_phase_digits<<<(int)std::min<uint64_t>((nph + 255) / 256, 4096), 256>>>(B.d_ph64.as<double2>(), nph,
-                                                                              phd.as<int4>());
+    k_phase_digits<<<(int)std::min<uint64_t>((nph + 255) / 256, 4096), 256>>>(B.secs[0].ph64, nph, phd.as<int4>());
     QS3_LAUNCHED();
     QS3_CUDA(cudaDeviceSynchronize());
     B.d_orb = std::move(orb);
@@ -796,8 +798,7 @@ static int build_table_nd(Basis &B, size_t max_bytes, DevBuf &reps, DevBuf &stab
     B.lv.orb = B.d_orb.as<uint32_t>();
     B.lv.n_orb = (uint32_t)n;
     for (int s = 0; s < B.S; ++s) B.secs[s].t2 = B.d_t2.as<int32_t>() + (size_t)s * n;
-    QS3_TRY(B.d_secs.upload(B.secs.data(), B.secs.size() * sizeof(SecView)));
-    return QS3_OK;
+    return put_secs(B);                      // after the wait: no kernel reads the old views
 }
 
 static int build_rep_table(Basis &B, size_t max_bytes, DevBuf &reps, DevBuf &stab, uint64_t n) {
@@ -858,6 +859,17 @@ __global__ void k_roots(int G, double2 *__restrict__ w) {
 }
 
 // ---------------------------------------------------------------- host side
+
+// tables laid out one after another, each on a 16-byte boundary
+struct TableImage {
+    std::vector<unsigned char> data;
+    template <class T> size_t add(const std::vector<T> &v) {
+        const size_t at = data.size();
+        data.resize((at + v.size() * sizeof(T) + 15) & ~(size_t)15);
+        if (!v.empty()) std::memcpy(data.data() + at, v.data(), v.size() * sizeof(T));
+        return at;
+    }
+};
 
 static bool binom_table(int N, int rows, std::vector<uint64_t> &t, uint64_t *cnd, int nd) {
     // t[m * (N+1) + c] = C(c, m), saturated at UINT64_MAX; returns false if C(N, nd) >= 2^63
@@ -995,7 +1007,11 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     B.total = B.offs[nsec];
     B.ntiles = B.tile0[nsec];
     B.nchunks = B.chunk0[nsec];
-    QS3_TRY(B.d_binom.upload(B.binom.data(), B.binom.size() * 8));
+
+    // every table of the lattice and of the sectors in one device image (one
+    // allocation and one copy: a basis of few rows is bound by those)
+    TableImage img;
+    const size_t o_binom = img.add(B.binom);
 
     // adjacency (CSR, both directions), diagonal constants
     std::vector<int> deg(N + 1, 0);
@@ -1020,34 +1036,24 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     }
     if (B.has_h)
         for (int i = 0; i < N; ++i) { u[i] += B.h[i]; c0 -= 0.5 * B.h[i]; }
-    QS3_TRY(B.d_adj_ptr.upload(deg.data(), deg.size() * 4));
-    QS3_TRY(B.d_adj_nbr.upload(nbr.data(), nbr.size() * 4));
-    QS3_TRY(B.d_adj_jxy.upload(ajxy.data(), ajxy.size() * 8));
-    QS3_TRY(B.d_adj_jz.upload(ajz.data(), ajz.size() * 8));
-    QS3_TRY(B.d_adj_jxy_f.upload(ajxyf.data(), ajxyf.size() * 4));
-    QS3_TRY(B.d_u.upload(u.data(), u.size() * 8));
-    std::vector<float> uf(u.begin(), u.end()), ajzf(ajz.begin(), ajz.end());
-    QS3_TRY(B.d_u_f.upload(uf.data(), uf.size() * 4));
-    QS3_TRY(B.d_adj_jz_f.upload(ajzf.data(), ajzf.size() * 4));
-    {
-        // double-float remainders (v - fl32(v), rounded to fp32)
-        auto rem = [](const std::vector<double> &v, const std::vector<float> &h) {
-            std::vector<float> r(v.size());
-            for (size_t i = 0; i < v.size(); ++i) r[i] = (float)(v[i] - (double)h[i]);
-            return r;
-        };
-        const std::vector<float> a = rem(ajxy, ajxyf), bu = rem(u, uf), cz = rem(ajz, ajzf);
-        QS3_TRY(B.d_adj_jxy_lo.upload(a.data(), a.size() * 4));
-        QS3_TRY(B.d_u_lo.upload(bu.data(), bu.size() * 4));
-        QS3_TRY(B.d_adj_jz_lo.upload(cz.data(), cz.size() * 4));
-    }
+    const std::vector<float> uf(u.begin(), u.end()), ajzf(ajz.begin(), ajz.end());
+    // double-float remainders (v - fl32(v), rounded to fp32)
+    auto rem = [](const std::vector<double> &v, const std::vector<float> &h) {
+        std::vector<float> r(v.size());
+        for (size_t i = 0; i < v.size(); ++i) r[i] = (float)(v[i] - (double)h[i]);
+        return r;
+    };
+    const size_t o_ptr = img.add(deg), o_nbr = img.add(nbr), o_jxy = img.add(ajxy), o_jz = img.add(ajz),
+                 o_jxyf = img.add(ajxyf), o_u = img.add(u), o_uf = img.add(uf), o_jzf = img.add(ajzf),
+                 o_jxyl = img.add(rem(ajxy, ajxyf)), o_ul = img.add(rem(u, uf)), o_jzl = img.add(rem(ajz, ajzf));
     // fixed-width copies of the adjacency for the U(1) kernels
     const int padw = K ? 0 : B.max_degree <= 2 ? 2 : B.max_degree <= 4 ? 4 : (B.max_degree <= 6 ? 6 : 0);
     const size_t np = (size_t)N * padw;
+    size_t o_pad = 0;
     if (padw) {
         // int4 | fp64 J^z | int2 | int2 transposed | fp32 J^z | fp32 J^z transposed
-        std::vector<unsigned char> img(np * (16 + 8 + 8 + 8 + 4 + 4), 0);
-        int4 *p64 = (int4 *)img.data();
+        std::vector<int4> pad(np * 3);
+        int4 *p64 = pad.data();
         double *z64 = (double *)(p64 + np);
         int2 *p32 = (int2 *)(z64 + np), *t32 = p32 + np;
         float *z32 = (float *)(t32 + np), *zt = z32 + np;
@@ -1067,7 +1073,7 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
                 p32[a] = t32[t] = make_int2(j, bf);
                 z32[a] = zt[t] = real ? ajzf[q] : 0.f;
             }
-        QS3_TRY(B.d_pad.upload(img.data(), img.size()));
+        o_pad = img.add(pad);
     }
     std::vector<uint32_t> xyz(N);
     for (int r = 0; r < N; ++r) {
@@ -1077,7 +1083,7 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
         // coordinates are only used with a translation group (x, y < 2048, z < 1024)
         xyz[r] = haveL ? ((uint32_t)x | ((uint32_t)y << 11) | ((uint32_t)z << 22)) : 0u;
     }
-    QS3_TRY(B.d_xyz.upload(xyz.data(), xyz.size() * 4));
+    const size_t o_xyz = img.add(xyz), o_tile = img.add(B.tile0), o_chunk = img.add(B.chunk0), o_K = img.add(B.K);
 
     int bits = 1;
     while ((1 << bits) < N) ++bits;
@@ -1089,33 +1095,12 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     L.has_k = B.has_k;
     L.key_bits = (bits * nd <= 64) ? bits : 0;
     L.mask_ok = L.key_bits > 0 && L.L[0] <= 32 && L.L[1] <= 32 && L.L[2] <= 32;
-    L.binom = B.d_binom.as<uint64_t>();
-    L.adj_ptr = B.d_adj_ptr.as<int>();
-    L.adj_nbr = B.d_adj_nbr.as<int>();
-    L.adj_jxy = B.d_adj_jxy.as<double>();
-    L.adj_jz = B.d_adj_jz.as<double>();
-    L.adj_jxy_f = B.d_adj_jxy_f.as<float>();
-    L.u = B.d_u.as<double>();
     L.c0 = c0;
     L.c0f = (float)c0;
-    L.u_f = B.d_u_f.as<float>();
-    L.adj_jz_f = B.d_adj_jz_f.as<float>();
-    L.adj_jxy_lo = B.d_adj_jxy_lo.as<float>();
-    L.u_lo = B.d_u_lo.as<float>();
-    L.adj_jz_lo = B.d_adj_jz_lo.as<float>();
     L.c0lo = (float)(c0 - (double)(float)c0);
-    L.xyz = B.d_xyz.as<uint32_t>();
     L.nsub = B.nsub;
     L.ncell = B.ncell;
     L.pad_w = padw;
-    if (padw) {
-        L.adj_pad64 = B.d_pad.as<int4>();
-        L.adj_jz_pad64 = (const double *)(L.adj_pad64 + np);
-        L.adj_pad = (const int2 *)(L.adj_jz_pad64 + np);
-        L.adjt = L.adj_pad + np;
-        L.adj_jz_pad = (const float *)(L.adjt + np);
-        L.adjt_jz = L.adj_jz_pad + np;
-    }
     L.jh_uniform = 0.0;
     if (nb > 0) {
         bool same = true;
@@ -1124,21 +1109,20 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     }
 
     L.diag_uniform = 0;
+    size_t o_pair = 0, npair = 0;
     if (B.has_k && nb > 0 && nd > 0) {
         bool same = true;
         for (int i = 1; i < N; ++i) same &= u[i] == u[0];
         for (size_t q = 1; q < ajz.size(); ++q) same &= ajz[q] == ajz[0];
         if (same) {
-            const size_t np = (size_t)nd * B.max_degree + 1;
-            std::vector<double> img(np + (np + 1) / 2, 0.0);
-            float *pf = (float *)(img.data() + np);
-            for (size_t n = 1; n < np; ++n) {
-                img[n] = img[n - 1] + ajz[0];
+            npair = (size_t)nd * B.max_degree + 1;
+            std::vector<double> sums(npair + (npair + 1) / 2, 0.0);
+            float *pf = (float *)(sums.data() + npair);
+            for (size_t n = 1; n < npair; ++n) {
+                sums[n] = sums[n - 1] + ajz[0];
                 pf[n] = pf[n - 1] + ajzf[0];
             }
-            QS3_TRY(B.d_pair.upload(img.data(), img.size() * 8));
-            L.pair_sum = B.d_pair.as<double>();
-            L.pair_sum_f = (const float *)(L.pair_sum + np);
+            o_pair = img.add(sums);
             L.e_row = c0;
             L.e_row_f = L.c0f;
             for (int k = 0; k < nd; ++k) {
@@ -1147,6 +1131,39 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
             }
             L.diag_uniform = 1;
         }
+    }
+
+    QS3_TRY(B.d_tab.upload(img.data.data(), img.data.size()));
+    {
+        const unsigned char *t = B.d_tab.as<unsigned char>();
+        L.binom = (const uint64_t *)(t + o_binom);
+        L.adj_ptr = (const int *)(t + o_ptr);
+        L.adj_nbr = (const int *)(t + o_nbr);
+        L.adj_jxy = (const double *)(t + o_jxy);
+        L.adj_jz = (const double *)(t + o_jz);
+        L.adj_jxy_f = (const float *)(t + o_jxyf);
+        L.u = (const double *)(t + o_u);
+        L.u_f = (const float *)(t + o_uf);
+        L.adj_jz_f = (const float *)(t + o_jzf);
+        L.adj_jxy_lo = (const float *)(t + o_jxyl);
+        L.u_lo = (const float *)(t + o_ul);
+        L.adj_jz_lo = (const float *)(t + o_jzl);
+        L.xyz = (const uint32_t *)(t + o_xyz);
+        if (padw) {
+            L.adj_pad64 = (const int4 *)(t + o_pad);
+            L.adj_jz_pad64 = (const double *)(L.adj_pad64 + np);
+            L.adj_pad = (const int2 *)(L.adj_jz_pad64 + np);
+            L.adjt = L.adj_pad + np;
+            L.adj_jz_pad = (const float *)(L.adjt + np);
+            L.adjt_jz = L.adj_jz_pad + np;
+        }
+        if (npair) {
+            L.pair_sum = (const double *)(t + o_pair);
+            L.pair_sum_f = (const float *)(L.pair_sum + npair);
+        }
+        B.tile0_d = (const int *)(t + o_tile);
+        B.chunk0_d = (const int *)(t + o_chunk);
+        B.K_d = (const int *)(t + o_K);
     }
 
     // sectors
@@ -1161,20 +1178,19 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
         QS3_TRY(build_sectors(B, oreps, ostab, n_orb));
     }
     B.secs.resize(nsec);
+    const size_t nph = B.has_k ? (size_t)nsec * N : 0;
     if (B.has_k) {
-        QS3_TRY(B.d_ph64.alloc((size_t)nsec * N * sizeof(double2)));
-        QS3_TRY(B.d_ph32.alloc((size_t)nsec * N * sizeof(float2)));
-        QS3_TRY(B.d_phdf.alloc((size_t)nsec * N * sizeof(float4)));
-        QS3_TRY(B.d_secs.upload(B.K.data(), B.K.size() * sizeof(int)));     // momenta for the table kernel
+        // double-float and complex128 phases, the roots of unity, complex64 phases
+        QS3_TRY(B.d_ph.alloc(nph * (sizeof(float4) + sizeof(double2) + sizeof(float2)) + (size_t)B.ncell * sizeof(double2)));
+        float4 *pdf = B.d_ph.as<float4>();
+        double2 *p64 = (double2 *)(pdf + nph), *rt = p64 + nph;
         const int tot = nsec * N;
-        k_phase_tables<<<(tot + 255) / 256, 256>>>(nsec, N, B.ncell, B.L[0], B.L[1], B.L[2], B.d_secs.as<int>(),
-                                                   B.d_ph64.as<double2>(), B.d_ph32.as<float2>(),
-                                                   B.d_phdf.as<float4>());
+        k_phase_tables<<<(tot + 255) / 256, 256>>>(nsec, N, B.ncell, B.L[0], B.L[1], B.L[2], B.K_d, p64,
+                                                   (float2 *)(rt + B.ncell), pdf);
         QS3_LAUNCHED();
-        QS3_TRY(B.d_roots.alloc((size_t)B.ncell * sizeof(double2)));
-        k_roots<<<(B.ncell + 255) / 256, 256>>>(B.ncell, B.d_roots.as<double2>());
+        k_roots<<<(B.ncell + 255) / 256, 256>>>(B.ncell, rt);
         QS3_LAUNCHED();
-        QS3_CUDA(cudaDeviceSynchronize());
+        B.roots_d = rt;
     }
     for (int s = 0; s < nsec; ++s) {
         SecView &v = B.secs[s];
@@ -1184,17 +1200,13 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
         v.off = B.offs[s];
         for (int a = 0; a < 3; ++a) v.K[a] = B.K[3 * s + a];
         v.tile0 = B.tile0[s];
-        v.ph64 = B.has_k ? B.d_ph64.as<double2>() + (size_t)s * N : nullptr;
-        v.ph32 = B.has_k ? B.d_ph32.as<float2>() + (size_t)s * N : nullptr;
-        v.phdf = B.has_k ? B.d_phdf.as<float4>() + (size_t)s * N : nullptr;
+        v.phdf = B.has_k ? B.d_ph.as<float4>() + (size_t)s * N : nullptr;
+        v.ph64 = B.has_k ? (const double2 *)(B.d_ph.as<float4>() + nph) + (size_t)s * N : nullptr;
+        v.ph32 = B.has_k ? (const float2 *)(B.roots_d + B.ncell) + (size_t)s * N : nullptr;
     }
-    QS3_TRY(B.d_secs.upload(B.secs.data(), B.secs.size() * sizeof(SecView)));
-    QS3_TRY(B.d_tile0.upload(B.tile0.data(), B.tile0.size() * 4));
-    QS3_TRY(B.d_chunk0.upload(B.chunk0.data(), B.chunk0.size() * 4));
-    if (B.has_k && nd > 0) {
-        QS3_TRY(build_index(B));
-        QS3_CUDA(cudaMemcpy(B.d_secs.p, B.secs.data(), B.secs.size() * sizeof(SecView), cudaMemcpyHostToDevice));
-    }
+    QS3_TRY(B.d_secs.alloc(B.secs.size() * sizeof(SecView)));
+    if (B.has_k && nd > 0) QS3_TRY(build_index(B));
+    QS3_TRY(put_secs(B));
     B.smem_bytes = row_kernel_smem(B, 0);
     if (B.smem_bytes > 200 * 1024)
         return set_err(QS3_ERR_OVERFLOW, "lattice tables need %zu bytes of shared memory", B.smem_bytes);
@@ -1218,6 +1230,7 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
             }
         }
     }
+    QS3_CUDA(cudaDeviceSynchronize());       // the handle may be used on any stream
     return QS3_OK;
 }
 
@@ -1245,7 +1258,7 @@ int qs3_basis_create(const qs3_lattice *lat, int32_t n_down, int32_t n_sectors, 
 int qs3_basis_destroy(qs3_basis_t b) {
     clear_err();
     delete b;
-    pool_trim();
+    pool_trim(POOL_IDLE_BYTES);
     return QS3_OK;
 }
 

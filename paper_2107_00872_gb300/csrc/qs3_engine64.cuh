@@ -1675,7 +1675,7 @@ struct Engine64 {
     VT *hin(int) { return hinb.as<VT>(); }
     VT *wv() { return wbuf.as<VT>(); }
     const SecView *secs() { return B.d_secs.as<SecView>(); }
-    const int *c0() { return B.d_chunk0.as<int>(); }
+    const int *c0() { return B.chunk0_d; }
     int *act() { return active.as<int>(); }
     int grid() const { return std::max(B.nchunks, 1); }
 

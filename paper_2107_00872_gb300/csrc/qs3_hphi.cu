@@ -726,7 +726,7 @@ static int tune_grid(KF kern, Basis &B, int occ, cudaStream_t st, const VT *phi,
                      int &best_bps, size_t smem = (size_t)-1) {
     if (smem == (size_t)-1) smem = B.smem_bytes;
     return tune_blocks(B, occ, st, best_bps, [&](int grid) {
-        kern<<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(), B.S, B.ntiles, phi, psi,
+        kern<<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d, B.S, B.ntiles, phi, psi,
                                            active);
     });
 }
@@ -748,7 +748,7 @@ static int hphi_ndt(Basis &B, const void *phi, void *psi, cudaStream_t st, const
         }
     }
     if (bps > 0) grid = std::max(1, std::min(B.ntiles, std::min(bps, occ) * num_sms()));
-    k_hphi<ND, VT, KS, TB><<<grid, NTHREADS, B.smem_bytes, st>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(),
+    k_hphi<ND, VT, KS, TB><<<grid, NTHREADS, B.smem_bytes, st>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d,
                                                                   B.S, B.ntiles, (const VT *)phi, (VT *)psi, active);
     QS3_LAUNCHED();
     return QS3_OK;
@@ -784,7 +784,7 @@ static int hphix_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
     QS3_TRY(launch_rows(k_hphi_x<ND>, B, B.smem_bytes, cache, &grid, &occ));
     if (B.ntiles == 0) return QS3_OK;
     auto launch = [&](int g) {
-        k_hphi_x<ND><<<g, NTHREADS, B.smem_bytes, st>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(), B.S,
+        k_hphi_x<ND><<<g, NTHREADS, B.smem_bytes, st>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d, B.S,
                                                          B.ntiles, hv, psi, active);
     };
     int &bps = B.tune_hphix;
@@ -977,7 +977,7 @@ static int count_nd(Basis &B, unsigned long long *d_out) {
     static std::atomic<unsigned long long> cache{0};
     int grid = 1;
     QS3_TRY(launch_rows(k_count<ND, KS>, B, B.smem_bytes, cache, &grid));
-    k_count<ND, KS><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(), B.S,
+    k_count<ND, KS><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d, B.S,
                                                        B.ntiles, d_out);
     QS3_LAUNCHED();
     return QS3_OK;

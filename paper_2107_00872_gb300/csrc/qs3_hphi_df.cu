@@ -238,7 +238,7 @@ static int hphi_df_ndt(Basis &B, const float4 *phi, const int *dx, uint64_t ld, 
     if (B.ntiles == 0) return QS3_OK;
     auto launch = [&](int g) {
         k_hphi_df<ND, TB, ODF, DEGB><<<g, NTHREADS, B.smem_bytes, st>>>(B.lv, B.d_secs.as<SecView>(),
-                                                                          B.d_tile0.as<int>(), B.S, B.ntiles, phi, psi,
+                                                                          B.tile0_d, B.S, B.ntiles, phi, psi,
                                                                           active, dx, ld);
     };
     int &bps = B.tune_hphi[QS3_C128DF];

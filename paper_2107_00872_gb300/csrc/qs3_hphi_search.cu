@@ -423,7 +423,7 @@ static int build_forms_nd(Basis &B) {
     const size_t smem = (size_t)(B.nd + 3) * (B.N + 1) * 8 + (size_t)B.N * 4;
     QS3_CUDA(cudaFuncSetAttribute(k_forms<ND, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
     QS3_CUDA(cudaFuncSetAttribute(k_form_fill<NO, KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-    const uint64_t *bin = B.d_binom.as<uint64_t>();
+    const uint64_t *bin = B.lv.binom;
     const int gp = (int)((np + 256) / 256);
     uint64_t base = 0;
     for (int s = 0; s < S; ++s) {
@@ -499,7 +499,7 @@ static int forms_run(Basis &B, const void *phi, void *psi, cudaStream_t st, cons
     const size_t smem = forms_smem(B);
     QS3_TRY(launch_rows(k_hphi_f<ND, VT, KT>, B, smem, cache, &grid, &occ));
     if (B.ntiles == 0) return QS3_OK;
-    k_hphi_f<ND, VT, KT><<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(), B.S, B.ntiles,
+    k_hphi_f<ND, VT, KT><<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d, B.S, B.ntiles,
                                                        (const VT *)phi, (VT *)psi, active, (unsigned)forms_off(B));
     QS3_LAUNCHED();
     if (B.tune_hphi[dt] == 0) B.tune_hphi[dt] = occ;             // always the whole occupancy

@@ -82,7 +82,12 @@ struct DevBuf {
 };
 
 constexpr size_t POOL_KEEP_BYTES = (size_t)512 << 20, POOL_MAX_BYTES = (size_t)256 << 20;
-void pool_trim();                                 // returns the current device's unused pool memory
+// the current device's unused pool memory goes back, but for `keep` bytes.
+// A basis that is destroyed leaves POOL_IDLE_BYTES, the pool's smallest unit:
+// with none left, the next small basis mapped it again and its destruction
+// unmapped it, 0.1 ms of the 0.83 ms that one sector of 5x5 took.
+void pool_trim(size_t keep);
+constexpr size_t POOL_IDLE_BYTES = (size_t)32 << 20;
 
 // ------------------------------------------------------- device-side views
 
@@ -190,16 +195,13 @@ struct Basis {
     std::vector<uint64_t> binom;            // host copy of the binomial rows 0 .. nd + 2
     bool has_h = false;
     // device data
-    DevBuf d_binom, d_adj_ptr, d_adj_nbr, d_adj_jxy, d_adj_jz, d_adj_jxy_f, d_u, d_xyz;
-    DevBuf d_u_f, d_adj_jz_f;
-    DevBuf d_pair;                          // LatView::pair_sum, pair_sum_f
-    DevBuf d_adj_jxy_lo, d_u_lo, d_adj_jz_lo;
-    DevBuf d_pad;                           // fixed-width adjacency (LatView::adj_pad ...)
+    DevBuf d_tab;                           // the tables that lv points to, tile0, chunk0 and K
+    const int *tile0_d = nullptr, *chunk0_d = nullptr, *K_d = nullptr;
     DevBuf d_sigma, d_stab, d_pinfo, d_sub;  // every sector's lists, one after another
     DevBuf d_orec, d_finfo, d_fsub;          // origin forms and their index (without a representative table)
-    DevBuf d_ph64, d_ph32, d_phdf;          // S x N per-site phase tables (k-sectors)
-    DevBuf d_roots;                         // e^{-2 pi i n / ncell}, n < ncell (k-sectors)
-    DevBuf d_secs, d_tile0, d_chunk0;
+    DevBuf d_ph;                            // S x N per-site phase tables and the roots (k-sectors)
+    const double2 *roots_d = nullptr;       // e^{-2 pi i n / ncell}, n < ncell
+    DevBuf d_secs;
     LatView lv{};
     std::vector<SecView> secs;
     uint64_t nnz = 0;                       // structural non-zeros (count_nnz), total and per sector

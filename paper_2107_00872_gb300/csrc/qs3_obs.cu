@@ -794,7 +794,7 @@ static int sq_t_nd(Basis &S, int ss, Basis &Dd, int sd, const int *Q, const doub
     reduced_q(S, Q, q);
     QS3_CUDA(cudaFuncSetAttribute(k_sq_t<ND, UP>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
     k_sq_t<ND, UP><<<grid_for(Dd.dims[sd]), NTHREADS, root_smem_bytes(S), st>>>(
-        S.lv, S.secs[ss], Dd.secs[sd], q[0], q[1], q[2], S.d_roots.as<double2>(), 1.0 / std::sqrt((double)S.N), phi, psi);
+        S.lv, S.secs[ss], Dd.secs[sd], q[0], q[1], q[2], S.roots_d, 1.0 / std::sqrt((double)S.N), phi, psi);
     QS3_LAUNCHED();
     return QS3_OK;
 }

@@ -1227,7 +1227,7 @@ struct Engine {
         if constexpr (DF) return rvec(rw); else return svec(x + 1);
     }
     const SecView *secs() { return B.d_secs.as<SecView>(); }
-    const int *c0() { return B.d_chunk0.as<int>(); }
+    const int *c0() { return B.chunk0_d; }
     int *act() { return active.as<int>(); }
 
     int init(int cap_, int nscratch) {
@@ -1712,10 +1712,10 @@ static int residuals(Basis &B, const WT *v, const std::vector<double> &e, cudaSt
     const qs3_dtype dt = sizeof(WT) == 8 ? QS3_F64 : QS3_C128;
     QS3_TRY(hphi_launch(B, dt, v, t.p, st, nullptr));
     k_resid<WT><<<B.nchunks, NTHREADS, 0, st>>>(t.as<WT>(), v, de.as<double>(), B.d_secs.as<SecView>(),
-                                                B.d_chunk0.as<int>(), B.S, part.as<double2>());
+                                                B.chunk0_d, B.S, part.as<double2>());
     QS3_LAUNCHED();
     dim3 g(1, B.S);
-    k_reduce<<<g, NTHREADS, 0, st>>>(part.as<double2>(), 1, B.d_chunk0.as<int>(), nullptr, out.as<double2>(), 1);
+    k_reduce<<<g, NTHREADS, 0, st>>>(part.as<double2>(), 1, B.chunk0_d, nullptr, out.as<double2>(), 1);
     QS3_LAUNCHED();
     std::vector<double2> h(B.S);
     QS3_CUDA(cudaMemcpyAsync(h.data(), out.p, B.S * sizeof(double2), cudaMemcpyDeviceToHost, st));
@@ -2578,7 +2578,7 @@ static int trl_entry(Basis &B, const qs3_solve_opts &o, double *evals, void *eve
             if (B.nchunks) {
                 k_combine<V64, V64><<<B.nchunks, NTHREADS, NK * sizeof(double), st>>>(
                     sum.as<V64>(), B.total, kept.as<V64>(), B.total, NK, 1, dC.as<double>(), NK,
-                    B.d_secs.as<SecView>(), B.d_chunk0.as<int>(), B.S, dm.as<int>());
+                    B.d_secs.as<SecView>(), B.chunk0_d, B.S, dm.as<int>());
                 QS3_LAUNCHED();
             }
             QS3_CUDA(cudaStreamSynchronize(st));
@@ -2675,7 +2675,7 @@ static int gs_dots_run(Basis &B, int m, const VT *V, uint64_t ldv, const VT *w, 
         QS3_LAUNCHED();
     }
     const SecView *secs = B.d_secs.as<SecView>();
-    const int *c0 = B.d_chunk0.as<int>();
+    const int *c0 = B.chunk0_d;
     if (mode == 0) {
         using G = typename DigT<VT>::T;
         QS3_TRY(dgt.alloc((uint64_t)m * D * sizeof(VT) + 16, st));      // k_dotb reads up to 16 bytes past
@@ -2749,7 +2749,7 @@ int hphi_x_binary64(Basis &B, const void *phi, void *psi, cudaStream_t st) {
                                       "amplitude");
     DevBuf hd;
     QS3_TRY(hd.alloc(B.total * sizeof(int4), st));
-    k_image<<<B.nchunks, XT, 0, st>>>((const double2 *)phi, hd.as<int4>(), B.d_secs.as<SecView>(), B.d_chunk0.as<int>(), B.S);
+    k_image<<<B.nchunks, XT, 0, st>>>((const double2 *)phi, hd.as<int4>(), B.d_secs.as<SecView>(), B.chunk0_d, B.S);
     QS3_LAUNCHED();
     return hphi_x_launch(B, {hd.as<int4>(), (const double2 *)phi, nullptr, B.total, nullptr}, psi, st, nullptr);
 }

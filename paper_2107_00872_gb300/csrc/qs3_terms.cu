@@ -203,12 +203,12 @@ static int build_terms_nd(Basis &B, size_t max_bytes) {
     const int grid = grid_tiles(B, 8);
     if (tb) {
         QS3_CUDA(cudaFuncSetAttribute(k_terms<ND, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-        k_terms<ND, true, false><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(),
+        k_terms<ND, true, false><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d,
                                                                    B.S, B.ntiles, cnt.as<uint64_t>(), nullptr,
                                                                    nullptr, nullptr, nullptr);
     } else {
         QS3_CUDA(cudaFuncSetAttribute(k_terms<ND, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-        k_terms<ND, false, false><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(),
+        k_terms<ND, false, false><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d,
                                                                     B.S, B.ntiles, cnt.as<uint64_t>(), nullptr,
                                                                     nullptr, nullptr, nullptr);
     }
@@ -232,13 +232,13 @@ static int build_terms_nd(Basis &B, size_t max_bytes) {
     QS3_TRY(dg.alloc(B.total * 8));
     if (tb) {
         QS3_CUDA(cudaFuncSetAttribute(k_terms<ND, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-        k_terms<ND, true, true><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(),
+        k_terms<ND, true, true><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d,
                                                                   B.S, B.ntiles, nullptr, rptr.as<uint64_t>(),
                                                                   col.as<uint32_t>(), code.as<uint32_t>(),
                                                                   dg.as<double>());
     } else {
         QS3_CUDA(cudaFuncSetAttribute(k_terms<ND, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
-        k_terms<ND, false, true><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(),
+        k_terms<ND, false, true><<<grid, NTHREADS, B.smem_bytes>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d,
                                                                    B.S, B.ntiles, nullptr, rptr.as<uint64_t>(),
                                                                    col.as<uint32_t>(), code.as<uint32_t>(),
                                                                    dg.as<double>());
@@ -286,7 +286,7 @@ static int hphi_st_vt(Basis &B, const void *phi, void *psi, cudaStream_t st, con
     using CT = typename VTr<VT>::C;
     const size_t smem = 16 * 18 + (size_t)B.N * sizeof(CT);
     const int grid = grid_tiles(B, 8);
-    k_hphi_st<VT><<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.d_tile0.as<int>(), B.S, B.ntiles,
+    k_hphi_st<VT><<<grid, NTHREADS, smem, st>>>(B.lv, B.d_secs.as<SecView>(), B.tile0_d, B.S, B.ntiles,
                                                  B.d_trp.as<uint64_t>(), B.d_tcol.as<uint32_t>(),
                                                  B.d_tcode.as<uint32_t>(), B.d_tdiag.as<double>(), (const VT *)phi,
                                                  (VT *)psi, active);

@@ -47,3 +47,27 @@ def test_index_beyond_32_bit_entries():
         lo, hi = b.offsets[s], b.offsets[s + 1]
         np.testing.assert_array_equal(b.ranks(s)[0], one.ranks()[0])
         assert torch.equal(one.hphi(phi[lo:hi].contiguous()), psi[lo:hi])
+
+
+# a basis of few rows is bound by the allocations of its creation, whose number
+# does not depend on the sectors; what the destruction leaves of the scratch is
+# mapped no more by the next creation
+@pytest.mark.parametrize("nk", [1, 4, 25])
+def test_creation_allocates_little(nk):
+    torch = torch_cuda()
+    import paper_2107_00872_gb300 as qs3
+    spec = qi.square(5)
+
+    def create():
+        qs3.inject_alloc_failure(1000)
+        try:
+            b = lib_basis(spec, 3, qi.all_k(spec.L)[:nk])
+        finally:
+            left = qs3.inject_alloc_failure(-1)
+        b.close()
+        return 1000 - left
+
+    create()
+    free = torch.cuda.mem_get_info()[0]
+    assert create() <= 24
+    assert abs(torch.cuda.mem_get_info()[0] - free) <= 4 << 20
