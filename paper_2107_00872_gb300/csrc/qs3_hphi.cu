@@ -251,15 +251,28 @@ __global__ void __launch_bounds__(NTHREADS, (KS && TB && sizeof(VT) == 16) ? 4 :
 // binary64 as in k_hphi.  The row sum is rounded to binary64 once, then
 // psi = J/2 sum + diag phi in binary64.
 // the row sum of the integer H Phi: (re, im) 2^(r - 1075), r the group
-// exponent of the largest term so far; a term T 2^(em - 1075) (|T| <= 2^54)
-// is rounded to nearest onto that grid, and a term of a coarser group first
-// moves the sum to its grid.  With at most 48 terms |sum| < 2^60, and the
-// error is at most (terms + moves) / 2 units of the final grid, i.e. about
-// 2^-54 of the largest term each (binary64 accumulation: 2^-53 of each
-// partial sum).
+// exponent of the largest term so far; a term T 2^(em - 1075) (|T| <= 2^53.5:
+// a phase of modulus 2^52 times two components of at most 2^53, over 2^52) is
+// rounded to nearest onto that grid, and a term of a coarser group first moves
+// the sum to its grid.  ROW_TERMS of them stay below 2^62, which rshift_round
+// needs and one more term keeps; rows of more terms are folded into binary64
+// (RowAcc::fold) every ROW_TERMS.  The error of a fold is at most (terms +
+// moves) / 2 units of its grid, i.e. about 2^-54 of the largest term each
+// (binary64 accumulation: 2^-53 of each partial sum).
+constexpr int ROW_TERMS = 256;
 struct RowAcc {
     long long re = 0, im = 0;
     int r = -100000;
+    __device__ __forceinline__ double2 value() const {
+        return make_double2(i128_ldexp(re, r - 1075), i128_ldexp(im, r - 1075));
+    }
+    __device__ __forceinline__ void fold(double2 &sum) {
+        const double2 v = value();
+        sum.x += v.x;
+        sum.y += v.y;
+        re = im = 0;
+        r = -100000;
+    }
 };
 // x 2^-d rounded to nearest, 0 <= d <= 63, |x| < 2^62 (0 for d = 63)
 __device__ __forceinline__ long long rshift_round(long long x, int d) {
@@ -333,6 +346,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
         const double rs = snorm[9 + st_row];
         double e = L.c0, dd = 0.0;
         RowAcc acc;
+        int nt = 0;
         double2 acc64 = make_double2(0.0, 0.0);
 #pragma unroll 1
         for (int m = 0; m < ND; ++m) {
@@ -378,6 +392,10 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
                     hd_unpack(__ldg(hv.hd + sv.off + idx), f1, f0, em);
                     long long tr, ti;
                     term_x(pd[u], f1, f0, tr, ti);
+                    if (++nt > ROW_TERMS) {
+                        acc.fold(acc64);
+                        nt = 1;
+                    }
                     row_add(acc, tr, ti, em);
                 } else {
                     double2 p = sv.ph64[u];
@@ -388,9 +406,9 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_x(LatView L, const SecView
                 }
             }
         }
-        double2 acch;
-        acch.x = i128_ldexp(acc.re, acc.r - 1075) + acc64.x;
-        acch.y = i128_ldexp(acc.im, acc.r - 1075) + acc64.y;
+        double2 acch = acc.value();
+        acch.x += acc64.x;
+        acch.y += acc64.y;
         const double ed = e + 0.5 * dd;
         double2 out;
         out.x = fma(ed, x0.x, juni * acch.x);
@@ -550,9 +568,9 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_o(LatView L, const SecView
                 }
             }
         }
-        double2 acch;
-        acch.x = i128_ldexp(acc.re, acc.r - 1075) + acc64.x;
-        acch.y = i128_ldexp(acc.im, acc.r - 1075) + acc64.y;
+        double2 acch = acc.value();
+        acch.x += acc64.x;
+        acch.y += acc64.y;
         const double2 x0 = hv.value(off + (uint32_t)row);
         double2 out;
         out.x = fma(ed, x0.x, juni * acch.x);
@@ -826,6 +844,7 @@ static int orb_group(const Basis &B, bool fp32) {
 // shared memory of the 32-bit binomials and the hop lists; 0: too many hops per row
 static size_t orb_smem(const Basis &B, int maxh) {
     const size_t lists = 18 * 8 + (size_t)maxh * NTHREADS * 5;
+    static_assert(MAX_DYN_SMEM / (NTHREADS * 5) < ROW_TERMS, "k_hphi_o sums a list without folds");
     if ((size_t)(B.nd + 3) * (B.N + 1) * 8 + lists > (size_t)MAX_DYN_SMEM) return 0;
     return (((size_t)(B.nd + 1) * (B.N + 1) + 1) & ~(size_t)1) * 4 + lists;
 }

@@ -1,0 +1,40 @@
+"""Lattices of many equal bonds (all pairs of a ring or a square): the products
+whose rows have hundreds of terms, against the binary64 FMA product.
+
+A row's sum of n terms, each of modulus at most |phi|max J / 2: the FMA product
+rounds every partial sum, the integer product each term on the grid of the
+largest and each fold once, so they differ by at most n^2 2^-52 of that modulus;
+the diagonal adds a few roundings of its own weight, (n + N_down^2 + N^2) |J^z|.
+"""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import qs3_inputs as qi
+from tests.gpu_common import lib_basis, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def _all_pairs(dims):
+    n = int(np.prod(dims))
+    bi, bj = np.triu_indices(n, 1)
+    L = tuple(dims) + (1,) * (3 - len(dims))
+    return qi.LatticeSpec(n, bi.astype(np.int32), bj.astype(np.int32), np.ones(len(bi)), np.full(len(bi), 0.01), None,
+                          L, "all pairs")
+
+
+def _tol(n_sites, nd, phi):
+    n = nd * (n_sites - nd)
+    return (n * n * 0.5 + 8 * 0.01 * n_sites ** 2) * 2.0 ** -52 * float(phi.abs().max())
+
+
+# rows of equal elements just below a power of two: every one of the 1028 terms
+# is the largest that the grid holds, at k = 0 in step
+@pytest.mark.parametrize("n,nd", [(261, 4), (100, 5)])
+def test_integer_product_of_many_terms(n, nd):
+    torch = torch_cuda()
+    b = lib_basis(_all_pairs((n,)), nd, [(0, 0, 0)])
+    phi = torch.full((b.total_dim,), (1 - 2.0 ** -53) * (1 - 1j), dtype=torch.complex128, device="cuda")
+    assert float((b.hphi(phi, integer=True) - b.hphi(phi)).abs().max()) <= _tol(n, nd, phi)
