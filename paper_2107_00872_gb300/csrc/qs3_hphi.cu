@@ -842,18 +842,17 @@ static int orb_group(const Basis &B, bool fp32) {
     return best;
 }
 // shared memory of the 32-bit binomials and the hop lists; 0: too many hops per row
-static size_t orb_smem(const Basis &B, int maxh) {
-    const size_t lists = 18 * 8 + (size_t)maxh * NTHREADS * 5;
+static size_t orb_smem(const Basis &B) {
+    const size_t maxh = (size_t)std::max(1, B.nd * B.max_degree);
+    const size_t smem = (((size_t)(B.nd + 1) * (B.N + 1) + 1) & ~(size_t)1) * 4 + 18 * 8 + maxh * NTHREADS * 5;
     static_assert(MAX_DYN_SMEM / (NTHREADS * 5) < ROW_TERMS, "k_hphi_o sums a list without folds");
-    if ((size_t)(B.nd + 3) * (B.N + 1) * 8 + lists > (size_t)MAX_DYN_SMEM) return 0;
-    return (((size_t)(B.nd + 1) * (B.N + 1) + 1) & ~(size_t)1) * 4 + lists;
+    return smem <= (size_t)MAX_DYN_SMEM ? smem : 0;
 }
 
 template <int ND>
 static int hphio_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, const int *active) {
     const int maxh = std::max(1, B.nd * B.max_degree);
-    const size_t smem = orb_smem(B, maxh);
-    if (!smem) return set_err(QS3_ERR_OVERFLOW, "hop lists of %d entries per row", maxh);
+    const size_t smem = orb_smem(B);
     static std::atomic<int> attr{0};
     if (attr.load(std::memory_order_acquire) == 0) {
         QS3_CUDA(cudaFuncSetAttribute(k_hphi_o<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM));
@@ -875,15 +874,14 @@ static int hphio_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
 // k_hphi_of: 10x10, N_down = 4 31 / 27 us a call, 12x12 53 / 37, 10x10x10, N_down =
 // 3 71 / 54; c64 21 / 18, 23 / 21, 44 / 38)
 static bool hphi_of_ok(const Basis &B) {
-    return B.has_k && B.lv.orb && B.d_oreps.p && B.lv.jh_uniform != 0.0 &&
-           orb_smem(B, std::max(1, B.nd * B.max_degree)) > 0;
+    return B.has_k && B.lv.orb && B.d_oreps.p && B.lv.jh_uniform != 0.0 && orb_smem(B) > 0;
 }
 
 template <int ND, typename VT>
 static int hphiof_nd(Basis &B, const void *phi, void *psi, cudaStream_t st, const int *active, int dt) {
     static std::atomic<unsigned long long> cache{0};
     const int maxh = std::max(1, B.nd * B.max_degree);
-    const size_t smem = orb_smem(B, maxh);
+    const size_t smem = orb_smem(B);
     int grid = 1, occ = 1;
     QS3_TRY(launch_rows(k_hphi_of<ND, VT>, B, smem, cache, &grid, &occ));
     if (B.tune_hphi[dt] == 0) B.tune_hphi[dt] = occ;             // the grid covers all orbits: nothing to tune
@@ -920,10 +918,10 @@ int hphi_x_launch(Basis &B, const HxVec &hv, void *psi, cudaStream_t st, const i
     if (!hphi_x_ok(B)) return set_err(QS3_ERR_STATE, "the integer H Phi needs a k-sector basis with the "
                                                      "representative table and one hop amplitude");
     double2 *o = (double2 *)psi;
-    // the orbit-batched kernel, except one sector with hop lists that do not
-    // fit (one sector, k_hphi_x / k_hphi_o: 10x10, N_down = 4 36 / 34 us a call,
-    // 10x10x10, N_down = 3 61 / 51, 12x12 40 / 40)
-    if (B.d_oreps.p && (B.S >= 2 || orb_smem(B, std::max(1, B.nd * B.max_degree)) > 0)) {
+    // the orbit-batched kernel, unless its hop lists do not fit (one sector,
+    // k_hphi_x / k_hphi_o: 10x10, N_down = 4 36 / 34 us a call, 10x10x10, N_down =
+    // 3 61 / 51, 12x12 40 / 40)
+    if (B.d_oreps.p && orb_smem(B) > 0) {
         switch (B.nd) {
             case 1: return hphio_nd<1>(B, hv, o, st, active);
             case 2: return hphio_nd<2>(B, hv, o, st, active);

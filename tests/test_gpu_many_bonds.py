@@ -38,3 +38,22 @@ def test_integer_product_of_many_terms(n, nd):
     b = lib_basis(_all_pairs((n,)), nd, [(0, 0, 0)])
     phi = torch.full((b.total_dim,), (1 - 2.0 ** -53) * (1 - 1j), dtype=torch.complex128, device="cuda")
     assert float((b.hphi(phi, integer=True) - b.hphi(phi)).abs().max()) <= _tol(n, nd, phi)
+
+
+# hop lists beyond shared memory (192 hops a row) over several sectors: the
+# product, and the binary64 solve that uses it, against binary64 FMAs
+def test_many_bonds_over_several_sectors():
+    torch = torch_cuda()
+    import paper_2107_00872_gb300 as qs3
+    spec, nd = _all_pairs((7, 7)), 4
+    b = lib_basis(spec, nd, [(0, 0, 0), (1, 3, 0)])
+    g = torch.Generator(device="cuda").manual_seed(2)
+    phi = torch.view_as_complex(torch.randn(b.total_dim, 2, generator=g, device="cuda", dtype=torch.float64))
+    got = b.hphi(phi, integer=True)
+    assert float((got - b.hphi(phi)).abs().max()) <= _tol(49, nd, phi)
+    e = []
+    for strict in (False, True):
+        ev, _, info = b.lanczos(qs3.SolveOpts(n_max=60, eps=1e-13, res_tol=1e-10, strict64=strict))
+        assert info["status"] == "QS3_OK"
+        e.append(ev[:, 0])
+    assert np.max(np.abs(e[0] - e[1])) <= 1e-11 * np.max(np.abs(e[1]))
