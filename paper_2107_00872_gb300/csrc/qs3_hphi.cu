@@ -870,11 +870,34 @@ static int hphio_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
 }
 
 // the orbit-batched FMA kernel serves bases with the representative table and
-// one hop amplitude whose hop lists fit, of one sector too (c128 k_hphi /
-// k_hphi_of: 10x10, N_down = 4 31 / 27 us a call, 12x12 53 / 37, 10x10x10, N_down =
-// 3 71 / 54; c64 21 / 18, 23 / 21, 44 / 38)
-static bool hphi_of_ok(const Basis &B) {
-    return B.has_k && B.lv.orb && B.d_oreps.p && B.lv.jh_uniform != 0.0 && orb_smem(B) > 0;
+// one hop amplitude, of one sector too (c128 k_hphi / k_hphi_of: 10x10, N_down =
+// 4 31 / 27 us a call, 12x12 53 / 37, 10x10x10, N_down = 3 71 / 54; c64 21 / 18, 23
+// / 21, 44 / 38), as far as its hop lists leave room: k_hphi lists nothing and
+// keeps its blocks and its L1 cache.  With three or four blocks resident that
+// leave the L1 60 KB (complex64: 80 KB) it is the faster one everywhere.  Fewer
+// blocks, or less L1, cost more than the sharing of few sectors gives, so the
+// rows must fill the chip (one block on every SM) as many times as `waves` says.
+// Square lattices of degree 8 to 48, k_hphi / k_hphi_of in us, c128 and c64:
+//   four blocks, little L1: 10x10, N_down = 3, 14 bonds a site, one sector 41 / 41
+//     and 27 / 31, 100 sectors 137 / 102 and 49 / 45; 14x14, 196 sectors 863 / 412
+//     and 246 / 147
+//   three blocks, 60 KB: 12x12, N_down = 4, 12 bonds, 1 sector 128 / 104 and 47 /
+//     68, 4 392 / 242 and 156 / 129
+//   two blocks: 10x10, N_down = 4, 20 bonds, 2 sectors 160 / 150 and 68 / 109, 16
+//     832 / 565 and 309 / 293; 14x14, N_down = 3, 28 bonds, 4 sectors 76 / 90 and
+//     51 / 65, 196 1671 / 1059 and 484 / 424
+//   one block: 10x10, N_down = 4, 36 bonds, 4 sectors 437 / 509 and 210 / 297, 8
+//     815 / 755 and 327 / 483, 100 8901 / 6480 and 2966 / 3111
+static bool hphi_of_ok(const Basis &B, bool fp32) {
+    if (!(B.has_k && B.lv.orb && B.d_oreps.p && B.lv.jh_uniform != 0.0) || !orb_smem(B)) return false;
+    const size_t per = orb_smem(B) / 1024 + 2;                   // KB; 1 KB of each block is the system's
+    const size_t blocks = std::min<size_t>(4, 228 / per), used = blocks * per;
+    uint64_t waves;
+    if (blocks >= 3) waves = fp32 ? (used > 196 ? 16 : used > 176 ? 4 : 0) : (used > 196 ? 1 : 0);
+    else if (blocks == 2) waves = fp32 ? (used > 196 ? 24 : 16) : (used > 196 ? 4 : 0);
+    else if (!fp32) waves = 8;
+    else return false;
+    return B.n_orb * (uint64_t)B.S >= waves * NTHREADS * (uint64_t)num_sms();
 }
 
 template <int ND, typename VT>
@@ -971,9 +994,9 @@ int hphi_launch(Basis &B, qs3_dtype dt, const void *phi, void *psi, cudaStream_t
         if (B.stored_terms && (dt == QS3_C64 || dt == QS3_C128)) return hphi_stored_launch(B, dt, phi, psi, st, active);
         if (!B.lv.orb && B.d_orec.p && (dt == QS3_C64 || dt == QS3_C128))
             return hphi_forms_launch(B, dt, phi, psi, st, active);
-        if (hphi_of_ok(B)) {
+        if ((dt == QS3_C64 || dt == QS3_C128) && hphi_of_ok(B, dt == QS3_C64)) {
             if (dt == QS3_C64) return hphiof_vt<float2>(B, phi, psi, st, active, dt);
-            if (dt == QS3_C128) return hphiof_vt<double2>(B, phi, psi, st, active, dt);
+            return hphiof_vt<double2>(B, phi, psi, st, active, dt);
         }
         if (dt == QS3_C64) return hphi_vt<float2, true>(B, phi, psi, st, active);
         if (dt == QS3_C128) return hphi_vt<double2, true>(B, phi, psi, st, active);

@@ -57,3 +57,31 @@ def test_many_bonds_over_several_sectors():
         assert info["status"] == "QS3_OK"
         e.append(ev[:, 0])
     assert np.max(np.abs(e[0] - e[1])) <= 1e-11 * np.max(np.abs(e[1]))
+
+
+# lattices of equal bonds to the nearest `degree` sites, where the number of
+# sectors decides between the orbit-batched kernel and the row kernel: all
+# momenta at once against one at a time, the same bits
+@pytest.mark.parametrize("dims,nd,degree", [((8, 8), 4, 10), ((8, 8), 4, 14), ((8, 8), 4, 20), ((8, 8), 4, 28),
+                                            ((5, 5), 6, 8), ((10, 10), 3, 18)])
+def test_batched_equals_single_with_many_bonds(dims, nd, degree):
+    torch = torch_cuda()
+    lx, ly = dims
+    near = sorted((min(x, lx - x) ** 2 + min(y, ly - y) ** 2, x, y) for x in range(lx) for y in range(ly))[1:]
+    d = set()
+    for _, x, y in near:
+        if len(d) < degree and (-x % lx, -y % ly) != (x, y):
+            d |= {(x, y), (-x % lx, -y % ly)}
+    pairs = [(r, (r % lx + x) % lx + lx * ((r // lx + y) % ly)) for r in range(lx * ly) for x, y in sorted(d)]
+    b = np.array([p for p in pairs if p[0] < p[1]], np.int32)
+    spec = qi.LatticeSpec(lx * ly, b[:, 0].copy(), b[:, 1].copy(), np.full(len(b), 0.7), np.full(len(b), 0.9), None,
+                          (lx, ly, 1), "near")
+    ks = qi.all_k(spec.L)
+    both = lib_basis(spec, nd, ks)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    x = torch.view_as_complex(torch.randn(both.total_dim, 2, generator=g, device="cuda", dtype=torch.float64))
+    for phi in (x, x.to(torch.complex64)):
+        psi = both.hphi(phi)
+        for s in (0, 1, len(ks) // 2):
+            lo, hi = both.offsets[s], both.offsets[s + 1]
+            assert torch.equal(lib_basis(spec, nd, [ks[s]]).hphi(phi[lo:hi].contiguous()), psi[lo:hi])
