@@ -153,7 +153,7 @@ int qs3_basis_rep_table(qs3_basis_t b, int32_t mode, int32_t *active);
 /* Autotuned launch choices of a basis (no counterpart in the paper).  On the
  * first direct (not stream-captured) use, the library times:
  *   - H Phi of the per-row k-sector kernels (no uniform J^xy with the table,
- *     the search, C128DF, hop lists beyond shared memory) with 1..4 fewer
+ *     the search, C128DF, many bonds a site) with 1..4 fewer
  *     resident 256-row blocks per SM than the occupancy limit (the persistent
  *     grid, i.e. rows in flight per SM), per vector dtype, and keeps the
  *     fastest.  The orbit-batched, origin-form and U(1) kernels take their

@@ -849,6 +849,19 @@ static size_t orb_smem(const Basis &B) {
     return smem <= (size_t)MAX_DYN_SMEM ? smem : 0;
 }
 
+// what the orbit-batched kernels have of an SM: resident blocks, and the shared
+// memory that those use in KB
+struct OrbRoom {
+    size_t blocks, used;
+};
+static OrbRoom orb_room(const Basis &B) {
+    const size_t per = orb_smem(B) / 1024 + 2;                   // 1 KB of each block is the system's
+    const size_t blocks = std::min<size_t>(4, 228 / per);
+    return {blocks, blocks * per};
+}
+// rows that put one block on every SM
+static uint64_t one_wave() { return NTHREADS * (uint64_t)num_sms(); }
+
 template <int ND>
 static int hphio_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, const int *active) {
     const int maxh = std::max(1, B.nd * B.max_degree);
@@ -890,14 +903,13 @@ static int hphio_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
 //     815 / 755 and 327 / 483, 100 8901 / 6480 and 2966 / 3111
 static bool hphi_of_ok(const Basis &B, bool fp32) {
     if (!(B.has_k && B.lv.orb && B.d_oreps.p && B.lv.jh_uniform != 0.0) || !orb_smem(B)) return false;
-    const size_t per = orb_smem(B) / 1024 + 2;                   // KB; 1 KB of each block is the system's
-    const size_t blocks = std::min<size_t>(4, 228 / per), used = blocks * per;
+    const auto [blocks, used] = orb_room(B);
     uint64_t waves;
     if (blocks >= 3) waves = fp32 ? (used > 196 ? 16 : used > 176 ? 4 : 0) : (used > 196 ? 1 : 0);
     else if (blocks == 2) waves = fp32 ? (used > 196 ? 24 : 16) : (used > 196 ? 4 : 0);
     else if (!fp32) waves = 8;
     else return false;
-    return B.n_orb * (uint64_t)B.S >= waves * NTHREADS * (uint64_t)num_sms();
+    return B.n_orb * (uint64_t)B.S >= waves * one_wave();
 }
 
 template <int ND, typename VT>
@@ -937,14 +949,26 @@ bool hphi_x_ok(const Basis &B) {
     return B.has_k && B.lv.orb && B.lv.jh_uniform != 0.0 && B.nd > 0 && !B.stored_terms && B.total > 0;
 }
 
+// the orbit-batched kernel, unless its hop lists do not fit.  One sector shares
+// no lists: there k_hphi_o gains what unranking and the lookups in flight give,
+// as long as four blocks are resident or the orbits are one wave of fewer, and
+// the L1 keeps 60 KB; a last wave that is nearly empty, or fewer warps over
+// several waves, cost more.  k_hphi_x / k_hphi_o in us a call: 4 bonds a site,
+// 10x10, N_down = 4 37 / 33, 12x12 40 / 39, 10x10x10, N_down = 3 61 / 51; 12
+// bonds (three blocks) 10x10 75 / 69, 12x12 86 / 108; 20 bonds (two) 116 / 115, 133
+// / 191; 28 bonds (one) 161 / 190, 183 / 347, 8x8 130 / 121
+static bool hphi_o_ok(const Basis &B) {
+    if (!B.d_oreps.p || !orb_smem(B)) return false;
+    if (B.S >= 2) return true;
+    const auto [blocks, used] = orb_room(B);
+    return used <= 196 && (blocks == 4 || B.n_orb <= blocks * one_wave());
+}
+
 int hphi_x_launch(Basis &B, const HxVec &hv, void *psi, cudaStream_t st, const int *active) {
     if (!hphi_x_ok(B)) return set_err(QS3_ERR_STATE, "the integer H Phi needs a k-sector basis with the "
                                                      "representative table and one hop amplitude");
     double2 *o = (double2 *)psi;
-    // the orbit-batched kernel, unless its hop lists do not fit (one sector,
-    // k_hphi_x / k_hphi_o: 10x10, N_down = 4 36 / 34 us a call, 10x10x10, N_down =
-    // 3 61 / 51, 12x12 40 / 40)
-    if (B.d_oreps.p && orb_smem(B) > 0) {
+    if (hphi_o_ok(B)) {
         switch (B.nd) {
             case 1: return hphio_nd<1>(B, hv, o, st, active);
             case 2: return hphio_nd<2>(B, hv, o, st, active);

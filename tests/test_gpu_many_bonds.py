@@ -85,3 +85,8 @@ def test_batched_equals_single_with_many_bonds(dims, nd, degree):
         for s in (0, 1, len(ks) // 2):
             lo, hi = both.offsets[s], both.offsets[s + 1]
             assert torch.equal(lib_basis(spec, nd, [ks[s]]).hphi(phi[lo:hi].contiguous()), psi[lo:hi])
+    psi = both.hphi(x, integer=True)
+    for s in (0, 1, len(ks) // 2):
+        lo, hi = both.offsets[s], both.offsets[s + 1]
+        one = lib_basis(spec, nd, [ks[s]]).hphi(x[lo:hi].contiguous(), integer=True)
+        assert float((one - psi[lo:hi]).abs().max()) <= 2 * _tol(lx * ly, nd, x)
