@@ -1046,6 +1046,7 @@ static int basis_create(const qs3_lattice *lat, int nd, int nsec, const int32_t 
     const size_t o_ptr = img.add(deg), o_nbr = img.add(nbr), o_jxy = img.add(ajxy), o_jz = img.add(ajz),
                  o_jxyf = img.add(ajxyf), o_u = img.add(u), o_uf = img.add(uf), o_jzf = img.add(ajzf),
                  o_jxyl = img.add(rem(ajxy, ajxyf)), o_ul = img.add(rem(u, uf)), o_jzl = img.add(rem(ajz, ajzf));
+    for (int b = 0; b < nb; ++b) B.n_long_bonds += std::abs(B.bi[b] - B.bj[b]) * SEG_REACH > N;
     // fixed-width copies of the adjacency for the U(1) kernels
     const int padw = K ? 0 : B.max_degree <= 2 ? 2 : B.max_degree <= 4 ? 4 : (B.max_degree <= 6 ? 6 : 0);
     const size_t np = (size_t)N * padw;

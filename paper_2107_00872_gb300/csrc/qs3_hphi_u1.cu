@@ -24,6 +24,7 @@
 // operations per row, 1083 us at the measured rate of the pipe.
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "qs3_hphi_common.cuh"
 
@@ -82,16 +83,29 @@ struct SegHop {
 
 constexpr int SEG_WARPS = NTHREADS / 32;
 constexpr int SEG_RUN = 4;                 // consecutive segments per run of a warp
-// k_hphi_u1s from a mean segment of so many rows on.  Open L x L lattices,
-// N_down = 3, fp32, k_hphi_u1s / k_hphi_u1n: L = 24 (mean 191) 394 / 410 us, 26
-// 624 / 659, 28 979 / 1032, 30 1447 / 1607, 32 (mean 341) 2100 / 2385 us; at L =
-// 20 (mean 133) 173 / 148, and with few segments (N_down = 2, N = 1024) 81 / 17,
-// so N_down = 3 only (more spins with such segments exceed 32-bit ranks).  Four
-// resident blocks (3: 2269, 5: 2237), runs of four segments (1: 2208, 8: 2368).
-// fp64 stays with k_hphi_u1n: the fp64 pipe bounds both (1176 / 1068 us at L = 24).
-constexpr int SEG_MIN = 160;
-// rows per lane and pass
-template <typename VT> constexpr int seg_r() { return sizeof(VT) == 4 ? 4 : 2; }
+// k_hphi_u1s serves real fp32 vectors of N_down = 3 (more spins with such segments
+// exceed 32-bit ranks; with N_down = 2 they are few: N = 1024 81 us, k_hphi_u1n 17)
+// on lattices of up to four neighbours, where the segments are long and few
+// hops of c_1 leave them: a lane whose hop passes c_2 sends its whole pass the
+// slow way.  N >= SEG_N (four neighbours: SEG_N_4) where every bond is at most N
+// / SEG_REACH sites long, or, with one longer bond, the closing one of a ring, N
+// >= SEG_N_RING.  k_hphi_u1n / k_hphi_u1s in us:
+//   rings 483 172 / 212, 600 321 / 325, 700 500 / 451, 1000 1550 / 1204, 1600 6680 /
+//   4377; open chains 483 170 / 156, 1000 1539 / 1019; open L x L 22 (bonds of N /
+//   22) 246 / 270, 23 315 / 324, 24 401 / 399, 28 1006 / 971, 32 2233 / 2106, 40 9025 /
+//   8232; open 8 x 64 281 / 270, 2 x 300 435 / 336; bonds of N / 8 (open 128 x 8) 2528 /
+//   2799; periodic 32 x 32 2293 / 2676, 3 x 200 446 / 466; six neighbours, open
+//   10x10x10 3046 / 3532; complex64, open 32 x 32 3295 / 3817 and ring 1000 1503 / 1870
+// Four resident blocks (open 32 x 32, 3: 2269, 5: 2237), runs of four segments (1:
+// 2208, 8: 2368).  fp64 stays with k_hphi_u1n: the fp64 pipe bounds both (1176 / 1068
+// us at L = 24).
+constexpr int SEG_N = 483, SEG_N_4 = 512, SEG_N_RING = 700;      // SEG_REACH: qs3_internal.cuh
+static bool segments_pay(const Basis &B) {
+    if (B.nd != 3 || B.lv.pad_w > 4) return false;
+    if (B.n_long_bonds) return B.n_long_bonds == 1 && B.N >= SEG_N_RING;
+    return B.N >= (B.lv.pad_w == 2 ? SEG_N : SEG_N_4);
+}
+constexpr int SEG_ROWS = 4;                // rows per lane and pass
 
 // a segment as its rows see it
 template <int ND> struct Seg {
@@ -102,11 +116,12 @@ template <int ND> struct Seg {
 };
 
 // the rows c_1 = x + lane + 32 r of a segment (FULL: all of them exist)
-template <int ND, typename VT, int DEG, int RL, bool FULL>
+template <int ND, int DEG, int RL, bool FULL>
 __device__ __forceinline__ void seg_rows(const U1View &L, const uint32_t *sC, const SegHop *hop,
                                          const Seg<ND> &sg, int x, int lane,
-                                         const VT *__restrict__ phi, VT *__restrict__ psi) {
-    using R = typename VTr<VT>::R;
+                                         const float *__restrict__ phi, float *__restrict__ psi) {
+    using VT = float;
+    using R = float;
     using CT = typename VTr<VT>::C;
     constexpr int NU = ND - 1;
     const int np1 = L.np1, N = L.N, len = sg.U[0];
@@ -203,11 +218,11 @@ __device__ __forceinline__ void seg_rows(const U1View &L, const uint32_t *sC, co
         }
 }
 
-template <int ND, typename VT, int DEG>
-__global__ void __launch_bounds__(NTHREADS, 4) k_hphi_u1s(U1View L, uint32_t nseg, const VT *__restrict__ phi,
-                                                          VT *__restrict__ psi, const int *__restrict__ active) {
+template <int ND, int DEG>
+__global__ void __launch_bounds__(NTHREADS, 4) k_hphi_u1s(U1View L, uint32_t nseg, const float *__restrict__ phi,
+                                                          float *__restrict__ psi, const int *__restrict__ active) {
     using R = float;
-    constexpr int NU = ND - 1, H = NU * DEG, RL = seg_r<VT>();
+    constexpr int NU = ND - 1, H = NU * DEG, RL = SEG_ROWS;
     static_assert(H <= 32, "one lane per hop of the upper spins");
     extern __shared__ __align__(16) unsigned char smem[];
     if (active && !active[0]) return;
@@ -278,8 +293,8 @@ __global__ void __launch_bounds__(NTHREADS, 4) k_hphi_u1s(U1View L, uint32_t nse
             }
             __syncwarp();
             int x = 0;
-            for (; x + 32 * RL <= len; x += 32 * RL) seg_rows<ND, VT, DEG, RL, true>(L, sC, hop, sg, x, lane, phi, psi);
-            for (; x < len; x += 32) seg_rows<ND, VT, DEG, 1, false>(L, sC, hop, sg, x, lane, phi, psi);
+            for (; x + 32 * RL <= len; x += 32 * RL) seg_rows<ND, DEG, RL, true>(L, sC, hop, sg, x, lane, phi, psi);
+            for (; x < len; x += 32) seg_rows<ND, DEG, 1, false>(L, sC, hop, sg, x, lane, phi, psi);
             if (++s >= s1) break;
             // the next list of upper spins
             bool carry = true;
@@ -370,6 +385,19 @@ __global__ void __launch_bounds__(NTHREADS, sizeof(typename VTr<VT>::R) == 8 || 
     }
 }
 
+// k_hphi_u1n in fp64: the rank and the load of every padded entry, and in
+// complex128 at N_down = 4 the registers of four spins' hops, cost what its 32-bit
+// ranks gain over the general kernel unless most entries are real.  General kernel
+// / k_hphi_u1n in us, fp64 and complex128 of N_down = 3: open 32 x 32 8968 / 5889 and
+// 12043 / 10440, ring 1000 4898 / 3493 and 6200 / 5735; five sixths real (open 6x6x6)
+// 96 / 95 and 143 / 148; three quarters (open 2 x 300) 1159 / 1132 and 1748 / 1983,
+// (honeycomb of 288 sites) 139 / 149 and 205 / 207.  N_down = 4: open 12 x 12 783 /
+// 771 and 1204 / 1287, ring 150 592 / 577 and 874 / 914, open 4x4x4 (three quarters) 51
+// / 53 and 72 / 80
+static bool fp64_rows_pay(const Basis &B, bool cplx) {
+    return (!cplx || B.nd <= 3) && 2.0 * B.nb >= (cplx ? 0.85 : 0.8) * (double)B.N * B.lv.pad_w;
+}
+
 // the persistent launch of kern (grid in blocks, at most `blocks`): every
 // resident block in fp32, four per SM in fp64, or as many as qs3_basis_tuning
 // imposed.  fp64, open lattices, blocks per SM 3 / 4 / 5 / 6: L = 16 110 / 108 /
@@ -396,26 +424,24 @@ static int u1_run(KF kern, Basis &B, size_t smem, uint64_t blocks, uint32_t n, c
 
 template <int ND, typename VT>
 static int u1_nd(Basis &B, const void *phi, void *psi, cudaStream_t st, const int *active, int dt, bool *done) {
-    using R = typename VTr<VT>::R;
     const int N = B.N;
-    (void)N;
     const VT *p = (const VT *)phi;
     VT *q = (VT *)psi;
     const size_t tab = (size_t)(ND + 1) * (N + 1) * sizeof(uint32_t);
-    if constexpr (ND == 3 && sizeof(R) == 4) {
-        // long segments, and many of them
+    if constexpr (ND == 3 && std::is_same_v<VT, float>) {
         const int dw = B.lv.pad_w;
         const size_t smem = tab + (size_t)SEG_WARPS * (ND - 1) * dw * sizeof(SegHop);
-        if (N - ND + 1 >= SEG_MIN * ND && smem <= (size_t)MAX_DYN_SMEM) {
+        if (segments_pay(B) && smem <= (size_t)MAX_DYN_SMEM) {
             const uint64_t nseg = (uint64_t)N * (N - 1) / 2;                 // C(N, N_down - 1)
             const uint64_t blocks = (nseg + SEG_WARPS * SEG_RUN - 1) / (SEG_WARPS * SEG_RUN);
             *done = true;
-            static std::atomic<unsigned long long> s2{0}, s4{0}, s6{0};
-            if (dw == 2) return u1_run(k_hphi_u1s<ND, VT, 2>, B, smem, blocks, (uint32_t)nseg, p, q, st, active, dt, s2);
-            if (dw == 4) return u1_run(k_hphi_u1s<ND, VT, 4>, B, smem, blocks, (uint32_t)nseg, p, q, st, active, dt, s4);
-            return u1_run(k_hphi_u1s<ND, VT, 6>, B, smem, blocks, (uint32_t)nseg, p, q, st, active, dt, s6);
+            static std::atomic<unsigned long long> s2{0}, s4{0};
+            if (dw == 2) return u1_run(k_hphi_u1s<ND, 2>, B, smem, blocks, (uint32_t)nseg, p, q, st, active, dt, s2);
+            return u1_run(k_hphi_u1s<ND, 4>, B, smem, blocks, (uint32_t)nseg, p, q, st, active, dt, s4);
         }
     }
+    if constexpr (sizeof(typename VTr<VT>::R) == 8)
+        if (!fp64_rows_pay(B, std::is_same_v<VT, double2>)) return QS3_OK;
     if constexpr (ND <= 4) {
         const uint64_t blocks = (B.total + NTHREADS - 1) / NTHREADS;
         *done = true;

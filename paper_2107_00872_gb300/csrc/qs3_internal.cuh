@@ -176,6 +176,8 @@ struct SecView {
 };
 
 // ---------------------------------------------------------- host basis
+constexpr int SEG_REACH = 24;
+
 struct Basis {
     int N = 0, nd = 0, nb = 0;
     int L[3] = {0, 0, 0};
@@ -194,6 +196,7 @@ struct Basis {
     std::vector<double> jxy, jz, h, pos;
     std::vector<uint64_t> binom;            // host copy of the binomial rows 0 .. nd + 2
     bool has_h = false;
+    int n_long_bonds = 0;                   // bonds of more than N / SEG_REACH sites' distance in the numbering
     // device data
     DevBuf d_tab;                           // the tables that lv points to, tile0, chunk0 and K
     const int *tile0_d = nullptr, *chunk0_d = nullptr, *K_d = nullptr;
