@@ -56,13 +56,11 @@ struct ObsSmem {
     double *snorm;   // [0..8] sqrt(s), [9..17] 1/sqrt(s)
 };
 
-__host__ __device__ inline size_t obs_smem_bytes(int nd_rows, int N, const int *L, bool hist) {
+__host__ __device__ inline size_t obs_smem_bytes(int nd_rows, int N, const int *L) {
     size_t s = (size_t)nd_rows * (N + 1) * 8 + (size_t)N * 4;
     s = (s + 15) & ~(size_t)15;
     s += 2 * (size_t)(L[0] + L[1] + L[2]) * 16 + 18 * 8;
-    s = (s + 15) & ~(size_t)15;
-    if (hist) s += (size_t)N * 16;
-    return s;
+    return (s + 15) & ~(size_t)15;
 }
 
 __device__ __forceinline__ ObsSmem obs_carve(const LatView &L, unsigned char *smem) {
@@ -205,6 +203,9 @@ __global__ void __launch_bounds__(NTHREADS) k_spsm_u1(LatView L, uint64_t dim, c
 // (7.0 ms of it the kernel).  d = 0 gives C = N_down |phi|^2.
 constexpr int CD = 8;
 constexpr int CORR_SMEM = 226 * 1024;      // the threads' sums (48 KB) beside the row tables
+static size_t corr_smem_bytes(const Basis &B) {
+    return 3 * CD * NTHREADS * 8 + (size_t)(B.nd + 3) * (B.N + 1) * 8 + (size_t)B.N * 4;
+}
 
 template <int ND, bool TB>
 __global__ void __launch_bounds__(NTHREADS) k_corr_k(LatView L, SecView sv, const double2 *__restrict__ phi, int do_pm,
@@ -770,7 +771,7 @@ static int corr_u1_nd(Basis &B, const double *phi, bool pm, double *G, double *M
 template <int ND>
 static int corr_k_nd(Basis &B, int s, const double2 *phi, bool pm, const int *dl, int ndl, int nb, double *part,
                      cudaStream_t st) {
-    const size_t smem = 3 * CD * NTHREADS * 8 + (size_t)(B.nd + 3) * (B.N + 1) * 8 + (size_t)B.N * 4;
+    const size_t smem = corr_smem_bytes(B);
     const dim3 grid(nb, (ndl + CD - 1) / CD);
     if (B.lv.orb) {
         QS3_CUDA(cudaFuncSetAttribute(k_corr_k<ND, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, CORR_SMEM));
@@ -805,7 +806,7 @@ static int smq_nd(Basis &S, int ss, Basis &Dd, int sd, const double2 *phs, const
     if constexpr (ND < 2) {
         return set_err(QS3_ERR_INVALID_ARG, "internal: smq_nd<%d>", ND);
     } else {
-        const size_t smem = obs_smem_bytes(S.nd + 3, S.N, S.L, false);
+        const size_t smem = obs_smem_bytes(S.nd + 3, S.N, S.L);
         if (smem > 200 * 1024) return set_err(QS3_ERR_OVERFLOW, "S^-_q tables need %zu bytes of shared memory", smem);
         const double isn = 1.0 / std::sqrt((double)S.N);
         if (S.has_k) {
@@ -918,7 +919,7 @@ int smq_launch(Basis &S, int ss, const void *phi, Basis &Dd, int sd, const int *
 template <int ND>
 static int szq_nd(Basis &S, int ss, Basis &Dd, int sd, const double2 *phs, double2 half_sum, const double2 *phi,
                   double2 *psi, cudaStream_t st) {
-    const size_t smem = obs_smem_bytes(S.nd + 3, S.N, S.L, false);
+    const size_t smem = obs_smem_bytes(S.nd + 3, S.N, S.L);
     if (smem > 200 * 1024) return set_err(QS3_ERR_OVERFLOW, "S^z_q tables need %zu bytes of shared memory", smem);
     const double isn = 1.0 / std::sqrt((double)S.N);
     if (S.has_k) {
@@ -937,7 +938,7 @@ static int szq_nd(Basis &S, int ss, Basis &Dd, int sd, const double2 *phs, doubl
 template <int ND>
 static int spq_nd(Basis &S, int ss, Basis &Dd, int sd, const double2 *phs, const double2 *phi, double2 *psi,
                   cudaStream_t st) {
-    const size_t smem = obs_smem_bytes(S.nd + 3, S.N, S.L, false);
+    const size_t smem = obs_smem_bytes(S.nd + 3, S.N, S.L);
     if (smem > 200 * 1024) return set_err(QS3_ERR_OVERFLOW, "S^+_q tables need %zu bytes of shared memory", smem);
     const double isn = 1.0 / std::sqrt((double)S.N);
     if (S.has_k) {
@@ -1063,9 +1064,8 @@ static int correlations(Basis &B, int s, const void *gs, int npairs, const int *
             return set_err(QS3_ERR_INVALID_ARG, "pair %d outside the lattice", p);
     if (B.dims[s] == 0) return set_err(QS3_ERR_INVALID_ARG, "sector %d is empty", s);
     const bool ks = B.has_k;
-    if (ks && nd > 0 && obs_smem_bytes(nd + 3, N, B.L, true) > 200 * 1024)
-        return set_err(QS3_ERR_OVERFLOW, "correlation tables need %zu bytes of shared memory",
-                       obs_smem_bytes(nd + 3, N, B.L, true));
+    if (ks && nd > 0 && corr_smem_bytes(B) > (size_t)CORR_SMEM)
+        return set_err(QS3_ERR_OVERFLOW, "correlation tables need %zu bytes of shared memory", corr_smem_bytes(B));
     // one displacement of every pair d, -d
     std::vector<int> dl;
     if (ks)
