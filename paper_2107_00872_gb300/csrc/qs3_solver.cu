@@ -1749,9 +1749,13 @@ static int residuals(Basis &B, const WT *v, const std::vector<double> &e, cudaSt
 // pivot, (a_k - x) - b_{k-1}^2 p_{k-1} / p_k - b_k^2 q_{k+2} / q_{k+1}, taken
 // times p_k q_{k+1}.  No division: a value and its predecessor are rescaled
 // together by a power of two when they leave [2^-lim, 2^lim], which keeps every
-// ratio exact.  bb[i] = b_{i-1}^2.  mild (|a - x| and b within [2^-41, 2^41]):
-// the test runs every fourth step only, at 2^400, which four steps take to
-// 2^724 at most.
+// ratio exact.  bb[i] = b_{i-1}^2.  mild (|a - x| <= 2 w, 2^-40 <= b <= w < 2^40
+// with w the Gershgorin width): the test runs every fourth step only, at 2^400.
+// Four steps multiply the larger of a value and its predecessor by less than
+// 2^205, and a minor that stays positive falls by b^2 / (4 w) >= 2^-122 a step at
+// most, the last one by the 2^-106 of a cancelled difference more: the values
+// stay within 2^605 and 2^-994, and none overflows or vanishes between two tests.
+// Elsewhere every step is tested; a minor that vanishes counts as not positive.
 struct Minor {
     double pm = 0.0, p = 1.0;
     bool neg = false;
@@ -1806,8 +1810,9 @@ __device__ int sturm_below_dev(int n, const double *__restrict__ a, const double
 __device__ double tri_lowest_warp(int n, const double *__restrict__ a, const double *__restrict__ b,
                                   const double *__restrict__ bb, double e_prev) {
     const int lane = threadIdx.x & 31;
-    double lo = 1e300, hi = -1e300;
+    double lo = 1e300, hi = -1e300, bmin = 1e300;
     for (int i = lane; i < n; i += 32) {
+        if (i) bmin = fmin(bmin, fabs(b[i - 1]));
         const double r = (i ? fabs(b[i - 1]) : 0.0) + (i < n - 1 ? fabs(b[i]) : 0.0);
         lo = fmin(lo, a[i] - r);
         hi = fmax(hi, a[i] + r);
@@ -1816,9 +1821,10 @@ __device__ double tri_lowest_warp(int n, const double *__restrict__ a, const dou
     for (int o = 16; o; o >>= 1) {
         lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
         hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        bmin = fmin(bmin, __shfl_xor_sync(0xffffffffu, bmin, o));
     }
     const double w = fmax(hi - lo, 1e-300);
-    const bool mild = w < 0x1p40 && w > 0x1p-40;      // |a - x| <= 2 w, b <= w
+    const bool mild = w < 0x1p40 && bmin >= 0x1p-40;
     lo -= 1e-3 * w;
     hi += 1e-3 * w;
     if (isfinite(e_prev) && e_prev > lo && e_prev < hi) {
