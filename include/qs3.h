@@ -138,8 +138,9 @@ int qs3_basis_nnz(qs3_basis_t b, uint64_t *nnz);
  *   mode = 1: build it (any size that fits); OVERFLOW when C(N, N_down) >= 2^32
  *             or there are 2^20 orbits or more, OOM when it does not fit,
  *             STATE on a U(1)-only basis or N_down = 0;
- *   mode = 0: release it (H Phi, S^-_q, S^+_q and the correlations then run
- *             the search);
+ *   mode = 0: release it, or the origin forms (H Phi, S^-_q, S^+_q and the
+ *             correlations then run the search; not while a product of the
+ *             basis is being issued by another thread);
  *   mode = -1: query only.
  * *active (may be NULL) receives 1 if the table is in use afterwards.  The
  * table occupies C(N, N_down) * 4 + n_sectors * n_orbits * 4 bytes of device

@@ -828,6 +828,18 @@ void drop_rep_table(Basis &B) {
     if (!B.secs.empty()) B.d_secs.upload(B.secs.data(), B.secs.size() * sizeof(SecView));
 }
 
+// the origin forms (qs3_hphi_search.cu); drop_rep_table then puts the views
+static void drop_forms(Basis &B) {
+    for (auto &v : B.secs) {
+        v.orec = nullptr;
+        v.finfo = nullptr;
+        v.fsub = nullptr;
+    }
+    B.d_orec.release();
+    B.d_finfo.release();
+    B.d_fsub.release();
+}
+
 // per-sector phase tables ph[s N + r] = exp(-2 pi i sum_alpha K_alpha r_alpha / L_alpha):
 // the phase e^{ik.t} of the translation t = -(r_x, r_y, r_z) that moves site r
 // to the origin; the angle is reduced exactly in integers
@@ -1304,6 +1316,7 @@ int qs3_basis_rep_table(qs3_basis_t b, int32_t mode, int32_t *active) {
     if (mode < -1 || mode > 1) return set_err(QS3_ERR_INVALID_ARG, "mode %d", mode);
     int st = QS3_OK;
     if (mode == 0) {
+        drop_forms(b->B);
         drop_rep_table(b->B);
     } else if (mode == 1) {
         size_t fr = 0, tt = 0;

@@ -71,3 +71,19 @@ def test_creation_allocates_little(nk):
     free = torch.cuda.mem_get_info()[0]
     assert create() <= 24
     assert abs(torch.cuda.mem_get_info()[0] - free) <= 4 << 20
+
+
+# a basis without the table holds the origin forms of its rows, about 20 bytes
+# each, and gives them back with mode 0; the search finds the same bits
+def test_origin_forms_are_given_back():
+    torch = torch_cuda()
+    b = lib_basis(qi.hypercubic((13, 5), True, 1.0, 0.9), 6, [(6, 2, 0)])
+    assert not b.rep_table()
+    phi = _randn(torch, b.total_dim, 5)
+    ref = [b.hphi(x) for x in (phi, phi.to(torch.complex128))]
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    assert not b.rep_table(0)
+    assert torch.cuda.mem_get_info()[0] - free >= 16 * b.total_dim
+    for x, r in zip((phi, phi.to(torch.complex128)), ref):
+        assert torch.equal(b.hphi(x), r)
