@@ -444,11 +444,11 @@ static int build_forms_nd(Basis &B) {
         k_form_first<KT><<<gp, 256>>>(key.as<KT>(), d, bits, NO, np, first.as<uint32_t>());
         QS3_LAUNCHED();
         QS3_CUDA(cudaMemsetAsync(size.as<uint32_t>() + np, 0, 4));
-        k_bucket_size<<<gp, 256>>>(NO, B.N + 1, 0, bin, 1, np, 0, first.as<uint32_t>(), size.as<uint32_t>());
+        k_bucket_size<false><<<gp, 256>>>(NO, B.N + 1, 0, bin, 1, np, 0, first.as<uint32_t>(), size.as<uint32_t>());
         QS3_LAUNCHED();
         size_t t2 = tb;
         QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, t2, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)np + 1));
-        k_bucket_info<<<gp, 256>>>(NO, B.N + 1, 0, bin, 1, np, 0, first.as<uint32_t>(), off.as<uint32_t>(), is, ss);
+        k_bucket_info<false><<<gp, 256>>>(NO, B.N + 1, 0, bin, 1, np, 0, first.as<uint32_t>(), off.as<uint32_t>(), is, ss);
         QS3_LAUNCHED();
         if (d > 0) {
             k_form_fill<NO, KT><<<g, NTHREADS, smem>>>(B.lv, key.as<KT>(), d, first.as<uint32_t>(), is, ss);

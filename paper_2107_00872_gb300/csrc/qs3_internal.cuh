@@ -148,6 +148,8 @@ struct LatView {
     const double *adj_jz_pad64;
 };
 
+constexpr uint32_t ONE_BUCKET = 0x80u;    // beyond every shift
+
 struct SecView {
     const uint64_t *sigma;        // sorted rank0 of the representatives (NULL: U(1))
     const uint8_t *stab;          // |Stab| of each representative
@@ -155,7 +157,8 @@ struct SecView {
     // sites (pre2; else the largest one), prefix P, are split by the rank of
     // their other sites into buckets of a few rows: pinfo[P] = (first entry o,
     // shift), rows of bucket q = low rank >> shift are sub[o + q] .. sub[o + q
-    // + 1] - 1
+    // + 1] - 1; a prefix of one bucket (up to three rows) has no entries but
+    // pinfo[P] = (first row, ONE_BUCKET | rows << 8), one dependent load less
     const uint2 *pinfo;
     const uint32_t *sub;
     int pre2;
@@ -760,6 +763,11 @@ __device__ __forceinline__ bool sigma_find(const SecView &sv, const int (&c)[ND]
                                            int np1, uint64_t r, uint32_t &idx) {
     uint64_t low;
     const uint2 pi = __ldg(sv.pinfo + prefix_of(c, sC, np1, sv.pre2, low));
+    if (pi.y & ONE_BUCKET) {
+        for (idx = pi.x; idx < pi.x + (pi.y >> 8); ++idx)
+            if (__ldg(sv.sigma + idx) == r) return true;
+        return false;
+    }
     const uint32_t *e = sv.sub + pi.x + (uint32_t)(low >> pi.y);
     return bucket_find(sv.sigma, __ldg(e), __ldg(e + 1), r, idx);
 }
@@ -772,7 +780,9 @@ __device__ __forceinline__ void stage_tables(const LatView &L, uint64_t *sC, uin
         for (int i = threadIdx.x; i < L.N; i += blockDim.x) sxyz[i] = L.xyz[i];
 }
 
-// entries of every (sector, prefix): its buckets plus the end
+// entries of every (sector, prefix): its buckets plus the end (ONE: none for one
+// bucket, whose rows are in its pinfo)
+template <bool ONE>
 static __global__ void k_bucket_size(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
                               int half, const uint32_t *__restrict__ first, uint32_t *__restrict__ size) {
     const uint64_t cnt = (uint64_t)S * np;
@@ -782,9 +792,10 @@ static __global__ void k_bucket_size(int nd, int np1, int pre2, const uint64_t *
         const uint32_t *f = first + s * (np + 1) + P;
         uint32_t nq;
         bucket_shift(P, (f[1] - f[0]) >> half, nd, pre2, binom, np1, nq);
-        size[i] = nq + 1;
+        size[i] = ONE && nq == 1 ? 0 : nq + 1;
     }
 }
+template <bool ONE>
 static __global__ void k_bucket_info(int nd, int np1, int pre2, const uint64_t *__restrict__ binom, int S, uint32_t np,
                               int half, const uint32_t *__restrict__ first, const uint32_t *__restrict__ off,
                               uint2 *__restrict__ pinfo, uint32_t *__restrict__ sub) {
@@ -795,6 +806,10 @@ static __global__ void k_bucket_info(int nd, int np1, int pre2, const uint64_t *
         const uint32_t *f = first + s * (np + 1) + P;
         uint32_t nq;
         const int sh = bucket_shift(P, (f[1] - f[0]) >> half, nd, pre2, binom, np1, nq);
+        if (ONE && nq == 1) {
+            pinfo[i] = make_uint2(f[0], ONE_BUCKET | (f[1] - f[0]) << 8);
+            continue;
+        }
         pinfo[i] = make_uint2(off[i], (uint32_t)sh);
         // an empty prefix: one empty bucket
         if (f[0] == f[1])
