@@ -886,30 +886,46 @@ static int hphio_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
 // one hop amplitude, of one sector too (c128 k_hphi / k_hphi_of: 10x10, N_down =
 // 4 31 / 27 us a call, 12x12 53 / 37, 10x10x10, N_down = 3 71 / 54; c64 21 / 18, 23
 // / 21, 44 / 38), as far as its hop lists leave room: k_hphi lists nothing and
-// keeps its blocks and its L1 cache.  With three or four blocks resident that
-// leave the L1 60 KB (complex64: 80 KB) it is the faster one everywhere.  Fewer
-// blocks, or less L1, cost more than the sharing of few sectors gives, so the
-// rows must fill the chip (one block on every SM) as many times as `waves` says.
-// Square lattices of degree 8 to 48, k_hphi / k_hphi_of in us, c128 and c64:
-//   four blocks, little L1: 10x10, N_down = 3, 14 bonds a site, one sector 41 / 41
-//     and 27 / 31, 100 sectors 137 / 102 and 49 / 45; 14x14, 196 sectors 863 / 412
-//     and 246 / 147
-//   three blocks, 60 KB: 12x12, N_down = 4, 12 bonds, 1 sector 128 / 104 and 47 /
-//     68, 4 392 / 242 and 156 / 129
+// keeps its blocks and its L1 cache, unless its 64-bit tables are large too.  With
+// three or four blocks resident that leave the L1 60 KB (complex64: 80 KB) the
+// orbits are faster everywhere, but for complex64 with one sector to share a list
+// over more than one wave.  Fewer blocks, or less L1, cost more than the sharing
+// of few sectors gives, so the rows must fill the chip (one block on every SM) as
+// many times as `waves` says, and the sectors be `share` at least.  Square
+// lattices of degree 8 to 48, k_hphi / k_hphi_of in us, c128 and c64:
+//   tables of 109 KB: 40x40, N_down = 3, 28 bonds a site (one block), one sector
+//     1325 / 940 and 1185 / 753
+//   four blocks, little L1: 10x10, N_down = 3, 14 bonds, one sector 41 / 41 and 27
+//     / 31, 100 sectors 137 / 102 and 49 / 45; 14x14, 196 sectors 863 / 412 and 246
+//     / 147
+//   three or four blocks: 16x16, N_down = 4, one sector, 4 bonds 201 / 131 and 74 /
+//     80, 12 bonds 547 / 379 and 203 / 253, two sectors 1086 / 580 and 371 / 337
 //   two blocks: 10x10, N_down = 4, 20 bonds, 2 sectors 160 / 150 and 68 / 109, 16
 //     832 / 565 and 309 / 293; 14x14, N_down = 3, 28 bonds, 4 sectors 76 / 90 and
-//     51 / 65, 196 1671 / 1059 and 484 / 424
+//     51 / 65, 196 1671 / 1059 and 484 / 424; 16x16, N_down = 4, 16 bonds, 2 sectors
+//     1439 / 920 and 500 / 533, 4 2785 / 1545 and 950 / 767
 //   one block: 10x10, N_down = 4, 36 bonds, 4 sectors 437 / 509 and 210 / 297, 8
-//     815 / 755 and 327 / 483, 100 8901 / 6480 and 2966 / 3111
+//     815 / 755 and 327 / 483, 100 8901 / 6480 and 2966 / 3111; 16x16, 24 bonds, one
+//     sector 1070 / 1361 in c128
+constexpr size_t HEAVY_TABLES = 64 * 1024;
 static bool hphi_of_ok(const Basis &B, bool fp32) {
     if (!(B.has_k && B.lv.orb && B.d_oreps.p && B.lv.jh_uniform != 0.0) || !orb_smem(B)) return false;
+    if (B.smem_bytes > HEAVY_TABLES) return true;
     const auto [blocks, used] = orb_room(B);
     uint64_t waves;
-    if (blocks >= 3) waves = fp32 ? (used > 196 ? 16 : used > 176 ? 4 : 0) : (used > 196 ? 1 : 0);
-    else if (blocks == 2) waves = fp32 ? (used > 196 ? 24 : 16) : (used > 196 ? 4 : 0);
-    else if (!fp32) waves = 8;
-    else return false;
-    return B.n_orb * (uint64_t)B.S >= waves * one_wave();
+    int share = 1;
+    if (blocks >= 3) {
+        waves = fp32 ? (used > 196 ? 16 : used > 176 ? 4 : 0) : (used > 196 ? 1 : 0);
+    } else if (blocks == 2) {
+        waves = fp32 ? (used > 196 ? 24 : 16) : (used > 196 ? 4 : 0);
+        share = fp32 ? 4 : 1;
+    } else {
+        if (fp32) return false;
+        waves = 8;
+        share = OSG;
+    }
+    if (fp32 && B.S == 1 && B.n_orb > blocks * one_wave()) return false;
+    return B.S >= share && B.n_orb * (uint64_t)B.S >= waves * one_wave();
 }
 
 template <int ND, typename VT>
