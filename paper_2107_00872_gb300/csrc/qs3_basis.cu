@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(NTHREADS) k_bucket_fill(LatView L, const SecVi
         const uint32_t P = prefix_of(c, sC, L.np1, secs[s].pre2, low);
         const uint32_t *f = first + (uint64_t)s * (np + 1) + P;
         const uint2 pi = pinfo[(uint64_t)s * np + P];
-        if (pi.y & ONE_BUCKET) continue;
+        if (ND <= 3 && (pi.y & ONE_BUCKET)) continue;
         uint32_t *e = sub + pi.x;
         const uint32_t q = (uint32_t)(low >> pi.y);
         uint32_t q0 = 0;
@@ -580,8 +580,8 @@ static int put_secs(Basis &B) {
 
 // the index over every sector's rows (SecView::pinfo, sub), as many sectors at
 // a time as INDEX_GROUP entries hold and at least one: the offsets in a group
-// are 32 bits (three entries per four rows at most), the groups' places in d_sub
-// 64; the scratch is three words per prefix of a group
+// are 32 bits (a sector of fewer than 2^32 rows has fewer than 3 2^30 + 2 np
+// entries), the groups' places in d_sub 64
 constexpr uint64_t INDEX_GROUP = (uint64_t)1 << 22;
 template <int ND>
 static int build_index_nd(Basis &B) {
@@ -592,8 +592,10 @@ static int build_index_nd(Basis &B) {
     const uint32_t np = pre2 ? (uint32_t)np2 : (uint32_t)B.N;
     for (auto &v : B.secs) v.pre2 = pre2;
     QS3_TRY(put_secs(B));
-    // a prefix of four rows or more has at most rows / 2 buckets and the end
-    auto entries = [&](int s) { return B.dims[s] / 4 * 3 + 4; };
+    // at most rows / 2 buckets and the end for a prefix of four rows or more, two
+    // entries for the others (ONE: none)
+    constexpr bool ONE = ND <= 3;
+    auto entries = [&](int s) { return B.dims[s] / 4 * 3 + 4 + (ONE ? 0 : 2 * (uint64_t)np); };
     std::vector<int> g0{0};
     uint64_t most = 0, in_group = 0, cnt_max = 0;
     for (int s = 0; s < S; ++s) {
@@ -629,11 +631,11 @@ static int build_index_nd(Basis &B) {
         k_first<<<g1, 256>>>(B.nd, B.N + 1, pre2, secs, ns, np, bin, first.as<uint32_t>());
         QS3_LAUNCHED();
         QS3_CUDA(cudaMemsetAsync(size.as<uint32_t>() + cnt, 0, 4));
-        k_bucket_size<true><<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, ns, np, 1, first.as<uint32_t>(), size.as<uint32_t>());
+        k_bucket_size<ONE><<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, ns, np, 1, first.as<uint32_t>(), size.as<uint32_t>());
         QS3_LAUNCHED();
         size_t t2 = tb;
         QS3_CUDA(cub::DeviceScan::ExclusiveSum(tmp.p, t2, size.as<uint32_t>(), off.as<uint32_t>(), (int64_t)(cnt + 1)));
-        k_bucket_info<true><<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, ns, np, 1, first.as<uint32_t>(), off.as<uint32_t>(), pinfo, sub);
+        k_bucket_info<ONE><<<g1, 256>>>(B.nd, B.N + 1, pre2, bin, ns, np, 1, first.as<uint32_t>(), off.as<uint32_t>(), pinfo, sub);
         QS3_LAUNCHED();
         const int t0 = B.tile0[s0], t1 = B.tile0[s0 + ns];
         if (t1 > t0) {

@@ -85,7 +85,7 @@ constexpr size_t POOL_KEEP_BYTES = (size_t)512 << 20, POOL_MAX_BYTES = (size_t)2
 // the current device's unused pool memory goes back, but for `keep` bytes.
 // A basis that is destroyed leaves POOL_IDLE_BYTES, the pool's smallest unit:
 // with none left, the next small basis mapped it again and its destruction
-// unmapped it, 0.1 ms of the 0.83 ms that one sector of 5x5 took.
+// unmapped it (one sector of 5x5: destruction 175 us, now 94).
 void pool_trim(size_t keep);
 constexpr size_t POOL_IDLE_BYTES = (size_t)32 << 20;
 
@@ -157,8 +157,9 @@ struct SecView {
     // sites (pre2; else the largest one), prefix P, are split by the rank of
     // their other sites into buckets of a few rows: pinfo[P] = (first entry o,
     // shift), rows of bucket q = low rank >> shift are sub[o + q] .. sub[o + q
-    // + 1] - 1; a prefix of one bucket (up to three rows) has no entries but
-    // pinfo[P] = (first row, ONE_BUCKET | rows << 8), one dependent load less
+    // + 1] - 1.  With N_down <= 3, where most prefixes have a row or two, a prefix
+    // of one bucket (up to three rows) has no entries but pinfo[P] = (first row,
+    // ONE_BUCKET | rows << 8), one dependent load less
     const uint2 *pinfo;
     const uint32_t *sub;
     int pre2;
@@ -763,13 +764,13 @@ __device__ __forceinline__ bool sigma_find(const SecView &sv, const int (&c)[ND]
                                            int np1, uint64_t r, uint32_t &idx) {
     uint64_t low;
     const uint2 pi = __ldg(sv.pinfo + prefix_of(c, sC, np1, sv.pre2, low));
-    if (pi.y & ONE_BUCKET) {
-        for (idx = pi.x; idx < pi.x + (pi.y >> 8); ++idx)
-            if (__ldg(sv.sigma + idx) == r) return true;
-        return false;
+    uint32_t lo = pi.x, hi = pi.x + (pi.y >> 8);
+    if (ND > 3 || !(pi.y & ONE_BUCKET)) {
+        const uint32_t *e = sv.sub + pi.x + (uint32_t)(low >> pi.y);
+        lo = __ldg(e);
+        hi = __ldg(e + 1);
     }
-    const uint32_t *e = sv.sub + pi.x + (uint32_t)(low >> pi.y);
-    return bucket_find(sv.sigma, __ldg(e), __ldg(e + 1), r, idx);
+    return bucket_find(sv.sigma, lo, hi, r, idx);
 }
 
 // stage the binomial table (rows 0..nd+2) and the coordinate table in smem

@@ -19,9 +19,9 @@ def _randn(torch, d, seed):
     return torch.view_as_complex(torch.randn(d, 2, generator=g, device="cuda", dtype=torch.float32))
 
 
-# 12x12, N_down = 4, all 144 momenta: up to 13 million entries, several groups; 9x5
-# and 6x4 stay within one (two-site and one-site prefixes)
-@pytest.mark.parametrize("dims,nd", [((12, 12), 4), ((9, 5), 4), ((6, 4), 2)])
+# 12x12, N_down = 4, all 144 momenta: about 11.6 million entries, several groups; 9x5
+# and 6x4 stay within one (two-site and one-site prefixes, lists and rows)
+@pytest.mark.parametrize("dims,nd", [((12, 12), 4), ((9, 5), 4), ((6, 4), 2), ((9, 5), 3), ((3, 2), 2), ((4, 2), 3)])
 def test_index_equals_table(dims, nd):
     torch = torch_cuda()
     spec = qi.hypercubic(dims, True, 1.0, 0.8)
