@@ -479,7 +479,7 @@ __device__ __forceinline__ int orbit_hops(const LatView &L, uint32_t rank, const
 // A table has fewer than 2^32 states, so ranks and binomials (rows 0 .. N_down)
 // are 32-bit words: 16 KB instead of 48 KB staged per block at N = 1000, and four
 // resident blocks instead of three (10x10x10, N_down = 3, 28 sectors: integer 674
-// -> 491 us, c128 720 -> 630, c64 406 -> 233, with the group rule's staging term).
+// -> 498 us, c128 720 -> 630, c64 406 -> 233, with the group rule's staging term).
 constexpr int OSG = 8;
 
 // the binary64 engine's product on the integer units: per term one row
@@ -829,7 +829,7 @@ static int hphix_nd(Basis &B, const HxVec &hv, double2 *psi, cudaStream_t st, co
 // 10x10, N_down = 4, 20 sectors, 1 / 2 / 4 per thread: c64 83 / 57 / 57 us,
 // c128 146 / 128 / 135, integer 146 / 114 / 120; all 100, 4 / 8 per thread: c64
 // 188 / 169, c128 507 / 519, integer 417 / 410; 10x10x10, N_down = 3 (16 loads a
-// thread), 28 sectors, 2 / 4 / 8: c64 347 / 268 / 233, integer 594 / 520 / 491.
+// thread), 28 sectors, 2 / 4 / 8: c64 347 / 268 / 233, integer 594 / 520 / 491 (one run).
 static int orb_group(const Basis &B, bool fp32) {
     const uint64_t wave = 4ull * NTHREADS * (uint64_t)num_sms();
     const int setup = (fp32 ? 2 : 1) + (B.nd + 1) * (B.N + 1) / (4 * NTHREADS);     // in half sectors

@@ -25,7 +25,9 @@
 // occupation masks; 13.2 with two-site prefixes, separate key and value lists
 // and the diagonal's fp64 additions per row); 8x8x8, N_down = 4, complex64:
 // 1.81 ms (3.45, 2.06).  About 480 instructions per warp and hop, half of the
-// issue slots; the loads' latency at 45 % occupancy is the rest.
+// issue slots; the loads' latency at 45 % occupancy is the rest.  At its bound of 64
+// registers the complex128 kernel spills (N_down = 5: 184 bytes stored and 260
+// loaded a thread, N_down = 4 116 / 136), the complex64 one from N_down = 6 on.
 #include <cub/cub.cuh>
 
 #include <algorithm>
