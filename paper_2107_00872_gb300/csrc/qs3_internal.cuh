@@ -676,7 +676,7 @@ __device__ __forceinline__ void unpack_key(uint64_t key, int kb, int (&rep)[ND])
 
 // the representative of the site list t, by whichever search applies: two spins
 // have nothing to gain from the masks (31x32, S^+_q from N_down = 2 without the
-// table 1401 us by canon_gen, 1620 by masks)
+// table 1483 us by canon_gen, 1620 by masks)
 template <int ND>
 __device__ __forceinline__ uint64_t canon(const int (&t)[ND], const LatView &L, const uint32_t *__restrict__ sxyz,
                                           const uint64_t *__restrict__ sC, int (&rep)[ND], int &ax, int &by,
